@@ -83,10 +83,27 @@ int apply_launch(hub_ctx *h, const double *x, double *y, cudaStream_t s) {
   return prof_mark(h, HUB_PROF_APPLY, false, s);
 }
 
+// Products of few terms go to the FP64 kernel: one launch.  Its 1.2e7 terms on the 12-site ring (6,6)
+// take 44 us against 69 us for the fixed-point path, whose launches alone take 45 us; beyond
+// about 2.2e7 terms (80 us) the FP64 unit costs more than the launches.
+constexpr double kF64Terms = 2.2e7;
+static bool f64_is_faster(const hub_ctx *h) {
+  const double nu = (double)h->count[0], nd = (double)h->count[1];
+  const double terms = (double)h->csr[0].nnz * nd + (double)h->csr[h->shared ? 0 : 1].nnz * nu + nu * nd;
+  return !h->k0 && !h->fail_waits && terms <= kF64Terms;   // the test hook needs kernels that wait
+}
+
 static int apply_kernels(hub_ctx *h, const double *x, double *y, cudaStream_t s) {
   const Ham H = h->view();
   if (H.n_up == 0 || H.n_dn == 0) return HUB_OK;
   if (h->k0) return k0_apply(h, x, y, s);
+  if (f64_is_faster(h)) return f64_apply(h, x, y, nullptr, s);
+  if (fix_apply_eligible(h)) {
+    const int rc = fix_apply(h, x, y, s);
+    if (rc != HUB_ERR_OOM) return rc;
+    h->fix_off = true;                // its vectors do not fit: the paths that need fewer
+    set_error("");
+  }
   if (use_fast(h)) return fast_apply_f64(h, x, y, s);
   return f64_apply(h, x, y, nullptr, s);
 }
@@ -152,7 +169,7 @@ extern "C" int hub_apply_host(hub_t h, const double *x_host, double *y_host, voi
   const int64_t D = vec_len(h);
   if ((rc = host_apply_buffers(h, &h->hx, &h->hy))) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  if (use_fast(h)) return fast_apply_host(h, x_host, y_host, h->hx, h->hy, s);
+  if (use_fast(h) && fast_host_pipelined(h)) return fast_apply_host(h, x_host, y_host, h->hx, h->hy, s);
   HUB_CUDA(cudaMemcpyAsync(h->hx, x_host, sizeof(double) * D, cudaMemcpyHostToDevice, s));
   rc = apply_launch(h, h->hx, h->hy, s);
   if (rc) return rc;

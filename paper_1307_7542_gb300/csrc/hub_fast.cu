@@ -114,6 +114,7 @@ struct FastView {
   int t_neg;                         // the kernels apply H / |t|: hopping sign(t), diagonal U k / |t|
   float2 Utab[32];                   // (U / |t|) k for k = popcount(I_up & I_dn)
   int *err;                          // device error flag (bounded waits)
+  const int *gate;                   // null, or a device flag: the kernels do nothing while it is 0
   int fail_waits;                    // test hook: take the given-up-wait exit once the copies landed
 };
 
@@ -161,7 +162,6 @@ __global__ void k_to_slots(int64_t n, const int32_t *__restrict__ slot_row, cons
 // the largest biased FP64 exponent in [kExpLo, kExpHi] and every nonzero entry's exponent
 // at most kExpSpan below it; FP64 subnormals, infinities and NaN are outside.  A vector
 // outside the window is multiplied by the FP64 kernel instead.
-constexpr int kExpSpan = 80, kExpLo = 200, kExpHi = 1900;
 
 // partials[block] = largest biased FP64 exponent of the block's elements (2047 for inf or
 // NaN), partials[nblk + block] = smallest biased exponent among its nonzero elements (0 for
@@ -263,7 +263,8 @@ __global__ void k_scale_all(const int *__restrict__ partials, int nblk, int n_se
 // scale[0] (0 when scale is null); one row per block and step
 __global__ void k_f64_to_df(int64_t r0, int64_t r1, int64_t n_up, int64_t ld, const double *__restrict__ x,
                             const int *__restrict__ scale, const int32_t *__restrict__ slot_row,
-                            float *__restrict__ out) {
+                            float *__restrict__ out, const int *__restrict__ gate) {
+  if (gate && gate[0] == 0) return;
   const int shift = scale ? scale[0] : 0;
   for (int64_t d = r0 + blockIdx.x; d < r1; d += gridDim.x) {
     float *__restrict__ row = out + d * 2 * ld;
@@ -282,8 +283,8 @@ __global__ void k_f64_to_df(int64_t r0, int64_t r1, int64_t n_up, int64_t ld, co
 // kernel writes y instead).  tabs = |t|: the kernels applied H / |t|.
 __global__ void k_unpermute(int64_t r0, int64_t r1, int64_t n_up, int64_t ld, const float *__restrict__ v,
                             const int32_t *__restrict__ slot_of, const int *__restrict__ scale, double tabs,
-                            double *__restrict__ y) {
-  if (scale[1]) return;
+                            double *__restrict__ y, const int *__restrict__ gate) {
+  if (scale[1] || (gate && gate[0] == 0)) return;
   const int shift = scale[0];
   for (int64_t d = r0 + blockIdx.x; d < r1; d += gridDim.x) {
     const float *__restrict__ row = v + d * 2 * ld;
@@ -312,22 +313,6 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
 // and serve as the column of idle schedule steps (adding zero is exact).
 constexpr int kUpPlane = 14080;
 
-// FP64 value of lane a + lane b of a packed (hi, lo) pair
-__device__ __forceinline__ double df2_lanes_to_f64(f2x h, f2x l) {
-  const float2 hh = upk2(h), ll = upk2(l);
-  return df_to_f64(make_float2(hh.x, ll.x), 0) + df_to_f64(make_float2(hh.y, ll.y), 0);
-}
-
-// The Lanczos recurrence fused into pass 1 (kUpd): the staged rows are those of w (the
-// previous step's pass-2 output); before the gathers each CTA forms r_j = w + c r_{j-1}
-// (c = -alpha_{j-1} / |r_{j-1}|, the update of Sec. IV's recurrence) in shared memory, writes
-// it back over w in HBM for pass 2 and the next steps, and accumulates |r_j|^2.
-#ifndef HUB_UPD_Q
-#define HUB_UPD_Q 1   // column quads per thread whose loads the fused update issues together
-#endif
-#ifndef HUB_FUSED_UPDATE
-#define HUB_FUSED_UPDATE 1   // 0: the Lanczos update as a separate vector pass before pass 1
-#endif
 #ifndef HUB_UP_PAIRED
 #define HUB_UP_PAIRED 1   // 1: pass 1 sums with DfSumP (low parts of a word's two entries paired); 0: DfSum4
 #endif
@@ -336,21 +321,10 @@ __device__ __forceinline__ double df2_lanes_to_f64(f2x h, f2x l) {
 #endif
 constexpr int kUpThreads = HUB_UP_THREADS;
 static_assert(kUpThreads % 32 == 0 && kUpThreads >= 512 && kUpThreads <= 1024, "pass-1 CTA size");
-constexpr int kUpdQ = HUB_UPD_Q;
-// Lanczos steps per host read-back for sectors of at most kBatchStepsMaxDim states
-constexpr int kMaxBatchSteps = 8;
-constexpr int64_t kBatchStepsMaxDim = 1 << 21;
-constexpr bool kFusedUpdate = HUB_FUSED_UPDATE != 0;
-
-struct UpdArgs {
-  const float *r_prev;               // r_{j-1} (planar rows)
-  const float2 *coef;                // coef[2] = c (double-float)
-  double *partials;                  // |r_j|^2 per CTA
-};
-
-template <typename Col, bool kUpd>
-__global__ void __launch_bounds__(kUpThreads, 1) k_up(const FastView F, float *x, float *__restrict__ z,
-                                                int64_t p_begin, int64_t p_end, UpdArgs U) {
+template <typename Col>
+__global__ void __launch_bounds__(kUpThreads, 1) k_up(const FastView F, const float *__restrict__ x,
+                                                      float *__restrict__ z, int64_t p_begin, int64_t p_end) {
+  if (F.gate && F.gate[0] == 0) return;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float *xs = reinterpret_cast<float *>(smem_raw);
   __shared__ __align__(8) uint64_t bar;
@@ -360,8 +334,6 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const FastView F, float *x
   const uint32_t pbytes = (uint32_t)(ld * sizeof(float));
   if (tid < 32) utab[tid] = F.Utab[tid];
   if (tid < 8) xs[(tid >> 1) * kUpPlane + ld + (tid & 1)] = 0.f;
-  __shared__ double wnorm[32];              // |r_j|^2 per warp, summed in a fixed order (kUpd)
-  if (kUpd && tid < 32) wnorm[tid] = 0.0;
   if (tid == 0) {
     mbar_init(&bar, 1);
     fence_mbar_init();
@@ -382,10 +354,6 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const FastView F, float *x
       if (pn < p_end) {
         prefetch_l2(x + 2 * pn * 2 * ld, 2 * pbytes);
         if (2 * pn + 1 < F.n_dn) prefetch_l2(x + (2 * pn + 1) * 2 * ld, 2 * pbytes);
-        if (kUpd) {
-          prefetch_l2(U.r_prev + 2 * pn * 2 * ld, 2 * pbytes);
-          if (2 * pn + 1 < F.n_dn) prefetch_l2(U.r_prev + (2 * pn + 1) * 2 * ld, 2 * pbytes);
-        }
       }
     }
     if (!mbar_wait_bounded(&bar, phase)) {
@@ -398,85 +366,6 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const FastView F, float *x
       return;
     }
     phase ^= 1u;
-    if (kUpd) {
-      // r_j = w + c r_{j-1} for both rows, four columns per thread step: in shared memory,
-      // in HBM over w, and into |r_j|^2 (lane b counted only when the rows differ)
-      const float *pr0 = U.r_prev + d0 * 2 * ld, *pr1 = U.r_prev + d1 * 2 * ld;
-      float *x0 = x + d0 * 2 * ld, *x1 = x + d1 * 2 * ld;
-      const float2 cf = U.coef[2];
-      const f2x cph = bcast2(cf.x), cpl = bcast2(cf.y);
-      DfAcc2 nacc{0ull, 0ull};
-      // kUpdQ quads per thread and batch, their global loads issued before any arithmetic
-      const int64_t stride = 4 * (int64_t)blockDim.x;
-      for (int64_t q0 = 4 * (int64_t)tid; q0 < ld; q0 += kUpdQ * stride) {
-        float4 ph0[kUpdQ], pl0[kUpdQ], ph1[kUpdQ], pl1[kUpdQ];
-#pragma unroll
-        for (int i = 0; i < kUpdQ; ++i) {
-          const int64_t q = q0 + i * stride;
-          if (q < ld) {
-            ph0[i] = *reinterpret_cast<const float4 *>(pr0 + q);
-            pl0[i] = *reinterpret_cast<const float4 *>(pr0 + ld + q);
-            ph1[i] = *reinterpret_cast<const float4 *>(pr1 + q);
-            pl1[i] = *reinterpret_cast<const float4 *>(pr1 + ld + q);
-          }
-        }
-#pragma unroll
-        for (int i = 0; i < kUpdQ; ++i) {
-          const int64_t q = q0 + i * stride;
-          if (q >= ld) break;
-          float4 *s0 = reinterpret_cast<float4 *>(xs + q), *s1 = reinterpret_cast<float4 *>(xs + kUpPlane + q);
-          float4 *s2 = reinterpret_cast<float4 *>(xs + 2 * kUpPlane + q);
-          float4 *s3 = reinterpret_cast<float4 *>(xs + 3 * kUpPlane + q);
-          const float4 wh0 = *s0, wl0 = *s1, wh1 = *s2, wl1 = *s3;
-          const float a_wh0[4] = {wh0.x, wh0.y, wh0.z, wh0.w}, a_wl0[4] = {wl0.x, wl0.y, wl0.z, wl0.w};
-          const float a_wh1[4] = {wh1.x, wh1.y, wh1.z, wh1.w}, a_wl1[4] = {wl1.x, wl1.y, wl1.z, wl1.w};
-          const float a_ph0[4] = {ph0[i].x, ph0[i].y, ph0[i].z, ph0[i].w};
-          const float a_pl0[4] = {pl0[i].x, pl0[i].y, pl0[i].z, pl0[i].w};
-          const float a_ph1[4] = {ph1[i].x, ph1[i].y, ph1[i].z, ph1[i].w};
-          const float a_pl1[4] = {pl1[i].x, pl1[i].y, pl1[i].z, pl1[i].w};
-          float rh0[4], rl0[4], rh1[4], rl1[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            f2x mh, ml, rh, rl, sh, sl;
-            df2_mul(cph, cpl, pk2(a_ph0[k], a_ph1[k]), pk2(a_pl0[k], a_pl1[k]), mh, ml);
-            df2_add(mh, ml, pk2(a_wh0[k], a_wh1[k]), pk2(a_wl0[k], a_wl1[k]), rh, rl);
-            df2_mul(rh, rl, rh, rl, sh, sl);
-            if (d1 == d0) {
-              sh &= 0xffffffffull;
-              sl &= 0xffffffffull;
-            }
-            acc2_add(nacc, sh, sl);
-            const float2 h2 = upk2(rh), l2 = upk2(rl);
-            rh0[k] = h2.x;
-            rh1[k] = h2.y;
-            rl0[k] = l2.x;
-            rl1[k] = l2.y;
-          }
-          const float4 oh0 = make_float4(rh0[0], rh0[1], rh0[2], rh0[3]);
-          const float4 ol0 = make_float4(rl0[0], rl0[1], rl0[2], rl0[3]);
-          const float4 oh1 = make_float4(rh1[0], rh1[1], rh1[2], rh1[3]);
-          const float4 ol1 = make_float4(rl1[0], rl1[1], rl1[2], rl1[3]);
-          *s0 = oh0;
-          *s1 = ol0;
-          *s2 = oh1;
-          *s3 = ol1;
-          *reinterpret_cast<float4 *>(x0 + q) = oh0;
-          *reinterpret_cast<float4 *>(x0 + ld + q) = ol0;
-          if (d1 != d0) {
-            *reinterpret_cast<float4 *>(x1 + q) = oh1;
-            *reinterpret_cast<float4 *>(x1 + ld + q) = ol1;
-          }
-        }
-      }
-      {
-        f2x h, l;
-        acc2_norm(nacc, h, l);
-        double v = df2_lanes_to_f64(h, l);
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if ((tid & 31) == 0) wnorm[tid >> 5] += v;
-      }
-      __syncthreads();
-    }
     const uint32_t I0 = F.basis_dn[d0], I1 = F.basis_dn[d1];
     float *__restrict__ z0 = z + d0 * 2 * ld;
     float *__restrict__ z1 = z + d1 * 2 * ld;
@@ -605,11 +494,6 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const FastView F, float *x
     }
     __syncthreads();
   }
-  if (kUpd && tid == 0) {                  // wnorm was last written before the loop's final barrier
-    double t = 0.0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += wnorm[k];
-    U.partials[blockIdx.x] = t;
-  }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -625,7 +509,9 @@ constexpr int kTile = 32;
 // columns), dst has n_c rows of plane length ld_d; dst columns n_r .. ld_d - 1 are zeroed.
 // Block (32, 8): a 32 x 32 tile of both planes through shared memory.
 __global__ void __launch_bounds__(256) k_transpose(int64_t n_r, int64_t n_c, int64_t ld_s, int64_t ld_d,
-                                                   const float *__restrict__ src, float *__restrict__ dst) {
+                                                   const float *__restrict__ src, float *__restrict__ dst,
+                                                   const int *__restrict__ gate) {
+  if (gate && gate[0] == 0) return;
   __shared__ float th[kTile][kTile + 1], tl[kTile][kTile + 1];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int64_t c0 = (int64_t)blockIdx.x * kTile, r0 = (int64_t)blockIdx.y * kTile;
@@ -673,52 +559,6 @@ struct Side {
   const void *col;
   int64_t r_begin = 0;               // first row a launch covers (rows r_begin .. n_rows - 1)
 };
-
-struct LzArgs {                      // Lanczos epilogue operands
-  const float *r_cur;                // r_j   (q_j = r_j / beta_cur)
-  const float *r_prev;               // r_{j-1}
-  const float2 *coef;                // [0] 1/beta_cur, [1] beta_cur/beta_prev (double-float)
-  const double *inv_beta;            // 1/beta_cur (FP64)
-  double *partials;                  // alpha partial per block
-};
-
-// Coefficients of the recurrence, computed once per step by one thread (keeps FP64
-// divisions out of the wide kernels).  scal: [0] alpha_j, [1] beta_cur, [2] beta_prev;
-// writes scal[6] = 1/beta_cur and, as double-floats, coef[0] = 1/beta_cur,
-// coef[1] = beta_cur/beta_prev (0 at the first step), coef[2] = -alpha_j/beta_cur.
-__global__ void k_coeffs(double *__restrict__ scal, float2 *__restrict__ coef) {
-  const double a = scal[0], bc = scal[1], bp = scal[2];
-  scal[6] = 1.0 / bc;
-  coef[0] = f64_to_df(1.0 / bc, 0);
-  coef[1] = f64_to_df(bp > 0.0 ? bc / bp : 0.0, 0);
-  coef[2] = f64_to_df(-a / bc, 0);
-}
-
-// scal[i] = v for the given slots (stream-ordered host -> device scalar writes)
-// beta_prev <- beta_cur, beta_cur <- beta_j (scal[2], scal[1], scal[3]) without a host value,
-// so that a captured iteration needs no per-iteration arguments.
-__global__ void k_rotate_beta(double *__restrict__ scal) {
-  const double b_cur = scal[1];
-  scal[1] = scal[3];
-  scal[2] = b_cur;
-}
-
-__global__ void k_set_scal(double *__restrict__ scal, int i0, double v0, int i1, double v1, int i2, double v2) {
-  if (i0 >= 0) scal[i0] = v0;
-  if (i1 >= 0) scal[i1] = v1;
-  if (i2 >= 0) scal[i2] = v2;
-}
-
-// Appends (alpha, |r|) = (scal[0], scal[1]) to hist (room for cap pairs) at the count kept
-// in scal[7], so that several steps can run between two host read-backs.
-__global__ void k_record(double *__restrict__ scal, double *__restrict__ hist, int cap) {
-  const int i = (int)scal[7];
-  if (i >= 0 && i < cap) {
-    hist[2 * i] = scal[0];
-    hist[2 * i + 1] = scal[1];
-  }
-  scal[7] = (double)(i + 1);
-}
 
 __device__ __forceinline__ f2x ld2(const float *p) { return *reinterpret_cast<const f2x *>(p); }
 __device__ __forceinline__ void st2(float *p, f2x v) { *reinterpret_cast<f2x *>(p) = v; }
@@ -815,13 +655,12 @@ __device__ __forceinline__ void dn_group(DfSumP (&acc)[kLane], const Side &S, co
 
 // kMode 0: w (planar double-float, slot order; may alias z) = Z + t S_dn, for hub_apply
 //          (the FP64 output in rank order is written afterwards by k_unpermute).
-// kMode 1: w = (Z + t S_dn)/beta_cur - (beta_cur/beta_prev) r_prev, partials <- <q_j, w>
-//          per block (= <r_j, w>/beta_cur).
 // kMode 2: pass 1 on X^T (side = spin up, rows of x are spin-up states, columns spin-down
 //          states): w = t S_up + diag x, diag from the two basis strings (no z).
 template <typename Col, int kMode>
 __global__ void __launch_bounds__(kDnThreads, HUB_DN_MINB) k_dn(const FastView F, const Side S, const float *__restrict__ x,
-                                                  const float *z, float *w, LzArgs L) {
+                                                  const float *z, float *w) {
+  if (F.gate && F.gate[0] == 0) return;
   constexpr int kLane = kDnLaneCols / 2;               // packed pairs per lane
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t ld = S.ld;
@@ -833,7 +672,6 @@ __global__ void __launch_bounds__(kDnThreads, HUB_DN_MINB) k_dn(const FastView F
   const int64_t u = (int64_t)blockIdx.y * kDnCols + kDnLaneCols * lane;
   const int64_t r0 = S.r_begin + (int64_t)blockIdx.x * kDnRows;
   const uint32_t row_bytes = (uint32_t)(2 * ld * sizeof(float));
-  DfAcc2 dacc{0ull, 0ull};
   const bool active = u < S.n_cols;                    // u + kDnLaneCols <= ld (see fast_build)
   const char *__restrict__ xh = reinterpret_cast<const char *>(x + u);
   const char *__restrict__ xl = reinterpret_cast<const char *>(x + ld + u);
@@ -891,189 +729,10 @@ __global__ void __launch_bounds__(kDnThreads, HUB_DN_MINB) k_dn(const FastView F
         df2_add(zh.v[i], zl.v[i], Sh, Sl, yh.v[i], yl.v[i]);
       }
     }
-    if (kMode != 1) {
-      stv<kLane>(wr + u, yh);
-      stv<kLane>(wr + ld + u, yl);
-    } else {
-      const float *rc = L.r_cur + d * 2 * ld, *rp = L.r_prev + d * 2 * ld;
-      const Vec<kLane> rph = ldv<kLane>(rp + u), rpl = ldv<kLane>(rp + ld + u);
-      const Vec<kLane> rch = ldv<kLane>(rc + u), rcl = ldv<kLane>(rc + ld + u);
-      // recurrence coefficients, read per row (L1-resident) rather than held across the
-      // hopping loop in registers
-      const float2 ib = L.coef[0], cp = L.coef[1];
-      const f2x ibh = bcast2(ib.x), ibl = bcast2(ib.y), cph = bcast2(cp.x), cpl = bcast2(cp.y);
-      Vec<kLane> wh, wl;
-#pragma unroll
-      for (int i = 0; i < kLane; ++i) {
-        f2x ah, al, bh, bl, qh, ql;
-        df2_mul(yh.v[i], yl.v[i], ibh, ibl, ah, al);
-        df2_mul(cph, cpl, rph.v[i], rpl.v[i], bh, bl);
-        df2_sub(ah, al, bh, bl, wh.v[i], wl.v[i]);
-        // keep padding columns zero: column u + 2i + 1 (lane b) and u + 2i (both lanes)
-        const int64_t c0 = u + 2 * i;
-        if (c0 >= S.n_cols) {
-          wh.v[i] = 0ull;
-          wl.v[i] = 0ull;
-        } else if (c0 + 1 >= S.n_cols) {
-          wh.v[i] &= 0xffffffffull;
-          wl.v[i] &= 0xffffffffull;
-        }
-        // <r_j, w>, accumulated in double-float, reduced in FP64 and scaled by 1/beta_cur
-        df2_mul(rch.v[i], rcl.v[i], wh.v[i], wl.v[i], qh, ql);
-        acc2_add(dacc, qh, ql);
-      }
-      stv<kLane>(wr + u, wh);
-      stv<kLane>(wr + ld + u, wl);
-    }
-  }
-  if (kMode == 1) {
-    f2x h, l;
-    acc2_norm(dacc, h, l);
-    double dot = df2_lanes_to_f64(h, l);
-    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-    __shared__ double ws[kDnThreads / 32];
-    if (lane == 0) ws[warp] = dot;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double s = 0.0;
-      for (int k = 0; k < kDnThreads / 32; ++k) s += ws[k];
-      L.partials[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = s * L.inv_beta[0];
-    }
+    stv<kLane>(wr + u, yh);
+    stv<kLane>(wr + ld + u, yl);
   }
 }
-
-// ---------------------------------------------------------------------------------------
-// Double-float Lanczos vector kernels (planar rows; padding columns stay zero).  Each
-// thread step takes four columns of one row: a 16-byte load per plane, two packed pairs.
-// ---------------------------------------------------------------------------------------
-__device__ __forceinline__ void block_sum_to(double v, double *partials) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __shared__ double ws[32];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) ws[wid] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += ws[k];
-    partials[blockIdx.x] = s;
-  }
-}
-
-// Column quads of a planar vector: quad k of n_rows * (ld / 4) starts at float offset
-// row * 2 ld + 4 q (hi) and + ld (lo).  The host keeps n_rows * ld / 4 below 2^32.
-struct Quads {
-  uint32_t per_row, n;
-  int64_t ld;
-  __device__ __forceinline__ int64_t at(uint32_t k) const {
-    const uint32_t d = k / per_row, q = k - d * per_row;
-    return (int64_t)d * 2 * ld + 4 * (int64_t)q;
-  }
-};
-__device__ __forceinline__ void ld4(const float *p, f2x &a, f2x &b) {
-  const float4 v = *reinterpret_cast<const float4 *>(p);
-  a = pk2(v.x, v.y);
-  b = pk2(v.z, v.w);
-}
-__device__ __forceinline__ void st4(float *p, f2x a, f2x b) {
-  const float2 u = upk2(a), v = upk2(b);
-  *reinterpret_cast<float4 *>(p) = make_float4(u.x, u.y, v.x, v.y);
-}
-
-// r_next = w + coef[2] r_cur = w - (alpha / beta_cur) r_cur  (in place over w);
-// partials <- |r_next|^2
-__global__ void k_df_update(Quads Q, float *__restrict__ w, const float *__restrict__ r_cur,
-                            const float2 *__restrict__ coef, double *__restrict__ partials) {
-  const float2 c = coef[2];
-  const f2x ch = bcast2(c.x), cl = bcast2(c.y);
-  DfAcc2 acc{0ull, 0ull};
-  for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < Q.n; k += (uint64_t)gridDim.x * blockDim.x) {
-    const int64_t o = Q.at((uint32_t)k);
-    f2x wh[2], wl[2], rh[2], rl[2];
-    ld4(w + o, wh[0], wh[1]);
-    ld4(w + o + Q.ld, wl[0], wl[1]);
-    ld4(r_cur + o, rh[0], rh[1]);
-    ld4(r_cur + o + Q.ld, rl[0], rl[1]);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      f2x ph, pl;
-      df2_mul(ch, cl, rh[i], rl[i], ph, pl);
-      df2_add(ph, pl, wh[i], wl[i], wh[i], wl[i]);
-      df2_mul(wh[i], wl[i], wh[i], wl[i], ph, pl);
-      acc2_add(acc, ph, pl);
-    }
-    st4(w + o, wh[0], wh[1]);
-    st4(w + o + Q.ld, wl[0], wl[1]);
-  }
-  f2x h, l;
-  acc2_norm(acc, h, l);
-  block_sum_to(df2_lanes_to_f64(h, l), partials);
-}
-
-// partials <- |v|^2
-__global__ void k_df_norm2(Quads Q, const float *__restrict__ v, double *__restrict__ partials) {
-  DfAcc2 acc{0ull, 0ull};
-  for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < Q.n; k += (uint64_t)gridDim.x * blockDim.x) {
-    const int64_t o = Q.at((uint32_t)k);
-    f2x vh[2], vl[2];
-    ld4(v + o, vh[0], vh[1]);
-    ld4(v + o + Q.ld, vl[0], vl[1]);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      f2x ph, pl;
-      df2_mul(vh[i], vl[i], vh[i], vl[i], ph, pl);
-      acc2_add(acc, ph, pl);
-    }
-  }
-  f2x h, l;
-  acc2_norm(acc, h, l);
-  block_sum_to(df2_lanes_to_f64(h, l), partials);
-}
-
-// psi += c r, c a double-float coefficient in coef[idx]
-__global__ void k_df_axpy(Quads Q, const float2 *__restrict__ coef, int idx, const float *__restrict__ r,
-                          float *__restrict__ psi) {
-  const float2 a = coef[idx];
-  const f2x ah = bcast2(a.x), al = bcast2(a.y);
-  for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < Q.n; k += (uint64_t)gridDim.x * blockDim.x) {
-    const int64_t o = Q.at((uint32_t)k);
-    f2x ph[2], pl[2], rh[2], rl[2];
-    ld4(psi + o, ph[0], ph[1]);
-    ld4(psi + o + Q.ld, pl[0], pl[1]);
-    ld4(r + o, rh[0], rh[1]);
-    ld4(r + o + Q.ld, rl[0], rl[1]);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      f2x mh, ml;
-      df2_mul(ah, al, rh[i], rl[i], mh, ml);
-      df2_add(mh, ml, ph[i], pl[i], ph[i], pl[i]);
-    }
-    st4(psi + o, ph[0], ph[1]);
-    st4(psi + o + Q.ld, pl[0], pl[1]);
-  }
-}
-
-// coef[3] = c / scal[1]  (psi coefficient v_j / beta_cur), one thread
-__global__ void k_psi_coef(const double *__restrict__ scal, double c, float2 *__restrict__ coef) {
-  coef[3] = f64_to_df(c / scal[1], 0);
-}
-
-// out (FP64, rank order) = v / |v|  with |v| = scal[idx]; one row per block and step
-__global__ void k_df_out_normalised(int64_t n_rows, int64_t n_up, int64_t ld, const float *__restrict__ v,
-                                    const double *__restrict__ scal, int idx, const int32_t *__restrict__ slot_of,
-                                    double *__restrict__ out) {
-  const float2 inv = f64_to_df(1.0 / scal[idx], 0);
-  for (int64_t d = blockIdx.x; d < n_rows; d += gridDim.x) {
-    const float *__restrict__ row = v + d * 2 * ld;
-    for (int64_t u = threadIdx.x; u < n_up; u += blockDim.x) {
-      const int32_t s = slot_of[u];
-      out[d * n_up + u] = df_to_f64(df_mul(make_float2(row[s], row[ld + s]), inv), 0);
-    }
-  }
-}
-
-// Second-pass recurrence with known coefficients: r_next = (H r_j)/1 ... computed as
-// w = (Z + t S)/beta_cur - (beta_cur/beta_prev) r_prev by k_dn<.,1>, then
-// r_next = w - (alpha/beta_cur) r_cur by k_df_update (alpha written into scal[0]).
 
 // ---------------------------------------------------------------------------------------
 // Host side.
@@ -1082,7 +741,6 @@ static int grid_vec() { return num_sms() * 4; }
 
 struct FastState {
   bool built = false;
-  float2 *coef = nullptr;                    // recurrence coefficients (double-float)
   bool col16 = true;
   int32_t *sp[2] = {nullptr, nullptr};
   uint32_t *sl_add = nullptr, *sl_sub = nullptr;
@@ -1097,10 +755,7 @@ struct FastState {
   int acc_terms = 0;                         // most terms one low-part accumulator sums (error bound)
   int64_t ld_t = 0;                          // plane length of X^T rows (count_dn padded)
   float *xt = nullptr, *zt = nullptr;        // X^T and Z^T (rows too long to stage)
-  float *lz[3] = {nullptr, nullptr, nullptr};
-  float *psi = nullptr;
   int *d_range = nullptr;                    // exponent partials [2 G], then scale[4] (k_scale)
-  double *d_hist = nullptr, *h_hist = nullptr;  // (alpha, |r|) of the steps since the last read-back
   int *d_err = nullptr;
   int64_t ld = 0;
   // pipelined host-buffer apply: copy stream, per-chunk events, exponent partials, flag
@@ -1110,13 +765,6 @@ struct FastState {
   // the multi-vector form: a second copy stream (outputs) and its own events
   cudaStream_t copy_out_stream = nullptr;
   std::vector<cudaEvent_t> many_events;
-  // CUDA graphs of one Lanczos iteration (first pass), one per rotation of the three
-  // vectors, captured on graph_stream and replayed on the caller's stream; lz_graph_key holds
-  // the operands they were captured with
-  cudaStream_t graph_stream = nullptr;
-  cudaGraphExec_t lz_graph[3] = {nullptr, nullptr, nullptr};
-  std::vector<unsigned char> lz_graph_key;
-  bool lz_graph_failed = false;
 };
 
 static FastState *fast_of(const hub_ctx *h) { return h->fast; }
@@ -1132,11 +780,7 @@ void fast_release(hub_ctx *h) {
   dev_free(f->zdf);
   dev_free(f->xt);
   dev_free(f->zt);
-  for (int k = 0; k < 3; ++k) dev_free(f->lz[k]);
-  dev_free(f->psi);
   dev_free(f->d_range);
-  dev_free(f->d_hist);
-  if (f->h_hist) cudaFreeHost(f->h_hist);
   dev_free(f->d_err);
   dev_free(f->d_range_chunks);
   dev_free(f->d_flag);
@@ -1145,10 +789,6 @@ void fast_release(hub_ctx *h) {
   if (f->copy_stream) cudaStreamDestroy(f->copy_stream);
   for (cudaEvent_t e : f->many_events) cudaEventDestroy(e);
   if (f->copy_out_stream) cudaStreamDestroy(f->copy_out_stream);
-  for (int k = 0; k < 3; ++k)
-    if (f->lz_graph[k]) cudaGraphExecDestroy(f->lz_graph[k]);
-  if (f->graph_stream) cudaStreamDestroy(f->graph_stream);
-  dev_free(f->coef);
   dev_free(f->sl_add);
   dev_free(f->sl_sub);
   dev_free(f->sl_off_add);
@@ -1402,17 +1042,16 @@ int fast_build(hub_ctx *h) {
       HUB_CUDA(cudaMemcpy(f->steps_sub, st[1].data(), sizeof(uint16_t) * nsl, cudaMemcpyHostToDevice));
     }
   }
-  if (!dev_alloc((void **)&f->d_err, sizeof(int) * 4, "error flag") ||
-      !dev_alloc((void **)&f->coef, sizeof(float2) * 8, "recurrence coefficients"))
-    return HUB_ERR_OOM;
+  if (!dev_alloc((void **)&f->d_err, sizeof(int) * 4, "error flag")) return HUB_ERR_OOM;
   HUB_CUDA(cudaMemset(f->d_err, 0, sizeof(int) * 4));
   HUB_CUDA(cudaDeviceSynchronize());
   f->built = true;
   return HUB_OK;
 }
 
-static FastView fast_view(const hub_ctx *h, const FastState *f) {
+static FastView fast_view(const hub_ctx *h, const FastState *f, const int *gate) {
   FastView v{};
+  v.gate = gate;
   v.n_up = h->count[0];
   v.n_dn = h->count[1];
   v.ld = f->ld;
@@ -1450,14 +1089,6 @@ static FastView fast_view(const hub_ctx *h, const FastState *f) {
   return v;
 }
 
-static Quads quads(const hub_ctx *h, const FastState *f) {
-  Quads q;
-  q.per_row = (uint32_t)(f->ld / 4);
-  q.n = (uint32_t)(h->count[1] * (f->ld / 4));
-  q.ld = f->ld;
-  return q;
-}
-
 static size_t up_smem(const FastState *f) { return sizeof(float) * (3 * (size_t)kUpPlane + (size_t)f->ld + 2); }
 constexpr size_t kMaxStage = 224 * 1024;
 static_assert(sizeof(float) * 4 * kUpPlane <= kMaxStage, "four staged planes must fit");
@@ -1476,28 +1107,26 @@ static dim3 dn_grid(const Side &S) {
 }
 
 template <typename Col, int kMode>
-static int launch_dn_t(const FastView &v, const Side &S, const float *x, const float *z, float *w, LzArgs L,
-                       cudaStream_t s) {
+static int launch_dn_t(const FastView &v, const Side &S, const float *x, const float *z, float *w, cudaStream_t s) {
   const dim3 g = dn_grid(S);
   if (g.y > 65535) return fail(HUB_ERR_ARG, "fast apply: too many column strips");
-  k_dn<Col, kMode><<<g, kDnThreads, 0, s>>>(v, S, x, z, w, L);
+  k_dn<Col, kMode><<<g, kDnThreads, 0, s>>>(v, S, x, z, w);
   HUB_LAUNCH_CHECK();
   return HUB_OK;
 }
 
 template <int kMode>
 static int launch_dn(const FastState *f, const FastView &v, const Side &S, const float *x, const float *z, float *w,
-                     LzArgs L, cudaStream_t s) {
-  return f->col16 ? launch_dn_t<uint16_t, kMode>(v, S, x, z, w, L, s)
-                  : launch_dn_t<uint32_t, kMode>(v, S, x, z, w, L, s);
+                     cudaStream_t s) {
+  return f->col16 ? launch_dn_t<uint16_t, kMode>(v, S, x, z, w, s) : launch_dn_t<uint32_t, kMode>(v, S, x, z, w, s);
 }
 
 // dst = src^T for planar matrices (see k_transpose)
 static int transpose(int64_t n_r, int64_t n_c, int64_t ld_s, int64_t ld_d, const float *src, float *dst,
-                     cudaStream_t s) {
+                     const int *gate, cudaStream_t s) {
   const dim3 g((unsigned)((n_c + kTile - 1) / kTile), (unsigned)((ld_d + kTile - 1) / kTile));
   if (g.y > 65535) return fail(HUB_ERR_ARG, "fast apply: matrix too large to transpose");
-  k_transpose<<<g, dim3(kTile, 8), 0, s>>>(n_r, n_c, ld_s, ld_d, src, dst);
+  k_transpose<<<g, dim3(kTile, 8), 0, s>>>(n_r, n_c, ld_s, ld_d, src, dst, gate);
   HUB_LAUNCH_CHECK();
   return HUB_OK;
 }
@@ -1505,62 +1134,43 @@ static int transpose(int64_t n_r, int64_t n_c, int64_t ld_s, int64_t ld_d, const
 static int ensure_vec(float **p, int64_t n, const char *what);
 
 // z <- pass 1 (x planar double-float); with staged rows, only the row pairs p0 .. p1 - 1
-// (p1 < 0: all pairs).  With upd: first x <- x + c r_prev (the Lanczos update, fused into the
-// staging of pass 1 when rows are staged, else a separate vector pass), |x|^2 partials into
-// upd->partials, their number in *n_part.
-static int run_up(hub_ctx *h, FastState *f, float *x, float *z, cudaStream_t s, int64_t p0 = 0, int64_t p1 = -1,
-                  const UpdArgs *upd = nullptr, int *n_part = nullptr) {
-  const FastView v = fast_view(h, f);
+// (p1 < 0: all pairs).
+static int run_up(hub_ctx *h, FastState *f, const float *x, float *z, cudaStream_t s, int64_t p0 = 0, int64_t p1 = -1,
+                  const int *gate = nullptr) {
+  const FastView v = fast_view(h, f, gate);
   if (p1 < 0) p1 = (v.n_dn + 1) / 2;
-  if ((!f->staged || upd) && (p0 != 0 || p1 != (v.n_dn + 1) / 2))
-    return fail(HUB_ERR_STATE, "pass 1: partial range");
+  if (!f->staged && (p0 != 0 || p1 != (v.n_dn + 1) / 2)) return fail(HUB_ERR_STATE, "pass 1: partial range");
   if (p1 <= p0) return HUB_OK;
   int rc;
-  const bool fused = upd && f->staged && kFusedUpdate;
-  if (upd && !fused) {                 // the update as its own pass, timed on its own
-    if ((rc = prof_mark(h, HUB_PROF_UPDATE, true, s))) return rc;
-    const int G = grid_vec();
-    count_launch(h);
-    k_df_update<<<G, 256, 0, s>>>(quads(h, f), x, upd->r_prev, upd->coef, upd->partials);
-    HUB_LAUNCH_CHECK();
-    if (n_part) *n_part = G;
-    if ((rc = prof_mark(h, HUB_PROF_UPDATE, false, s))) return rc;
-  }
   if ((rc = prof_mark(h, HUB_PROF_UP, true, s))) return rc;
   if (f->staged) {
     count_launch(h);
     const int threads = v.n_up >= 4096 ? kUpThreads : (v.n_up >= 1024 ? 512 : (v.n_up >= 256 ? 256 : 128));
     const int grid = (int)std::min<int64_t>(p1 - p0, (int64_t)num_sms());
     const size_t smem = up_smem(f);
-    const UpdArgs U = fused ? *upd : UpdArgs{};
-    if (fused && n_part) *n_part = grid;
-#define HUB_UP(C, K)                                                                                      \
-  do {                                                                                                    \
-    HUB_CUDA(cudaFuncSetAttribute(k_up<C, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxStage)); \
-    k_up<C, K><<<grid, threads, smem, s>>>(v, x, z, p0, p1, U);                                          \
+#define HUB_UP(C)                                                                                          \
+  do {                                                                                                     \
+    HUB_CUDA(cudaFuncSetAttribute(k_up<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxStage));  \
+    k_up<C><<<grid, threads, smem, s>>>(v, x, z, p0, p1);                                                  \
   } while (0)
-    if (f->col16) {
-      if (fused) HUB_UP(uint16_t, true); else HUB_UP(uint16_t, false);
-    } else {
-      if (fused) HUB_UP(uint32_t, true); else HUB_UP(uint32_t, false);
-    }
+    if (f->col16) HUB_UP(uint16_t); else HUB_UP(uint32_t);
 #undef HUB_UP
     HUB_LAUNCH_CHECK();
   } else {
     const int64_t Dt = h->count[0] * 2 * f->ld_t;
     if ((rc = ensure_vec(&f->xt, Dt, "transposed x")) || (rc = ensure_vec(&f->zt, Dt, "transposed z"))) return rc;
     count_launch(h, 3);
-    if ((rc = transpose(h->count[1], h->count[0], f->ld, f->ld_t, x, f->xt, s))) return rc;
-    if ((rc = launch_dn<2>(f, v, side_up(h, f), f->xt, nullptr, f->zt, LzArgs{}, s))) return rc;
-    if ((rc = transpose(h->count[0], h->count[1], f->ld_t, f->ld, f->zt, z, s))) return rc;
+    if ((rc = transpose(h->count[1], h->count[0], f->ld, f->ld_t, x, f->xt, gate, s))) return rc;
+    if ((rc = launch_dn<2>(f, v, side_up(h, f), f->xt, nullptr, f->zt, s))) return rc;
+    if ((rc = transpose(h->count[0], h->count[1], f->ld_t, f->ld, f->zt, z, gate, s))) return rc;
   }
   return prof_mark(h, HUB_PROF_UP, false, s);
 }
 
 // pass 2 on the rows r0 .. r1 - 1 of X (r1 < 0: all rows)
-static int run_dn(hub_ctx *h, FastState *f, int mode, const float *x, const float *z, float *w, LzArgs L,
-                  cudaStream_t s, int64_t r0 = 0, int64_t r1 = -1) {
-  const FastView v = fast_view(h, f);
+static int run_dn(hub_ctx *h, FastState *f, const float *x, const float *z, float *w, cudaStream_t s, int64_t r0 = 0,
+                  int64_t r1 = -1, const int *gate = nullptr) {
+  const FastView v = fast_view(h, f, gate);
   count_launch(h);
   int rc = prof_mark(h, HUB_PROF_DN, true, s);
   if (rc) return rc;
@@ -1568,8 +1178,7 @@ static int run_dn(hub_ctx *h, FastState *f, int mode, const float *x, const floa
   S.r_begin = r0;
   if (r1 >= 0) S.n_rows = r1;
   if (S.n_rows <= S.r_begin) return prof_mark(h, HUB_PROF_DN, false, s);
-  rc = mode == 0 ? launch_dn<0>(f, v, S, x, z, w, L, s) : launch_dn<1>(f, v, S, x, z, w, L, s);
-  if (rc) return rc;
+  if ((rc = launch_dn<0>(f, v, S, x, z, w, s))) return rc;
   return prof_mark(h, HUB_PROF_DN, false, s);
 }
 
@@ -1587,31 +1196,72 @@ static int *range_buf(FastState *f) {
   return f->d_range;
 }
 
-// hub_apply on the fast path: FP64 in, FP64 out.  A vector outside the double-float window
+// Floats of a scratch vector: a planar vector, or a fixed-point one in either order.
+static int64_t scratch_floats(const hub_ctx *h, const FastState *f) {
+  return 2 * std::max(h->count[1] * f->ld, h->count[0] * f->ld_t);
+}
+
+int fast_scratch(hub_ctx *h, int n, float **v) {
+  FastState *f = fast_of(h);
+  float **const all[4] = {&f->xdf, &f->zdf, &f->xt, &f->zt};
+  for (int k = 0; k < n; ++k) {
+    const int rc = ensure_vec(all[k], scratch_floats(h, f), "apply scratch");
+    if (rc) return rc;
+    v[k] = *all[k];
+  }
+  return HUB_OK;
+}
+
+int fast_exp_range(hub_ctx *h, const double *x, int64_t D, int **part, int *nblk, cudaStream_t s) {
+  FastState *f = fast_of(h);
+  *nblk = grid_vec();
+  if (!(*part = range_buf(f))) return HUB_ERR_OOM;
+  count_launch(h);
+  k_exp_range<<<*nblk, 256, 0, s>>>(D, x, *part);
+  HUB_LAUNCH_CHECK();
+  return HUB_OK;
+}
+
+int *fast_err(const hub_ctx *h) { return fast_of(h)->d_err; }
+
+// Conversion, both passes and the un-permutation of a product whose scale is known.
+static int df_apply(hub_ctx *h, FastState *f, const double *x, double *y, const int *scale, const int *gate,
+                    cudaStream_t s) {
+  int rc;
+  count_launch(h);
+  k_f64_to_df<<<row_grid(h), 256, 0, s>>>(0, h->count[1], h->count[0], f->ld, x, scale, f->slot_row, f->xdf, gate);
+  HUB_LAUNCH_CHECK();
+  if ((rc = run_up(h, f, f->xdf, f->zdf, s, 0, -1, gate))) return rc;
+  if ((rc = run_dn(h, f, f->xdf, f->zdf, f->zdf, s, 0, -1, gate))) return rc;
+  count_launch(h);
+  k_unpermute<<<row_grid(h), 512, 0, s>>>(0, h->count[1], h->count[0], f->ld, f->zdf, f->slot_of, scale,
+                                          std::fabs(h->t[0]), y, gate);
+  HUB_LAUNCH_CHECK();
+  return HUB_OK;
+}
+
+int fast_apply_gated(hub_ctx *h, const double *x, double *y, const int *scale, const int *gate, cudaStream_t s) {
+  FastState *f = fast_of(h);
+  float *v[2];
+  const int rc = fast_scratch(h, 2, v);
+  return rc ? rc : df_apply(h, f, x, y, scale, gate, s);
+}
+
+// hub_apply on the double-float path: FP64 in, FP64 out.  A vector outside the double-float window
 // (kExpSpan) is multiplied by the FP64 kernel instead: both are launched, the device-side
 // flag scale[1] decides which one writes y, so the call stays asynchronous.
 int fast_apply_f64(hub_ctx *h, const double *x, double *y, cudaStream_t s) {
   FastState *f = fast_of(h);
   if (!f || !f->built) return fail(HUB_ERR_STATE, "fast apply: not built");
-  const int64_t Dp = h->count[1] * 2 * f->ld, D = h->count[0] * h->count[1];
-  int rc;
-  if ((rc = ensure_vec(&f->xdf, Dp, "apply scratch x")) || (rc = ensure_vec(&f->zdf, Dp, "apply scratch z")))
-    return rc;
-  const int G = grid_vec();
-  int *part = range_buf(f);
-  if (!part) return HUB_ERR_OOM;
+  float *v[2];
+  int *part = nullptr, G = 0, rc;
+  if ((rc = fast_scratch(h, 2, v))) return rc;
+  if ((rc = fast_exp_range(h, x, h->count[0] * h->count[1], &part, &G, s))) return rc;
   int *scale = part + 2 * G;
-  count_launch(h, 3);
-  k_exp_range<<<G, 256, 0, s>>>(D, x, part);
-  k_scale<<<1, 256, 0, s>>>(part, G, scale);
-  k_f64_to_df<<<row_grid(h), 256, 0, s>>>(0, h->count[1], h->count[0], f->ld, x, scale, f->slot_row, f->xdf);
-  HUB_LAUNCH_CHECK();
-  if ((rc = run_up(h, f, f->xdf, f->zdf, s))) return rc;
-  if ((rc = run_dn(h, f, 0, f->xdf, f->zdf, f->zdf, LzArgs{}, s))) return rc;
   count_launch(h);
-  k_unpermute<<<row_grid(h), 512, 0, s>>>(0, h->count[1], h->count[0], f->ld, f->zdf, f->slot_of, scale,
-                                          std::fabs(h->t[0]), y);
+  k_scale<<<1, 256, 0, s>>>(part, G, scale);
   HUB_LAUNCH_CHECK();
+  if ((rc = df_apply(h, f, x, y, scale, nullptr, s))) return rc;
   return f64_apply(h, x, y, scale + 1, s);
 }
 
@@ -1655,10 +1305,10 @@ static HostChunks host_chunks(int64_t n_dn) {
 
 // Scratch of the chunked host-buffer apply: double-float x and z, per-chunk exponent
 // partials, the scale words, the route flag (device and pinned host) and the input copy stream.
-static int host_pipe_buffers(FastState *f, int64_t Dp) {
-  int rc;
-  if ((rc = ensure_vec(&f->xdf, Dp, "apply scratch x")) || (rc = ensure_vec(&f->zdf, Dp, "apply scratch z")))
-    return rc;
+static int host_pipe_buffers(hub_ctx *h, FastState *f) {
+  float *v[2];
+  const int rc = fast_scratch(h, 2, v);
+  if (rc) return rc;
   if (!f->d_range_chunks &&
       !dev_alloc((void **)&f->d_range_chunks, sizeof(int) * 2 * grid_vec() * kHostChunks, "exponent partials"))
     return HUB_ERR_OOM;
@@ -1697,7 +1347,7 @@ static int host_pass1(hub_ctx *h, FastState *f, const double *xd, const int64_t 
     count_launch(h, c == 0 ? 3 : 2);
     k_exp_range<<<G, 256, 0, s>>>((b[c + 1] - b[c]) * n_up, xd + b[c] * n_up, part + 2 * c * G);
     if (c == 0) k_scale<<<1, 256, 0, s>>>(part, G, scale);
-    k_f64_to_df<<<rg, 256, 0, s>>>(b[c], b[c + 1], n_up, f->ld, xd, scale, f->slot_row, f->xdf);
+    k_f64_to_df<<<rg, 256, 0, s>>>(b[c], b[c + 1], n_up, f->ld, xd, scale, f->slot_row, f->xdf, nullptr);
     HUB_LAUNCH_CHECK();
     if ((rc = run_up(h, f, f->xdf, f->zdf, s, b[c] / 2, (b[c + 1] + 1) / 2))) return rc;
   }
@@ -1712,7 +1362,8 @@ static int host_pass1(hub_ctx *h, FastState *f, const double *xd, const int64_t 
 static int host_redo(hub_ctx *h, FastState *f, const double *xd, cudaStream_t s) {
   int *scale = f->d_range + 2 * grid_vec();
   count_launch(h);
-  k_f64_to_df<<<row_grid(h), 256, 0, s>>>(0, h->count[1], h->count[0], f->ld, xd, scale + 2, f->slot_row, f->xdf);
+  k_f64_to_df<<<row_grid(h), 256, 0, s>>>(0, h->count[1], h->count[0], f->ld, xd, scale + 2, f->slot_row, f->xdf,
+                                          nullptr);
   HUB_LAUNCH_CHECK();
   return run_up(h, f, f->xdf, f->zdf, s);
 }
@@ -1728,10 +1379,10 @@ static int host_pass2(hub_ctx *h, FastState *f, double *yd, double *y_host, cons
   const int rg = (int)std::min<int64_t>(per, (int64_t)num_sms() * 8);
   int rc;
   for (int c = 0; c < nc; ++c) {
-    if ((rc = run_dn(h, f, 0, f->xdf, f->zdf, f->zdf, LzArgs{}, s, b[c], b[c + 1]))) return rc;
+    if ((rc = run_dn(h, f, f->xdf, f->zdf, f->zdf, s, b[c], b[c + 1]))) return rc;
     count_launch(h);
     k_unpermute<<<rg, 512, 0, s>>>(b[c], b[c + 1], n_up, f->ld, f->zdf, f->slot_of, scale + 2,
-                                   std::fabs(h->t[0]), yd);
+                                   std::fabs(h->t[0]), yd, nullptr);
     HUB_LAUNCH_CHECK();
     HUB_CUDA(cudaEventRecord(ev_out[c], s));
     HUB_CUDA(cudaStreamWaitEvent(sc, ev_out[c], 0));
@@ -1741,9 +1392,14 @@ static int host_pass2(hub_ctx *h, FastState *f, double *yd, double *y_host, cons
   return HUB_OK;
 }
 
+// Sectors below this are multiplied in one piece (copy in, hub_apply, copy out): their copies take
+// less than the chunks' launches.
+constexpr int64_t kHostPipelineMin = (int64_t)1 << 22;
+
 bool fast_host_pipelined(const hub_ctx *h) {
   const FastState *f = fast_of(h);
-  return f && f->built && f->staged && h->count[1] >= 2 * kHostChunks;
+  return f && f->built && f->staged && h->count[1] >= 2 * kHostChunks &&
+         h->count[0] * h->count[1] >= kHostPipelineMin;
 }
 
 // The chunked copies and passes of fast_apply_host: input chunks on the copy stream, pass 1
@@ -1786,16 +1442,9 @@ int fast_apply_host(hub_ctx *h, const double *x_host, double *y_host, double *xd
   FastState *f = fast_of(h);
   if (!f || !f->built) return fail(HUB_ERR_STATE, "fast apply: not built");
   const int64_t n_up = h->count[0], n_dn = h->count[1];
-  if (!fast_host_pipelined(h)) {   // one piece: copy in, apply, copy out
-    HUB_CUDA(cudaMemcpyAsync(xd, x_host, sizeof(double) * n_up * n_dn, cudaMemcpyHostToDevice, s));
-    int rc = fast_apply_f64(h, xd, yd, s);
-    if (rc) return rc;
-    HUB_CUDA(cudaMemcpyAsync(y_host, yd, sizeof(double) * n_up * n_dn, cudaMemcpyDeviceToHost, s));
-    HUB_CUDA(cudaStreamSynchronize(s));
-    return HUB_OK;
-  }
+  if (!fast_host_pipelined(h)) return fail(HUB_ERR_STATE, "fast apply: no row-chunk pipeline for this sector");
   int rc;
-  if ((rc = host_pipe_buffers(f, n_dn * 2 * f->ld))) return rc;
+  if ((rc = host_pipe_buffers(h, f))) return rc;
   // events: [kHostChunks] input chunks, [kHostChunks] output chunks, start, end
   if ((rc = ensure_events(f->events, 2 * kHostChunks + 2))) return rc;
   cudaStream_t sc = f->copy_stream;
@@ -1827,7 +1476,7 @@ int fast_apply_host_many(hub_ctx *h, int64_t n_vec, const double *x_host, double
   if (!fast_host_pipelined(h)) return fail(HUB_ERR_STATE, "fast apply: no row-chunk pipeline for this sector");
   const int64_t n_up = h->count[0], n_dn = h->count[1], D = n_up * n_dn;
   int rc;
-  if ((rc = host_pipe_buffers(f, n_dn * 2 * f->ld))) return rc;
+  if ((rc = host_pipe_buffers(h, f))) return rc;
   if (!f->copy_out_stream) HUB_CUDA(cudaStreamCreateWithFlags(&f->copy_out_stream, cudaStreamNonBlocking));
   // events: [2][kHostChunks] input chunks (by buffer), [kHostChunks] output chunks,
   // x_free[2], y_free[2], start, end
@@ -1898,286 +1547,6 @@ int fast_check_error(hub_ctx *h) {
     return fail(HUB_ERR_TIMEOUT, "a bounded wait for a staged row gave up (row copy never completed)");
   }
   return HUB_OK;
-}
-
-// ---------------------------------------------------------------------------------------
-// Double-float Lanczos (same recurrence as the FP64 driver; vectors kept unnormalised,
-// r_j = beta_{j-1} q_j, so the normalisation is folded into the apply's epilogue).
-// scal: [0] alpha_j, [1] beta_cur = |r_j|, [2] beta_prev = |r_{j-1}| (0 at the start),
-// [3] beta_j, [5] |psi|, [6] 1/beta_cur.
-// ---------------------------------------------------------------------------------------
-// Captures `iteration` once per rotation of the three Lanczos vectors (graphs replayed in
-// turn on the caller's stream) unless the cached graphs were captured with the same operands.
-// Returns false, with the CUDA error state cleared, if capture is not possible; the caller
-// then launches each kernel itself.
-template <class F>
-static bool lz_graphs(hub_ctx *h, FastState *f, float *v0, float *v1, float *v2, F &iteration) {
-  if (f->lz_graph_failed) return false;
-  std::vector<unsigned char> key;
-  auto add = [&](const void *p, size_t n) {
-    const unsigned char *b = (const unsigned char *)p;
-    key.insert(key.end(), b, b + n);
-  };
-  const FastView v = fast_view(h, f);
-  const Side S = side_dn(h, f);
-  const void *ptrs[9] = {v0, v1, v2, f->zdf, h->partials, h->d_scal, h->h_scal, f->coef, f->d_err};
-  add(&v, sizeof(v));
-  add(&S.n_rows, sizeof(S.n_rows));
-  add(&S.ld, sizeof(S.ld));
-  add(ptrs, sizeof(ptrs));
-  add(&h->partials_n, sizeof(h->partials_n));
-  if (f->lz_graph[0] && key == f->lz_graph_key) return true;
-  for (int k = 0; k < 3; ++k)
-    if (f->lz_graph[k]) {
-      cudaGraphExecDestroy(f->lz_graph[k]);
-      f->lz_graph[k] = nullptr;
-    }
-  if (!f->graph_stream && cudaStreamCreateWithFlags(&f->graph_stream, cudaStreamNonBlocking) != cudaSuccess) {
-    f->graph_stream = nullptr;
-    f->lz_graph_failed = true;
-    cudaGetLastError();
-    return false;
-  }
-  float *r[3] = {v0, v1, v2};
-  bool ok = true;
-  for (int k = 0; k < 3 && ok; ++k) {
-    if (cudaStreamBeginCapture(f->graph_stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
-      ok = false;
-      break;
-    }
-    const int rc = iteration(r[k % 3], r[(k + 1) % 3], r[(k + 2) % 3], f->graph_stream);
-    cudaGraph_t g = nullptr;
-    const cudaError_t e = cudaStreamEndCapture(f->graph_stream, &g);
-    ok = rc == HUB_OK && e == cudaSuccess && g != nullptr &&
-         cudaGraphInstantiate(&f->lz_graph[k], g, 0) == cudaSuccess;
-    if (g) cudaGraphDestroy(g);
-  }
-  if (!ok) {
-    for (int k = 0; k < 3; ++k)
-      if (f->lz_graph[k]) {
-        cudaGraphExecDestroy(f->lz_graph[k]);
-        f->lz_graph[k] = nullptr;
-      }
-    f->lz_graph_failed = true;
-    cudaGetLastError();
-    set_error("");
-    return false;
-  }
-  f->lz_graph_key = key;
-  return true;
-}
-
-int fast_lanczos(hub_ctx *h, const double *x0, int maxit, double tol, double *E0, double *psi_out,
-                 int *iters, cudaStream_t s) {
-  FastState *f = fast_of(h);
-  if (!f || !f->built) return fail(HUB_ERR_STATE, "fast Lanczos: not built");
-  const int64_t Dp = h->count[1] * 2 * f->ld;
-  int rc;
-  for (int k = 0; k < 3; ++k)
-    if ((rc = ensure_vec(&f->lz[k], Dp, "Lanczos vector"))) return rc;
-  if ((rc = ensure_vec(&f->zdf, Dp, "apply scratch z"))) return rc;
-  const int G = grid_vec();
-  const Quads Q = quads(h, f);
-  const dim3 gd = dn_grid(side_dn(h, f));
-  const int64_t n_dn_blocks = (int64_t)gd.x * gd.y;
-  constexpr int kTmp = 2048;                      // first-stage slots of the alpha reduction
-  if ((rc = ensure_partials(h, std::max<int64_t>(n_dn_blocks, G) + kTmp))) return rc;
-  int *part = range_buf(f);
-  if (!part) return HUB_ERR_OOM;
-  int *scale = part + 2 * G;
-  if (!h->d_scal && !dev_alloc((void **)&h->d_scal, sizeof(double) * 8, "Lanczos scalars")) return HUB_ERR_OOM;
-  if (!h->h_scal) HUB_CUDA(cudaMallocHost((void **)&h->h_scal, sizeof(double) * 8));
-  double *scal = h->d_scal, *P = h->partials;
-  float2 *coef = f->coef;
-
-  // r_1 = 2^-shift x0 as double-float (max |r_1| in [1, 2): the FP32 exponent range holds
-  // any scale of x0; entries below 2^-126 max |x0| lose bits, which E0 and psi do not
-  // notice), scal[1] = |r_1|, scal[0] = scal[2] = 0, coef[2] = 0 (no update before step 1)
-  const int64_t D = h->count[0] * h->count[1];
-  auto start = [&](float *r) -> int {
-    count_launch(h, 6);
-    k_exp_range<<<G, 256, 0, s>>>(D, x0, part);
-    k_scale<<<1, 256, 0, s>>>(part, G, scale);
-    k_f64_to_df<<<row_grid(h), 256, 0, s>>>(0, h->count[1], h->count[0], f->ld, x0, scale, f->slot_row, r);
-    k_df_norm2<<<G, 256, 0, s>>>(Q, r, P);
-    HUB_LAUNCH_CHECK();
-    int rc2 = reduce_partials(P, G, scal + 1, 1, s);
-    if (rc2) return rc2;
-    k_set_scal<<<1, 1, 0, s>>>(scal, 0, 0.0, 2, 0.0, -1, 0.0);
-    k_coeffs<<<1, 1, 0, s>>>(scal, coef);
-    HUB_LAUNCH_CHECK();
-    return HUB_OK;
-  };
-  // One step of the recurrence on (rp, wb, ot) = (r_{j-1}, w_{j-1}, free):
-  //   pass 1 forms r_j = w_{j-1} - (alpha_{j-1} / |r_{j-1}|) r_{j-1} over wb (fused update),
-  //   Z = (H_up + diag) r_j and |r_j|^2;  beta: scal[2] <- |r_{j-1}|, scal[1] <- |r_j|;
-  //   pass 2 writes w_j = H r_j / |r_j| - (|r_j| / |r_{j-1}|) r_{j-1} into ot and the alpha
-  //   partials <q_j, w_j>;  alpha_j -> scal[0], coef[2] <- -alpha_j / |r_j| for the next
-  //   step;  (alpha_j, |r_j|) appended to the step record.  With full == false only pass 1
-  //   and the norm (the last step of the second pass).
-  auto iteration = [&](float *rp, float *wb, float *ot, cudaStream_t st, bool full) -> int {
-    int rc2 = prof_mark(h, HUB_PROF_APPLY, true, st);
-    if (rc2) return rc2;
-    const UpdArgs U{rp, coef, P};
-    int n_norm = 0;
-    if ((rc2 = run_up(h, f, wb, f->zdf, st, 0, -1, &U, &n_norm))) return rc2;
-    if ((rc2 = reduce_partials(P, n_norm, scal + 3, 1, st))) return rc2;
-    count_launch(h, 2);
-    k_rotate_beta<<<1, 1, 0, st>>>(scal);
-    k_coeffs<<<1, 1, 0, st>>>(scal, coef);
-    HUB_LAUNCH_CHECK();
-    if (!full) return prof_mark(h, HUB_PROF_APPLY, false, st);
-    LzArgs L{wb, rp, coef, scal + 6, P};
-    if ((rc2 = run_dn(h, f, 1, wb, f->zdf, ot, L, st))) return rc2;
-    if ((rc2 = prof_mark(h, HUB_PROF_APPLY, false, st))) return rc2;
-    if ((rc2 = reduce_partials_2stage(P, (int)n_dn_blocks, P + std::max<int64_t>(n_dn_blocks, G), kTmp, scal + 0, 0,
-                                      st)))
-      return rc2;
-    count_launch(h, 2);
-    k_coeffs<<<1, 1, 0, st>>>(scal, coef);
-    k_record<<<1, 1, 0, st>>>(scal, f->d_hist, kMaxBatchSteps);
-    HUB_LAUNCH_CHECK();
-    return HUB_OK;
-  };
-  auto full_step = [&](float *rp, float *wb, float *ot, cudaStream_t st) -> int {
-    return iteration(rp, wb, ot, st, true);
-  };
-
-  float *rp = f->lz[0], *wb = f->lz[1], *ot = f->lz[2];
-  float *const vecs[3] = {f->lz[0], f->lz[1], f->lz[2]};   // step j works on (vecs[j%3], [j+1], [j+2])
-  if (!f->d_hist && !dev_alloc((void **)&f->d_hist, sizeof(double) * 2 * kMaxBatchSteps, "step record"))
-    return HUB_ERR_OOM;
-  if (!f->h_hist) HUB_CUDA(cudaMallocHost((void **)&f->h_hist, sizeof(double) * 2 * kMaxBatchSteps));
-  // Replay captured iterations unless profiling (event pairs per launch) is on; rows that
-  // take the transposed pass 1 allocate on first use and are not captured.
-  const bool graphs = !h->prof && f->staged && lz_graphs(h, f, rp, wb, ot, full_step);
-  if ((rc = start(wb))) return rc;
-  HUB_CUDA(cudaMemsetAsync(rp, 0, sizeof(float) * Dp, s));
-  HUB_CUDA(cudaMemcpyAsync(h->h_scal + 1, scal + 1, sizeof(double), cudaMemcpyDeviceToHost, s));
-  int shift = 0;
-  HUB_CUDA(cudaMemcpyAsync(&shift, scale, sizeof(int), cudaMemcpyDeviceToHost, s));
-  HUB_CUDA(cudaStreamSynchronize(s));
-  h->start_norm = std::ldexp(h->h_scal[1], shift);   // |x0|
-  if (!(h->h_scal[1] > 0.0) || !std::isfinite(h->h_scal[1]))
-    return fail(HUB_ERR_ARG, "hub_lanczos_ground: start vector is zero or not finite");
-
-  h->alpha.clear();
-  h->beta.clear();
-  // the device recurrence runs on H / |t|: its alpha and beta times |t| are those of H
-  const double tabs = std::fabs(h->t[0]);
-  // Small sectors run several steps per host read-back (a step costs less than the read-back's
-  // latency); the steps after the stopping one are discarded, so E0, the iteration count and
-  // the coefficients are those of one step per read-back.
-  const int batch = D <= kBatchStepsMaxDim ? kMaxBatchSteps : 1;
-  double E = 0.0, E_prev = 0.0;
-  LowestTracker lowest;
-  int status = HUB_ERR_NOCONV;
-  int computed = 0;                                // steps run on the device
-  bool done = false;
-  for (int j = 0; j < maxit && !done;) {
-    const int nb = std::min(batch, maxit - j);
-    count_launch(h);
-    k_set_scal<<<1, 1, 0, s>>>(scal, 7, 0.0, -1, 0.0, -1, 0.0);
-    HUB_LAUNCH_CHECK();
-    for (int b = 0; b < nb; ++b) {
-      const int jj = j + b;
-      if (graphs) {
-        HUB_CUDA(cudaGraphLaunch(f->lz_graph[jj % 3], s));
-      } else if ((rc = full_step(vecs[jj % 3], vecs[(jj + 1) % 3], vecs[(jj + 2) % 3], s))) {
-        return rc;
-      }
-    }
-    HUB_CUDA(cudaMemcpyAsync(f->h_hist, f->d_hist, sizeof(double) * 2 * nb, cudaMemcpyDeviceToHost, s));
-    HUB_CUDA(cudaStreamSynchronize(s));
-    computed = j + nb;
-    for (int b = 0; b < nb && !done; ++b) {
-      const int jj = j + b;
-      const double a_dev = f->h_hist[2 * b], r_dev = f->h_hist[2 * b + 1];   // alpha_{jj+1}, |r_{jj+1}|
-      if (!std::isfinite(r_dev)) {
-        if ((rc = fast_check_error(h))) return rc;       // a given-up wait left the step incomplete
-        return fail(HUB_ERR_CUDA, "hub_lanczos_ground: non-finite beta");
-      }
-      if (jj > 0) {
-        // |r_{jj+1}| is beta_jj, the coupling of q_jj and q_{jj+1}: on breakdown T_jj is final
-        // and this step's alpha (formed with 1/beta_jj) is dropped
-        h->beta.push_back(tabs * r_dev);
-        if (tabs * r_dev <= 1e-14 * std::fmax(1.0, std::fabs(h->alpha.back()))) {
-          status = HUB_CONVERGED_BREAKDOWN;
-          done = true;
-          break;
-        }
-      }
-      if (!std::isfinite(a_dev)) {
-        if ((rc = fast_check_error(h))) return rc;
-        return fail(HUB_ERR_CUDA, "hub_lanczos_ground: non-finite alpha");
-      }
-      h->alpha.push_back(tabs * a_dev);
-      if (tol > 0) E = lowest.next(h->alpha.data(), h->beta.data(), (int)h->alpha.size());   // else at the end
-      if (tol > 0 && jj > 0 && std::fabs(E - E_prev) < tol) {
-        status = HUB_OK;
-        done = true;
-        break;
-      }
-      E_prev = E;
-    }
-    j += nb;
-  }
-  if (tol <= 0 && status == HUB_ERR_NOCONV) status = HUB_OK;
-  if (tol <= 0 && !h->alpha.empty()) E = tridiag_lowest(h->alpha.data(), h->beta.data(), (int)h->alpha.size());
-  if ((rc = fast_check_error(h))) return rc;
-  const int last = (int)h->alpha.size() - 1;        // 0-based index of the last kept step
-  if (status != HUB_CONVERGED_BREAKDOWN && last >= 0) {
-    // beta_k = |w_k - (alpha_k / |r_k|) r_k|: recorded by the following step if it ran in the
-    // same batch, else formed now by that step's update (coef[2] is still the last step's)
-    if (last + 1 < computed && (last + 1) / batch == last / batch) {
-      h->beta.push_back(tabs * f->h_hist[2 * ((last + 1) % batch) + 1]);
-    } else {
-      count_launch(h);
-      k_df_update<<<G, 256, 0, s>>>(Q, vecs[(last + 2) % 3], vecs[(last + 1) % 3], coef, P);
-      HUB_LAUNCH_CHECK();
-      if ((rc = reduce_partials(P, G, scal + 3, 1, s))) return rc;
-      HUB_CUDA(cudaMemcpyAsync(h->h_scal + 3, scal + 3, sizeof(double), cudaMemcpyDeviceToHost, s));
-      HUB_CUDA(cudaStreamSynchronize(s));
-      h->beta.push_back(tabs * h->h_scal[3]);
-    }
-  }
-  *E0 = E;
-  const int k = (int)h->alpha.size();
-  if (iters) *iters = k;
-
-  if (psi_out) {
-    // second pass, the same deterministic steps again: psi = sum_j v_j q_j = sum_j v_j r_j / |r_j|
-    std::vector<double> vv = tridiag_vector(h->alpha.data(), h->beta.data(), k, psi_eigenvalue(h, E));
-    if ((rc = ensure_vec(&f->psi, Dp, "ground-state vector"))) return rc;
-    rp = f->lz[0];
-    wb = f->lz[1];
-    ot = f->lz[2];
-    if ((rc = start(wb))) return rc;
-    HUB_CUDA(cudaMemsetAsync(rp, 0, sizeof(float) * Dp, s));
-    HUB_CUDA(cudaMemsetAsync(f->psi, 0, sizeof(float) * Dp, s));
-    for (int j = 0; j < k; ++j) {
-      if ((rc = iteration(rp, wb, ot, s, j + 1 < k))) return rc;
-      count_launch(h, 2);
-      k_psi_coef<<<1, 1, 0, s>>>(scal, vv[j], coef);
-      k_df_axpy<<<G, 256, 0, s>>>(Q, coef, 3, wb, f->psi);
-      HUB_LAUNCH_CHECK();
-      float *t0 = rp;
-      rp = wb;
-      wb = ot;
-      ot = t0;
-    }
-    count_launch(h, 3);
-    k_df_norm2<<<G, 256, 0, s>>>(Q, f->psi, P);
-    HUB_LAUNCH_CHECK();
-    if ((rc = reduce_partials(P, G, scal + 5, 1, s))) return rc;
-    k_df_out_normalised<<<row_grid(h), 256, 0, s>>>(h->count[1], h->count[0], f->ld, f->psi, scal, 5, f->slot_of,
-                                                    psi_out);
-    HUB_LAUNCH_CHECK();
-    HUB_CUDA(cudaStreamSynchronize(s));
-    if ((rc = fast_check_error(h))) return rc;
-  }
-  if (status == HUB_ERR_NOCONV) set_error("hub_lanczos_ground: maxit reached before |dE0| < tol");
-  return status;
 }
 
 }  // namespace hub

@@ -1,0 +1,1927 @@
+// hub_fix.cu -- the product (Eq. 11) and the Lanczos recurrence (Sec. IV, V) in 64-bit fixed
+// point on the integer pipe, for uniform t and U without site energies.
+//
+// GB300 issues FP64 at about 1/70 of its integer rate, and a hopping term of the product is
+// +-t x_m: with all entries of a vector on one power-of-two grid, x_m = X_m 2^e with X_m a
+// 64-bit integer, a sum of terms is a sum of integers -- exact, and the same in any order.  What
+// limits the product is then moving the terms.
+//
+// Each spin's hops run as one of two kernels.  Gathers (k_fix_gather): rows along which the spin
+// varies are staged whole in shared memory, each thread sums the terms of its position; for up to
+// kStageMax states.  Row combinations (k_fix_comb): the rows of the order along which the other
+// spin varies are added and subtracted; for spins with more states.  Where both spins are of the
+// same kind the vector is held in both orders (count_dn x count_up and its transpose), and whoever
+// writes it -- the conversion of a caller's vector, the Lanczos update -- writes both, through a
+// shared-memory tile; where they differ one order serves both passes.  The two passes write one
+// contribution each, the second with the diagonal; k_fix_out or k_fix_update adds them.
+//
+// Grid.  |X_m| <= 2^B, B = min(56, 62 - hh), 2^hh >= the largest number of hopping terms of an
+// entry, so that no sum overflows.  A rounded entry is off by at most 1/2 of 2^e, 2^-(B+1) of
+// the vector's largest entry.  Y is kept on the grid 2^(e + g), g >= 0 chosen for the diagonal.
+//
+// Lanczos vectors.  The vectors are kept unnormalised and monic, s_{j+1} = H s_j - alpha_j s_j -
+// beta_j^2 s_{j-1} (q_j = s_j / |s_j|, beta_{j+1} = |s_{j+1}| / |s_j|), each on its own grid, so
+// only shifts and two multiplications by a 55-bit coefficient are needed per entry, and the
+// dot products <s_j, H s_j>, <s_j, s_{j-1}> and |s_{j+1}|^2 are integer sums: no result depends on
+// the order in which blocks finish.  A start vector of random numbers keeps max |s_j| / rms(s_j)
+// below 2^6.5, so an entry carries 49 bits and more below the rms, against 48 significant bits of
+// double-float arithmetic.  Against long double (12-site ring, 12 steps) alpha and beta are off by
+// 1.4e-14 and 1.8e-15 at U = 7.25, by 6e-10 and 2.5e-10 at U = 4000 (double-float 5.7e-14, 1.8e-15,
+// 1.1e-9 and 6.7e-10).
+//
+// Products for a caller (hub_apply) must keep every entry within 1e-13 (|H||x|)_n, which a grid
+// fixed by the largest entry does not give where (|H||x|)_n is small.  k_fix_out sees the entry's
+// two sums: if neither reaches the threshold that proves the bound, the entry's index is recorded
+// and k_fix_entries recomputes it in FP64.  A vector with many small entries (a sample decides
+// beforehand), or with more such entries than the list holds, is multiplied by the double-float
+// or FP64 kernels instead, all on device flags, without a host round trip.
+//
+// Measured on the 4x4 cluster at half filling (1.66e8 states): a Lanczos step 4.15 ms (passes 1.32
+// and 1.32, update 1.44) against 4.96 ms in double-float; a product 4.4 ms against 6.2 ms.
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <new>
+#include <vector>
+
+#include "hub_internal.cuh"
+
+namespace hub {
+
+std::vector<double> tridiag_vector(const double *a, const double *b, int k, double lam);
+
+typedef long long i64;
+typedef unsigned long long u64;
+
+constexpr int kFixMaxBits = 56;     // largest B
+constexpr int kFixSpare = 2;        // bits beyond B that an update may use before k_fix_rescale
+constexpr int kStageMax = 14384;    // longest rows that are staged: two of 115 KB
+constexpr int kCombCols = 128;      // columns of a combination strip: four per lane
+constexpr int kCombThreads = 256;
+constexpr int kCombPairs = 3;       // pairs of rows loaded before the first is added
+constexpr int kCombRows = 64;       // most rows of a tile
+constexpr int kTileThreads = 256;
+constexpr int kUpdateBlocks = 4;    // resident update CTAs per SM (64 registers a thread)
+constexpr int kFixSlots = 64;       // copies of the accumulators (fewer collisions of atomics)
+constexpr int kFixHist = 8;         // Lanczos steps recorded between two host read-backs
+constexpr int kFixFrac = 4;         // fraction bits of the update's sums
+
+// ctl words of a product (device): see k_fix_plan
+enum { kCtlShift = 0, kCtlSkip = 1, kCtlCount = 2, kCtlDf = 3, kCtlF64 = 4, kCtlDfScale = 6, kCtlWords = 8 };
+
+// One spin's hopping matrix as row combinations: a row's entries are ordered adding pairs,
+// subtracting pairs, then the last adding and the last subtracting one where their numbers are odd.
+struct CombLists {
+  int R;                              // rows of a tile
+  const int32_t *rp;                  // row starts
+  const uint32_t *cnt;                // adding entries | subtracting entries << 16
+  const uint32_t *word;               // entries: rows of the vector
+};
+// The same as gathers inside a row: slices of two groups of 16 positions whose schedules (see
+// k_fix_schedule) are of nearly the same length; a group is four quads of consecutive positions.  A
+// step's entry is 16 bits, the position and +-1 as the top two bits; a lane's 16 bytes are eight
+// steps, at word[(l * cap + j / 8) * 32 + lane] for step j of slice l; meta[l * 32 + lane] = the lane's position
+// | the slice's steps (even) << 16.
+struct GatherLists {
+  const uint4 *word;
+  const uint32_t *meta;
+  int cap, slices;
+};
+
+// Diagonal in fixed point: d = U n
+struct FixDiag {
+  int kind;                           // 0: zero; 1: n times an integer; 2: table of n
+  int mul;                            // kind 1: U / tau
+  int shift;                          // bits the (high) product is shifted right
+  i64 tab[32];                        // kind 2, in units of tau 2^(dh - 62)
+};
+
+// One contribution to the product: rows x positions of one order of the vector.
+struct FixPass {
+  i64 n_rows, n_pos, ld;              // ld: row stride in entries
+  const i64 *x;
+  i64 *out;
+  const uint32_t *bits_row, *bits_pos;
+  FixDiag diag;                       // kind 0 in the pass that leaves the diagonal to the other
+  int q, g;                           // 62 - B; bits the grid of the output is coarser by
+  int t_neg;                          // uniform t < 0: the sums change sign
+  int *err;                           // device error flag
+  int fail_waits;                     // test hook
+  const int *skip;                    // apply: device flag, nothing to do
+  u64 *acc;                           // Lanczos: dot product and maximum into these slots
+  struct FixScal *scal;               // Lanczos, second pass of a step: its last block ends the step
+  int second;
+};
+
+// Lanczos scalars on the device.
+struct FixScal {
+  double N, N_prev;                   // |S_j|^2 and |S_{j-1}|^2 (integers on their grids)
+  double alpha, beta2;                // of step j
+  double overlap;                     // <S_j, S_{j-1}>
+  double max_cur, max_prev;           // bounds on |S_j|, |S_{j-1}|
+  int rel;                            // exponent of S_{j-1}'s grid minus that of S_j's
+  int sh;                             // exponent of S_{j+1}'s grid minus that of S_j's
+  i64 ma, mb;                         // coefficients of the update (55-bit mantissas) ...
+  int sy, sa, sb;                     // ... and the shifts of its three terms (right, left, left)
+  double bound, ratio;                // on |S_{j+1}| on its grid; the last step's max |S_{j+1}| / bound
+  int rescale;                        // bits S_{j+1} is too large by
+  int step, hist_n;
+  unsigned ticket_dn, ticket_up;
+  double hist[3 * kFixHist];          // (alpha_j, beta_{j+1}, |S_j|^2) of the steps since the last read-back
+};
+// Accumulators: [kFixSlots][kAcc] 64-bit words: hh and mid sums split in 32-bit halves, two maxima, and
+// the sums of a second dot product
+constexpr int kAcc = 10;
+
+__device__ __forceinline__ i64 shr_any(i64 v, int s) {   // v 2^-s, truncated
+  return s >= 0 ? v >> min(s, 63) : (i64)((u64)v << min(-s, 62));
+}
+// v = hi 2^28 + lo, -2^27 <= lo < 2^27
+__device__ __forceinline__ void limbs28(i64 v, int &hi, int &lo) {
+  lo = (int)((unsigned)v << 4) >> 4;
+  hi = (int)((v - lo) >> 28);
+}
+// A vector whose rows are staged for gathers holds its entries as the two limbs, lo in the low word:
+// a sum of 8 terms +-X is then one multiply-add by +-1 per limb and term, without carries.
+__device__ __forceinline__ i64 limbs_pack(i64 v) {
+  int h, l;
+  limbs28(v, h, l);
+  return (i64)(((u64)(unsigned)h << 32) | (unsigned)l);
+}
+__device__ __forceinline__ void limbs_of(i64 p, int &hi, int &lo) {
+  lo = (int)p;
+  hi = (int)((u64)p >> 32);
+}
+__device__ __forceinline__ i64 limbs_value(int hi, int lo) { return (i64)hi * (1 << 28) + lo; }
+template <bool kLimb>
+__device__ __forceinline__ i64 fix_store(i64 v) {
+  return kLimb ? limbs_pack(v) : v;
+}
+template <bool kLimb>
+__device__ __forceinline__ void fix_load(i64 p, int &hi, int &lo) {
+  if (kLimb)
+    limbs_of(p, hi, lo);
+  else
+    limbs28(p, hi, lo);
+}
+__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {   // multiples of 16
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ i64 int2_bits(int2 v) { return (i64)(((u64)(unsigned)v.y << 32) | (unsigned)v.x); }
+__device__ __forceinline__ i64 entry_of(int2 v) { return int2_bits(v); }     // of a vector stored plainly
+// Sum of products: hh 2^56 + mid 2^28
+struct Dot {
+  i64 hh, mid;
+  __device__ __forceinline__ void add(int ah, int al, int bh, int bl) {   // 0 <= bl < 2^28, the others signed limbs
+    hh += (i64)ah * bh;
+    mid += (i64)ah * bl;
+    mid += (i64)al * bh;
+    mid += (i64)__mulhi(al << 4, bl);
+  }
+  // without the product of the low limbs: their signs are independent, so that it adds 2^-48 /
+  // sqrt(D) of the squared norms
+  __device__ __forceinline__ void add_high(int ah, int al, int bh, int bl) {
+    hh += (i64)ah * bh;
+    mid += (i64)ah * bl;
+    mid += (i64)al * bh;
+  }
+  __device__ __forceinline__ void square(int ah, int al) {
+    hh += (i64)ah * ah;
+    mid += (i64)(2 * ah) * al;
+    mid += (i64)__mulhi(al << 2, al << 2);
+  }
+};
+// Dot sums with their halves apart, so that a thread can add any number of them
+struct DotLong {
+  i64 v[4];
+  __device__ __forceinline__ void take(Dot &d) {
+    v[0] += d.hh >> 32;
+    v[1] += d.hh & 0xffffffffll;
+    v[2] += d.mid >> 32;
+    v[3] += d.mid & 0xffffffffll;
+    d.hh = d.mid = 0;
+  }
+  __device__ __forceinline__ void take_squares(Dot &d) {   // sums of squares up to 2^64
+    v[0] += (i64)((u64)d.hh >> 32) - (d.hh >> 32);
+    take(d);
+  }
+};
+
+// x = X 2^e rounded to the nearest integer X (an FP64 subnormal counts as zero)
+__device__ __forceinline__ i64 f64_to_fix(double x, int e) {
+  const u64 b = (u64)__double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  if (ex == 0) return 0;
+  const u64 m = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
+  const int s = ex - 1075 - e;
+  u64 v;
+  if (s >= 0) {
+    v = m << min(s, 8);
+  } else {
+    const int r = -s;
+    v = r >= 55 ? 0ull : (m + (1ull << (r - 1))) >> r;
+  }
+  return (b >> 63) ? -(i64)v : (i64)v;
+}
+
+// v 2^e rounded to FP64 (results in the normal range)
+__device__ __forceinline__ double fix_to_f64(i64 v, int e) {
+  if (v == 0) return 0.0;
+  const u64 sign = (u64)v & 0x8000000000000000ull;
+  u64 m = v < 0 ? (u64)0 - (u64)v : (u64)v;
+  const int lz = __clzll((i64)m);
+  m <<= lz;
+  u64 r = m >> 11;
+  const unsigned rem = (unsigned)m & 0x7ffu;
+  r += (rem > 0x400u || (rem == 0x400u && (r & 1ull))) ? 1ull : 0ull;
+  const int E = 63 - lz + e + 1023;
+  return __longlong_as_double((i64)(sign | (((u64)(unsigned)(E - 1) << 52) + r)));
+}
+
+// ---------------------------------------------------------------------------------------
+// Scale and route of a caller's vector.  partials: k_exp_range's, nblk maxima then nblk minima
+// of the biased exponents.  ctl[kCtlShift]: exponent of max |x|; [kCtlSkip]: not for this path;
+// [kCtlF64] / [kCtlDf]: the FP64 / double-float kernels multiply it instead.  A vector outside
+// the double-float window (kExp*) goes to FP64 as before.  `wide` vectors -- more than one in
+// eight of 4096 sampled entries below 2^-8 of the largest -- would fill the list of entries to
+// recompute; random numbers have 2 % there (max 6 sigma), a ground state of the 12-site ring
+// 40 % and more.  Only time depends on the sample: the list catches what it misses.
+// ---------------------------------------------------------------------------------------
+constexpr int kPlanThreads = 256, kPlanSamples = 4096;
+__global__ void k_fix_plan(const int *__restrict__ partials, int nblk, i64 D, const double *__restrict__ x, int df_ok,
+                           int *__restrict__ ctl) {
+  __shared__ int smax, smin, small;
+  if (threadIdx.x == 0) {
+    smax = 0;
+    smin = 2048;
+    small = 0;
+  }
+  __syncthreads();
+  int a = 0, c = 2048;
+  for (int k = threadIdx.x; k < nblk; k += blockDim.x) {
+    a = max(a, partials[k]);
+    c = min(c, partials[nblk + k]);
+  }
+  atomicMax(&smax, a);
+  atomicMin(&smin, c);
+  __syncthreads();
+  const int emax = smax, emin = smin;
+  int n = 0;
+  {
+    const i64 step = D > kPlanSamples ? D / kPlanSamples : 1;
+    for (int k = threadIdx.x; k < kPlanSamples; k += blockDim.x) {
+      const i64 at = k * step;
+      if (at < D) n += (int)(((u64)__double_as_longlong(x[at]) >> 52) & 0x7ff) < emax - 8 ? 1 : 0;
+    }
+    atomicAdd(&small, n);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const bool out = emax != 0 && (emax < kExpLo || emax > kExpHi || emin < emax - kExpSpan);
+    const i64 samples = D < kPlanSamples ? D : kPlanSamples;
+    const bool wide = emax == 0 || 8 * (i64)small > samples;
+    ctl[kCtlShift] = ctl[kCtlDfScale] = emax == 0 ? 0 : emax - 1023;
+    ctl[kCtlDfScale + 1] = 0;
+    ctl[kCtlSkip] = out || wide ? 1 : 0;
+    ctl[kCtlCount] = 0;
+    ctl[kCtlDf] = !out && wide && df_ok ? 1 : 0;
+    ctl[kCtlF64] = out || (wide && !df_ok) ? 1 : 0;
+  }
+}
+
+// A thread's sums (N = 4: one dot product, 8: two) into the block's slot; vmax (top word of the
+// largest magnitude) into maximum number `which`.
+template <int N>
+__device__ __forceinline__ void block_sums(i64 (&v)[N], unsigned vmax, int which, u64 *__restrict__ acc) {
+  __shared__ i64 sv[N][32];
+  __shared__ unsigned sm[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
+  const i64 total = warp_totals<N>(v);
+  vmax = __reduce_max_sync(0xffffffffu, vmax);
+  if (lane < N) sv[lane][warp] = total;
+  if (lane == 0) sm[warp] = vmax;
+  __syncthreads();
+  if (warp == 0) {
+    u64 *slot = acc + (size_t)(blockIdx.x % kFixSlots) * kAcc;
+    if (lane < N) {
+      i64 t = 0;
+      for (int k = 0; k < nw; ++k) t += sv[lane][k];
+      atomicAdd(slot + (lane < 4 ? lane : lane + 2), (u64)t);
+    }
+    vmax = __reduce_max_sync(0xffffffffu, lane < nw ? sm[lane] : 0u);
+    if (lane == 0) atomicMax(slot + 4 + which, (u64)vmax);
+  }
+}
+
+// True in exactly one block, the last to arrive; all slots are then complete.  Leaves the
+// ticket at zero.
+__device__ __forceinline__ bool last_block(unsigned *ticket) {
+  __shared__ bool last;
+  if (threadIdx.x < 32) __threadfence();     // the adding threads
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (last && threadIdx.x == 0) *ticket = 0;
+  return last;
+}
+
+// hh 2^56 + mid 2^28 of summed halves as a double, exact to 2^-53 of the total
+__device__ __forceinline__ double dot_value(const i64 *s) {
+  const i64 mid_hi = s[2] + (s[3] >> 32), mid_lo = s[3] & 0xffffffffll;
+  const i64 hh_hi = s[0] + (s[1] >> 32), hh_lo = s[1] & 0xffffffffll;
+  return (double)hh_hi * 0x1p88 + ((double)hh_lo * 0x1p56 + ((double)mid_hi * 0x1p60 + (double)mid_lo * 0x1p28));
+}
+// Sums of the slots (first warp): the two dot products and bounds on the two maxima; the slots are
+// left at zero for the next kernel.
+struct SlotSums {
+  double dot, dot2, max0, max1;
+};
+__device__ __forceinline__ SlotSums take_slots(u64 *acc) {
+  __threadfence();
+  i64 s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  unsigned m0 = 0, m1 = 0;
+  for (int k = threadIdx.x; k < kFixSlots; k += 32) {
+    u64 *p = acc + (size_t)k * kAcc;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      s[i] += (i64)__ldcg(p + i);
+      s[4 + i] += (i64)__ldcg(p + 6 + i);
+    }
+    m0 = max(m0, (unsigned)__ldcg(p + 4));
+    m1 = max(m1, (unsigned)__ldcg(p + 5));
+    for (int i = 0; i < kAcc; ++i) p[i] = 0;
+  }
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s[i] += __shfl_xor_sync(0xffffffffu, s[i], o);
+  return SlotSums{dot_value(s), dot_value(s + 4), ((double)__reduce_max_sync(0xffffffffu, m0) + 1.0) * 0x1p32,
+                  ((double)__reduce_max_sync(0xffffffffu, m1) + 1.0) * 0x1p32};
+}
+
+// diag(row, position) X on the output's grid, X = xh 2^28 + xl
+__device__ __forceinline__ i64 diag_term(const FixPass &P, const i64 *__restrict__ tab, uint32_t Ir, uint32_t Ip,
+                                         int xh, int xl) {
+  const FixDiag &G = P.diag;
+  const uint32_t both = Ir & Ip;
+  if (G.kind == 1) {
+    const int k = G.mul * __popc(both);
+    const i64 v = (i64)xl * k + ((i64)xh * k) * (1 << 28);
+    return G.shift ? (v + (1ll << (G.shift - 1))) >> G.shift : v;
+  }
+  const i64 X = limbs_value(xh, xl);
+  return shr_any(__mul64hi(tab[__popc(both)], (i64)((u64)X << P.q)), G.shift);
+}
+
+// An entry of a pass: hopping sum s, own entry X.  Returns the output; kLz: adds to the dot
+// product <X, output 2^-7> and the maximum.
+template <bool kLz>
+__device__ __forceinline__ i64 pass_entry(const FixPass &P, const i64 *__restrict__ tab, i64 s, int xh, int xl,
+                                          uint32_t Ir, uint32_t Ip, Dot &dot, unsigned &vmax) {
+  if (P.g) s = (s + (1ll << (P.g - 1))) >> P.g;
+  if (P.diag.kind) s += diag_term(P, tab, Ir, Ip, xh, xl);
+  if (kLz) {
+    const int yh = (int)((u64)s >> 32);
+    dot.add(xh, xl, yh >> 3, (int)((unsigned)(s >> 7) & 0x0fffffffu));
+    vmax = max(vmax, (unsigned)abs(yh));
+  }
+  return s;
+}
+
+// The end of a pass: sums into the slots; the last block of a step's second pass turns them into
+// alpha_j and the coefficients of the update
+//   S_{j+1} = 2^-sh (2^g (out_1 + out_2) - alpha S_j - beta^2 2^rel S_{j-1}),
+// sh from a bound on its entries, which keeps them below 2^(B + kFixSpare), and from the part of the
+// bound that the last step's largest entry reached (a third as a rule, nearly the same from step to
+// step), so that they come to lie between 2^(B-1) and 2^B; where they do not, k_fix_rescale takes
+// the spare bits off.
+__device__ __forceinline__ void pass_end(const FixPass &P, const DotLong &dot, unsigned vmax) {
+  i64 v[4] = {dot.v[0], dot.v[1], dot.v[2], dot.v[3]};
+  block_sums<4>(v, vmax, P.second, P.acc);
+  if (!P.second || !last_block(&P.scal->ticket_dn) || threadIdx.x >= 32) return;
+  const SlotSums t = take_slots(P.acc);
+  const double d = t.dot * 128.0, m0 = t.max0, m1 = t.max1;
+  if (threadIdx.x != 0) return;
+  FixScal &q = *P.scal;
+  const int B = 62 - P.q;
+  // alpha_j = <q_j, H q_j - beta_j q_{j-1}>: the overlap of S_j and S_{j-1} is rounding only, but
+  // without its term it would double from step to step
+  const double bp = ldexp(q.beta2, q.rel), G = (double)(1ll << P.g), alpha = (d * G - bp * q.overlap) / q.N;
+  const double bound = (m0 + m1) * G + fabs(alpha) * q.max_cur + bp * q.max_prev;
+  int sh = 0, least = 0, xa = 0, xb = 0;
+  frexp(bound, &least);                    // bound < 2^least
+  frexp(bound * fmin(1.0, 1.05 * q.ratio), &sh);
+  sh = max(sh - B, least - B - kFixSpare);
+  q.bound = ldexp(bound, -sh);
+  const double fa = frexp(ldexp(alpha, -sh), &xa), fb = frexp(ldexp(bp, -sh), &xb);
+  q.alpha = alpha;
+  q.sh = sh;
+  q.ma = (i64)ldexp(fa, 55);
+  q.mb = (i64)ldexp(fb, 55);
+  q.sy = sh - P.g - kFixFrac;
+  q.sa = xa + kFixFrac + 1;                // fa 2^55 S 2^-56 2^sa = alpha 2^-sh S 2^kFixFrac
+  q.sb = xb + kFixFrac + 1;
+}
+
+// ---------------------------------------------------------------------------------------
+// Gathers: the hops of the positions' spin.  A CTA stages two rows of the vector whole in shared
+// memory (bulk copies completing on an mbarrier), then each thread sums the hopping row of its
+// position for both rows.  What bounds it is the shared-memory bandwidth, 8 bytes per term, so the
+// schedule lets a half-warp's 16 eight-byte loads hit 16 different bank pairs (position mod
+// 16), idle steps reading a zero of a bank left free.  Issue slots come next: a term's sign is a
+// factor +-1 of one multiply-add per limb, which leaves the schedule free to mix signs (steps of one
+// sign each save a third of the instructions but need 13 % more steps, and ran 20 % slower).
+// ---------------------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t phase) {   // bounded: about 2^24 polls
+  for (uint32_t it = 0; it < (1u << 24); ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(smem_addr(bar)), "r"(phase)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+
+// kPlane: entries from one staged row to the next (a constant, so that both rows' loads of a term
+// share one address).  kLimb: entries stored as limbs.
+template <int kPlane, bool kLz, bool kLimb>
+__global__ void __launch_bounds__(1024, 1) k_fix_gather(const FixPass P, const GatherLists L) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  int2 *const x0 = reinterpret_cast<int2 *>(smem), *const x1 = x0 + kPlane;   // entries ld .. ld + 15 are zero
+  __shared__ __align__(8) uint64_t bar;
+  __shared__ i64 utab[32];
+  if (P.skip && __ldg(P.skip)) return;
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid < 32) {
+    utab[tid] = P.diag.tab[tid];
+    (tid < 16 ? x0 : x1)[P.ld + (tid & 15)] = make_int2(0, 0);     // idle steps read one of these
+  }
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  const uint32_t bytes = (uint32_t)(P.ld * sizeof(i64));
+  const i64 pairs = (P.n_rows + 1) / 2;
+  const int n_pos = (int)P.n_pos;
+  uint32_t phase = 0;
+  DotLong dots{{0, 0, 0, 0}};
+  unsigned vmax = 0;
+  for (i64 p = blockIdx.x; p < pairs; p += gridDim.x) {
+    const i64 r0 = 2 * p;
+    const bool two = r0 + 1 < P.n_rows;
+    const i64 *s0 = P.x + r0 * P.ld, *s1 = two ? s0 + P.ld : s0;   // odd tail: the same row twice
+    if (tid == 0) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&bar)), "r"(2 * bytes)
+                   : "memory");
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                       smem_addr(x0)),
+                   "l"(s0), "r"(bytes), "r"(smem_addr(&bar))
+                   : "memory");
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                       smem_addr(x1)),
+                   "l"(s1), "r"(bytes), "r"(smem_addr(&bar))
+                   : "memory");
+      const i64 pn = p + gridDim.x;           // the CTA's next pair into L2 meanwhile
+      if (pn < pairs)
+        prefetch_l2(P.x + 2 * pn * P.ld, 2 * pn + 1 < P.n_rows ? 2 * bytes : bytes);
+    }
+    const uint32_t I0 = P.diag.kind ? P.bits_row[r0] : 0u, I1 = P.diag.kind && two ? P.bits_row[r0 + 1] : I0;
+    if (!mbar_wait(&bar, phase)) {
+      if (tid == 0) atomicExch(P.err, 1);
+      mbar_wait(&bar, phase);                 // give a late copy one more bounded chance to land
+      return;
+    }
+    if (P.fail_waits) {                       // test hook: the same exit, after the copies landed
+      if (tid == 0) atomicExch(P.err, 1);
+      return;
+    }
+    phase ^= 1u;
+    i64 *const o0 = P.out + r0 * P.ld, *const o1 = o0 + P.ld;
+    Dot dot{0, 0};
+    const int nw = (int)(blockDim.x >> 5);
+    const uint4 *__restrict__ wp = L.word + (uint32_t)((tid >> 5) * L.cap * 32 + lane);
+    int sl = tid >> 5;
+    uint32_t meta = 0;
+    uint4 qn = make_uint4(0u, 0u, 0u, 0u);
+    if (sl < L.slices) {
+      meta = L.meta[sl * 32 + lane];
+      qn = wp[0];
+    }
+    for (; sl < L.slices; sl += nw) {
+      const int s = (int)(meta & 0xffffu);
+      int n = (int)(meta >> 16);
+      const uint4 *__restrict__ w4 = wp;
+      wp += (uint32_t)(nw * L.cap * 32);
+      const bool more = sl + nw < L.slices;
+      if (more) meta = L.meta[(sl + nw) * 32 + lane];
+      i64 a0 = 0, a1 = 0;
+#define FIX_TERM(ADDR, SGN)                                                  \
+  do {                                                                       \
+    const int2 *at_ = reinterpret_cast<const int2 *>(smem + (ADDR));         \
+    const int2 u_ = at_[0], v_ = at_[kPlane];                                \
+    const int s_ = (SGN);                                                    \
+    if (kLimb) {                                                             \
+      l0 = u_.x * s_ + l0;                                                   \
+      h0 = u_.y * s_ + h0;                                                   \
+      l1 = v_.x * s_ + l1;                                                   \
+      h1 = v_.y * s_ + h1;                                                   \
+    } else {                                                                 \
+      a0 += s_ < 0 ? -entry_of(u_) : entry_of(u_);                           \
+      a1 += s_ < 0 ? -entry_of(v_) : entry_of(v_);                           \
+    }                                                                        \
+  } while (0)
+#define FIX_WORD(W)                                                          \
+  do {                                                                       \
+    const uint32_t w_ = (W);                                                 \
+    FIX_TERM((w_ << 3) & 0x1fff8u, (int)(w_ << 16) >> 30);                   \
+    FIX_TERM((w_ >> 13) & 0x1fff8u, (int)w_ >> 30);                          \
+  } while (0)
+      for (; n > 0; n -= 8) {
+        const uint4 q = qn;
+        int h0 = 0, l0 = 0, h1 = 0, l1 = 0;   // limb sums of 8 terms, below 2^31
+        if (n >= 8) {
+          w4 += 32;
+          if (n > 8) qn = w4[0];              // next batch in flight
+          FIX_WORD(q.x);
+          FIX_WORD(q.y);
+          FIX_WORD(q.z);
+          FIX_WORD(q.w);
+        } else {
+          FIX_WORD(q.x);
+          if (n > 2) FIX_WORD(q.y);
+          if (n > 4) FIX_WORD(q.z);
+        }
+        if (kLimb) {
+          a0 += limbs_value(h0, l0);
+          a1 += limbs_value(h1, l1);
+        }
+      }
+#undef FIX_WORD
+#undef FIX_TERM
+      if (more) qn = wp[0];                   // the next slice's first batch
+      if (P.t_neg) {
+        a0 = -a0;
+        a1 = -a1;
+      }
+      if (s >= n_pos) continue;
+      const uint32_t Ip = P.diag.kind ? P.bits_pos[s] : 0u;
+      const int2 u = x0[s], v = x1[s];
+      int uh, ul, vh, vl;
+      fix_load<kLimb>(int2_bits(u), uh, ul);
+      fix_load<kLimb>(int2_bits(v), vh, vl);
+      o0[s] = pass_entry<kLz>(P, utab, a0, uh, ul, I0, Ip, dot, vmax);
+      if (two) o1[s] = pass_entry<kLz>(P, utab, a1, vh, vl, I1, Ip, dot, vmax);
+    }
+    if (kLz) dots.take(dot);
+    __syncthreads();
+  }
+  if (kLz) pass_end(P, dots, vmax);
+}
+
+// Schedule of a group of 16 positions, the lanes of a half-warp: a colouring of the bipartite graph
+// lanes x banks (position mod 16) whose edges are the group's entries -- no two edges of a lane or
+// of a bank share a step.  By Koenig's theorem as many steps suffice as the largest degree has
+// edges; they are found edge by edge, exchanging two colours along an alternating path where the
+// lane and the bank have no free step in common.  A bank with more entries than cap_steps takes
+// the rest in steps of its lanes alone (conflicts, but the schedule stays bounded).  One thread
+// per group (quads 4 g .. 4 g + 3 of quad).  deg[g] = its steps.
+constexpr int kSchedRow = 64;         // longest hopping row of the gather form
+constexpr int kSchedMax = 2 * kSchedRow;
+constexpr uint16_t kNoEntry = 0xffff;
+__global__ void __launch_bounds__(32) k_fix_schedule(int n, int groups, int idle, int cap_steps,
+                                                     const int32_t *__restrict__ quad,
+                                                     const int32_t *__restrict__ rp,
+                                                     const uint32_t *__restrict__ scol, uint16_t *__restrict__ word,
+                                                     uint16_t *__restrict__ deg) {
+  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= groups) return;
+  uint16_t at[16][kSchedMax];         // entry of a lane at a step
+  int8_t who[16][kSchedMax];          // lane that reads a bank at a step
+  int load[16];
+  for (int b = 0; b < 16; ++b) {
+    load[b] = 0;
+    for (int j = 0; j < cap_steps; ++j) {
+      at[b][j] = kNoEntry;
+      who[b][j] = -1;
+    }
+  }
+  int steps = 0;
+  for (int l = 0; l < 16; ++l) {
+    const int r = quad[4 * g + (l >> 2)] * 4 + (l & 3);
+    if (r >= n) continue;
+    steps = max(steps, rp[r + 1] - rp[r]);
+    for (int32_t k = rp[r]; k < rp[r + 1]; ++k) ++load[scol[k] & 15];
+  }
+  for (int b = 0; b < 16; ++b) steps = max(steps, load[b]);
+  steps = min(steps, cap_steps);
+  for (int l = 0; l < 16; ++l) {
+    const int r = quad[4 * g + (l >> 2)] * 4 + (l & 3);
+    if (r >= n) continue;
+    for (int32_t k = rp[r]; k < rp[r + 1]; ++k) {
+      const uint32_t w = scol[k];
+      const uint16_t v = (uint16_t)((w & 0x3fffu) | (w >> 31 ? 0x4000u : 0xc000u));     // esign -1 adds
+      const int b = w & 15;
+      int x = -1, y = -1;             // a free step of the lane, one of the bank, one of both
+      for (int j = 0; j < steps; ++j) {
+        const bool fl = at[l][j] == kNoEntry, fb = who[b][j] < 0;
+        if (fl && fb) {
+          x = y = j;
+          break;
+        }
+        if (fl && x < 0) x = j;
+        if (fb && y < 0) y = j;
+      }
+      bool ok = y >= 0;
+      if (ok && x != y) {
+        // exchange steps x and y along the path b -x- lane -y- bank -x- ...: frees step x of b
+        int8_t pl[34], pb[34];
+        uint16_t pv[34];
+        int m = 0;
+        for (int cb = b; ok;) {
+          const int l1 = who[cb][x];
+          if (l1 < 0) break;
+          pl[m] = (int8_t)l1;
+          pb[m] = (int8_t)cb;
+          pv[m++] = at[l1][x];
+          const uint16_t v2 = at[l1][y];
+          if (v2 == kNoEntry) break;
+          cb = v2 & 15;
+          pl[m] = (int8_t)l1;
+          pb[m] = (int8_t)cb;
+          pv[m++] = v2;
+          ok = who[cb][y] == l1 && m < 32;   // else it meets an entry without a bank of its own
+        }
+        for (int i = 0; ok && i < m; ++i) {
+          at[(int)pl[i]][i & 1 ? y : x] = kNoEntry;
+          who[(int)pb[i]][i & 1 ? y : x] = -1;
+        }
+        for (int i = 0; ok && i < m; ++i) {
+          at[(int)pl[i]][i & 1 ? x : y] = pv[i];
+          who[(int)pb[i]][i & 1 ? x : y] = pl[i];
+        }
+      }
+      at[l][x] = v;                   // the lane has a free step: steps >= its entries
+      if (ok) who[b][x] = (int8_t)l;
+    }
+  }
+  // idle lanes read the zero of a bank the step leaves free
+  uint16_t *out = word + (size_t)g * cap_steps * 16;
+  for (int j = 0; j < cap_steps; ++j) {
+    int fb = 0;
+    while (fb < 15 && who[fb][j] >= 0) ++fb;
+    const uint16_t z = (uint16_t)((idle + ((fb - idle) & 15)) | 0x4000);
+    for (int l = 0; l < 16; ++l) out[j * 16 + l] = at[l][j] == kNoEntry ? z : at[l][j];
+  }
+  deg[g] = (uint16_t)steps;
+}
+// The groups' schedules side by side in the slices' layout.
+__global__ void k_fix_pack(const int32_t *__restrict__ group, int cap_steps, const uint16_t *__restrict__ in,
+                           uint16_t *__restrict__ word) {
+  const int sl = blockIdx.x, lane = threadIdx.x, g = group[2 * sl + (lane >> 4)];
+  for (int j = 0; j < cap_steps; ++j)
+    word[(((size_t)sl * (cap_steps / 8) + (j >> 3)) * 32 + lane) * 8 + (j & 7)] =
+        in[((size_t)g * cap_steps + j) * 16 + (lane & 15)];
+}
+
+// ---------------------------------------------------------------------------------------
+// Row combinations: the hops of the rows' spin, where its rows are too long to stage.  Tile = R rows x 128 columns; tiles of one column strip are adjacent in the
+// grid, so that the strip of x (n_rows x 128 values, 13 MB at 4x4) stays in L2 while all its
+// row tiles combine it.  A warp takes a row at a time, lane l the columns 2l, 2l + 1, 64 + 2l and
+// 65 + 2l: every load is a coalesced 512-byte segment, the index, address and branch work of an
+// entry is shared by 128 sums, and pairs of equal sign take one three-operand add per word.
+// ---------------------------------------------------------------------------------------
+
+// four columns of a lane
+struct Quad {
+  i64 v[4];
+};
+__device__ __forceinline__ Quad ld_quad(const char *__restrict__ p, uint32_t up) {
+  const longlong2 a = *reinterpret_cast<const longlong2 *>(p), b = *reinterpret_cast<const longlong2 *>(p + up);
+  return Quad{{a.x, a.y, b.x, b.y}};
+}
+
+// A hopping row (entries k0 ..) summed over the lane's columns into s.  w: the words of its first
+// 32 entries, one per lane (loaded while the previous row was summed); longer rows take them 32
+// at a time.  up: byte offset of the lane's second pair of columns (0 where it has none).
+__device__ __forceinline__ void comb_row(const CombLists &S, const char *__restrict__ xb, uint32_t row_bytes, uint32_t up,
+                                         int lane, int32_t k0, uint32_t cnt, uint32_t w, Quad &s) {
+  constexpr int kP = kCombPairs;
+  const int na = cnt & 0xffff, ns = cnt >> 16, all = na + ns;
+  const int pa = na & ~1, pe = pa + (ns & ~1);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) s.v[i] = 0;
+  for (int base = 0; base < all; base += 32) {
+    if (base) w = S.word[k0 + base + lane];
+    const int n = min(32, all - base);
+    const int np = min(max(pe - base, 0), n), ae = pa - base;    // paired entries here, adding ones first
+    Quad o0, o1;                                                 // the odd ones
+    const bool odd0 = np < n, odd1 = np + 1 < n;
+    const uint32_t c0 = __shfl_sync(0xffffffffu, w, np & 31), c1 = __shfl_sync(0xffffffffu, w, (np + 1) & 31);
+    if (odd0) o0 = ld_quad(xb + (u64)c0 * row_bytes, up);
+    if (odd1) o1 = ld_quad(xb + (u64)c1 * row_bytes, up);
+    for (int j = 0; j < np; j += 2 * kP) {
+      Quad v[2 * kP];
+#pragma unroll
+      for (int t = 0; t < kP; ++t) {
+        const uint32_t ca = __shfl_sync(0xffffffffu, w, j + 2 * t), cb = __shfl_sync(0xffffffffu, w, j + 2 * t + 1);
+        if (j + 2 * t < np) {
+          v[2 * t] = ld_quad(xb + (u64)ca * row_bytes, up);
+          v[2 * t + 1] = ld_quad(xb + (u64)cb * row_bytes, up);
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < kP; ++t) {
+        if (j + 2 * t < ae) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) s.v[i] = s.v[i] + v[2 * t].v[i] + v[2 * t + 1].v[i];
+        } else if (j + 2 * t < np) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) s.v[i] = s.v[i] - v[2 * t].v[i] - v[2 * t + 1].v[i];
+        }
+      }
+    }
+    if (odd0) {                       // the adding one, unless there is none
+      if (na & 1) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s.v[i] += o0.v[i];
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s.v[i] -= o0.v[i];
+      }
+    }
+    if (odd1) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s.v[i] -= o1.v[i];
+    }
+  }
+}
+
+template <bool kLz>
+__global__ void __launch_bounds__(kCombThreads, 2) k_fix_comb(const FixPass P, const CombLists S) {
+  constexpr int kWarps = kCombThreads / 32;
+  __shared__ i64 utab[32];
+  if (P.skip && __ldg(P.skip)) return;
+  if (P.fail_waits) {                       // test hook: report as a given-up wait would
+    if (threadIdx.x == 0) atomicExch(P.err, 1);
+    return;
+  }
+  if (threadIdx.x < 32) utab[threadIdx.x] = P.diag.tab[threadIdx.x];
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t tiles = (uint32_t)((P.n_rows + S.R - 1) / S.R);
+  const uint32_t strip = blockIdx.x / tiles;
+  const i64 r0 = (i64)(blockIdx.x - strip * tiles) * S.R;
+  const int nr = (int)min((i64)S.R, P.n_rows - r0);
+  // the lane's columns c, c + 1 and c + 64, c + 65; lanes past the last column repeat the first
+  // one (their sums are dropped)
+  const i64 c = (i64)strip * kCombCols + 2 * lane;
+  const bool in[2] = {c < P.n_pos, c + 64 < P.n_pos}, second[2] = {c + 1 < P.n_pos, c + 65 < P.n_pos};
+  const uint32_t row_bytes = (uint32_t)(P.ld * sizeof(i64)), up = in[1] ? 512u : 0u;
+  const char *__restrict__ xb = reinterpret_cast<const char *>(P.x + (in[0] ? c : 0));
+  uint32_t Ip[4] = {0, 0, 0, 0};
+  if (P.diag.kind) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const i64 u = c + 64 * (i >> 1) + (i & 1);
+      if (u < P.n_pos) Ip[i] = P.bits_pos[u];
+    }
+  }
+  // the warp's rows are warp, warp + kWarps, ...: start, counts and words of the next one are
+  // loaded while the current one is summed
+  int32_t k0 = 0, k0n = 0;
+  uint32_t cnt = 0, cntn = 0, w = 0;
+  if (warp < nr) {
+    k0 = S.rp[r0 + warp];
+    cnt = S.cnt[r0 + warp];
+    w = S.word[k0 + lane];                   // padded by 32 words
+  }
+  if (warp + kWarps < nr) {
+    k0n = S.rp[r0 + warp + kWarps];
+    cntn = S.cnt[r0 + warp + kWarps];
+  }
+  DotLong dots{{0, 0, 0, 0}};
+  unsigned vmax = 0;
+#pragma unroll 1
+  for (int rr = warp; rr < nr; rr += kWarps) {
+    Quad s;
+    const i64 d = r0 + rr;
+    uint32_t wn = 0, cnt2 = 0;
+    int32_t k2 = 0;
+    if (rr + kWarps < nr) wn = S.word[k0n + lane];
+    if (rr + 2 * kWarps < nr) {
+      k2 = S.rp[d + 2 * kWarps];
+      cnt2 = S.cnt[d + 2 * kWarps];
+    }
+    comb_row(S, xb, row_bytes, up, lane, k0, cnt, w, s);
+    if (P.t_neg) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s.v[i] = -s.v[i];
+    }
+    k0 = k0n;
+    cnt = cntn;
+    w = wn;
+    k0n = k2;
+    cntn = cnt2;
+    const uint32_t Ir = P.diag.kind ? P.bits_row[d] : 0u;
+    Dot dot{0, 0};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (!in[h]) break;
+      const i64 at = d * P.ld + c + 64 * h;
+      const longlong2 xv = *reinterpret_cast<const longlong2 *>(P.x + at);
+      int xh, xl;
+      limbs28(xv.x, xh, xl);
+      const i64 y0 = pass_entry<kLz>(P, utab, s.v[2 * h], xh, xl, Ir, Ip[2 * h], dot, vmax);
+      i64 y1 = 0;
+      if (second[h]) {
+        limbs28(xv.y, xh, xl);
+        y1 = pass_entry<kLz>(P, utab, s.v[2 * h + 1], xh, xl, Ir, Ip[2 * h + 1], dot, vmax);
+      }
+      *reinterpret_cast<longlong2 *>(P.out + at) = make_longlong2(y0, y1);
+    }
+    if (kLz) dots.take(dot);
+  }
+  if (kLz) pass_end(P, dots, vmax);
+}
+
+// ---------------------------------------------------------------------------------------
+// Kernels that write both orders: tiles of 64 x 64 entries, rows read and written as 512-byte
+// segments, the transposed copy through shared memory.  HBM-bound.
+// ---------------------------------------------------------------------------------------
+
+// T x T tile t of a transposed matrix (its rows c0 .., positions r0 ..) between memory and shared
+// memory, which holds it as [row][position] of the untransposed one.  A thread has two entries of
+// T / 2 T / 256 rows; an odd last position comes with the padding behind it.
+template <int T>
+struct TileBuf {
+  i64 v[T][T + 1];
+};
+template <int T>
+struct TileAt {                       // the thread's place: columns c, c + 1 of rows k0, k0 + kStep, ..
+  static constexpr int kStep = 2 * kTileThreads / T;
+  const int c = 2 * (int)(threadIdx.x % (T / 2)), k0 = (int)(threadIdx.x / (T / 2));
+};
+template <int T>
+__device__ __forceinline__ void tile_in_t(TileBuf<T> &t, const i64 *__restrict__ m, i64 ldm, i64 r0, i64 c0, i64 n_r,
+                                          i64 n_c) {
+  const TileAt<T> at;
+#pragma unroll
+  for (int i = 0; i < T / TileAt<T>::kStep; ++i) {
+    const int k = at.k0 + i * TileAt<T>::kStep;
+    if (c0 + k < n_c && r0 + at.c < n_r) {
+      const longlong2 v = *reinterpret_cast<const longlong2 *>(m + (c0 + k) * ldm + r0 + at.c);
+      t.v[at.c][k] = v.x;
+      t.v[at.c + 1][k] = v.y;
+    }
+  }
+}
+template <int T>
+__device__ __forceinline__ void tile_out_t(const TileBuf<T> &t, i64 *__restrict__ m, i64 ldm, i64 r0, i64 c0, i64 n_r,
+                                           i64 n_c) {
+  const TileAt<T> at;
+#pragma unroll
+  for (int i = 0; i < T / TileAt<T>::kStep; ++i) {
+    const int k = at.k0 + i * TileAt<T>::kStep;
+    if (c0 + k < n_c && r0 + at.c < n_r)
+      *reinterpret_cast<longlong2 *>(m + (c0 + k) * ldm + r0 + at.c) = make_longlong2(t.v[at.c][k], t.v[at.c + 1][k]);
+  }
+}
+// Corner of a tile, rows of tiles in turn (numbered along strips of 24 tile columns, so that the tiles in
+// work cover a square, the update took 1.60 ms instead of 1.44 at 4x4).
+template <int T>
+__device__ __forceinline__ void tile_at(uint32_t tile, i64 n_c, i64 *r0, i64 *c0) {
+  const uint32_t tx = (uint32_t)((n_c + T - 1) / T), by = tile / tx;
+  *c0 = (i64)(tile - by * tx) * T;
+  *r0 = (i64)by * T;
+}
+__device__ __forceinline__ double2 ld_two(const double *p, bool vec, bool second) {
+  if (vec) return *reinterpret_cast<const double2 *>(p);
+  return make_double2(p[0], second ? p[1] : 0.0);
+}
+
+// X (stride ld) and XT (transposed, stride ldt), either may be null, from FP64 x (n_r x n_c) on the
+// grid of ctl[kCtlShift].  acc != null: also |X|^2 into the slots.
+template <int T, bool kLimb>
+__global__ void __launch_bounds__(kTileThreads) k_fix_in(i64 n_r, i64 n_c, i64 ld, i64 ldt,
+                                                         const double *__restrict__ x, const int *__restrict__ ctl,
+                                                         int use_skip, int B, i64 *__restrict__ X,
+                                                         i64 *__restrict__ XT, u64 *__restrict__ acc) {
+  __shared__ TileBuf<T> t;
+  if (use_skip && __ldg(ctl + kCtlSkip)) return;
+  const int e = ctl[kCtlShift] - (B - 2);
+  i64 r0, c0;
+  tile_at<T>(blockIdx.x, n_c, &r0, &c0);
+  const TileAt<T> at;
+  const i64 u = c0 + at.c;
+  const bool in = u < n_c, second = u + 1 < n_c;
+  const bool vec = (n_c & 1) == 0 && ((uintptr_t)x & 15) == 0;
+  constexpr int kN = T / TileAt<T>::kStep;
+  double2 xv[kN];
+#pragma unroll
+  for (int i = 0; i < kN; ++i) {
+    const i64 d = r0 + at.k0 + i * TileAt<T>::kStep;
+    xv[i] = make_double2(0.0, 0.0);
+    if (d < n_r && in) xv[i] = ld_two(x + d * n_c + u, vec, second);
+  }
+  Dot dot{0, 0};
+#pragma unroll
+  for (int i = 0; i < kN; ++i) {
+    const int k = at.k0 + i * TileAt<T>::kStep;
+    i64 v[2] = {f64_to_fix(xv[i].x, e), f64_to_fix(xv[i].y, e)};
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      if (acc) {
+        int h, l;
+        limbs28(v[j], h, l);
+        dot.square(h, l);
+      }
+      v[j] = fix_store<kLimb>(v[j]);
+      t.v[k][at.c + j] = v[j];
+    }
+    if (X && r0 + k < n_r && in) *reinterpret_cast<longlong2 *>(X + (r0 + k) * ld + u) = make_longlong2(v[0], v[1]);
+  }
+  if (XT) {
+    __syncthreads();
+    tile_out_t<T>(t, XT, ldt, r0, c0, n_r, n_c);
+  }
+  if (acc) {
+    DotLong dots{{0, 0, 0, 0}};
+    dots.take(dot);
+    block_sums<4>(dots.v, 0u, 0, acc);
+  }
+}
+
+// Scalars of a Lanczos start: |S_1|^2 from k_fix_in's slots.
+__global__ void k_fix_start(u64 *acc, int B, FixScal *q) {
+  const double N = take_slots(acc).dot;
+  if (threadIdx.x == 0) {
+    q->N = N;
+    q->overlap = 0.0;
+    q->N_prev = 1.0;
+    q->alpha = q->beta2 = 0.0;
+    q->max_cur = ldexp(1.0, B - 1);
+    q->rescale = 0;
+    q->max_prev = 0.0;
+    q->ratio = 0.5;
+    q->rel = q->sh = 0;
+    q->step = q->hist_n = 0;
+    q->ticket_dn = q->ticket_up = 0;
+  }
+}
+
+__global__ void k_fix_rewind(FixScal *q) { q->hist_n = 0; }
+
+// S_{j+1} over S_{j-1}, from the two contributions a (order of S) and b (kBt: the other order); kBt:
+// S_{j+1} in the other order too, into ST (which may be b).  Adds |S_{j+1}|^2 and <S_{j+1}, S_j> and
+// finds max |S_{j+1}|; the last block moves the scalars on.  Memory bounds it: 48 bytes per entry,
+// 1.38 ms at 4x4 (5.8 TB/s; in double-float 1.35 ms for 40 bytes).  A CTA takes tiles in turn and
+// adds up its sums once at the end (1.48 ms with a CTA per tile); more loads in flight per thread
+// (unrolled by 2 to 8, with 64 or 80 registers) were slower, 1.48 to 1.56 ms.  psi != null: psi += v_j q_j first (v: the eigenvector of T;
+// psi in the caller's order, rows and positions swapped if swap).
+template <int T, bool kBt, bool kLimb, bool kPsi>
+__global__ void __launch_bounds__(kTileThreads, kUpdateBlocks) k_fix_update(i64 n_r, i64 n_c, i64 ld, i64 ldt,
+                                                             const i64 *__restrict__ a, const i64 *b,
+                                                             const i64 *__restrict__ cur, i64 *__restrict__ prev,
+                                                             i64 *ST, FixScal *__restrict__ q, u64 *__restrict__ acc,
+                                                             const double *__restrict__ v, double *__restrict__ psi,
+                                                             int swap, int B) {
+  __shared__ TileBuf<T> t;
+  int mah, mal, mbh, mbl;
+  limbs28(q->ma, mah, mal);
+  limbs28(q->mb, mbh, mbl);
+  const int sy = q->sy, sa = q->sa, sb = q->sb;
+  const bool plain_shifts = sy >= 0 && sy < 64 && sa >= 0 && sa <= 28 && sb >= 0 && sb <= 28;
+  const double pc = kPsi ? v[q->step] / sqrt(q->N) : 0.0;
+  DotLong dots{{0, 0, 0, 0}}, overs{{0, 0, 0, 0}};
+  unsigned vmax = 0;
+  const TileAt<T> at;
+  const int c = at.c;
+  const uint32_t tiles = (uint32_t)(((n_c + T - 1) / T) * ((n_r + T - 1) / T));   // below 2^31 (fix_fits)
+  for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    i64 r0, c0;
+    tile_at<T>(tile, n_c, &r0, &c0);
+    if (kBt) {
+      if (tile != blockIdx.x) __syncthreads();            // the tile before has been written out
+      tile_in_t<T>(t, b, ldt, r0, c0, n_r, n_c);
+      __syncthreads();
+    } else if (kPsi && swap && tile != blockIdx.x) {
+      __syncthreads();
+    }
+    Dot dot{0, 0}, over{0, 0};
+    const i64 u = c0 + c;
+    const bool second = u + 1 < n_c;
+#pragma unroll 1
+    for (int k = at.k0, it = 0; k < T; k += TileAt<T>::kStep, ++it) {
+      if (it == 4) dots.take_squares(dot);     // entries may reach 2^(B + kFixSpare): eight squares 2^63
+      const i64 d = r0 + k;
+      if (d >= n_r || u >= n_c) continue;
+      const i64 o = d * ld + u;
+      const longlong2 sc = *reinterpret_cast<const longlong2 *>(cur + o), sp = *reinterpret_cast<const longlong2 *>(prev + o);
+      const longlong2 ya = *reinterpret_cast<const longlong2 *>(a + o);
+      longlong2 yb;
+      if (kBt)
+        yb = make_longlong2(t.v[k][c], t.v[k][c + 1]);
+      else
+        yb = *reinterpret_cast<const longlong2 *>(b + o);
+      const i64 y2[2] = {ya.x + yb.x, ya.y + yb.y};
+      int ch[2], cl[2];
+      fix_load<kLimb>(sc.x, ch[0], cl[0]);
+      fix_load<kLimb>(sc.y, ch[1], cl[1]);
+      i64 s[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        int ph, pl;
+        fix_load<kLimb>(i ? sp.y : sp.x, ph, pl);
+        // alpha S_j and beta^2 S_{j-1} from their limb products
+        const i64 ah = (i64)ch[i] * mah, am = (i64)ch[i] * mal + (i64)cl[i] * mah + __mulhi(cl[i] << 2, mal << 2);
+        const i64 bh = (i64)ph * mbh, bm = (i64)ph * mbl + (i64)pl * mbh + __mulhi(pl << 2, mbl << 2);
+        i64 t3;
+        if (plain_shifts)
+          t3 = (y2[i] >> sy) - ((ah << sa) + (am >> (28 - sa))) - ((bh << sb) + (bm >> (28 - sb)));
+        else
+          t3 = shr_any(y2[i], sy) - (shr_any(ah, -sa) + shr_any(am, 28 - sa)) - (shr_any(bh, -sb) + shr_any(bm, 28 - sb));
+        s[i] = (t3 + (1ll << (kFixFrac - 1))) >> kFixFrac;
+      }
+      if (!second) s[1] = 0;
+      if (kPsi) {
+        const i64 c2[2] = {limbs_value(ch[0], cl[0]), limbs_value(ch[1], cl[1])};
+        if (!kBt && swap) {
+          t.v[k][c] = c2[0];                    // written below, along the caller's rows
+          t.v[k][c + 1] = c2[1];
+        } else {
+          psi[d * n_c + u] += pc * (double)c2[0];
+          if (second) psi[d * n_c + u + 1] += pc * (double)c2[1];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        int h, l;
+        limbs28(s[i], h, l);
+        dot.square(h, l);
+        over.add_high(h, l, ch[i], cl[i]);
+        vmax = max(vmax, (unsigned)abs((int)(s[i] >> 32)));
+        if (kLimb) s[i] = (i64)(((u64)(unsigned)h << 32) | (unsigned)l);
+      }
+      *reinterpret_cast<longlong2 *>(prev + o) = make_longlong2(s[0], s[1]);
+      if (kBt) {
+        t.v[k][c] = s[0];
+        t.v[k][c + 1] = s[1];
+      }
+    }
+    if (kBt) {
+      __syncthreads();
+      tile_out_t<T>(t, ST, ldt, r0, c0, n_r, n_c);
+    } else if (kPsi && swap) {
+      __syncthreads();
+      const int r = (int)(threadIdx.x % T);
+      for (int k = (int)(threadIdx.x / T); k < T; k += kTileThreads / T)
+        if (c0 + k < n_c && r0 + r < n_r) psi[(c0 + k) * n_r + r0 + r] += pc * (double)t.v[r][k];
+    }
+    dots.take_squares(dot);
+    overs.take(over);
+  }
+  i64 sums8[8];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    sums8[i] = dots.v[i];
+    sums8[i + 4] = overs.v[i];
+  }
+  block_sums<8>(sums8, vmax, 0, acc);
+  if (!last_block(&q->ticket_up) || threadIdx.x >= 32) return;
+  const SlotSums sums = take_slots(acc);
+  if (threadIdx.x == 0) {
+    // bits to take off: entries below 2^B (1 - 2^-15), so that the top limbs of eight add up below 2^31
+    int r = 0;
+    while (r < kFixSpare && sums.max0 > ldexp(1.0 - 0x1p-15, B + r)) ++r;
+    const double N = ldexp(sums.dot, -2 * r), b2 = ldexp(N / q->N, 2 * (q->sh + r));
+    const int i = q->hist_n;
+    if (i < kFixHist) {
+      q->hist[3 * i] = q->alpha;
+      q->hist[3 * i + 1] = sqrt(b2);
+      q->hist[3 * i + 2] = q->N;
+    }
+    q->hist_n = i + 1;
+    q->step += 1;
+    q->N_prev = q->N;
+    q->N = N;
+    q->beta2 = b2;
+    q->rel = -(q->sh + r);
+    q->max_prev = q->max_cur;
+    q->max_cur = ldexp(sums.max0, -r) + 1.0;
+    q->overlap = ldexp(sums.dot2, -r);
+    q->rescale = r;
+    q->ratio = sums.max0 / q->bound;
+  }
+}
+
+// S_{j+1} (and its other order) 2^-rescale, rounded: nothing to do as a rule
+template <bool kLimb>
+__global__ void __launch_bounds__(256) k_fix_rescale(const FixScal *__restrict__ q, i64 n, i64 *__restrict__ S, i64 nt,
+                                                     i64 *__restrict__ ST) {
+  const int r = q->rescale;
+  if (r == 0) return;
+  for (i64 k = blockIdx.x * (i64)blockDim.x + threadIdx.x; k < n + nt; k += (i64)gridDim.x * blockDim.x) {
+    i64 *p = k < n ? S + k : ST + (k - n);
+    int h, l;
+    fix_load<kLimb>(*p, h, l);
+    *p = fix_store<kLimb>((limbs_value(h, l) + (1ll << (r - 1))) >> r);
+  }
+}
+
+// y (n_r x n_c, caller's order) = tabs 2^.. (a + b), a and b each in that order or (kAt, kBt) the other
+// one.  An entry whose contributions' magnitudes -- a lower bound of (|H||x|)_n -- do
+// not reach thr is recorded in list (see k_fix_entries).
+template <int T, bool kAt, bool kBt>
+__global__ void __launch_bounds__(kTileThreads) k_fix_out(i64 n_r, i64 n_c, i64 ld, i64 ldt, const i64 *__restrict__ a,
+                                                          const i64 *__restrict__ b, int eg, i64 thr, double tabs,
+                                                          int *__restrict__ ctl, i64 *__restrict__ list, int cap,
+                                                          double *__restrict__ y) {
+  __shared__ TileBuf<T> t;
+  if (ctl[kCtlSkip]) return;
+  const int e = ctl[kCtlShift] + eg;
+  i64 r0, c0;
+  tile_at<T>(blockIdx.x, n_c, &r0, &c0);
+  const TileAt<T> at;
+  const i64 u = c0 + at.c;
+  const bool in = u < n_c, second = u + 1 < n_c;
+  const bool vec = (n_c & 1) == 0 && ((uintptr_t)y & 15) == 0;
+  constexpr int kN = T / TileAt<T>::kStep;
+  longlong2 sa[kN], sb[kN];
+#pragma unroll
+  for (int i = 0; i < kN; ++i) {             // what needs no transposing, in flight first
+    const i64 d = r0 + at.k0 + i * TileAt<T>::kStep;
+    sa[i] = sb[i] = make_longlong2(0, 0);
+    if (!kAt && d < n_r && in) sa[i] = *reinterpret_cast<const longlong2 *>(a + d * ld + u);
+    if (!kBt && d < n_r && in) sb[i] = *reinterpret_cast<const longlong2 *>(b + d * ld + u);
+  }
+  if (kBt) {
+    tile_in_t<T>(t, b, ldt, r0, c0, n_r, n_c);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kN; ++i) {
+      const int k = at.k0 + i * TileAt<T>::kStep;
+      sb[i] = make_longlong2(t.v[k][at.c], t.v[k][at.c + 1]);
+    }
+  }
+  if (kAt) {
+    if (kBt) __syncthreads();
+    tile_in_t<T>(t, a, ldt, r0, c0, n_r, n_c);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kN; ++i) {
+      const int k = at.k0 + i * TileAt<T>::kStep;
+      sa[i] = make_longlong2(t.v[k][at.c], t.v[k][at.c + 1]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < kN; ++i) {
+    const i64 d = r0 + at.k0 + i * TileAt<T>::kStep;
+    if (d >= n_r || !in) continue;
+    const i64 n = d * n_c + u;
+    const i64 s0[2] = {sa[i].x, sa[i].y}, s1[2] = {sb[i].x, sb[i].y};
+    double v[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      v[j] = fix_to_f64(s0[j] + s1[j], e);
+      if (tabs != 1.0) v[j] *= tabs;
+      if ((j == 0 || second) && llabs(s0[j]) + llabs(s1[j]) < thr) {
+        const int k = atomicAdd(ctl + kCtlCount, 1);
+        if (k < cap) list[k] = n + j;
+      }
+    }
+    if (vec) {
+      *reinterpret_cast<double2 *>(y + n) = make_double2(v[0], v[1]);
+    } else {
+      y[n] = v[0];
+      if (second) y[n + 1] = v[1];
+    }
+  }
+}
+
+// psi += v_j q_j alone (the last vector)
+template <bool kLimb>
+__global__ void k_fix_axpy(i64 n_r, i64 n_c, i64 ld, const i64 *__restrict__ cur, const FixScal *__restrict__ q,
+                           const double *__restrict__ v, double *__restrict__ psi, int swap) {
+  const double pc = v[q->step] / sqrt(q->N);
+  const i64 D = n_r * n_c;
+  for (i64 k = blockIdx.x * (i64)blockDim.x + threadIdx.x; k < D; k += (i64)gridDim.x * blockDim.x) {
+    const i64 d = k / n_c, u = k - d * n_c;
+    int hi, lo;
+    fix_load<kLimb>(cur[d * ld + u], hi, lo);
+    psi[swap ? u * n_r + d : k] += pc * (double)limbs_value(hi, lo);
+  }
+}
+
+// The recorded entries in FP64, one warp each: hops gathered by the lanes.  More entries than
+// the list holds: the whole vector goes to the double-float (or FP64) kernels.
+__global__ void __launch_bounds__(256) k_fix_entries(const Ham H, const double *__restrict__ x, double *__restrict__ y,
+                                                     int *__restrict__ ctl, const i64 *__restrict__ list, int cap,
+                                                     int df_ok) {
+  if (ctl[kCtlSkip]) return;
+  const int n = ctl[kCtlCount];
+  if (n > cap) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl[df_ok ? kCtlDf : kCtlF64] = 1;
+    return;
+  }
+  const int lane = threadIdx.x & 31;
+  const int w0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nw = (int)((gridDim.x * blockDim.x) >> 5);
+  for (int k = w0; k < n; k += nw) {
+    const i64 at = list[k], d = at / H.n_up, u = at - d * H.n_up;
+    double v = lane == 0 ? diag_of(H, H.basis_up[u], H.basis_dn[d], u, d) * x[at] : 0.0;
+    for (int32_t j = H.rp_up[u] + lane; j < H.rp_up[u + 1]; j += 32) v = fma(H.val_up[j], x[d * H.n_up + H.col_up[j]], v);
+    for (int32_t j = H.rp_dn[d] + lane; j < H.rp_dn[d + 1]; j += 32)
+      v = fma(H.val_dn[j], x[(i64)H.col_dn[j] * H.n_up + u], v);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) y[at] = v;
+  }
+}
+
+// Entry lists of a spin (see CombLists) from its CSR matrix.
+__global__ void k_fix_lists(i64 n, const int32_t *__restrict__ rp, const uint32_t *__restrict__ scol,
+                            uint32_t *__restrict__ cnt, uint32_t *__restrict__ word) {
+  for (i64 r = blockIdx.x * (i64)blockDim.x + threadIdx.x; r < n; r += (i64)gridDim.x * blockDim.x) {
+    const int32_t a = rp[r], b = rp[r + 1];
+    int na = 0;
+    for (int32_t k = a; k < b; ++k) na += (int)(scol[k] >> 31);
+    const int ns = b - a - na, pa = na & ~1, pe = pa + (ns & ~1);
+    int ia = 0, is = 0;
+    for (int32_t k = a; k < b; ++k) {
+      const bool add = (scol[k] >> 31) != 0;
+      int at;
+      if (add) {
+        at = ia < pa ? ia : pe;
+        ++ia;
+      } else {
+        at = is < (ns & ~1) ? pa + is : pe + (na & 1);
+        ++is;
+      }
+      word[a + at] = scol[k] & 0x7fffffffu;
+    }
+    cnt[r] = (uint32_t)na | ((uint32_t)ns << 16);
+  }
+}
+
+// ---------------------------------------------------------------------------------------
+// Host side.
+// ---------------------------------------------------------------------------------------
+struct FixState {
+  bool lists_ready = false;           // entry lists of the spins: gather schedule or row combinations
+  uint32_t *cnt[2] = {nullptr, nullptr}, *word[2] = {nullptr, nullptr};
+  uint16_t *sched[2] = {nullptr, nullptr};
+  uint32_t *meta[2] = {nullptr, nullptr};
+  int cap_steps[2] = {0, 0}, slices[2] = {0, 0};
+  int *ctl = nullptr;
+  i64 *list = nullptr;
+  int cap = 0;
+  u64 *acc = nullptr;
+  FixScal *scal = nullptr, *h_scal = nullptr;
+  i64 *vec[2] = {nullptr, nullptr};   // S_j, S_{j-1}
+  double *v = nullptr;                // eigenvector of T
+  int v_cap = 0;
+  cudaStream_t gs = nullptr;
+  cudaGraphExec_t graph[2] = {nullptr, nullptr};
+  std::vector<unsigned char> graph_key;
+  bool graph_failed = false;
+};
+
+void fix_release(hub_ctx *h) {
+  FixState *f = h->fix;
+  if (!f) return;
+  for (int s = 0; s < 2; ++s) {
+    dev_free(f->cnt[s]);
+    dev_free(f->word[s]);
+    dev_free(f->sched[s]);
+    dev_free(f->meta[s]);
+    dev_free(f->vec[s]);
+    if (f->graph[s]) cudaGraphExecDestroy(f->graph[s]);
+  }
+  dev_free(f->ctl);
+  dev_free(f->list);
+  dev_free(f->acc);
+  dev_free(f->scal);
+  if (f->h_scal) cudaFreeHost(f->h_scal);
+  dev_free(f->v);
+  if (f->gs) cudaStreamDestroy(f->gs);
+  delete f;
+  h->fix = nullptr;
+}
+
+static int ceil_log2(double v) {      // smallest n with v <= 2^n (v > 0)
+  int n = 0;
+  const double m = std::frexp(v, &n);
+  return m == 0.5 ? n - 1 : n;
+}
+
+// What the fixed-point path needs to know about the model; ok == false: not for this path.
+struct FixPlan {
+  bool ok = false;
+  bool gather[2] = {false, false};    // the spin's hops as gathers inside staged rows
+  double tau = 1.0, units = 0.0;      // |t|; worst-case error of an entry in units of 2^e
+  int hh = 0, B = 0, q = 0, g = 0, dh = 0;
+  int kind = 0;
+  bool limbs() const { return gather[0] && gather[1]; }   // the vectors' storage
+};
+
+static FixPlan fix_plan(const hub_ctx *h) {
+  FixPlan p;
+  if (h->mode != HUB_MODE_AUTO || h->fix_off || h->k0 || !h->have_hop || !h->have_U || !h->fast) return p;
+  if (h->count[0] <= 0 || h->count[1] <= 0) return p;
+  // t uniform, U uniform, no site energies (the other models keep the 53-bit entries of the FP64
+  // kernels, which the grid does not quite reach)
+  if (!h->uniform_U || h->has_eps || h->t.empty()) return p;
+  for (double t : h->t)
+    if (t != h->t[0]) return p;
+  p.tau = std::fabs(h->t[0]);
+  if (!(p.tau >= 0x1p-500 && p.tau <= 0x1p500)) return p;
+  const int rows = h->csr[0].max_row + h->csr[h->shared ? 0 : 1].max_row;
+  for (int s = 0; s < 2; ++s)
+    p.gather[s] = h->count[s] <= kStageMax && h->csr[h->shared ? 0 : s].max_row <= kSchedRow;
+  p.hh = ceil_log2(std::max(rows, 1));
+  p.B = std::min(kFixMaxBits, 62 - p.hh);
+  p.q = 62 - p.B;
+  const double r = h->U0 / p.tau, dmax = std::fabs(r) * std::min(h->N[0], h->N[1]);
+  if (!std::isfinite(dmax) || dmax > 0x1p24) return p;
+  if (dmax > 0.0) {
+    p.kind = r == std::floor(r) && dmax <= std::ldexp(1.0, p.q) ? 1 : 2;
+    p.dh = std::max(ceil_log2(dmax), -40);
+    // |Y| <= 2^(B - g) (rows + dmax) < 2^63; the general diagonal's high product must not be
+    // shifted left
+    p.g = std::max(0, ceil_log2(1.07 * (std::max(rows, 1) + dmax)) + p.B - 63);
+    if (p.kind == 2) p.g = std::max(p.g, p.dh + 2 - p.q);
+  }
+  // rounding of the entries (1/2 each), of the shift to Y's grid and of the diagonal's product (2^g
+  // each at most)
+  p.units = 0.5 * (rows + dmax) + (p.g || p.kind == 2 ? std::ldexp(2.0, p.g) : 0.0) + 1.0;
+  p.ok = true;
+  return p;
+}
+
+static FixState *fix_state(hub_ctx *h) {
+  if (!h->fix) h->fix = new (std::nothrow) FixState();
+  return h->fix;
+}
+
+// Row stride in entries: rows start on 32-byte sectors.
+static i64 fix_ld(i64 n) { return (n + 3) & ~(i64)3; }
+static int grid_of(i64 n) { return (int)std::max<i64>(1, std::min<i64>((n + 255) / 256, (i64)num_sms() * 16)); }
+
+// Groups of 16 positions for a gather schedule: four quads of consecutive positions each (the
+// outputs of a quad are one 32-byte sector), chosen greedily among the next 64 quads, longest rows
+// first, so that the group's busiest bank stays low; or the quads in their own order where that
+// needs no more steps.  At 4x4 1.17 steps per entry of a row against 1.26.
+static std::vector<int32_t> gather_groups(int n, const SpinCSR &c, int *rc) {
+  const int groups = (n + 31) / 32 * 2, quads = 4 * groups;
+  std::vector<int32_t> rp(n + 1), natural(quads), best(quads);
+  std::vector<uint32_t> sc(std::max<i64>(c.nnz, 1));
+  cudaError_t e = cudaMemcpy(rp.data(), c.rowptr, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess && c.nnz) e = cudaMemcpy(sc.data(), c.scol, sizeof(uint32_t) * c.nnz, cudaMemcpyDeviceToHost);
+  *rc = e == cudaSuccess ? HUB_OK : cuda_fail(e, "gather groups", __FILE__, __LINE__);
+  if (*rc) return natural;
+  std::vector<int32_t> load(16 * (size_t)quads, 0), len(quads, 0);
+  for (int r = 0; r < n; ++r) {
+    len[r / 4] = std::max(len[r / 4], rp[r + 1] - rp[r]);
+    for (int32_t k = rp[r]; k < rp[r + 1]; ++k) ++load[16 * (size_t)(r / 4) + (sc[k] & 15)];
+  }
+  for (int q = 0; q < quads; ++q) natural[q] = q;
+  auto steps = [&](const std::vector<int32_t> &order) {
+    i64 total = 0;
+    for (int g = 0; g < groups; ++g) {
+      int m = 0;
+      for (int b = 0; b < 16; ++b) {
+        int s = 0;
+        for (int k = 0; k < 4; ++k) s += load[16 * (size_t)order[4 * g + k] + b];
+        m = std::max(m, s);
+      }
+      for (int k = 0; k < 4; ++k) m = std::max(m, len[order[4 * g + k]]);
+      total += m;
+    }
+    return total;
+  };
+  std::vector<int32_t> left = natural;
+  std::stable_sort(left.begin(), left.end(), [&](int a, int b) { return len[a] > len[b]; });
+  size_t head = 0;
+  for (int g = 0; g < groups; ++g) {
+    int sum[16] = {0};
+    for (int k = 0; k < 4; ++k) {
+      size_t pick = head;
+      i64 score = INT64_MAX;
+      for (size_t i = head; i < std::min(left.size(), head + (k ? 64 : 1)); ++i) {
+        const int32_t *l = &load[16 * (size_t)left[i]];
+        i64 m = 0, sq = 0;
+        for (int b = 0; b < 16; ++b) {
+          const i64 v = sum[b] + l[b];
+          m = std::max(m, v);
+          sq += v * v;
+        }
+        if ((m << 32) + sq < score) {
+          score = (m << 32) + sq;
+          pick = i;
+        }
+      }
+      best[4 * g + k] = left[pick];
+      for (int b = 0; b < 16; ++b) sum[b] += load[16 * (size_t)left[pick] + b];
+      for (size_t i = pick; i > head; --i) left[i] = left[i - 1];
+      ++head;
+    }
+  }
+  return steps(best) < steps(natural) ? best : natural;
+}
+
+// Gather schedule of a spin: the groups coloured on the device, then paired by length into slices.
+static int gather_tables(FixState *f, int s, int n, const SpinCSR &c) {
+  const int slices = (n + 31) / 32, groups = 2 * slices;
+  const int cap = std::min(kSchedMax, (2 * std::max(c.max_row, 1) + 7) / 8 * 8);
+  uint16_t *tmp = nullptr, *deg = nullptr;
+  int32_t *grp = nullptr, *quad = nullptr;
+  std::vector<uint16_t> d(groups);
+  std::vector<int32_t> order(groups);
+  std::vector<uint32_t> meta(32 * (size_t)slices);
+  int rc = HUB_OK;
+  const std::vector<int32_t> q = gather_groups(n, c, &rc);
+  if (rc) return rc;
+  f->cap_steps[s] = cap;
+  f->slices[s] = slices;
+  if (!dev_alloc((void **)&f->sched[s], sizeof(uint16_t) * 32 * (size_t)slices * cap, "gather schedule") ||
+      !dev_alloc((void **)&f->meta[s], sizeof(uint32_t) * meta.size(), "gather slices") ||
+      !dev_alloc((void **)&quad, sizeof(int32_t) * q.size(), "gather groups") ||
+      !dev_alloc((void **)&grp, sizeof(int32_t) * groups, "gather groups") ||
+      !dev_alloc((void **)&tmp, sizeof(uint16_t) * 32 * (size_t)slices * cap, "gather schedule") ||
+      !dev_alloc((void **)&deg, sizeof(uint16_t) * groups, "gather steps"))
+    rc = HUB_ERR_OOM;
+  cudaError_t e = cudaSuccess;
+  if (rc == HUB_OK) e = cudaMemcpy(quad, q.data(), sizeof(int32_t) * q.size(), cudaMemcpyHostToDevice);
+  if (rc == HUB_OK && e == cudaSuccess) {
+    k_fix_schedule<<<(groups + 31) / 32, 32>>>(n, groups, (int)fix_ld(n), cap, quad, c.rowptr, c.scol, tmp, deg);
+    e = cudaMemcpy(d.data(), deg, sizeof(uint16_t) * groups, cudaMemcpyDeviceToHost);
+    for (int g = 0; g < groups; ++g) order[g] = g;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return d[a] > d[b]; });
+    for (int k = 0; k < slices; ++k)
+      for (int l = 0; l < 32; ++l) {          // words hold two steps
+        const uint32_t steps = (d[order[2 * k]] + 1u) & ~1u;
+        const uint32_t at = (uint32_t)q[4 * order[2 * k + (l >> 4)] + ((l >> 2) & 3)] * 4 + (l & 3);
+        meta[32 * (size_t)k + l] = at | (steps << 16);
+      }
+    if (e == cudaSuccess) e = cudaMemcpy(grp, order.data(), sizeof(int32_t) * groups, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(f->meta[s], meta.data(), sizeof(uint32_t) * meta.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+      k_fix_pack<<<slices, 32>>>(grp, cap, tmp, f->sched[s]);
+      e = cudaDeviceSynchronize();
+    }
+  }
+  dev_free(tmp);
+  dev_free(deg);
+  dev_free(grp);
+  dev_free(quad);
+  if (rc == HUB_OK) HUB_CUDA(e);
+  return rc;
+}
+
+// Tables of the plan: entry lists, coefficients and diagonal.
+static int fix_tables(hub_ctx *h, FixState *f, const FixPlan &p) {
+  if (!f->lists_ready) {
+    for (int s = 0; s < (h->shared ? 1 : 2); ++s) {
+      const SpinCSR &c = h->csr[s];
+      const i64 nnz = c.nnz, n = h->count[s];
+      if (p.gather[s]) {
+        const int rc = gather_tables(f, s, (int)n, c);
+        if (rc) return rc;
+        continue;
+      }
+      if (!dev_alloc((void **)&f->cnt[s], sizeof(uint32_t) * n, "hopping entry counts") ||
+          !dev_alloc((void **)&f->word[s], sizeof(uint32_t) * (nnz + 32), "hopping entries"))
+        return HUB_ERR_OOM;
+      HUB_CUDA(cudaMemset(f->word[s], 0, sizeof(uint32_t) * (nnz + 32)));
+      k_fix_lists<<<grid_of(n), 256>>>(n, c.rowptr, c.scol, f->cnt[s], f->word[s]);
+      HUB_LAUNCH_CHECK();
+    }
+    HUB_CUDA(cudaDeviceSynchronize());
+    f->lists_ready = true;
+  }
+  return HUB_OK;
+}
+
+// A pass over the order of the vector whose rows are spin a's states.
+static FixPass fix_pass(const hub_ctx *h, const FixState *f, const FixPlan &p, int a, bool diag) {
+  const int b = 1 - a;
+  FixPass P{};
+  P.n_rows = h->count[a];
+  P.n_pos = h->count[b];
+  P.ld = fix_ld(P.n_pos);
+  P.bits_row = h->basis[a];
+  P.bits_pos = h->basis[b];
+  P.q = p.q;
+  P.g = p.g;
+  P.t_neg = h->t[0] < 0.0;
+  P.err = fast_err(h);
+  P.fail_waits = h->fail_waits ? 1 : 0;
+  if (!diag) return P;
+  FixDiag &d = P.diag;
+  d.kind = p.kind;
+  if (p.kind == 1) {
+    d.mul = (int)(h->U0 / p.tau);
+    d.shift = p.g;
+  }
+  if (p.kind == 2) {
+    d.shift = p.q - 2 - p.dh + p.g;
+    for (int k = 0; k <= std::min(h->N[0], h->N[1]); ++k)
+      d.tab[k] = (i64)std::llrint(std::ldexp(h->U0 * k / p.tau, 62 - p.dh));
+  }
+  return P;
+}
+
+// Rows of a combination tile, fewer where the grid would leave SMs idle (two CTAs each).
+static int tile_rows(i64 n_rows, i64 n_cols) {
+  const i64 strips = (n_cols + kCombCols - 1) / kCombCols;
+  const i64 want = n_rows * strips / (2 * num_sms());
+  return (int)std::min<i64>(kCombRows, std::max<i64>(1, want / 8) * 8);
+}
+static i64 comb_blocks(i64 n_rows, i64 n_cols) {
+  const int R = tile_rows(n_rows, n_cols);
+  return ((n_rows + R - 1) / R) * ((n_cols + kCombCols - 1) / kCombCols);
+}
+// Tiles of 64 x 64 entries, or 32 x 32 where the larger ones would leave SMs idle.
+static bool small_tiles(const hub_ctx *h) { return h->count[0] * h->count[1] < (i64)64 * 64 * 8 * num_sms(); }
+static i64 tile_blocks(const hub_ctx *h) {
+  const i64 T = small_tiles(h) ? 32 : 64;
+  return ((h->count[0] + T - 1) / T) * ((h->count[1] + T - 1) / T);
+}
+// grids are one-dimensional, row strides in bytes 32-bit
+static bool fix_fits(const hub_ctx *h) {
+  const i64 lim = ((i64)1 << 31) - 1;
+  for (int s = 0; s < 2; ++s)
+    if (comb_blocks(h->count[s], h->count[1 - s]) > lim || fix_ld(h->count[s]) * 8 > (i64)0xffffffff) return false;
+  return tile_blocks(h) <= lim;
+}
+
+// out = the hops of the rows' (comb) or the positions' spin (gather) applied to P.x
+static int launch_comb(const hub_ctx *h, const FixState *f, const FixPass &P, int a, cudaStream_t s) {
+  const int t = h->shared ? 0 : a;
+  CombLists L{tile_rows(P.n_rows, P.n_pos), h->csr[t].rowptr, f->cnt[t], f->word[t]};
+  const int g = (int)comb_blocks(P.n_rows, P.n_pos);
+  (P.acc ? k_fix_comb<true> : k_fix_comb<false>)<<<g, kCombThreads, 0, s>>>(P, L);
+  HUB_LAUNCH_CHECK();
+  return HUB_OK;
+}
+template <int kPlane, bool kLimb>
+static int launch_gather_t(const FixPass &P, const GatherLists &L, cudaStream_t s) {
+  static_assert(kPlane % 16 == 0, "both rows in the same banks");
+  const size_t smem = 2 * sizeof(i64) * (size_t)kPlane;
+  const int threads = kPlane > 2048 ? 1024 : (P.n_pos >= 256 ? 256 : 128);
+  const i64 per_sm = std::max<i64>(1, std::min<i64>((i64)(220 * 1024 / smem), 1024 / threads));
+  const int grid = (int)std::min<i64>((P.n_rows + 1) / 2, per_sm * num_sms());
+  const auto k = P.acc ? k_fix_gather<kPlane, true, kLimb> : k_fix_gather<kPlane, false, kLimb>;
+  HUB_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k<<<grid, threads, smem, s>>>(P, L);
+  HUB_LAUNCH_CHECK();
+  return HUB_OK;
+}
+template <int kPlane>
+static int launch_gather_p(const FixPlan &p, const FixPass &P, const GatherLists &L, cudaStream_t s) {
+  return p.limbs() ? launch_gather_t<kPlane, true>(P, L, s) : launch_gather_t<kPlane, false>(P, L, s);
+}
+static int launch_gather(const hub_ctx *h, const FixState *f, const FixPlan &p, const FixPass &P, int b, cudaStream_t s) {
+  const int t = h->shared ? 0 : b;
+  const GatherLists L{(const uint4 *)f->sched[t], f->meta[t], f->cap_steps[t] / 8, f->slices[t]};
+  return P.ld + 16 <= 2048 ? launch_gather_p<2048>(p, P, L, s) : launch_gather_p<kStageMax + 16>(p, P, L, s);
+}
+
+// How the two spins' hops are run.  `a` is the spin whose states are the rows of the order the
+// Lanczos vectors are kept in.
+//   both as gathers: the positions' spin on that order, the rows' spin on the other one;
+//   both as combinations: the rows' spin on that order, the positions' spin on the other one;
+//   one of each: the gathered spin are the positions, both on that order, the other is not kept.
+struct FixShape {
+  int a = 1;                          // rows: spin down (the caller's order) unless only it gathers
+  bool both = true;                   // two orders of the vector
+};
+static FixShape fix_shape(const FixPlan &p) {
+  FixShape F;
+  if (p.gather[0] != p.gather[1]) {
+    F.both = false;
+    F.a = p.gather[0] ? 1 : 0;
+  }
+  return F;
+}
+
+// The two contributions to the product of S (order of rows a; ST: the other order): out0 in the
+// order of a, out1 in the other one if F.both, else in the same.  Where a pass gathers, its output
+// may be its input.  lz: Lanczos sums into f->acc.
+static int fix_product(hub_ctx *h, FixState *f, const FixPlan &p, const FixShape &F, const i64 *S, const i64 *ST,
+                       i64 *out0, i64 *out1, const int *skip, bool lz, cudaStream_t s) {
+  int rc;
+  count_launch(h, 2);
+  FixPass P0 = fix_pass(h, f, p, F.a, true), P1 = fix_pass(h, f, p, F.both ? 1 - F.a : F.a, false);
+  P0.x = S;
+  P0.out = out0;
+  P1.x = F.both ? ST : S;
+  P1.out = out1;
+  P0.skip = P1.skip = skip;
+  if (lz) {
+    P0.acc = P1.acc = f->acc;
+    P0.scal = P1.scal = f->scal;
+  }
+  // one of each: the combination first, so that the gather may work in place
+  const bool swap = !F.both;
+  (swap ? P0 : P1).second = 1;
+  for (int k = 0; k < 2; ++k) {
+    const bool first = (k == 0) != swap;      // P0's turn
+    const FixPass &P = first ? P0 : P1;
+    // P0 runs the positions' spin where spins gather (and the rows' spin where both combine)
+    const int rows = first || !F.both ? F.a : 1 - F.a;
+    const bool gather = F.both ? p.gather[0] : first;
+    const int kind = k == 0 ? HUB_PROF_UP : HUB_PROF_DN;
+    if ((rc = prof_mark(h, kind, true, s))) return rc;
+    if ((rc = gather ? launch_gather(h, f, p, P, 1 - rows, s) : launch_comb(h, f, P, rows, s))) return rc;
+    if ((rc = prof_mark(h, kind, false, s))) return rc;
+  }
+  return HUB_OK;
+}
+
+// Scale and route words of x (k_exp_range's partials live with the double-float path)
+static int plan_vector(hub_ctx *h, FixState *f, const double *x, i64 D, int df_ok, cudaStream_t s) {
+  int *part = nullptr, nblk = 0;
+  const int rc = fast_exp_range(h, x, D, &part, &nblk, s);
+  if (rc) return rc;
+  count_launch(h);
+  k_fix_plan<<<1, kPlanThreads, 0, s>>>(part, nblk, D, x, df_ok, f->ctl);
+  HUB_LAUNCH_CHECK();
+  return HUB_OK;
+}
+
+// Vectors of the handle's scratch a product needs: S, ST and, for combinations, their outputs.
+static int scratch_vectors(const FixPlan &p, const FixShape &F) { return F.both && !p.gather[0] ? 4 : 2; }
+
+// hub_apply in fixed point, the other kernels launched behind it on device flags.
+bool fix_apply_eligible(const hub_ctx *h) {
+  if (h->fail_waits) return false;    // the test hook exercises the double-float kernels' waits
+  const FixPlan p = fix_plan(h);
+  // an entry's worst-case error has to lie well inside the bound for vectors of ordinary shape
+  return p.ok && p.units <= 128.0 && fix_fits(h);
+}
+
+int fix_apply(hub_ctx *h, const double *x, double *y, cudaStream_t s) {
+  const FixPlan p = fix_plan(h);
+  const FixShape F = fix_shape(p);
+  FixState *f = fix_state(h);
+  if (!f) return fail(HUB_ERR_OOM, "fixed-point apply: host allocation failed");
+  int rc = fix_tables(h, f, p);
+  if (rc) return rc;
+  const i64 n_up = h->count[0], n_dn = h->count[1], D = n_up * n_dn;
+  float *buf[4] = {nullptr, nullptr, nullptr, nullptr};
+  if ((rc = fast_scratch(h, scratch_vectors(p, F), buf))) return rc;
+  if (!f->ctl && !dev_alloc((void **)&f->ctl, sizeof(int) * kCtlWords, "product flags")) return HUB_ERR_OOM;
+  if (!f->list) {
+    f->cap = (int)std::min<i64>(std::max<i64>(D / 64, 1024), (i64)1 << 24);
+    if (!dev_alloc((void **)&f->list, sizeof(i64) * f->cap, "entries to recompute")) return HUB_ERR_OOM;
+  }
+  const int df_ok = use_fast(h) ? 1 : 0;
+  if ((rc = plan_vector(h, f, x, D, df_ok, s))) return rc;
+  // X: rows spin down (the caller's order); XT: rows spin up
+  const bool cx = F.both || F.a == 1, ct = F.both || F.a == 0;
+  i64 *X = (i64 *)buf[0], *XT = (i64 *)buf[1];
+  const i64 ld = fix_ld(n_up), ldt = fix_ld(n_dn);
+  const int tb = (int)tile_blocks(h), *skip = f->ctl + kCtlSkip;
+  count_launch(h, 3);
+  const bool st = small_tiles(h);
+  (p.limbs() ? (st ? k_fix_in<32, true> : k_fix_in<64, true>)
+             : (st ? k_fix_in<32, false> : k_fix_in<64, false>))<<<tb, kTileThreads, 0, s>>>(
+      n_dn, n_up, ld, ldt, x, f->ctl, 1, p.B, cx ? X : nullptr, ct ? XT : nullptr, nullptr);
+  HUB_LAUNCH_CHECK();
+  i64 *in0 = F.a == 1 ? X : XT, *in1 = F.a == 1 ? XT : X, *out0 = in0, *out1 = in1;   // gathers: in place
+  if (F.both && !p.gather[0]) {
+    out0 = (i64 *)buf[2];
+    out1 = (i64 *)buf[3];
+  }
+  if ((rc = fix_product(h, f, p, F, in0, in1, out0, out1, skip, false, s))) return rc;
+  const i64 thr = ((i64)std::ceil(p.units * 1.25e13) >> p.g) + 1;   // |error| <= units 2^e <= 0.8e-13 thr 2^(e + g)
+  const int eg = p.g - (p.B - 2);
+#define FIX_OUT(AT, BT)                                                                                               \
+  (st ? k_fix_out<32, AT, BT> : k_fix_out<64, AT, BT>)<<<tb, kTileThreads, 0, s>>>(n_dn, n_up, ld, ldt, out0, out1, eg, \
+                                                                                   thr, p.tau, f->ctl, f->list, f->cap, y)
+  if (F.both)
+    FIX_OUT(false, true);
+  else if (F.a == 1)
+    FIX_OUT(false, false);
+  else
+    FIX_OUT(true, true);
+#undef FIX_OUT
+  HUB_LAUNCH_CHECK();
+  k_fix_entries<<<num_sms() * 4, 256, 0, s>>>(h->view(), x, y, f->ctl, f->list, f->cap, df_ok);
+  HUB_LAUNCH_CHECK();
+  if (df_ok && (rc = fast_apply_gated(h, x, y, f->ctl + kCtlDfScale, f->ctl + kCtlDf, s))) return rc;
+  return f64_apply(h, x, y, f->ctl + kCtlF64, s);
+}
+
+// ---------------------------------------------------------------------------------------
+// Lanczos driver: three kernels per step, replayed as a graph (one per rotation of the two
+// vectors), the scalars of the recurrence kept on the device.
+// ---------------------------------------------------------------------------------------
+bool fix_lanczos_eligible(const hub_ctx *h) { return fix_plan(h).ok && fix_fits(h); }
+
+int fix_lanczos(hub_ctx *h, const double *x0, int maxit, double tol, double *E0, double *psi_out, int *iters,
+                cudaStream_t s) {
+  const FixPlan p = fix_plan(h);
+  FixState *f = fix_state(h);
+  if (!f) return fail(HUB_ERR_OOM, "fixed-point Lanczos: host allocation failed");
+  int rc = fix_tables(h, f, p);
+  if (rc) return rc;
+  const FixShape F = fix_shape(p);
+  const i64 n_up = h->count[0], n_dn = h->count[1], D = n_up * n_dn;
+  const i64 n_r = h->count[F.a], n_c = h->count[1 - F.a], ld = fix_ld(n_c), ldt = fix_ld(n_r);
+  // out0; the other order (its gather works in place) or out1; out1 of combinations in both orders
+  const bool third = F.both && !p.gather[0];
+  float *buf[4] = {nullptr, nullptr, nullptr, nullptr};
+  if ((rc = fast_scratch(h, third ? 3 : 2, buf))) return rc;
+  i64 *const out0 = (i64 *)buf[0], *const ST = (i64 *)buf[1], *const out1 = third ? (i64 *)buf[2] : ST;
+  for (int k = 0; k < 2; ++k)
+    if (!f->vec[k] && !dev_alloc((void **)&f->vec[k], sizeof(i64) * n_r * ld, "Lanczos vector")) return HUB_ERR_OOM;
+  if ((!f->acc && !dev_alloc((void **)&f->acc, sizeof(u64) * kFixSlots * kAcc, "Lanczos sums")) ||
+      (!f->scal && !dev_alloc((void **)&f->scal, sizeof(FixScal), "Lanczos scalars")) ||
+      (!f->ctl && !dev_alloc((void **)&f->ctl, sizeof(int) * kCtlWords, "product flags")))
+    return HUB_ERR_OOM;
+  if (!f->h_scal) HUB_CUDA(cudaMallocHost((void **)&f->h_scal, sizeof(FixScal)));
+  const int tb = (int)tile_blocks(h), ub = std::min(tb, kUpdateBlocks * num_sms());
+  const int swap = F.a == 0;
+  const bool st32 = small_tiles(h);
+
+  // S_1 = x0 on the grid of its largest entry
+  auto start = [&]() -> int {
+    int rc2 = plan_vector(h, f, x0, D, 0, s);
+    if (rc2) return rc2;
+    count_launch(h, 2);
+    HUB_CUDA(cudaMemsetAsync(f->acc, 0, sizeof(u64) * kFixSlots * kAcc, s));
+    HUB_CUDA(cudaMemsetAsync(f->vec[1], 0, sizeof(i64) * n_r * ld, s));
+    (p.limbs() ? (st32 ? k_fix_in<32, true> : k_fix_in<64, true>)
+               : (st32 ? k_fix_in<32, false> : k_fix_in<64, false>))<<<tb, kTileThreads, 0, s>>>(
+        n_dn, n_up, fix_ld(n_up), fix_ld(n_dn), x0, f->ctl, 0, p.B, swap ? nullptr : f->vec[0],
+        swap ? f->vec[0] : (F.both ? ST : nullptr), f->acc);
+    HUB_LAUNCH_CHECK();
+    k_fix_start<<<1, 32, 0, s>>>(f->acc, p.B, f->scal);
+    HUB_LAUNCH_CHECK();
+    return HUB_OK;
+  };
+  // one step on (cur, prev): prev becomes S_{j+1}
+  auto step = [&](i64 *cur, i64 *prev, double *psi, cudaStream_t st) -> int {
+    int rc2 = prof_mark(h, HUB_PROF_APPLY, true, st);
+    if (rc2 || (rc2 = fix_product(h, f, p, F, cur, ST, out0, out1, nullptr, true, st)) ||
+        (rc2 = prof_mark(h, HUB_PROF_APPLY, false, st)) || (rc2 = prof_mark(h, HUB_PROF_UPDATE, true, st)))
+      return rc2;
+    count_launch(h);
+#define FIX_UPDATE_T(T, BT, LIMB)                                                                                   \
+  (psi ? k_fix_update<T, BT, LIMB, true> : k_fix_update<T, BT, LIMB, false>)<<<ub, kTileThreads, 0, st>>>(          \
+      n_r, n_c, ld, ldt, out0, out1, cur, prev, ST, f->scal, f->acc, psi ? f->v : nullptr, psi, swap, p.B)
+#define FIX_UPDATE(BT, LIMB)                                                                                        \
+  do {                                                                                                              \
+    if (st32)                                                                                                       \
+      FIX_UPDATE_T(32, BT, LIMB);                                                                                   \
+    else                                                                                                            \
+      FIX_UPDATE_T(64, BT, LIMB);                                                                                   \
+  } while (0)
+    if (!F.both)
+      FIX_UPDATE(false, false);
+    else if (p.limbs())
+      FIX_UPDATE(true, true);
+    else
+      FIX_UPDATE(true, false);
+#undef FIX_UPDATE
+#undef FIX_UPDATE_T
+    HUB_LAUNCH_CHECK();
+    count_launch(h);
+    (p.limbs() ? k_fix_rescale<true> : k_fix_rescale<false>)<<<grid_of(D), 256, 0, st>>>(
+        f->scal, n_r * ld, prev, F.both ? n_c * ldt : 0, ST);
+    HUB_LAUNCH_CHECK();
+    return prof_mark(h, HUB_PROF_UPDATE, false, st);
+  };
+
+  if ((rc = start())) return rc;
+  int ctl[kCtlWords];
+  HUB_CUDA(cudaMemcpyAsync(ctl, f->ctl, sizeof(ctl), cudaMemcpyDeviceToHost, s));
+  HUB_CUDA(cudaMemcpyAsync(f->h_scal, f->scal, sizeof(FixScal), cudaMemcpyDeviceToHost, s));
+  HUB_CUDA(cudaStreamSynchronize(s));
+  if (ctl[kCtlShift] == 2047 - 1023 || !(f->h_scal->N > 0.0))
+    return fail(HUB_ERR_ARG, "hub_lanczos_ground: start vector is zero or not finite");
+  h->start_norm = std::ldexp(std::sqrt(f->h_scal->N), ctl[kCtlShift] - (p.B - 2));
+
+  // graphs of one step, kept while their operands stay the same
+  bool graphs = !h->prof && !f->graph_failed;
+  if (graphs) {
+    std::vector<unsigned char> key;
+    auto add = [&](const void *q, size_t n) { key.insert(key.end(), (const unsigned char *)q, (const unsigned char *)q + n); };
+    const FixPass P0 = fix_pass(h, f, p, F.a, true);
+    const void *ptrs[8] = {out0, ST, out1, f->vec[0], f->vec[1], f->acc, f->scal, nullptr};
+    add(&P0, sizeof(P0));
+    add(ptrs, sizeof(ptrs));
+    if (!f->graph[0] || key != f->graph_key) {
+      bool ok = f->gs || cudaStreamCreateWithFlags(&f->gs, cudaStreamNonBlocking) == cudaSuccess;
+      for (int k = 0; k < 2 && ok; ++k) {
+        if (f->graph[k]) cudaGraphExecDestroy(f->graph[k]);
+        f->graph[k] = nullptr;
+        cudaGraph_t g = nullptr;
+        ok = cudaStreamBeginCapture(f->gs, cudaStreamCaptureModeRelaxed) == cudaSuccess;
+        if (!ok) break;
+        const int r2 = step(f->vec[k], f->vec[1 - k], nullptr, f->gs);
+        ok = cudaStreamEndCapture(f->gs, &g) == cudaSuccess && r2 == HUB_OK && g &&
+             cudaGraphInstantiate(&f->graph[k], g, 0) == cudaSuccess;
+        if (g) cudaGraphDestroy(g);
+      }
+      if (!ok) {
+        for (int k = 0; k < 2; ++k) {
+          if (f->graph[k]) cudaGraphExecDestroy(f->graph[k]);
+          f->graph[k] = nullptr;
+        }
+        f->graph_failed = true;
+        cudaGetLastError();
+        set_error("");
+      } else {
+        f->graph_key = key;
+      }
+    }
+    graphs = f->graph[0] != nullptr;
+  }
+
+  h->alpha.clear();
+  h->beta.clear();
+  // Small sectors run several steps per host read-back; steps past the stopping one are dropped.
+  const int batch = D <= ((i64)1 << 21) ? kFixHist : 1;
+  double E = 0.0, E_prev = 0.0;
+  LowestTracker lowest;
+  int status = HUB_ERR_NOCONV;
+  bool done = false;
+  for (int j = 0; j < maxit && !done;) {
+    const int nb = std::min(batch, maxit - j);
+    count_launch(h);
+    k_fix_rewind<<<1, 1, 0, s>>>(f->scal);
+    HUB_LAUNCH_CHECK();
+    for (int b = 0; b < nb; ++b) {
+      const int k = (j + b) & 1;
+      if (graphs) {
+        HUB_CUDA(cudaGraphLaunch(f->graph[k], s));
+      } else if ((rc = step(f->vec[k], f->vec[1 - k], nullptr, s))) {
+        return rc;
+      }
+    }
+    HUB_CUDA(cudaMemcpyAsync(f->h_scal, f->scal, sizeof(FixScal), cudaMemcpyDeviceToHost, s));
+    HUB_CUDA(cudaStreamSynchronize(s));
+    for (int b = 0; b < nb; ++b) {
+      const double a = p.tau * f->h_scal->hist[3 * b], be = p.tau * f->h_scal->hist[3 * b + 1];
+      if (!std::isfinite(a) || !std::isfinite(be)) {
+        if ((rc = fast_check_error(h))) return rc;
+        return fail(HUB_ERR_CUDA, "hub_lanczos_ground: non-finite alpha/beta");
+      }
+      h->alpha.push_back(a);
+      h->beta.push_back(be);
+      if (tol > 0) E = lowest.next(h->alpha.data(), h->beta.data(), (int)h->alpha.size());   // else at the end
+      if (tol > 0 && j + b > 0 && std::fabs(E - E_prev) < tol) {
+        status = HUB_OK;
+        done = true;
+        break;
+      }
+      E_prev = E;
+      if (be <= 1e-14 * std::fmax(1.0, std::fabs(a))) {
+        status = HUB_CONVERGED_BREAKDOWN;
+        done = true;
+        break;
+      }
+    }
+    j += nb;
+  }
+  if (tol <= 0 && status == HUB_ERR_NOCONV) status = HUB_OK;
+  if (tol <= 0) E = tridiag_lowest(h->alpha.data(), h->beta.data(), (int)h->alpha.size());
+  if ((rc = fast_check_error(h))) return rc;
+  *E0 = E;
+  const int k = (int)h->alpha.size();
+  if (iters) *iters = k;
+
+  if (psi_out) {
+    // second pass: the same integer steps again, psi = sum_j v_j q_j
+    const std::vector<double> vv = tridiag_vector(h->alpha.data(), h->beta.data(), k, psi_eigenvalue(h, E));
+    if (f->v_cap < k) {
+      dev_free(f->v);
+      f->v = nullptr;
+      f->v_cap = 0;
+      if (!dev_alloc((void **)&f->v, sizeof(double) * k, "eigenvector of T")) return HUB_ERR_OOM;
+      f->v_cap = k;
+    }
+    HUB_CUDA(cudaMemcpyAsync(f->v, vv.data(), sizeof(double) * k, cudaMemcpyHostToDevice, s));
+    HUB_CUDA(cudaMemsetAsync(psi_out, 0, sizeof(double) * D, s));
+    if ((rc = start())) return rc;
+    for (int j = 0; j + 1 < k; ++j)
+      if ((rc = step(f->vec[j & 1], f->vec[1 - (j & 1)], psi_out, s))) return rc;
+    count_launch(h);
+    (p.limbs() ? k_fix_axpy<true> : k_fix_axpy<false>)<<<grid_of(D), 256, 0, s>>>(
+        n_r, n_c, ld, f->vec[(k - 1) & 1], f->scal, f->v, psi_out, swap);
+    HUB_LAUNCH_CHECK();
+    if ((rc = f64_normalise(h, D, psi_out, s))) return rc;
+    HUB_CUDA(cudaStreamSynchronize(s));
+    if ((rc = fast_check_error(h))) return rc;
+  }
+  if (status == HUB_ERR_NOCONV) set_error("hub_lanczos_ground: maxit reached before |dE0| < tol");
+  return status;
+}
+
+}  // namespace hub

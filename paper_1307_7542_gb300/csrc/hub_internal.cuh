@@ -46,6 +46,7 @@ struct SpinCSR {
 struct FastState;   // fast-path tables and scratch (hub_fast.cu)
 struct K0State;     // k = 0 translation-sector tables (hub_k0.cu)
 struct SmallState;  // single-launch Lanczos of small sectors (hub_small.cu)
+struct FixState;    // fixed-point product and Lanczos (hub_fix.cu)
 
 // Read-only view of everything a kernel needs, passed by value.
 struct Ham {
@@ -64,6 +65,26 @@ struct Ham {
   double t0;
   int has_eps;
 };
+
+// Lane l of the warp: the warp's total of v[l % N].  Each of the first log2(N) exchanges sends one of
+// a pair and keeps the other, so that N totals take N + 4 - log2(N) shuffles instead of 5 N.
+template <int N, typename T>
+__device__ __forceinline__ T warp_totals(T (&v)[N]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int m = N / 2, o = 1; m > 0; m >>= 1, o <<= 1) {
+    const bool odd = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < m; ++k) {
+      const T keep = odd ? v[2 * k + 1] : v[2 * k], send = odd ? v[2 * k] : v[2 * k + 1];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  T t = v[0];
+#pragma unroll
+  for (int o = N; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
 
 }  // namespace hub
 
@@ -135,6 +156,10 @@ struct hub_ctx {
   int64_t small_max_dim = int64_t(1) << 18;
   hub::SmallState *small = nullptr;
 
+  // fixed-point product and Lanczos (hub_fix.cu): tables, flags and vectors
+  hub::FixState *fix = nullptr;
+  bool fix_off = false;                // its vectors did not fit: the other paths until hub_hopping
+
   hub::Ham view() const;
 };
 
@@ -172,8 +197,15 @@ int fast_apply_host(hub_ctx *h, const double *x_host, double *y_host, double *xd
 bool fast_host_pipelined(const hub_ctx *h);
 int fast_apply_host_many(hub_ctx *h, int64_t n_vec, const double *x_host, double *y_host, double *const xd[2],
                          double *const yd[2], cudaStream_t s);
-int fast_lanczos(hub_ctx *h, const double *x0, int maxit, double tol, double *E0, double *psi_out, int *iters,
-                 cudaStream_t s);
+// The same product behind the fixed-point one: every kernel does nothing unless gate[0] != 0 when
+// it runs; scale: the vector's power-of-two exponent and a zero.
+int fast_apply_gated(hub_ctx *h, const double *x, double *y, const int *scale, const int *gate, cudaStream_t s);
+// The first n <= 4 scratch vectors of the handle, each large enough for a vector in either order.
+int fast_scratch(hub_ctx *h, int n, float **v);
+// Largest and smallest biased exponents of x per block: part[0 .. nblk) and part[nblk .. 2 nblk).
+int fast_exp_range(hub_ctx *h, const double *x, int64_t D, int **part, int *nblk, cudaStream_t s);
+// The handle's device error flag.
+int *fast_err(const hub_ctx *h);
 int fast_check_error(hub_ctx *h);
 // Lowest eigenvalues of the successive tridiagonals T_1, T_2, ... of one Lanczos run (host),
 // each by bisection on the Sturm count like tridiag_lowest, but started from a bracket around
@@ -193,6 +225,20 @@ double psi_eigenvalue(hub_ctx *h, double E0);
 inline bool use_fast(const hub_ctx *h) {
   return h->mode == HUB_MODE_AUTO && h->fast && !h->k0 && fast_eligible(h);
 }
+
+// The double-float window (hub_fast.cu): biased FP64 exponents of the largest entry, and how far
+// below it a nonzero entry may lie.
+constexpr int kExpSpan = 80, kExpLo = 200, kExpHi = 1900;
+
+// Fixed-point product and Lanczos (hub_fix.cu).
+bool fix_apply_eligible(const hub_ctx *h);
+int fix_apply(hub_ctx *h, const double *x, double *y, cudaStream_t s);
+bool fix_lanczos_eligible(const hub_ctx *h);
+int fix_lanczos(hub_ctx *h, const double *x0, int maxit, double tol, double *E0, double *psi_out, int *iters,
+                cudaStream_t s);
+void fix_release(hub_ctx *h);
+// v /= |v| (hub_lanczos.cu)
+int f64_normalise(hub_ctx *h, int64_t D, double *v, cudaStream_t s);
 
 // Single-launch Lanczos of small sectors (hub_small.cu).
 bool small_eligible(const hub_ctx *h);

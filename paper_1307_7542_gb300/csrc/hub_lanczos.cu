@@ -190,9 +190,14 @@ double LowestTracker::next(const double *a, const double *b, int k) {
 }
 
 // Eigenvector of T for eigenvalue lam by inverse iteration (tridiagonal LU with partial
-// pivoting), normalised, first nonzero component positive.
+// pivoting), normalised, first nonzero component positive.  The iteration starts from the first
+// unit vector: where T holds spurious copies of lam it then converges to their combination with
+// the largest first component, whose Ritz vector has norm 1 and the smallest residual (a start
+// from all ones gives an arbitrary combination: residuals of 1e-6 against 1e-11 once a level has
+// a second copy).
 std::vector<double> tridiag_vector(const double *a, const double *b, int k, double lam) {
-  std::vector<double> v(k, 1.0);
+  std::vector<double> v(k, 0.0);
+  v[0] = 1.0;
   if (k == 1) return v;
   const double scale = fabs(lam) + 1.0;
   const double shift = lam - 1e-13 * scale;   // keep T - shift*I nonsingular
@@ -298,12 +303,29 @@ static int k0_start(hub_ctx *h, const double **x0, double *w, cudaStream_t s) {
   return k0_project_inplace(h, w, s);
 }
 
-static int ensure_workspace(hub_ctx *h, int64_t D) {
-  for (int k = 0; k < 3; ++k)
-    if (!h->work[k] && !dev_alloc((void **)&h->work[k], sizeof(double) * D, "Lanczos vector")) return HUB_ERR_OOM;
+static int ensure_scalars(hub_ctx *h) {
   if (!h->d_scal && !dev_alloc((void **)&h->d_scal, sizeof(double) * 8, "Lanczos scalars")) return HUB_ERR_OOM;
   if (!h->h_scal) HUB_CUDA(cudaMallocHost((void **)&h->h_scal, sizeof(double) * 8));
   return ensure_partials(h, vec_grid());
+}
+
+int f64_normalise(hub_ctx *h, int64_t D, double *v, cudaStream_t s) {
+  int rc = ensure_scalars(h);
+  if (rc) return rc;
+  const int G = vec_grid(), T = kVecThreads;
+  count_launch(h, 3);
+  k_dot<<<G, T, 0, s>>>(D, v, v, h->partials);
+  HUB_LAUNCH_CHECK();
+  if ((rc = reduce_partials(h->partials, G, h->d_scal + 4, 1, s))) return rc;
+  k_scale_by<<<G, T, 0, s>>>(D, v, h->d_scal + 4);
+  HUB_LAUNCH_CHECK();
+  return HUB_OK;
+}
+
+static int ensure_workspace(hub_ctx *h, int64_t D) {
+  for (int k = 0; k < 3; ++k)
+    if (!h->work[k] && !dev_alloc((void **)&h->work[k], sizeof(double) * D, "Lanczos vector")) return HUB_ERR_OOM;
+  return ensure_scalars(h);
 }
 
 }  // namespace hub
@@ -319,15 +341,20 @@ extern "C" int hub_lanczos_ground(hub_t h, const double *x0_dev, int maxit, doub
   const int64_t D = vec_len(h);
   if (D == 0) return fail(HUB_ERR_ARG, "hub_lanczos_ground: empty sector");
   if (small_eligible(h)) return small_lanczos(h, x0_dev, maxit, tol, E0, psi_dev, iters, (cudaStream_t)stream);
-  if (use_fast(h)) {
-    if (!x0_dev) {
-      // the fast driver converts an FP64 start vector: draw it into the FP64 workspace
+  if (fix_lanczos_eligible(h)) {
+    const double *x0 = x0_dev;
+    if (!x0) {
+      // the fixed-point driver converts an FP64 start vector: draw it into the FP64 workspace
       if (!h->work[2] && !dev_alloc((void **)&h->work[2], sizeof(double) * D, "start vector")) return HUB_ERR_OOM;
       k_splitmix_uniform<<<vec_grid(), kVecThreads, 0, (cudaStream_t)stream>>>(D, h->work[2]);
       HUB_LAUNCH_CHECK();
-      x0_dev = h->work[2];
+      x0 = h->work[2];
     }
-    return fast_lanczos(h, x0_dev, maxit, tol, E0, psi_dev, iters, (cudaStream_t)stream);
+    rc = fix_lanczos(h, x0, maxit, tol, E0, psi_dev, iters, (cudaStream_t)stream);
+    if (rc != HUB_ERR_OOM) return rc;
+    fix_release(h);                   // its vectors do not fit: three FP64 ones may
+    h->fix_off = true;
+    set_error("");
   }
   rc = ensure_workspace(h, D);
   if (rc) return rc;
@@ -431,11 +458,7 @@ extern "C" int hub_lanczos_ground(hub_t h, const double *x0_dev, int maxit, doub
       w = t0;
     }
     // normalise psi
-    k_dot<<<G, T, 0, s>>>(D, psi_dev, psi_dev, P);
-    HUB_LAUNCH_CHECK();
-    if ((rc = reduce_partials(P, G, scal + 4, 1, s))) return rc;
-    k_scale_by<<<G, T, 0, s>>>(D, psi_dev, scal + 4);
-    HUB_LAUNCH_CHECK();
+    if ((rc = f64_normalise(h, D, psi_dev, s))) return rc;
     HUB_CUDA(cudaStreamSynchronize(s));
   }
   if (status == HUB_ERR_NOCONV) set_error("hub_lanczos_ground: maxit reached before |dE0| < tol");

@@ -445,6 +445,8 @@ extern "C" int hub_hopping(hub_t h, int n_bonds, const int32_t *bonds_host, cons
     bt.t[b] = t_host[b];
   }
   k0_leave(h);
+  fix_release(h);
+  h->fix_off = false;
   h->have_hop = false;
   h->n_bonds = n_bonds;
   h->bonds.assign(bonds_host, bonds_host + 2 * n_bonds);
@@ -556,6 +558,7 @@ extern "C" void hub_free(hub_t h) {
   dev_free(h->hx2);
   dev_free(h->hy2);
   fast_release(h);
+  fix_release(h);
   k0_release(h);
   small_release(h);
   for (int k = 0; k < hub_ctx::kProfKinds; ++k) {
