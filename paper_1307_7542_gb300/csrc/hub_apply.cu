@@ -8,47 +8,112 @@
 // The diagonal (Sec. III.B) is sum_i U_i bit_i(I_up & I_dn) + eps(I_up) + eps(I_dn),
 // computed on the fly from popcount instead of Algorithm II's index_U tables.
 //
-// Kernel shape (FP64 path): one CTA per row d of X (grid-stride).  The CTA stages row d
-// in shared memory when it fits; each thread owns columns u and sums the H_up row of u
-// (gather from shared memory) and the H_dn row of d (coalesced loads of the neighbour
-// rows X[d'][u], served from L2).
+// Kernel shape (FP64 path): a CTA takes two rows d of X and a chunk of columns u.  It stages both
+// rows in shared memory when they fit; each thread owns columns u and sums the H_up row of u
+// (gathers from shared memory; an entry is loaded once for both rows) and the H_dn rows of both d
+// (coalesced loads of the neighbour rows X[d'][u], served from L2).  The FP64 unit bounds it: one
+// multiply-add per term, at about 1/70 of the integer rate (disordered 3x4 lattice, 853,776 states,
+// 26 hops each: 56 us, with the Lanczos step around it 74 us; 47 us of FP64 issue).  Columns are cut
+// at multiples of a warp, since a partial warp costs the unit a whole one.
 #include "hub_internal.cuh"
 
 namespace hub {
 
-// gate: null, or a device flag; the kernel does nothing while gate[0] is 0 (the fast path
-// passes its out-of-window flag, so that this kernel multiplies exactly the vectors the
-// double-float kernels cannot).
-template <bool kStage>
-__global__ void __launch_bounds__(512) k_apply_f64(const Ham H, const double *__restrict__ x,
-                                                   double *__restrict__ y, const int *__restrict__ gate) {
+// The diagonal with the sums over doubly occupied sites from a table: one lookup per four sites
+// instead of one divergent read of the parameters per set bit.
+__device__ __forceinline__ double f64_diag(const Ham &H, const double (*s_U)[16], uint32_t both, int64_t u, int64_t d) {
+  double v;
+  if (H.uniform_U) {
+    v = H.U0 * (double)__popc(both);
+  } else {
+    v = s_U[0][both & 15];
+    for (int k = 1; 4 * k < H.M; ++k) v += s_U[k][(both >> 4 * k) & 15];
+  }
+  if (H.has_eps) v += H.eps_up[u] + H.eps_dn[d];
+  return v;
+}
+// The Lanczos step around a product, in the same kernel (hub_lanczos.cu): see F64Step.
+// kMode 0: y = H x.  kMode 1: y = inv (H x) - c prev and the CTA's part of inv <x, y>.
+// kMode 2: psi += v x, y = (H x - a x - c prev) inv (second pass, known coefficients).
+// gate: null, or a device flag; the kernel does nothing while gate[0] is 0 (the other paths
+// pass their out-of-window flag, so that this kernel multiplies exactly the vectors they cannot).
+template <bool kStage, int kMode, int kF64Rows>
+__global__ void __launch_bounds__(256, 6) k_apply_f64(const Ham H, const double *__restrict__ x, double *y,
+                                                   const int *__restrict__ gate, int chunks, const F64Step L) {
   if (gate && gate[0] == 0) return;
   extern __shared__ double xs[];
+  __shared__ double s_U[8][16];                  // sums of U_i over the set bits of each four sites
+  if (!H.uniform_U) {
+    if (threadIdx.x < 128 || blockDim.x < 128)
+      for (int k = threadIdx.x; k < 128; k += min(blockDim.x, 128)) {
+        double v = 0.0;
+        for (int i = 0; i < 4; ++i)
+          if (((k >> i) & 1) && (k >> 4) * 4 + i < H.M) v += H.U[(k >> 4) * 4 + i];
+        s_U[k >> 4][k & 15] = v;
+      }
+    __syncthreads();
+  }
   const int64_t nu = H.n_up, nd = H.n_dn;
-  for (int64_t d = blockIdx.x; d < nd; d += gridDim.x) {
+  const int64_t width = ((nu + chunks - 1) / chunks + 31) & ~(int64_t)31, items = (nd + kF64Rows - 1) / kF64Rows * chunks;
+  double inv = 1.0, c = 0.0, dot = 0.0;
+  if (kMode == 1) {
+    inv = L.scal->inv;
+    c = L.scal->c;
+  }
+  for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
+    const int64_t d = item / chunks * kF64Rows, u0 = item % chunks * width, u1 = min(nu, u0 + width);
+    const int rows = kF64Rows == 1 ? 1 : (int)min((int64_t)kF64Rows, nd - d);
     const double *__restrict__ xrow = x + d * nu;
     if (kStage) {
-      for (int64_t u = threadIdx.x; u < nu; u += blockDim.x) xs[u] = xrow[u];
+      if (item != blockIdx.x) __syncthreads();
+#pragma unroll 4
+      for (int64_t u = threadIdx.x; u < rows * nu; u += blockDim.x) xs[u] = xrow[u];
       __syncthreads();
     }
-    const uint32_t Id = H.basis_dn[d];
-    const int32_t k0 = H.rp_dn[d], k1 = H.rp_dn[d + 1];
-    for (int64_t u = threadIdx.x; u < nu; u += blockDim.x) {
-      const double xv = kStage ? xs[u] : xrow[u];
-      double acc = diag_of(H, H.basis_up[u], Id, u, d) * xv;
+    const double *r0 = kStage ? xs : xrow, *r1 = rows > 1 ? r0 + nu : r0;
+    const uint32_t Id0 = H.basis_dn[d], Id1 = rows > 1 ? H.basis_dn[d + 1] : 0u;
+    const int32_t k0 = H.rp_dn[d], k1 = H.rp_dn[d + 1], k2 = rows > 1 ? H.rp_dn[d + 2] : k1;
+    for (int64_t u = u0 + threadIdx.x; u < u1; u += blockDim.x) {
+      const double x0 = r0[u], x1 = r1[u];
+      const uint32_t Iu = H.basis_up[u];
+      double acc0 = f64_diag(H, s_U, Iu & Id0, u, d) * x0;
+      double acc1 = rows > 1 ? f64_diag(H, s_U, Iu & Id1, u, d + 1) * x1 : 0.0;
       const int32_t j0 = H.rp_up[u], j1 = H.rp_up[u + 1];
+#pragma unroll 2
       for (int32_t k = j0; k < j1; ++k) {
-        const int32_t c = H.col_up[k];
-        acc = fma(H.val_up[k], kStage ? xs[c] : xrow[c], acc);
+        const int32_t e = H.col_up[k];
+        const double v = H.val_up[k];
+        acc0 = fma(v, r0[e], acc0);
+        if (rows > 1) acc1 = fma(v, r1[e], acc1);
       }
-      for (int32_t k = k0; k < k1; ++k) acc = fma(H.val_dn[k], x[(int64_t)H.col_dn[k] * nu + u], acc);
-      y[d * nu + u] = acc;
+#pragma unroll 4
+      for (int32_t k = k0; k < k1; ++k) acc0 = fma(H.val_dn[k], x[(int64_t)H.col_dn[k] * nu + u], acc0);
+#pragma unroll 4
+      for (int32_t k = k1; k < k2; ++k) acc1 = fma(H.val_dn[k], x[(int64_t)H.col_dn[k] * nu + u], acc1);
+#pragma unroll
+      for (int r = 0; r < kF64Rows; ++r) {
+        if (r >= rows) break;
+        const int64_t o = (d + r) * nu + u;
+        double v = r ? acc1 : acc0;
+        const double xv = r ? x1 : x0;
+        if (kMode == 1) {
+          v = fma(-c, L.prev[o], inv * v);
+          dot = fma(xv, v, dot);
+        } else if (kMode == 2) {
+          L.psi[o] = fma(L.v, xv, L.psi[o]);
+          v = (fma(-L.a, xv, v) - L.b * L.prev[o]) * L.inv;
+        }
+        y[o] = v;
+      }
     }
-    if (kStage) __syncthreads();
   }
+  if (kMode == 1) f64_step_alpha(L, dot);
 }
 
-static size_t stage_bytes(const Ham &H) { return sizeof(double) * (size_t)H.n_up; }
+// Rows of a CTA: two; one where rows are so narrow that a CTA has few threads at work (12 columns x 924
+// rows: 8.1 us, 10.7 with two).
+static int f64_rows(const Ham &H) { return H.n_up > 128 ? 2 : 1; }
+static size_t stage_bytes(const Ham &H) { return sizeof(double) * (size_t)H.n_up * f64_rows(H); }
 
 static int apply_kernels(hub_ctx *h, const double *x, double *y, cudaStream_t s);
 
@@ -108,22 +173,43 @@ static int apply_kernels(hub_ctx *h, const double *x, double *y, cudaStream_t s)
   return f64_apply(h, x, y, nullptr, s);
 }
 
-int f64_apply(hub_ctx *h, const double *x, double *y, const int *gate, cudaStream_t s) {
+// Columns of a CTA: chunks of 256 and less where the row is short, so that a small matrix still makes
+// several CTAs per SM; a quarter of a longer row, which is staged once per chunk.
+static int f64_chunks(const Ham &H) { return (int)std::min<int64_t>(4, (H.n_up + 255) / 256); }
+int64_t f64_grid(const Ham &H) {
+  const int rows = f64_rows(H);
+  return std::min<int64_t>((H.n_dn + rows - 1) / rows * f64_chunks(H), (int64_t)num_sms() * 16);
+}
+bool f64_product(hub_ctx *h) {
+  return !h->k0 && (f64_is_faster(h) || (!fix_apply_eligible(h) && !use_fast(h)));
+}
+template <int kMode>
+static int f64_launch(hub_ctx *h, const double *x, double *y, const int *gate, const F64Step &L, cudaStream_t s) {
   const Ham H = h->view();
   count_launch(h);
   const size_t smem = stage_bytes(H);
-  const int threads = H.n_up >= 512 ? 512 : (H.n_up >= 128 ? 256 : 64);
-  int64_t grid = H.n_dn;
-  const int64_t cap = (int64_t)num_sms() * 8;
-  if (grid > cap) grid = cap;
-  if (smem <= 200 * 1024) {
-    HUB_CUDA(cudaFuncSetAttribute(k_apply_f64<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    k_apply_f64<true><<<(int)grid, threads, smem, s>>>(H, x, y, gate);
+  const int chunks = f64_chunks(H);
+  const int64_t width = (H.n_up + chunks - 1) / chunks;
+  const int threads = width > 128 ? 256 : (width > 64 ? 128 : 64);
+  const int grid = (int)f64_grid(H);
+  if (smem > 200 * 1024) {
+    k_apply_f64<false, kMode, 2><<<grid, threads, 0, s>>>(H, x, y, gate, chunks, L);
+  } else if (f64_rows(H) == 1) {
+    k_apply_f64<true, kMode, 1><<<grid, threads, smem, s>>>(H, x, y, gate, chunks, L);
   } else {
-    k_apply_f64<false><<<(int)grid, threads, 0, s>>>(H, x, y, gate);
+    HUB_CUDA(cudaFuncSetAttribute(k_apply_f64<true, kMode, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    k_apply_f64<true, kMode, 2><<<grid, threads, smem, s>>>(H, x, y, gate, chunks, L);
   }
   HUB_LAUNCH_CHECK();
   return HUB_OK;
+}
+int f64_apply(hub_ctx *h, const double *x, double *y, const int *gate, cudaStream_t s) {
+  return f64_launch<0>(h, x, y, gate, F64Step(), s);
+}
+int f64_apply_step(hub_ctx *h, const double *x, double *y, const F64Step &L, bool second, cudaStream_t s) {
+  int rc = prof_mark(h, HUB_PROF_APPLY, true, s);
+  if (rc || (rc = second ? f64_launch<2>(h, x, y, nullptr, L, s) : f64_launch<1>(h, x, y, nullptr, L, s))) return rc;
+  return prof_mark(h, HUB_PROF_APPLY, false, s);
 }
 
 static int check_ready(const hub_ctx *h, const char *who) {

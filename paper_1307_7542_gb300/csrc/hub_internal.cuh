@@ -86,6 +86,58 @@ __device__ __forceinline__ T warp_totals(T (&v)[N]) {
   return t;
 }
 
+// Scalars of the FP64 Lanczos recurrence on the device (hub_lanczos.cu).  The vectors are kept as they
+// leave the update, r_j = beta_j q_j; inv = 1 / beta_j and c = beta_j / beta_{j-1} scale the next product.
+struct F64Scal {
+  double inv, c, alpha;
+  double hist[2][2];                  // (alpha_j, beta_{j+1}) of the last two steps
+  unsigned ticket[2];
+};
+struct F64Step {
+  F64Scal *scal = nullptr;
+  double *partials = nullptr;
+  const double *prev = nullptr;       // may be the output
+  double *psi = nullptr;
+  double a = 0.0, b = 0.0, inv = 1.0, v = 0.0;   // second pass: alpha_j, beta_j, 1 / beta_{j+1}, v_j
+};
+
+// Adds the CTAs' values; true in the first thread of the last CTA to arrive, with *sum the total in
+// a fixed order.  Leaves the ticket at zero.  All threads of all CTAs of the launch take part.
+__device__ __forceinline__ bool grid_sum(double v, double *__restrict__ partials, unsigned *ticket, double *sum) {
+  __shared__ double ws[32];
+  __shared__ bool last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) ws[warp] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int k = 0; k < nw; ++k) s += ws[k];
+    partials[blockIdx.x] = s;
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    if (last) *ticket = 0;
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  double t = 0.0;
+  for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) t += __ldcg(partials + k);
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (lane == 0) ws[warp] = t;
+  __syncthreads();
+  if (threadIdx.x != 0) return false;
+  t = 0.0;
+  for (int k = 0; k < nw; ++k) t += ws[k];
+  *sum = t;
+  return true;
+}
+// The end of a step's first kernel: alpha_j from the parts of <r_j, w> / beta_j.
+__device__ __forceinline__ void f64_step_alpha(const F64Step &L, double dot) {
+  double sum;
+  if (grid_sum(dot, L.partials, &L.scal->ticket[0], &sum)) L.scal->alpha = L.scal->inv * sum;
+}
+
 }  // namespace hub
 
 // The handle behind the opaque hub_t.
@@ -185,6 +237,11 @@ int apply_launch(hub_ctx *h, const double *x, double *y, cudaStream_t s);
 // The FP64 product kernel of the full sector; with a gate it does nothing unless gate[0] != 0
 // when it runs (a device flag written earlier on the stream).
 int f64_apply(hub_ctx *h, const double *x, double *y, const int *gate, cudaStream_t s);
+// Whether products of the handle's vectors go to the FP64 kernel; its grid; and the product with the
+// Lanczos step around it (second: the pass that builds the Ritz vector).
+bool f64_product(hub_ctx *h);
+int64_t f64_grid(const hub::Ham &H);
+int f64_apply_step(hub_ctx *h, const double *x, double *y, const hub::F64Step &L, bool second, cudaStream_t s);
 
 // Fast path (hub_fast.cu).
 bool fast_eligible(const hub_ctx *h);

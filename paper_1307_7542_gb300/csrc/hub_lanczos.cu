@@ -51,39 +51,52 @@ __global__ void k_dot(int64_t n, const double *__restrict__ a, const double *__r
   block_partial(v, partials);
 }
 
-// w -= (*beta_prev) q_prev;  partials <- <q, w>
-__global__ void k_sub_dot(int64_t n, double *__restrict__ w, const double *__restrict__ q_prev,
-                          const double *__restrict__ q, const double *__restrict__ beta_prev,
-                          double *__restrict__ partials) {
-  const double bp = *beta_prev;
+// After a product y = H r_j of another path:  w = inv y - c r_{j-1} over y;  alpha_j = inv <r_j, w>.
+__global__ void k_step_dot(int64_t n, double *__restrict__ w, const double *__restrict__ r, const F64Step L) {
+  const double inv = L.scal->inv, c = L.scal->c;
   double v = 0.0;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-    double wk = fma(-bp, q_prev[k], w[k]);
+    const double wk = fma(-c, L.prev[k], inv * w[k]);
     w[k] = wk;
-    v = fma(q[k], wk, v);
+    v = fma(r[k], wk, v);
   }
-  block_partial(v, partials);
+  f64_step_alpha(L, v);
 }
 
-// w -= (*alpha) q;  partials <- |w|^2
-__global__ void k_sub_norm(int64_t n, double *__restrict__ w, const double *__restrict__ q,
-                           const double *__restrict__ alpha, double *__restrict__ partials) {
-  const double a = *alpha;
-  double v = 0.0;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-    double wk = fma(-a, q[k], w[k]);
-    w[k] = wk;
-    v = fma(wk, wk, v);
+// r_{j+1} = w - alpha_j q_j over w, beta_{j+1} = |r_{j+1}|; the last CTA moves the scalars on.
+__global__ void k_step_norm(int64_t n, double *__restrict__ w, const double *__restrict__ r, F64Scal *q, int slot,
+                            double *__restrict__ partials) {
+  const double a = q->alpha * q->inv;
+  double v = 0.0, sum;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t k0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k0 < n; k0 += 4 * stride) {
+    double x[4], y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int64_t k = k0 + i * stride;
+      x[i] = k < n ? r[k] : 0.0;
+      y[i] = k < n ? w[k] : 0.0;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int64_t k = k0 + i * stride;
+      if (k >= n) break;
+      y[i] = fma(-a, x[i], y[i]);
+      w[k] = y[i];
+      v = fma(y[i], y[i], v);
+    }
   }
-  block_partial(v, partials);
+  if (!grid_sum(v, partials, &q->ticket[1], &sum)) return;
+  const double beta = sqrt(sum);
+  q->hist[slot][0] = q->alpha;
+  q->hist[slot][1] = beta;
+  q->c = beta * q->inv;
+  q->inv = 1.0 / beta;
 }
 
-// w /= *beta; the first thread also records beta as the next beta_prev.
-__global__ void k_scale_inv(int64_t n, double *__restrict__ w, double *__restrict__ scal) {
-  const double inv = 1.0 / scal[1];
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-    w[k] *= inv;
-  if (blockIdx.x == 0 && threadIdx.x == 0) scal[2] = scal[1];
+__global__ void k_step_first(F64Scal *q) {
+  *q = F64Scal();
+  q->inv = 1.0;
 }
 
 // dst = src / *nrm
@@ -107,11 +120,13 @@ __global__ void k_axpy(int64_t n, double a, const double *__restrict__ x, double
     y[k] = fma(a, x[k], y[k]);
 }
 
-// w = H q already in w:  w -= a q + b q_prev;  then w /= c  (second pass, known coefficients)
-__global__ void k_recur(int64_t n, double *__restrict__ w, const double *__restrict__ q,
-                        const double *__restrict__ q_prev, double a, double b, double inv_c) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-    w[k] = (w[k] - a * q[k] - b * q_prev[k]) * inv_c;
+// w = H q already in w:  psi += v q, w -= a q + b q_prev;  then w /= c  (second pass, known coefficients)
+__global__ void k_recur(int64_t n, double *__restrict__ w, const double *__restrict__ q, const F64Step L) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+    const double qk = q[k];
+    L.psi[k] = fma(L.v, qk, L.psi[k]);
+    w[k] = (w[k] - L.a * qk - L.b * L.prev[k]) * L.inv;
+  }
 }
 
 // Start vector for x0 == NULL: uniform [-1, 1) from SplitMix64 (seed 0, counter k).
@@ -303,10 +318,12 @@ static int k0_start(hub_ctx *h, const double **x0, double *w, cudaStream_t s) {
   return k0_project_inplace(h, w, s);
 }
 
+constexpr size_t kStepScal = (sizeof(F64Scal) + sizeof(double) - 1) / sizeof(double);   // after d_scal's eight
+
 static int ensure_scalars(hub_ctx *h) {
-  if (!h->d_scal && !dev_alloc((void **)&h->d_scal, sizeof(double) * 8, "Lanczos scalars")) return HUB_ERR_OOM;
+  if (!h->d_scal && !dev_alloc((void **)&h->d_scal, sizeof(double) * (8 + kStepScal), "Lanczos scalars")) return HUB_ERR_OOM;
   if (!h->h_scal) HUB_CUDA(cudaMallocHost((void **)&h->h_scal, sizeof(double) * 8));
-  return ensure_partials(h, vec_grid());
+  return ensure_partials(h, std::max<int64_t>(vec_grid(), f64_grid(h->view())));
 }
 
 int f64_normalise(hub_ctx *h, int64_t D, double *v, cudaStream_t s) {
@@ -321,6 +338,18 @@ int f64_normalise(hub_ctx *h, int64_t D, double *v, cudaStream_t s) {
   HUB_LAUNCH_CHECK();
   return HUB_OK;
 }
+
+struct StepEvents {
+  cudaEvent_t e[2] = {nullptr, nullptr};
+  int create() {
+    for (cudaEvent_t &x : e) HUB_CUDA(cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
+    return HUB_OK;
+  }
+  ~StepEvents() {
+    for (cudaEvent_t x : e)
+      if (x) cudaEventDestroy(x);
+  }
+};
 
 static int ensure_workspace(hub_ctx *h, int64_t D) {
   for (int k = 0; k < 3; ++k)
@@ -377,7 +406,9 @@ extern "C" int hub_lanczos_ground(hub_t h, const double *x0_dev, int maxit, doub
   if ((rc = reduce_partials(P, G, scal + 3, 1, s))) return rc;
   k_copy_scaled<<<G, T, 0, s>>>(D, q, x0, scal + 3);
   HUB_CUDA(cudaMemsetAsync(qp, 0, sizeof(double) * D, s));
-  HUB_CUDA(cudaMemsetAsync(scal + 2, 0, sizeof(double), s));
+  F64Scal *sc = reinterpret_cast<F64Scal *>(scal + 8);
+  k_step_first<<<1, 1, 0, s>>>(sc);
+  HUB_LAUNCH_CHECK();
   HUB_CUDA(cudaMemcpyAsync(h->h_scal + 3, scal + 3, sizeof(double), cudaMemcpyDeviceToHost, s));
   HUB_CUDA(cudaStreamSynchronize(s));
   h->start_norm = h->h_scal[3];
@@ -389,18 +420,44 @@ extern "C" int hub_lanczos_ground(hub_t h, const double *x0_dev, int maxit, doub
   double E = 0.0, E_prev = 0.0;
   LowestTracker lowest;
   int status = HUB_ERR_NOCONV;
+  // Step j, its coefficients on the way to the host.  The product carries the step's first half where it
+  // runs in the FP64 kernel.
+  const bool fused = f64_product(h);
+  StepEvents ev;
+  if ((rc = ev.create())) return rc;
+  auto step = [&](int j) -> int {
+    F64Step L;
+    L.scal = sc;
+    L.partials = P;
+    L.prev = qp;
+    int rc2 = fused ? f64_apply_step(h, q, w, L, false, s) : apply_launch(h, q, w, s);
+    if (rc2) return rc2;
+    if (!fused) {
+      count_launch(h);
+      k_step_dot<<<G, T, 0, s>>>(D, w, q, L);
+      HUB_LAUNCH_CHECK();
+    }
+    count_launch(h);
+    k_step_norm<<<G, T, 0, s>>>(D, w, q, sc, j & 1, P);
+    HUB_LAUNCH_CHECK();
+    HUB_CUDA(cudaMemcpyAsync(h->h_scal + 2 * (j & 1), sc->hist[j & 1], 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
+    HUB_CUDA(cudaEventRecord(ev.e[j & 1], s));
+    double *t0 = qp;
+    qp = q;
+    q = w;
+    w = t0;
+    return HUB_OK;
+  };
+  // The next step is enqueued before the last one's coefficients are looked at, so that the device does
+  // not wait for the host (10 us and more of a step's 40 at 0.85 M states); a converged run has then
+  // taken one step too many, which is why larger vectors, whose steps hide the host, do not.
+  const bool ahead = tol <= 0 || D <= (int64_t)1 << 22;
+  int queued = 0;
   for (int j = 0; j < maxit; ++j) {
-    if ((rc = apply_launch(h, q, w, s))) return rc;
-    count_launch(h, 5);   // sub_dot, reduce, sub_norm, reduce, scale_inv
-    k_sub_dot<<<G, T, 0, s>>>(D, w, qp, q, scal + 2, P);
-    HUB_LAUNCH_CHECK();
-    if ((rc = reduce_partials(P, G, scal + 0, 0, s))) return rc;
-    k_sub_norm<<<G, T, 0, s>>>(D, w, q, scal + 0, P);
-    HUB_LAUNCH_CHECK();
-    if ((rc = reduce_partials(P, G, scal + 1, 1, s))) return rc;
-    HUB_CUDA(cudaMemcpyAsync(h->h_scal, scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
-    HUB_CUDA(cudaStreamSynchronize(s));
-    const double a = h->h_scal[0], b = h->h_scal[1];
+    for (; queued <= (ahead ? std::min(j + 1, maxit - 1) : j); ++queued)
+      if ((rc = step(queued))) return rc;
+    HUB_CUDA(cudaEventSynchronize(ev.e[j & 1]));
+    const double a = h->h_scal[2 * (j & 1)], b = h->h_scal[2 * (j & 1) + 1];
     if (!std::isfinite(a) || !std::isfinite(b)) return fail(HUB_ERR_CUDA, "hub_lanczos_ground: non-finite alpha/beta");
     h->alpha.push_back(a);
     h->beta.push_back(b);
@@ -414,15 +471,8 @@ extern "C" int hub_lanczos_ground(hub_t h, const double *x0_dev, int maxit, doub
       status = HUB_CONVERGED_BREAKDOWN;
       break;
     }
-    if (j + 1 < maxit) {
-      k_scale_inv<<<G, T, 0, s>>>(D, w, scal);
-      HUB_LAUNCH_CHECK();
-      double *t0 = qp;
-      qp = q;
-      q = w;
-      w = t0;
-    }
   }
+  HUB_CUDA(cudaStreamSynchronize(s));
   if (tol <= 0 && status == HUB_ERR_NOCONV) status = HUB_OK;
   if (tol <= 0) E = tridiag_lowest(h->alpha.data(), h->beta.data(), (int)h->alpha.size());
   *E0 = E;
@@ -446,12 +496,23 @@ extern "C" int hub_lanczos_ground(hub_t h, const double *x0_dev, int maxit, doub
     HUB_CUDA(cudaMemsetAsync(qp, 0, sizeof(double) * D, s));
     HUB_CUDA(cudaMemsetAsync(psi_dev, 0, sizeof(double) * D, s));
     for (int j = 0; j < k; ++j) {
-      k_axpy<<<G, T, 0, s>>>(D, v[j], q, psi_dev);
-      HUB_LAUNCH_CHECK();
-      if (j + 1 == k) break;
-      if ((rc = apply_launch(h, q, w, s))) return rc;
-      k_recur<<<G, T, 0, s>>>(D, w, q, qp, h->alpha[j], j ? h->beta[j - 1] : 0.0, 1.0 / h->beta[j]);
-      HUB_LAUNCH_CHECK();
+      if (j + 1 == k) {
+        k_axpy<<<G, T, 0, s>>>(D, v[j], q, psi_dev);
+        HUB_LAUNCH_CHECK();
+        break;
+      }
+      F64Step L;
+      L.prev = qp;
+      L.psi = psi_dev;
+      L.a = h->alpha[j];
+      L.b = j ? h->beta[j - 1] : 0.0;
+      L.inv = 1.0 / h->beta[j];
+      L.v = v[j];
+      if ((rc = fused ? f64_apply_step(h, q, w, L, true, s) : apply_launch(h, q, w, s))) return rc;
+      if (!fused) {
+        k_recur<<<G, T, 0, s>>>(D, w, q, L);
+        HUB_LAUNCH_CHECK();
+      }
       double *t0 = qp;
       qp = q;
       q = w;
