@@ -82,7 +82,7 @@ struct SmallState {
 struct SmallArgs {
   Ham H;
   int64_t D;
-  double *V0, *V1, *V2;        // Lanczos vectors in slot j % 3 (S_j in the grid form, q_j in the cluster form)
+  double *V0, *V1, *V2;        // Lanczos vectors in slot j % 3 (S_j in the grid form, r_j in the cluster form)
   const double *x0;            // start vector (nullptr: SplitMix64 uniform [-1, 1), seed 0)
   double *part, *hist, *start;
   const double *coef;          // mode 1: y
@@ -108,9 +108,9 @@ __device__ __forceinline__ double cta_sum(double v, double *red) {
   __syncthreads();
   if (lane == 0) red[wid] = v;
   __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0)
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += red[k];
+  if (wid != 0) return 0.0;
+  double s = lane < (int)(blockDim.x >> 5) ? red[lane] : 0.0;
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   return s;
 }
 
@@ -346,15 +346,16 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_lanczos(const SmallA
 
 // ---------------------------------------------------------------------------------------
 // Sectors of at most kSmallClusterMax states: one thread-block cluster (at most 16 CTAs, one
-// GPC).  Here the Lanczos vectors are normalised explicitly (q_j); each thread keeps its states'
-// q_j, q_{j-1} and w in registers, and every CTA holds the whole of q_j in shared memory: once
-// beta_j is known each CTA writes its slice of q_{j+1} into the shared memory of every CTA of
-// the cluster (distributed shared memory), so inside a launch no vector passes through L2.
-// Per iteration three cluster barriers: after the <q_j, w> partials, after the |w|^2 partials,
-// after the broadcast of q_{j+1} (shared-memory copies alternate, so a broadcast never
-// overwrites the copy a slower CTA is still reading).  The last two vectors of a launch also go
-// to global memory (slot j % 3), where the next launch of the run finds q_{j0} and q_{j0-1}; the
-// psi pass repeats the same operations with the recorded alpha_j, beta_j.
+// GPC).  Each thread keeps its states' r_j, r_{j-1} and w in registers (r_j = beta_{j-1} q_j, as the
+// update leaves it), and every CTA holds the whole of r_j in shared memory: each CTA writes its slice
+// of r_{j+1} into the shared memory of every CTA of the cluster (distributed shared memory), so
+// inside a launch no vector passes through L2.  Per iteration two cluster barriers, which is what
+// bounds it together with the latency of the FP64 sums: after the <r_j, w> partials, and after the
+// |w|^2 partials and r_{j+1} (shared-memory copies alternate, so a broadcast never overwrites the
+// copy a slower CTA is still reading: that one has passed a barrier since).  8-site ring, 57 iterations
+// and psi: 0.97 ms; 1.13 ms with a third barrier for the normalised vector, set-up per iteration and
+// serial sums over the warps.  The last two vectors of a launch also go to global memory (slot j % 3), where the next launch of the run
+// finds them; the psi pass repeats the same operations with the recorded alpha_j, beta_j.
 // ---------------------------------------------------------------------------------------
 constexpr int kClusterE = 3;        // states per thread at most
 
@@ -383,35 +384,51 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_cluster(const SmallA
     return;
   }
   int64_t nid[kClusterE];
-  double q[kClusterE], qp[kClusterE], w[kClusterE], psi[kClusterE];
+  double r[kClusterE], rp[kClusterE], w[kClusterE], psi[kClusterE], dg[kClusterE];
+  int row[kClusterE], col[kClusterE], up0[kClusterE], up1[kClusterE], dn0[kClusterE], dn1[kClusterE];
 #pragma unroll
   for (int e = 0; e < kClusterE; ++e) {
     nid[e] = lo + threadIdx.x + (int64_t)e * blockDim.x;
-    q[e] = qp[e] = w[e] = psi[e] = 0.0;
+    r[e] = rp[e] = w[e] = psi[e] = dg[e] = 0.0;
+    row[e] = col[e] = up0[e] = up1[e] = dn0[e] = dn1[e] = 0;
+    if (nid[e] < hi) {                // the state's place, diagonal and entries stay the same
+      const int n = (int)nid[e], d = n / (int)nu, u = n - d * (int)nu;
+      const uint32_t Iu = __ldg(H.basis_up + u), Id = __ldg(H.basis_dn + d);
+      dg[e] = (H.uniform_U && !H.has_eps) ? s_diag[__popc(Iu & Id)] : diag_of(H, Iu, Id, u, d);
+      row[e] = d * (int)nu;
+      col[e] = u;
+      up0[e] = __ldg(H.rp_up + u);
+      up1[e] = __ldg(H.rp_up + u + 1);
+      dn0[e] = __ldg(H.rp_dn + d);
+      dn1[e] = __ldg(H.rp_dn + d + 1);
+    }
   }
   auto own = [&](int e) { return nid[e] < hi; };
   double *cur = xs, *nxt = xs + D;
-  // q (q_{j+1}) into every CTA's copy dst and, when `global`, into global slot k: the next launch
+  // v into every CTA's copy dst and, when `global`, into global slot k: the next launch
   // of the run reads only the last two vectors of this one, so only those are stored (fewer
   // stores for the cluster barrier's release to wait for)
-  auto publish = [&](double *dst, int k, bool global) {
+  auto publish = [&](const double *v, double *dst, int k, bool global) {
 #pragma unroll
     for (int e = 0; e < kClusterE; ++e)
       if (own(e)) {
-        if (global) V(k)[nid[e]] = q[e];
-        for (int r = 0; r < G; ++r) cl.map_shared_rank(dst, (unsigned)r)[nid[e]] = q[e];
+        if (global) V(k)[nid[e]] = v[e];
+        for (int b = 0; b < G; ++b) cl.map_shared_rank(dst, (unsigned)b)[nid[e]] = v[e];
       }
   };
-  double bp = 0.0;
-  if (A.j0 == 0) {                    // q_0 = x0 / |x0|
+  double inv, c = 0.0;                // q_j = inv r_j;  beta_{j-1} q_{j-1} = c r_{j-1}
+  if (A.j0 == 0) {                    // r_0 = x0
     double nn = 0.0;
 #pragma unroll
     for (int e = 0; e < kClusterE; ++e)
       if (own(e)) {
-        q[e] = A.x0 ? A.x0[nid[e]] : splitmix_uniform(nid[e]);
-        nn = fma(q[e], q[e], nn);
+        r[e] = A.x0 ? A.x0[nid[e]] : splitmix_uniform(nid[e]);
+        nn = fma(r[e], r[e], nn);
       }
     double s2;
+    // no CTA may write into another's shared memory before that one runs
+    cl.sync();
+    publish(r, cur, 0, A.mode == 0);
     gs.total(nn, &s2);
     const double s = sqrt(s2);
     const bool good = s > 0.0 && isfinite(s);
@@ -423,28 +440,26 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_cluster(const SmallA
       gs.leave();
       return;
     }
-    const double inv = 1.0 / s;
-#pragma unroll
-    for (int e = 0; e < kClusterE; ++e) q[e] *= inv;
-    publish(cur, 0, A.mode == 0);
-    cl.sync();
-  } else {                            // q_{j0}, q_{j0-1} and beta_{j0-1} from the earlier launches
-    bp = __ldcg(A.hist + 2 * (A.j0 - 1) + 1);
+    inv = 1.0 / s;
+  } else {                            // r_{j0}, r_{j0-1} and their norms from the earlier launches
+    const double b = __ldcg(A.hist + 2 * (A.j0 - 1) + 1);
+    inv = 1.0 / b;
+    c = b / (A.j0 >= 2 ? __ldcg(A.hist + 2 * (A.j0 - 2) + 1) : __ldcg(A.start));
     const double *Q = V(A.j0 % 3), *Qp = V((A.j0 + 2) % 3);
 #pragma unroll
     for (int e = 0; e < kClusterE; ++e)
       if (own(e)) {
-        q[e] = __ldcg(Q + nid[e]);
-        qp[e] = __ldcg(Qp + nid[e]);
+        r[e] = __ldcg(Q + nid[e]);
+        rp[e] = __ldcg(Qp + nid[e]);
       }
     for (int64_t k = threadIdx.x; k < D; k += blockDim.x) cur[k] = __ldcg(Q + k);
     __syncthreads();
   }
   for (int j = A.j0; j < A.j1; ++j) {
     if (A.mode == 1) {                // psi += y_j q_j
-      const double y = A.coef[j];
+      const double y = A.coef[j] * inv;
 #pragma unroll
-      for (int e = 0; e < kClusterE; ++e) psi[e] = j == 0 ? y * q[e] : fma(y, q[e], psi[e]);
+      for (int e = 0; e < kClusterE; ++e) psi[e] = j == 0 ? y * r[e] : fma(y, r[e], psi[e]);
       if (j + 1 == A.j1) break;
     }
     // w = H q_j - beta_{j-1} q_{j-1}
@@ -452,32 +467,36 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_cluster(const SmallA
 #pragma unroll
     for (int e = 0; e < kClusterE; ++e)
       if (own(e)) {
-        const int64_t n = nid[e], d = n / nu, u = n - d * nu;
-        const uint32_t Iu = __ldg(H.basis_up + u), Id = __ldg(H.basis_dn + d);
-        const double dg = (H.uniform_U && !H.has_eps) ? s_diag[__popc(Iu & Id)] : diag_of(H, Iu, Id, u, d);
         double acc_up = 0.0, acc_dn = 0.0;
-        const double *row = cur + d * nu;
-        for (int32_t k = __ldg(H.rp_up + u), k1 = __ldg(H.rp_up + u + 1); k < k1; ++k)
-          acc_up = fma(__ldg(H.val_up + k), row[__ldg(H.col_up + k)], acc_up);
-        for (int32_t k = __ldg(H.rp_dn + d), k1 = __ldg(H.rp_dn + d + 1); k < k1; ++k)
-          acc_dn = fma(__ldg(H.val_dn + k), cur[(int64_t)__ldg(H.col_dn + k) * nu + u], acc_dn);
-        double v = fma(dg, q[e], acc_up + acc_dn);
-        if (j) v = fma(-bp, qp[e], v);
+#pragma unroll 4
+        for (int k = up0[e]; k < up1[e]; ++k)
+          acc_up = fma(__ldg(H.val_up + k), cur[row[e] + __ldg(H.col_up + k)], acc_up);
+#pragma unroll 4
+        for (int k = dn0[e]; k < dn1[e]; ++k)
+          acc_dn = fma(__ldg(H.val_dn + k), cur[__ldg(H.col_dn + k) * (int)nu + col[e]], acc_dn);
+        const double v = fma(-c, rp[e], inv * fma(dg[e], r[e], acc_up + acc_dn));
         w[e] = v;
-        dot = fma(q[e], v, dot);
+        dot = fma(r[e], v, dot);
       }
-    double b;
+    double a, b;
     if (A.mode == 0) {
-      double a, b2;
       gs.total(dot, &a);
-      double nn = 0.0;
+      a *= inv;
+    } else {                          // psi pass: the recorded coefficients
+      a = __ldcg(A.hist + 2 * j);
+    }
+    double nn = 0.0;
+    const double ai = a * inv;
 #pragma unroll
-      for (int e = 0; e < kClusterE; ++e)
-        if (own(e)) {
-          w[e] = fma(-a, q[e], w[e]);
-          nn = fma(w[e], w[e], nn);
-        }
-      gs.total(nn, &b2);
+    for (int e = 0; e < kClusterE; ++e)
+      if (own(e)) {
+        w[e] = fma(-ai, r[e], w[e]);
+        nn = fma(w[e], w[e], nn);
+      }
+    publish(w, nxt, (j + 1) % 3, A.mode == 0 && j + 2 >= A.j1);
+    if (A.mode == 0) {
+      double b2;
+      gs.total(nn, &b2);              // its barrier completes r_{j+1} too
       b = sqrt(b2);
       if (lead) {
         A.hist[2 * j] = a;
@@ -489,24 +508,20 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_cluster(const SmallA
         gs.leave();
         return;
       }
-    } else {                          // psi pass: the recorded coefficients
-      const double a = __ldcg(A.hist + 2 * j);
-#pragma unroll
-      for (int e = 0; e < kClusterE; ++e) w[e] = fma(-a, q[e], w[e]);
+    } else {
       b = __ldcg(A.hist + 2 * j + 1);
+      cl.sync();
     }
-    const double inv = 1.0 / b;       // q_{j+1} = w / beta_j
 #pragma unroll
     for (int e = 0; e < kClusterE; ++e) {
-      qp[e] = q[e];
-      q[e] = w[e] * inv;
+      rp[e] = r[e];
+      r[e] = w[e];
     }
-    publish(nxt, (j + 1) % 3, A.mode == 0 && j + 2 >= A.j1);
-    cl.sync();
+    c = b * inv;
+    inv = 1.0 / b;
     double *t = cur;
     cur = nxt;
     nxt = t;
-    bp = b;
   }
   if (A.mode == 1) {                  // psi /= |psi|
     double nn = 0.0, p2;
@@ -514,10 +529,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_cluster(const SmallA
     for (int e = 0; e < kClusterE; ++e)
       if (own(e)) nn = fma(psi[e], psi[e], nn);
     gs.total(nn, &p2);
-    const double inv = 1.0 / sqrt(p2);
+    const double s = 1.0 / sqrt(p2);
 #pragma unroll
     for (int e = 0; e < kClusterE; ++e)
-      if (own(e)) A.psi[nid[e]] = psi[e] * inv;
+      if (own(e)) A.psi[nid[e]] = psi[e] * s;
   }
   gs.leave();
 }
