@@ -588,8 +588,9 @@ __global__ void __launch_bounds__(1024, 1) k_fix_gather(const FixPass P, const G
 // of a bank share a step.  By Koenig's theorem as many steps suffice as the largest degree has
 // edges; they are found edge by edge, exchanging two colours along an alternating path where the
 // lane and the bank have no free step in common.  A bank with more entries than cap_steps takes
-// the rest in steps of its lanes alone (conflicts, but the schedule stays bounded).  One thread
-// per group (quads 4 g .. 4 g + 3 of quad).  deg[g] = its steps.
+// the rest in steps of its lanes alone (conflicts, but the schedule stays bounded).  A warp per
+// group (quads 4 g .. 4 g + 3 of quad), one lane of which colours, with the free steps of lanes and
+// banks as bit masks: 93 us at 4x4 (a thread per group and linear searches: 0.8 ms).  deg[g] = its steps.
 constexpr int kSchedRow = 64;         // longest hopping row of the gather form
 constexpr int kSchedMax = 2 * kSchedRow;
 constexpr uint16_t kNoEntry = 0xffff;
@@ -598,43 +599,45 @@ __global__ void __launch_bounds__(32) k_fix_schedule(int n, int groups, int idle
                                                      const int32_t *__restrict__ rp,
                                                      const uint32_t *__restrict__ scol, uint16_t *__restrict__ word,
                                                      uint16_t *__restrict__ deg) {
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  const int g = blockIdx.x, lane = threadIdx.x;
   if (g >= groups) return;
-  uint16_t at[16][kSchedMax];         // entry of a lane at a step
-  int8_t who[16][kSchedMax];          // lane that reads a bank at a step
-  int load[16];
-  for (int b = 0; b < 16; ++b) {
-    load[b] = 0;
-    for (int j = 0; j < cap_steps; ++j) {
-      at[b][j] = kNoEntry;
-      who[b][j] = -1;
-    }
+  __shared__ uint16_t at[16][kSchedMax];         // entry of a lane at a step
+  __shared__ int8_t who[16][kSchedMax];          // lane that reads a bank at a step
+  __shared__ u64 free_l[16][2], free_b[16][2];   // free steps
+  __shared__ int load[16];
+  if (lane < 16) load[lane] = 0;
+  for (int k = lane; k < 16 * kSchedMax; k += 32) {
+    at[k / kSchedMax][k % kSchedMax] = kNoEntry;
+    who[k / kSchedMax][k % kSchedMax] = -1;
   }
+  __syncwarp();
+  const int own = quad[4 * g + ((lane & 15) >> 2)] * 4 + (lane & 3);
   int steps = 0;
-  for (int l = 0; l < 16; ++l) {
-    const int r = quad[4 * g + (l >> 2)] * 4 + (l & 3);
-    if (r >= n) continue;
-    steps = max(steps, rp[r + 1] - rp[r]);
-    for (int32_t k = rp[r]; k < rp[r + 1]; ++k) ++load[scol[k] & 15];
+  if (lane < 16 && own < n) {
+    steps = rp[own + 1] - rp[own];
+    for (int32_t k = rp[own]; k < rp[own + 1]; ++k) atomicAdd(&load[scol[k] & 15], 1);
   }
-  for (int b = 0; b < 16; ++b) steps = max(steps, load[b]);
-  steps = min(steps, cap_steps);
-  for (int l = 0; l < 16; ++l) {
+  __syncwarp();
+  steps = min(__reduce_max_sync(0xffffffffu, max(steps, load[lane & 15])), cap_steps);
+  if (lane < 16)
+    for (int h = 0; h < 2; ++h) {
+      const int m = min(max(steps - 64 * h, 0), 64);
+      free_l[lane][h] = free_b[lane][h] = m == 64 ? ~0ull : (1ull << m) - 1ull;
+    }
+  __syncwarp();
+  auto first = [](u64 a, u64 b) { return a ? __ffsll((long long)a) - 1 : (b ? 63 + __ffsll((long long)b) : -1); };
+  for (int l = 0; lane == 0 && l < 16; ++l) {
     const int r = quad[4 * g + (l >> 2)] * 4 + (l & 3);
     if (r >= n) continue;
     for (int32_t k = rp[r]; k < rp[r + 1]; ++k) {
       const uint32_t w = scol[k];
       const uint16_t v = (uint16_t)((w & 0x3fffu) | (w >> 31 ? 0x4000u : 0xc000u));     // esign -1 adds
       const int b = w & 15;
-      int x = -1, y = -1;             // a free step of the lane, one of the bank, one of both
-      for (int j = 0; j < steps; ++j) {
-        const bool fl = at[l][j] == kNoEntry, fb = who[b][j] < 0;
-        if (fl && fb) {
-          x = y = j;
-          break;
-        }
-        if (fl && x < 0) x = j;
-        if (fb && y < 0) y = j;
+      // a step free for both, or one of the lane and one of the bank
+      int x = first(free_l[l][0] & free_b[b][0], free_l[l][1] & free_b[b][1]), y = x;
+      if (x < 0) {
+        x = first(free_l[l][0], free_l[l][1]);
+        y = first(free_b[b][0], free_b[b][1]);
       }
       bool ok = y >= 0;
       if (ok && x != y) {
@@ -657,27 +660,38 @@ __global__ void __launch_bounds__(32) k_fix_schedule(int n, int groups, int idle
           ok = who[cb][y] == l1 && m < 32;   // else it meets an entry without a bank of its own
         }
         for (int i = 0; ok && i < m; ++i) {
-          at[(int)pl[i]][i & 1 ? y : x] = kNoEntry;
-          who[(int)pb[i]][i & 1 ? y : x] = -1;
+          const int t = i & 1 ? y : x;
+          at[(int)pl[i]][t] = kNoEntry;
+          who[(int)pb[i]][t] = -1;
+          free_l[(int)pl[i]][t >> 6] |= 1ull << (t & 63);
+          free_b[(int)pb[i]][t >> 6] |= 1ull << (t & 63);
         }
         for (int i = 0; ok && i < m; ++i) {
-          at[(int)pl[i]][i & 1 ? x : y] = pv[i];
-          who[(int)pb[i]][i & 1 ? x : y] = pl[i];
+          const int t = i & 1 ? x : y;
+          at[(int)pl[i]][t] = pv[i];
+          who[(int)pb[i]][t] = pl[i];
+          free_l[(int)pl[i]][t >> 6] &= ~(1ull << (t & 63));
+          free_b[(int)pb[i]][t >> 6] &= ~(1ull << (t & 63));
         }
       }
       at[l][x] = v;                   // the lane has a free step: steps >= its entries
-      if (ok) who[b][x] = (int8_t)l;
+      free_l[l][x >> 6] &= ~(1ull << (x & 63));
+      if (ok) {
+        who[b][x] = (int8_t)l;
+        free_b[b][x >> 6] &= ~(1ull << (x & 63));
+      }
     }
   }
+  __syncwarp();
   // idle lanes read the zero of a bank the step leaves free
   uint16_t *out = word + (size_t)g * cap_steps * 16;
-  for (int j = 0; j < cap_steps; ++j) {
+  for (int j = lane; j < cap_steps; j += 32) {
     int fb = 0;
     while (fb < 15 && who[fb][j] >= 0) ++fb;
     const uint16_t z = (uint16_t)((idle + ((fb - idle) & 15)) | 0x4000);
     for (int l = 0; l < 16; ++l) out[j * 16 + l] = at[l][j] == kNoEntry ? z : at[l][j];
   }
-  deg[g] = (uint16_t)steps;
+  if (lane == 0) deg[g] = (uint16_t)steps;
 }
 // The groups' schedules side by side in the slices' layout.
 __global__ void k_fix_pack(const int32_t *__restrict__ group, int cap_steps, const uint16_t *__restrict__ in,
@@ -1371,7 +1385,7 @@ static i64 fix_ld(i64 n) { return (n + 3) & ~(i64)3; }
 static int grid_of(i64 n) { return (int)std::max<i64>(1, std::min<i64>((n + 255) / 256, (i64)num_sms() * 16)); }
 
 // Groups of 16 positions for a gather schedule: four quads of consecutive positions each (the
-// outputs of a quad are one 32-byte sector), chosen greedily among the next 64 quads, longest rows
+// outputs of a quad are one 32-byte sector), chosen greedily among the next 32 quads, longest rows
 // first, so that the group's busiest bank stays low; or the quads in their own order where that
 // needs no more steps.  At 4x4 1.17 steps per entry of a row against 1.26.
 static std::vector<int32_t> gather_groups(int n, const SpinCSR &c, int *rc) {
@@ -1406,20 +1420,21 @@ static std::vector<int32_t> gather_groups(int n, const SpinCSR &c, int *rc) {
   std::stable_sort(left.begin(), left.end(), [&](int a, int b) { return len[a] > len[b]; });
   size_t head = 0;
   for (int g = 0; g < groups; ++g) {
-    int sum[16] = {0};
+    int32_t sum[16] = {0};               // at most 4 quads of 4 rows of kSchedRow entries: 2^10
     for (int k = 0; k < 4; ++k) {
       size_t pick = head;
-      i64 score = INT64_MAX;
-      for (size_t i = head; i < std::min(left.size(), head + (k ? 64 : 1)); ++i) {
+      int64_t score = INT64_MAX;
+      for (size_t i = head; i < std::min(left.size(), head + (k ? 32 : 1)); ++i) {
         const int32_t *l = &load[16 * (size_t)left[i]];
-        i64 m = 0, sq = 0;
+        int32_t m = 0, sq = 0;
         for (int b = 0; b < 16; ++b) {
-          const i64 v = sum[b] + l[b];
+          const int32_t v = sum[b] + l[b];
           m = std::max(m, v);
           sq += v * v;
         }
-        if ((m << 32) + sq < score) {
-          score = (m << 32) + sq;
+        const int64_t sc2 = ((int64_t)m << 32) + sq;
+        if (sc2 < score) {
+          score = sc2;
           pick = i;
         }
       }
@@ -1456,7 +1471,7 @@ static int gather_tables(FixState *f, int s, int n, const SpinCSR &c) {
   cudaError_t e = cudaSuccess;
   if (rc == HUB_OK) e = cudaMemcpy(quad, q.data(), sizeof(int32_t) * q.size(), cudaMemcpyHostToDevice);
   if (rc == HUB_OK && e == cudaSuccess) {
-    k_fix_schedule<<<(groups + 31) / 32, 32>>>(n, groups, (int)fix_ld(n), cap, quad, c.rowptr, c.scol, tmp, deg);
+    k_fix_schedule<<<groups, 32>>>(n, groups, (int)fix_ld(n), cap, quad, c.rowptr, c.scol, tmp, deg);
     e = cudaMemcpy(d.data(), deg, sizeof(uint16_t) * groups, cudaMemcpyDeviceToHost);
     for (int g = 0; g < groups; ++g) order[g] = g;
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return d[a] > d[b]; });
