@@ -26,7 +26,7 @@
 // the order in which blocks finish.  A start vector of random numbers keeps max |s_j| / rms(s_j)
 // below 2^6.5, so an entry carries 49 bits and more below the rms, against 48 significant bits of
 // double-float arithmetic.  Against long double (12-site ring, 12 steps) alpha and beta are off by
-// 1.4e-14 and 1.8e-15 at U = 7.25, by 6e-10 and 2.5e-10 at U = 4000 (double-float 5.7e-14, 1.8e-15,
+// 1.4e-14 and 1.8e-15 at U = 7.25, by 9.9e-10 and 4.2e-10 at U = 4000 (double-float 5.7e-14, 1.8e-15,
 // 1.1e-9 and 6.7e-10).
 //
 // Products for a caller (hub_apply) must keep every entry within 1e-13 (|H||x|)_n, which a grid
@@ -36,8 +36,8 @@
 // beforehand), or with more such entries than the list holds, is multiplied by the double-float
 // or FP64 kernels instead, all on device flags, without a host round trip.
 //
-// Measured on the 4x4 cluster at half filling (1.66e8 states): a Lanczos step 4.15 ms (passes 1.32
-// and 1.32, update 1.44) against 4.96 ms in double-float; a product 4.4 ms against 6.2 ms.
+// Measured on the 4x4 cluster at half filling (1.66e8 states): a Lanczos step 4.12 ms (passes 1.32
+// and 1.31, update 1.38) against 5.0 ms in double-float; a product 4.2 ms against 6.1 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -1149,63 +1149,52 @@ __global__ void __launch_bounds__(256) k_fix_rescale(const FixScal *__restrict__
 
 // y (n_r x n_c, caller's order) = tabs 2^.. (a + b), a and b each in that order or (kAt, kBt) the other
 // one.  An entry whose contributions' magnitudes -- a lower bound of (|H||x|)_n -- do
-// not reach thr is recorded in list (see k_fix_entries).
+// not reach thr is recorded in list (see k_fix_entries).  Memory bounds it (24 bytes per entry, 0.59 ms
+// at 4x4): 0.69 ms with four CTAs per SM and loads as they are needed, 0.85 ms with a tile's loads in
+// registers first (116 of them, two CTAs); unrolled by 2 or 4, or five CTAs, 0 to 0.09 ms slower.
 template <int T, bool kAt, bool kBt>
-__global__ void __launch_bounds__(kTileThreads) k_fix_out(i64 n_r, i64 n_c, i64 ld, i64 ldt, const i64 *__restrict__ a,
-                                                          const i64 *__restrict__ b, int eg, i64 thr, double tabs,
+__global__ void __launch_bounds__(kTileThreads, kUpdateBlocks) k_fix_out(i64 n_r, i64 n_c, i64 ld, i64 ldt,
+                                                                         const i64 *__restrict__ a, const i64 *__restrict__ b, int eg, i64 thr, double tabs,
                                                           int *__restrict__ ctl, i64 *__restrict__ list, int cap,
                                                           double *__restrict__ y) {
+  static_assert(T == 32 || !(kAt && kBt), "two tiles in 48 KB");
   __shared__ TileBuf<T> t;
+  __shared__ TileBuf<kAt && kBt ? T : 2> t2;
   if (ctl[kCtlSkip]) return;
   const int e = ctl[kCtlShift] + eg;
   i64 r0, c0;
   tile_at<T>(blockIdx.x, n_c, &r0, &c0);
   const TileAt<T> at;
   const i64 u = c0 + at.c;
-  const bool in = u < n_c, second = u + 1 < n_c;
+  const bool second = u + 1 < n_c;
   const bool vec = (n_c & 1) == 0 && ((uintptr_t)y & 15) == 0;
-  constexpr int kN = T / TileAt<T>::kStep;
-  longlong2 sa[kN], sb[kN];
-#pragma unroll
-  for (int i = 0; i < kN; ++i) {             // what needs no transposing, in flight first
-    const i64 d = r0 + at.k0 + i * TileAt<T>::kStep;
-    sa[i] = sb[i] = make_longlong2(0, 0);
-    if (!kAt && d < n_r && in) sa[i] = *reinterpret_cast<const longlong2 *>(a + d * ld + u);
-    if (!kBt && d < n_r && in) sb[i] = *reinterpret_cast<const longlong2 *>(b + d * ld + u);
-  }
-  if (kBt) {
-    tile_in_t<T>(t, b, ldt, r0, c0, n_r, n_c);
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < kN; ++i) {
-      const int k = at.k0 + i * TileAt<T>::kStep;
-      sb[i] = make_longlong2(t.v[k][at.c], t.v[k][at.c + 1]);
-    }
-  }
-  if (kAt) {
-    if (kBt) __syncthreads();
+  if (kBt) tile_in_t<T>(t, b, ldt, r0, c0, n_r, n_c);
+  if constexpr (kAt && kBt)
+    tile_in_t<T>(t2, a, ldt, r0, c0, n_r, n_c);
+  else if (kAt)
     tile_in_t<T>(t, a, ldt, r0, c0, n_r, n_c);
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < kN; ++i) {
-      const int k = at.k0 + i * TileAt<T>::kStep;
-      sa[i] = make_longlong2(t.v[k][at.c], t.v[k][at.c + 1]);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < kN; ++i) {
-    const i64 d = r0 + at.k0 + i * TileAt<T>::kStep;
-    if (d >= n_r || !in) continue;
+  if (kAt || kBt) __syncthreads();
+#pragma unroll 1
+  for (int k = at.k0; k < T; k += TileAt<T>::kStep) {
+    const i64 d = r0 + k;
+    if (d >= n_r || u >= n_c) continue;
+    longlong2 va;
+    if constexpr (kAt && kBt)
+      va = make_longlong2(t2.v[k][at.c], t2.v[k][at.c + 1]);
+    else
+      va = kAt ? make_longlong2(t.v[k][at.c], t.v[k][at.c + 1]) : *reinterpret_cast<const longlong2 *>(a + d * ld + u);
+    const longlong2 vb = kBt ? make_longlong2(t.v[k][at.c], t.v[k][at.c + 1])
+                             : *reinterpret_cast<const longlong2 *>(b + d * ld + u);
     const i64 n = d * n_c + u;
-    const i64 s0[2] = {sa[i].x, sa[i].y}, s1[2] = {sb[i].x, sb[i].y};
+    const i64 s0[2] = {va.x, va.y}, s1[2] = {vb.x, vb.y};
     double v[2];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       v[j] = fix_to_f64(s0[j] + s1[j], e);
       if (tabs != 1.0) v[j] *= tabs;
       if ((j == 0 || second) && llabs(s0[j]) + llabs(s1[j]) < thr) {
-        const int k = atomicAdd(ctl + kCtlCount, 1);
-        if (k < cap) list[k] = n + j;
+        const int at_list = atomicAdd(ctl + kCtlCount, 1);
+        if (at_list < cap) list[at_list] = n + j;
       }
     }
     if (vec) {
@@ -1561,16 +1550,16 @@ static i64 comb_blocks(i64 n_rows, i64 n_cols) {
 }
 // Tiles of 64 x 64 entries, or 32 x 32 where the larger ones would leave SMs idle.
 static bool small_tiles(const hub_ctx *h) { return h->count[0] * h->count[1] < (i64)64 * 64 * 8 * num_sms(); }
-static i64 tile_blocks(const hub_ctx *h) {
-  const i64 T = small_tiles(h) ? 32 : 64;
+static i64 tile_blocks(const hub_ctx *h, i64 T) {
   return ((h->count[0] + T - 1) / T) * ((h->count[1] + T - 1) / T);
 }
+static i64 tile_blocks(const hub_ctx *h) { return tile_blocks(h, small_tiles(h) ? 32 : 64); }
 // grids are one-dimensional, row strides in bytes 32-bit
 static bool fix_fits(const hub_ctx *h) {
   const i64 lim = ((i64)1 << 31) - 1;
   for (int s = 0; s < 2; ++s)
     if (comb_blocks(h->count[s], h->count[1 - s]) > lim || fix_ld(h->count[s]) * 8 > (i64)0xffffffff) return false;
-  return tile_blocks(h) <= lim;
+  return tile_blocks(h, 32) <= lim;
 }
 
 // out = the hops of the rows' (comb) or the positions' spin (gather) applied to P.x
@@ -1715,15 +1704,17 @@ int fix_apply(hub_ctx *h, const double *x, double *y, cudaStream_t s) {
   if ((rc = fix_product(h, f, p, F, in0, in1, out0, out1, skip, false, s))) return rc;
   const i64 thr = ((i64)std::ceil(p.units * 1.25e13) >> p.g) + 1;   // |error| <= units 2^e <= 0.8e-13 thr 2^(e + g)
   const int eg = p.g - (p.B - 2);
-#define FIX_OUT(AT, BT)                                                                                               \
-  (st ? k_fix_out<32, AT, BT> : k_fix_out<64, AT, BT>)<<<tb, kTileThreads, 0, s>>>(n_dn, n_up, ld, ldt, out0, out1, eg, \
-                                                                                   thr, p.tau, f->ctl, f->list, f->cap, y)
-  if (F.both)
-    FIX_OUT(false, true);
+#define FIX_OUT(T, AT, BT)                                                                                      \
+  k_fix_out<T, AT, BT><<<(int)tile_blocks(h, T), kTileThreads, 0, s>>>(n_dn, n_up, ld, ldt, out0, out1, eg, thr, \
+                                                                       p.tau, f->ctl, f->list, f->cap, y)
+  if (F.both && st)
+    FIX_OUT(32, false, true);
+  else if (F.both)
+    FIX_OUT(64, false, true);
   else if (F.a == 1)
-    FIX_OUT(false, false);
+    FIX_OUT(64, false, false);
   else
-    FIX_OUT(true, true);
+    FIX_OUT(32, true, true);
 #undef FIX_OUT
   HUB_LAUNCH_CHECK();
   k_fix_entries<<<num_sms() * 4, 256, 0, s>>>(h->view(), x, y, f->ctl, f->list, f->cap, df_ok);
