@@ -31,17 +31,14 @@ FALLBACK_HBM_GBS = 6800.0
 # flops, i.e. 152 SMs x 2 FP64 instructions/clock x 2.07 GHz = 0.629e12 instructions/s.
 FP64_INSTR_PEAK = 152 * 2 * 2.07e9
 SMEM_PEAK_TBS = 28.7          # shared-memory load bandwidth, conflict-free, all SMs (probe)
-# FP32 pipe: 152 SMs x 128 lanes x 2.07 GHz (a packed f32x2 instruction occupies two lanes)
-FP32_PEAK_TOPS = 152 * 128 * 2.07e9 / 1e12
-FP32_OPS_PER_TERM = 14        # compensated double-float sum: TwoSum, TwoSum of its error, two adds
-# DRAM bytes (read + write) per element of X from one ncu capture of each kernel on the 4x4
-# (6,6) sector (profiles/k_up_4x4_sector66.md, profiles/k_dn_4x4_sector66.md); the
-# per-element traffic does not depend on the sector, so a launch's traffic is this times D.
-NCU_DRAM_BYTES_PER_ELEMENT = {"k_up": 0.98165581e9 / 64128064, "k_dn": 2.0847303e9 / 64128064}
-STAGE_MAX_COLS = 14076        # rows up to this length are staged in shared memory by pass 1
-# arithmetic of the timed fast path: vectors as pairs of FP32 numbers (48-bit significands),
-# compensated sums; FP64 at the interface
-DTYPE_FAST = "df32 (FP32 pairs, compensated sums; FP64 in/out)"
+# DRAM bytes (read + write) per element of X from one ncu capture of each pass on the 4x4
+# (6,6) sector (profiles/k_fix_gather_4x4_sector66.md); the per-element traffic does not
+# depend on the sector, so a launch's traffic is this times D.
+NCU_DRAM_BYTES_PER_ELEMENT = {"up": 0.981e9 / 64128064, "dn": 0.969e9 / 64128064}
+STAGE_MAX_COLS = 14384        # rows up to this length are staged in shared memory
+# arithmetic of the timed fast path: vectors as 64-bit integers on a power-of-two grid (56 bits
+# below the largest entry), exact sums; FP64 at the interface
+DTYPE_FAST = "int64 fixed point (57-bit entries, exact sums; FP64 in/out)"
 
 
 def parse():
@@ -322,8 +319,8 @@ def extras(hub, W, torch):
     m.close()
     torch.cuda.empty_cache()
     out["square3x6"] = {"workload": "3x6 PBC (9,9), t=1, U=4", "dim": D, "lanczos_step_ms": 1000 * el / 4,
-                        "apply_ms": ap_ms / max(n_ap, 1), "k_up_ms": up_ms / max(n_up_l, 1),
-                        "k_dn_ms": dn_ms / max(n_dn_l, 1),
+                        "apply_ms": ap_ms / max(n_ap, 1), "up_ms": up_ms / max(n_up_l, 1),
+                        "dn_ms": dn_ms / max(n_dn_l, 1),
                         "apply_gbs_16B_per_element": 16 * D / (ap_ms / max(n_ap, 1) / 1000) / 1e9}
     # (4) zero-temperature Green's function (Sec. VII) at 4x4 PBC, half filling, site 0, spin up:
     # ground state of (8,8), c+ psi0 into (9,8) and c psi0 into (7,8), 100 continued-fraction
@@ -552,47 +549,37 @@ def run_gpu(a):
              "fp64_equiv_rate_T": nnz_H / (apply_avg_ms / 1000.0) / 1e12,
              "fp64_alu_frac": nnz_H / (apply_avg_ms / 1000.0) / FP64_INSTR_PEAK}
     if n_up_l and n_dn_l:
-        # fast path, each pass timed by its own event pair.  HBM bytes per element (double-float
-        # vectors, 8 B): pass 1 reads X and writes Z (16 B); pass 2 (Lanczos epilogue) reads X by
-        # strips, Z, r_j, r_{j-1} and writes w (40 B); the update reads w and r_{j-1} and writes
-        # r_j (24 B).  FP32 pipe: each hopping term costs 14 FP32 operations in the compensated
-        # double-float sum (both passes).
-        up_avg, dn_avg = up_ms / n_up_l, dn_ms / n_dn_l
-        terms = {"k_up": nnz_u * m.count_dn, "k_dn": nnz_d * m.count_up}
-        passes = {"k_up": {"ms": up_avg, "algorithmic_bytes": 16 * D, "gbs": gb(16 * D, up_avg)},
-                  "k_dn": {"ms": dn_avg, "algorithmic_bytes": 40 * D, "gbs": gb(40 * D, dn_avg)}}
+        # fast path, each pass timed by its own event pair.  HBM bytes per element (8-byte
+        # entries): a pass reads X in its order and writes its contribution (16 B); the update
+        # reads both contributions, r_j and r_{j-1} and writes r_{j+1} in both orders (48 B).
+        # Shared memory: 8 B per hopping term where the pass gathers inside staged rows.
+        passes = {}
+        for k_, ms_, n_, nnz_, rows_, cols_ in (("up", up_ms, n_up_l, nnz_u, m.count_dn, m.count_up),
+                                                ("dn", dn_ms, n_dn_l, nnz_d, m.count_up, m.count_dn)):
+            avg, smem = ms_ / n_, 8 * nnz_ * rows_
+            passes[k_] = {"ms": avg, "algorithmic_bytes": 16 * D, "gbs": gb(16 * D, avg),
+                          "hbm_frac": gb(16 * D, avg) / hbm_gbs, "terms": nnz_ * rows_}
+            if cols_ <= STAGE_MAX_COLS:
+                passes[k_]["shared_memory"] = {
+                    "algorithmic_bytes": smem, "tbs": gb(smem, avg) / 1000.0, "peak_tbs": SMEM_PEAK_TBS,
+                    "frac": gb(smem, avg) / 1000.0 / SMEM_PEAK_TBS}
         update = None
         if n_ud_l:
             ud_avg = ud_ms / n_ud_l
-            update = {"kernel": "k_df_update", "ms": ud_avg, "launches": n_ud_l, "algorithmic_bytes": 24 * D,
-                      "gbs": gb(24 * D, ud_avg), "hbm_frac": gb(24 * D, ud_avg) / hbm_gbs}
-        for k_, v_ in passes.items():
-            ops = FP32_OPS_PER_TERM * terms[k_]
-            v_["hbm_frac"] = v_["gbs"] / hbm_gbs
-            v_["fp32_ops"] = ops
-            v_["fp32_tops"] = ops / (v_["ms"] / 1000.0) / 1e12
-            v_["fp32_frac"] = v_["fp32_tops"] / FP32_PEAK_TOPS
-        if m.count_up <= STAGE_MAX_COLS:
-            # pass 1 gathers from shared memory: 8 B (high and low word) per spin-up hop and
-            # for the diagonal's own element, per element of X
-            smem_bytes = 8 * (nnz_u + m.count_up) * m.count_dn
-            passes["k_up"]["shared_memory"] = {
-                "algorithmic_bytes": smem_bytes, "tbs": gb(smem_bytes, up_avg) / 1000.0,
-                "peak_tbs": SMEM_PEAK_TBS, "frac": gb(smem_bytes, up_avg) / 1000.0 / SMEM_PEAK_TBS,
-                "peak_source": "probe: conflict-free 64-bit shared loads, all SMs (GB300)"}
+            update = {"kernel": "k_fix_update", "ms": ud_avg, "launches": n_ud_l, "algorithmic_bytes": 48 * D,
+                      "gbs": gb(48 * D, ud_avg), "hbm_frac": gb(48 * D, ud_avg) / hbm_gbs}
         dom = max(passes, key=lambda k: passes[k]["ms"])
         staged_4x4 = a.workload.startswith("4x4") and m.count_up <= STAGE_MAX_COLS
         traffic = NCU_DRAM_BYTES_PER_ELEMENT[dom] * D if staged_4x4 and dom in NCU_DRAM_BYTES_PER_ELEMENT else None
         pd = passes[dom]
-        if pd["fp32_frac"] >= pd["hbm_frac"]:
-            roofline = {"bound": "alu", "kernel": dom, "achieved": pd["fp32_tops"], "peak": FP32_PEAK_TOPS,
-                        "unit": "T FP32 op/s", "frac": pd["fp32_frac"],
-                        "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2.07 GHz",
-                        "hbm": {"achieved": pd["gbs"], "peak": hbm_gbs, "unit": "GB/s", "frac": pd["hbm_frac"],
-                                "peak_source": peak_src}}
+        hbm = {"achieved": pd["gbs"], "peak": hbm_gbs, "unit": "GB/s", "frac": pd["hbm_frac"], "peak_source": peak_src}
+        if "shared_memory" in pd:
+            sm = pd["shared_memory"]
+            roofline = {"bound": "smem", "kernel": "k_fix_gather (%s)" % dom, "achieved": sm["tbs"],
+                        "peak": SMEM_PEAK_TBS, "unit": "TB/s", "frac": sm["frac"],
+                        "peak_source": "probe: conflict-free 64-bit shared loads, all SMs (GB300)", "hbm": hbm}
         else:
-            roofline = {"bound": "hbm", "kernel": dom, "achieved": pd["gbs"], "peak": hbm_gbs, "unit": "GB/s",
-                        "frac": pd["hbm_frac"], "peak_source": peak_src}
+            roofline = dict(hbm, bound="hbm", kernel="k_fix_comb (%s)" % dom)
         roofline.update({"traffic": traffic,
                          "traffic_source": ("ncu dram__bytes_read.sum + dram__bytes_write.sum of the same kernel "
                                             "on the 4x4 (6,6) sector, scaled by elements" if traffic else None),

@@ -53,8 +53,8 @@ extern "C" {
 #define HUB_SPIN_UP 0
 #define HUB_SPIN_DN 1
 
-#define HUB_MODE_AUTO 0   /* fast double-float path when t and U are uniform (window and
-                             bound: see hub_apply), else FP64; in a momentum sector:
+#define HUB_MODE_AUTO 0   /* fixed-point or double-float path when t and U are uniform (window
+                             and bound: see hub_apply), else FP64; in a momentum sector:
                              integer-pipe sums when t is uniform                         */
 #define HUB_MODE_FP64 1   /* always the native FP64 kernels                              */
 
@@ -115,11 +115,15 @@ int hub_get_csr(hub_t h, int spin, int32_t *rowptr_host, int32_t *cols_host, dou
  *
  * Accuracy: every entry satisfies |y_n - (Hx)_n| <= 1e-13 (|H||x|)_n, |H| the entrywise
  * absolute matrix.  The native FP64 kernel (HUB_MODE_FP64; non-uniform t or U) does
- * this with FP64 multiply-adds.  In HUB_MODE_AUTO with uniform t and U the product runs
- * in double-float arithmetic (pairs of FP32 numbers, 48 significant bits; compensated
+ * this with FP64 multiply-adds, also for products of few terms (one launch).  In
+ * HUB_MODE_AUTO with uniform t and U larger products run in 64-bit fixed point: the entries on
+ * one power-of-two grid, 2^-(B+1) of the largest |x_n| (B = 56 or 62 minus the bits of the
+ * number of hopping terms), sums exact; an entry whose two sums are too small for the grid to
+ * meet the bound is computed again in FP64, and a vector with many such entries is multiplied in
+ * double-float arithmetic (pairs of FP32 numbers, 48 significant bits; compensated
  * sums) with a derived worst-case error of max(N + 10.1, 16) * 2^-48 (|H||x|)_n, N <= 15 the
  * most terms one low-part accumulator takes (N = 9 on the 4x4 lattice: 6.8e-14 (|H||x|)_n).
- * That bound needs a window, checked on the device for every call: the largest |x_n| in
+ * These need a window, checked on the device for every call: the largest |x_n| in
  * [2^-823, 2^877], every nonzero |x_n| at least 2^-80 times the largest (no FP64
  * subnormals, infinities or NaN); and a model with uniform t != 0 and U, no site energies,
  * |t| and U/|t| either 0 or in [2^-16, 2^16].  A vector or model outside it is multiplied by the FP64 kernel
@@ -142,7 +146,8 @@ int hub_apply_host(hub_t h, const double *x_host, double *y_host, void *stream);
  * are either the same array (the product in place) or do not overlap at all; page-locked
  * buffers let the copies run at the link's rate.  Each result is bit for bit that of
  * hub_apply_host on the same vector (same kernels, window check and routing).  On the fast
- * path with row-chunked copies (pass 1 staging rows, at least 16 rows) the copies of
+ * path with row-chunked copies (rows that are staged, at least 16 rows, at least 2^22 states; in
+ * double-float arithmetic, pass by pass as the chunks arrive) the copies of
  * neighbouring vectors overlap: vector v + 1 comes in and vector v - 1 goes back while vector
  * v is computed, on two copy streams of the handle; this takes a second pair of device
  * vectors (2 D doubles more), allocated on first use.  Elsewhere it is one hub_apply_host
@@ -162,10 +167,10 @@ int hub_apply_host_many(hub_t h, int64_t n_vec, const double *x_host, double *y_
  * HUB_ERR_NOCONV, *E0 still set).  If psi_dev != NULL the recurrence is run a second
  * time to form the normalised ground-state vector.  Blocks until done; *E0 and *iters
  * are host pointers (iters may be NULL).  Workspace: three device vectors.
- * In HUB_MODE_AUTO with uniform t and U (and t, U, eps in hub_apply's parameter range)
- * the Lanczos vectors are held in double-float form: x0 is scaled by a power of two so
- * that its largest entry lies in [1, 2), and components smaller than about 2^-126 times
- * the largest entry of a Lanczos vector are flushed.  Neither changes E0 at the 1e-10
+ * In HUB_MODE_AUTO with uniform t and U and no site energies (and t, U in hub_apply's parameter
+ * range) the Lanczos vectors are held in 64-bit fixed point, each on a grid of its own
+ * 2^-56 of about its largest entry, and the dot products are integer sums.  This does not change
+ * E0 at the 1e-10
  * level; HUB_MODE_FP64 keeps every vector in FP64.  Sectors of at most hub_set_small_dim's
  * bound (default 262144 states; not in a momentum sector) run instead in one cooperative
  * kernel per batch of iterations, FP64 throughout, in either mode: the same recurrence and

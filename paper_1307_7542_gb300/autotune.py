@@ -1,6 +1,6 @@
 """Autotuner for the kernel shape knobs (run on the GPU it tunes for).
 
-The fast apply (csrc/hub_fast.cu) and the batched solver (csrc/hub_batch.cu) take their launch
+The double-float products (csrc/hub_fast.cu) and the batched solver (csrc/hub_batch.cu) take their launch
 shapes from compile-time knobs:
 
 * ``HUB_DN_LANE_COLS`` -- columns a pass-2 lane owns (2: 64-bit loads, 4: 128-bit loads);
@@ -8,22 +8,20 @@ shapes from compile-time knobs:
 * ``HUB_DN_MINB``      -- resident pass-2 CTAs per SM the register allocation aims for;
 * ``HUB_BANK_CAP``     -- distinct columns per shared-memory bank and step in the pass-1
   schedule (k > 0 fixed, 0 adaptive, -k adaptive capped at k);
-* ``HUB_FUSED_UPDATE`` -- 1: the Lanczos update r_j = w - c r_{j-1} is formed by pass 1 while
-  it stages the rows; 0: a separate vector pass before pass 1;
-* ``HUB_UPD_Q``        -- column quads per thread whose loads the fused update issues together;
 * ``HUB_UP_THREADS``   -- threads of the pass-1 CTA (1024, 768 or 512; fewer leave more registers);
 * ``HUB_UP_PAIRED``    -- 1: pass 1 adds the low parts of a column word's two entries together
   before accumulating them (two accumulators, as pass 2); 0: four accumulators of single terms;
-* ``HUB_BATCH_THREADS`` -- threads per CTA of the batched persistent solver;
+* ``HUB_BATCH_THREADS`` -- threads per CTA of the batched persistent solver's large jobs;
 * ``HUB_BATCH_SPLIT``  -- jobs of at most this many states run in a second launch of the batched
-  solver, its shared memory sized for them (0: one launch);
+  solver, in small CTAs sized for them (0: one launch);
 * ``HUB_SMALL_CLUSTER_MAX``, ``HUB_SMALL_THREADS``, ``HUB_SMALL_PER_THREAD``,
   ``HUB_SMALL_BATCH`` -- the largest sector the single-launch small-sector Lanczos
   (csrc/hub_small.cu) runs as one thread-block cluster (0: always the cooperative grid), its
   threads per CTA, states per thread the grid is sized for, and iterations per launch.
 
 For each candidate setting this module builds one copy of the library, times on the GPU what
-the knob affects (one Lanczos step at 4x4 half filling for the apply knobs; the 5184-job
+the knob affects (one product at 4x4 half filling for the apply knobs, of a vector whose entries
+span many orders of magnitude, which is what the double-float kernels multiply; the 5184-job
 impurity batch of 81 sectors x 64 parameter sets for the batched knob; the 8-site ring's ground
 state to |dE0| < 1e-12 for the small-sector knobs), each in a fresh process, and keeps the
 fastest by coordinate descent from the current setting (a change is kept only if it is at least
@@ -51,8 +49,6 @@ APPLY_SPACE = {
     "HUB_DN_BATCH": [2, 4],
     "HUB_DN_MINB": [3, 4, 5, 6],
     "HUB_BANK_CAP": [2, 1, 3, 0, -2],
-    "HUB_FUSED_UPDATE": [1, 0],
-    "HUB_UPD_Q": [1, 2],
     "HUB_UP_THREADS": [1024, 768, 512],
     "HUB_UP_PAIRED": [1, 0],
 }
@@ -60,11 +56,12 @@ BATCH_SPACE = {"HUB_BATCH_THREADS": [256, 512, 1024], "HUB_BATCH_SPLIT": [2048, 
 SMALL_SPACE = {"HUB_SMALL_CLUSTER_MAX": [8192, 12800, 0], "HUB_SMALL_THREADS": [128, 256, 320, 384, 512],
                "HUB_SMALL_PER_THREAD": [1, 2, 4], "HUB_SMALL_BATCH": [8, 4, 16]}
 DEFAULTS = {"HUB_DN_LANE_COLS": 4, "HUB_DN_BATCH": 2, "HUB_DN_MINB": 4, "HUB_BANK_CAP": 2,
-            "HUB_FUSED_UPDATE": 0, "HUB_UPD_Q": 1, "HUB_UP_THREADS": 1024, "HUB_UP_PAIRED": 1,
+            "HUB_UP_THREADS": 1024, "HUB_UP_PAIRED": 1,
             "HUB_BATCH_THREADS": 256, "HUB_BATCH_SPLIT": 2048,
             "HUB_SMALL_CLUSTER_MAX": 8192, "HUB_SMALL_THREADS": 320, "HUB_SMALL_PER_THREAD": 1,
             "HUB_SMALL_BATCH": 8}
-# tuned.json key of each group's timing
+# tuned.json key of each group's timing ("lanczos_step_ms_4x4": the apply group's, recorded while
+# the Lanczos step ran on its kernels; now a product)
 RESULT_KEYS = {"apply": "lanczos_step_ms_4x4", "batch": "aim_batch_ms", "small": "ring8_ground_ms"}
 MARGIN = 0.01
 
@@ -74,22 +71,25 @@ def _tag(knobs: dict) -> str:
 
 
 def _child_apply(lib_path: str, steps: int) -> float:
-    """ms per Lanczos step at 4x4 PBC (8,8), U = 4, with the library at lib_path."""
+    """ms per product at 4x4 PBC (8,8), U = 4, of a vector with entries over 30 binary orders, with
+    the library at lib_path."""
     import torch
     from paper_1307_7542_gb300 import hub, workloads as W
     hub.LIB_PATH = lib_path
     hub._lib = None
     w = W.square4x4(4.0)
     m = hub.Hubbard(16, 8, 8, w["bonds"], w["t"], w["U"], w["eps"])
-    x0 = torch.from_numpy(W.normal(0, m.D)).cuda()
-    m.ground(x0, maxit=3, tol=0.0)
-    torch.cuda.synchronize()
+    x = torch.from_numpy(W.normal(0, m.D)).cuda()
+    x *= torch.exp2(-30.0 * torch.rand(m.D, device="cuda", dtype=torch.float64))
+    y = torch.empty_like(x)
+    for _ in range(3):
+        m.apply(x, y)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     e0.record()
-    r = m.ground(x0, maxit=steps, tol=0.0)
+    for _ in range(steps):
+        m.apply(x, y)
     e1.record()
     torch.cuda.synchronize()
-    assert r["iters"] == steps
     m.close()
     return e0.elapsed_time(e1) / steps
 

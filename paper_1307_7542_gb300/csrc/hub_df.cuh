@@ -16,55 +16,10 @@
 
 namespace hub {
 
-// (s, e) with s + e == a + b exactly (round-to-nearest FP32, no overflow).
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
-  s = __fadd_rn(a, b);
-  float bb = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-
 // (s, e) with s + e == a + b exactly, valid when |a| >= |b| (or a == 0).
 __device__ __forceinline__ void fast_two_sum(float a, float b, float &s, float &e) {
   s = __fadd_rn(a, b);
   e = __fsub_rn(b, __fsub_rn(s, a));
-}
-
-// Accumulator: the exact sum of the high parts is kept as H plus the rounding errors,
-// which go to L together with the low parts (used for the long dot products of Lanczos;
-// the hopping sums of the product use the compensated DfSumP or DfSum4 below).
-struct DfAcc {
-  float H, L;
-};
-
-__device__ __forceinline__ void acc_add(DfAcc &a, float2 v) {
-  float s, e;
-  two_sum(a.H, v.x, s, e);
-  a.H = s;
-  a.L = __fadd_rn(__fadd_rn(a.L, v.y), e);
-}
-
-__device__ __forceinline__ void acc_sub(DfAcc &a, float2 v) {
-  float s, e;
-  two_sum(a.H, -v.x, s, e);
-  a.H = s;
-  a.L = __fadd_rn(__fsub_rn(a.L, v.y), e);
-}
-
-// Normalised double-float value of an accumulator.
-__device__ __forceinline__ float2 acc_value(const DfAcc &a) {
-  float s, e;
-  two_sum(a.H, a.L, s, e);
-  return make_float2(s, e);
-}
-
-// a + b for normalised double-floats (sloppy addition: TwoSum of the high parts).
-__device__ __forceinline__ float2 df_add(float2 a, float2 b) {
-  float s, e;
-  two_sum(a.x, b.x, s, e);
-  e = __fadd_rn(e, __fadd_rn(a.y, b.y));
-  float r, f;
-  fast_two_sum(s, e, r, f);
-  return make_float2(r, f);
 }
 
 // a * b for double-floats (TwoProd of the high parts plus the cross terms).
@@ -77,9 +32,6 @@ __device__ __forceinline__ float2 df_mul(float2 a, float2 b) {
   fast_two_sum(p, e, r, f);
   return make_float2(r, f);
 }
-
-// a * b + c for double-floats.
-__device__ __forceinline__ float2 df_fma(float2 a, float2 b, float2 c) { return df_add(df_mul(a, b), c); }
 
 // ---------------------------------------------------------------------------------------
 // Two independent double-float accumulators advanced together with the packed FP32x2
@@ -124,33 +76,8 @@ __device__ __forceinline__ f2x sub2(f2x a, f2x b) {
 #endif
 }
 
-__device__ __forceinline__ f2x bcast2(float a) { return pk2(a, a); }
-
 // sign bits of both lanes (XOR negates both exactly)
 constexpr f2x kSign2 = 0x8000000080000000ull;
-
-struct DfAcc2 {
-  f2x H, L;   // high parts (exact running sums) and low parts + TwoSum errors, per lane
-};
-
-// a += v (v = vh + vl per lane): TwoSum of the high parts, errors and low parts into L.
-__device__ __forceinline__ void acc2_add(DfAcc2 &a, f2x vh, f2x vl) {
-  const f2x s = add2(a.H, vh);
-  const f2x bb = sub2(s, a.H);
-  const f2x e = add2(sub2(a.H, sub2(s, bb)), sub2(vh, bb));
-  a.H = s;
-  a.L = add2(add2(a.L, vl), e);
-}
-
-// a -= v: the TwoSum of (a.H, -vh) written with subtractions (negation is exact, so this
-// is the same error-free transformation as acc2_add of -v).
-__device__ __forceinline__ void acc2_sub(DfAcc2 &a, f2x vh, f2x vl) {
-  const f2x s = sub2(a.H, vh);
-  const f2x bb = sub2(s, a.H);
-  const f2x e = sub2(sub2(a.H, sub2(s, bb)), add2(vh, bb));
-  a.H = s;
-  a.L = add2(sub2(a.L, vl), e);
-}
 
 // ---------------------------------------------------------------------------------------
 // Compensated paired sum for the hopping terms of the product (sums of +-v, v = vh + vl a
@@ -256,14 +183,6 @@ __device__ __forceinline__ void sump_norm(const DfSumP &a, f2x &h, f2x &l) {
   two_sum2(s, add2(e, C), h, l);
 }
 
-// Normalised (hi, lo) per lane of a paired accumulator.
-__device__ __forceinline__ void acc2_norm(const DfAcc2 &a, f2x &h, f2x &l) {
-  const f2x s = add2(a.H, a.L);
-  const f2x bb = sub2(s, a.H);
-  l = add2(sub2(a.H, sub2(s, bb)), sub2(a.L, bb));
-  h = s;
-}
-
 // Packed double-float arithmetic on two lanes; the same operation sequences as df_add and
 // df_mul.
 __device__ __forceinline__ void df2_add(f2x ah, f2x al, f2x bh, f2x bl, f2x &rh, f2x &rl) {
@@ -271,14 +190,6 @@ __device__ __forceinline__ void df2_add(f2x ah, f2x al, f2x bh, f2x bl, f2x &rh,
   const f2x bb = sub2(s, ah);
   f2x e = add2(sub2(ah, sub2(s, bb)), sub2(bh, bb));
   e = add2(e, add2(al, bl));
-  rh = add2(s, e);
-  rl = sub2(e, sub2(rh, s));
-}
-__device__ __forceinline__ void df2_sub(f2x ah, f2x al, f2x bh, f2x bl, f2x &rh, f2x &rl) {
-  const f2x s = sub2(ah, bh);
-  const f2x bb = sub2(s, ah);
-  f2x e = sub2(sub2(ah, sub2(s, bb)), add2(bh, bb));
-  e = add2(e, sub2(al, bl));
   rh = add2(s, e);
   rl = sub2(e, sub2(rh, s));
 }
@@ -292,12 +203,6 @@ __device__ __forceinline__ void df2_mul(f2x ah, f2x al, f2x bh, f2x bl, f2x &rh,
   const float2 r1 = df_mul(make_float2(a_h.y, a_l.y), make_float2(b_h.y, b_l.y));
   rh = pk2(r0.x, r1.x);
   rl = pk2(r0.y, r1.y);
-}
-
-// Lane a / lane b of a paired accumulator as a plain accumulator.
-__device__ __forceinline__ DfAcc acc2_lane(const DfAcc2 &a, int lane) {
-  const float2 h = upk2(a.H), l = upk2(a.L);
-  return lane == 0 ? DfAcc{h.x, l.x} : DfAcc{h.y, l.y};
 }
 
 // 2^k as a float for -126 <= k <= 127.

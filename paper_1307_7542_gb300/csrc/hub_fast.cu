@@ -1,5 +1,5 @@
-// hub_fast.cu -- the fast apply for uniform hopping (K3 fast path) and the double-float
-// Lanczos built on it.
+// hub_fast.cu -- double-float products for uniform hopping: of vectors that the fixed-point path
+// (hub_fix.cu) does not serve, and of host buffers in row chunks.
 //
 // The product is Eq. 11 of Sec. IV.A on the count_dn x count_up state matrix X (Eq.
 // count2):  Y = X H_up^T + H_dn X + diag o X, with every hopping element -t * esign
