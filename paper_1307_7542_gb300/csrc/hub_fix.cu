@@ -1298,8 +1298,7 @@ void fix_release(hub_ctx *h) {
   for (int s = 0; s < 2; ++s) {
     dev_free(f->cnt[s]);
     dev_free(f->word[s]);
-    dev_free(f->sched[s]);
-    dev_free(f->meta[s]);
+    dev_free(f->sched[s]);              // meta lies in the same allocation
     dev_free(f->vec[s]);
     if (f->graph[s]) cudaGraphExecDestroy(f->graph[s]);
   }
@@ -1437,52 +1436,44 @@ static std::vector<int32_t> gather_groups(int n, const SpinCSR &c, int *rc) {
 }
 
 // Gather schedule of a spin: the groups coloured on the device, then paired by length into slices.
+// One allocation for the schedule and what it is made from (a first product pays for each).
 static int gather_tables(FixState *f, int s, int n, const SpinCSR &c) {
   const int slices = (n + 31) / 32, groups = 2 * slices;
   const int cap = std::min(kSchedMax, (2 * std::max(c.max_row, 1) + 7) / 8 * 8);
-  uint16_t *tmp = nullptr, *deg = nullptr;
-  int32_t *grp = nullptr, *quad = nullptr;
   std::vector<uint16_t> d(groups);
   std::vector<int32_t> order(groups);
-  std::vector<uint32_t> meta(32 * (size_t)slices);
   int rc = HUB_OK;
   const std::vector<int32_t> q = gather_groups(n, c, &rc);
   if (rc) return rc;
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  const size_t words = up(sizeof(uint16_t) * 32 * (size_t)slices * cap), lanes = 32 * (size_t)slices;
+  const size_t o_meta = 2 * words, o_quad = o_meta + up(sizeof(uint32_t) * (lanes + groups));
+  const size_t o_deg = o_quad + up(sizeof(int32_t) * q.size()), bytes = o_deg + up(sizeof(uint16_t) * groups);
+  if (!f->sched[s] && !dev_alloc((void **)&f->sched[s], bytes, "gather schedule")) return HUB_ERR_OOM;
+  char *base = (char *)f->sched[s];
+  f->meta[s] = (uint32_t *)(base + o_meta);
   f->cap_steps[s] = cap;
   f->slices[s] = slices;
-  if (!dev_alloc((void **)&f->sched[s], sizeof(uint16_t) * 32 * (size_t)slices * cap, "gather schedule") ||
-      !dev_alloc((void **)&f->meta[s], sizeof(uint32_t) * meta.size(), "gather slices") ||
-      !dev_alloc((void **)&quad, sizeof(int32_t) * q.size(), "gather groups") ||
-      !dev_alloc((void **)&grp, sizeof(int32_t) * groups, "gather groups") ||
-      !dev_alloc((void **)&tmp, sizeof(uint16_t) * 32 * (size_t)slices * cap, "gather schedule") ||
-      !dev_alloc((void **)&deg, sizeof(uint16_t) * groups, "gather steps"))
-    rc = HUB_ERR_OOM;
-  cudaError_t e = cudaSuccess;
-  if (rc == HUB_OK) e = cudaMemcpy(quad, q.data(), sizeof(int32_t) * q.size(), cudaMemcpyHostToDevice);
-  if (rc == HUB_OK && e == cudaSuccess) {
-    k_fix_schedule<<<groups, 32>>>(n, groups, (int)fix_ld(n), cap, quad, c.rowptr, c.scol, tmp, deg);
-    e = cudaMemcpy(d.data(), deg, sizeof(uint16_t) * groups, cudaMemcpyDeviceToHost);
-    for (int g = 0; g < groups; ++g) order[g] = g;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return d[a] > d[b]; });
-    for (int k = 0; k < slices; ++k)
-      for (int l = 0; l < 32; ++l) {          // words hold two steps
-        const uint32_t steps = (d[order[2 * k]] + 1u) & ~1u;
-        const uint32_t at = (uint32_t)q[4 * order[2 * k + (l >> 4)] + ((l >> 2) & 3)] * 4 + (l & 3);
-        meta[32 * (size_t)k + l] = at | (steps << 16);
-      }
-    if (e == cudaSuccess) e = cudaMemcpy(grp, order.data(), sizeof(int32_t) * groups, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(f->meta[s], meta.data(), sizeof(uint32_t) * meta.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) {
-      k_fix_pack<<<slices, 32>>>(grp, cap, tmp, f->sched[s]);
-      e = cudaDeviceSynchronize();
+  uint16_t *tmp = (uint16_t *)(base + words), *deg = (uint16_t *)(base + o_deg);
+  int32_t *quad = (int32_t *)(base + o_quad), *grp = (int32_t *)(f->meta[s] + lanes);
+  HUB_CUDA(cudaMemcpy(quad, q.data(), sizeof(int32_t) * q.size(), cudaMemcpyHostToDevice));
+  k_fix_schedule<<<groups, 32>>>(n, groups, (int)fix_ld(n), cap, quad, c.rowptr, c.scol, tmp, deg);
+  HUB_LAUNCH_CHECK();
+  HUB_CUDA(cudaMemcpy(d.data(), deg, sizeof(uint16_t) * groups, cudaMemcpyDeviceToHost));
+  for (int g = 0; g < groups; ++g) order[g] = g;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return d[a] > d[b]; });
+  std::vector<uint32_t> meta(lanes + groups);
+  for (int k = 0; k < slices; ++k)
+    for (int l = 0; l < 32; ++l) {          // words hold two steps
+      const uint32_t steps = (d[order[2 * k]] + 1u) & ~1u;
+      const uint32_t at = (uint32_t)q[4 * order[2 * k + (l >> 4)] + ((l >> 2) & 3)] * 4 + (l & 3);
+      meta[32 * (size_t)k + l] = at | (steps << 16);
     }
-  }
-  dev_free(tmp);
-  dev_free(deg);
-  dev_free(grp);
-  dev_free(quad);
-  if (rc == HUB_OK) HUB_CUDA(e);
-  return rc;
+  for (int g = 0; g < groups; ++g) meta[lanes + g] = (uint32_t)order[g];
+  HUB_CUDA(cudaMemcpy(f->meta[s], meta.data(), sizeof(uint32_t) * meta.size(), cudaMemcpyHostToDevice));
+  k_fix_pack<<<slices, 32>>>(grp, cap, tmp, f->sched[s]);
+  HUB_LAUNCH_CHECK();
+  return HUB_OK;
 }
 
 // Tables of the plan: entry lists, coefficients and diagonal.
@@ -1496,8 +1487,8 @@ static int fix_tables(hub_ctx *h, FixState *f, const FixPlan &p) {
         if (rc) return rc;
         continue;
       }
-      if (!dev_alloc((void **)&f->cnt[s], sizeof(uint32_t) * n, "hopping entry counts") ||
-          !dev_alloc((void **)&f->word[s], sizeof(uint32_t) * (nnz + 32), "hopping entries"))
+      if ((!f->cnt[s] && !dev_alloc((void **)&f->cnt[s], sizeof(uint32_t) * n, "hopping entry counts")) ||
+          (!f->word[s] && !dev_alloc((void **)&f->word[s], sizeof(uint32_t) * (nnz + 32), "hopping entries")))
         return HUB_ERR_OOM;
       HUB_CUDA(cudaMemset(f->word[s], 0, sizeof(uint32_t) * (nnz + 32)));
       k_fix_lists<<<grid_of(n), 256>>>(n, c.rowptr, c.scol, f->cnt[s], f->word[s]);
