@@ -165,8 +165,8 @@ int hub_apply_host_many(hub_t h, int64_t n_vec, const double *x_host, double *y_
  * |E0_j - E0_{j-1}| < tol (tol <= 0: run exactly maxit iterations), on breakdown
  * (beta_j <= 1e-14 |alpha_j|, returns HUB_CONVERGED_BREAKDOWN) or at maxit (returns
  * HUB_ERR_NOCONV, *E0 still set).  If psi_dev != NULL the recurrence is run a second
- * time to form the normalised ground-state vector.  Blocks until done; *E0 and *iters
- * are host pointers (iters may be NULL).  Workspace: three device vectors.
+ * time to form the normalised ground-state vector, which may lie over x0.  Blocks until done;
+ * *E0 and *iters are host pointers (iters may be NULL).  Workspace: three device vectors.
  * In HUB_MODE_AUTO with uniform t and U and no site energies (and t, U in hub_apply's parameter
  * range) the Lanczos vectors are held in 64-bit fixed point, each on a grid of its own
  * 2^-56 of about its largest entry, and the dot products are integer sums.  This does not change
@@ -225,7 +225,7 @@ int hub_lanczos_block(hub_t h, int k, const double *X0_dev, int steps, int n_eig
  * from x0_dev (NULL: the seeded start vector), then the second pass of hub_lanczos_ground
  * forms the normalised Ritz vector psi_dev (device, count_up * count_dn) for the eigenvalue
  * of T nearest `target` (e.g. one returned by hub_lanczos_spectrum with the same x0 and
- * maxit); *ritz_host receives that eigenvalue.  1 <= maxit <= 3000; blocks until done.
+ * maxit); *ritz_host receives that eigenvalue.  psi may lie over x0.  1 <= maxit <= 3000; blocks until done.
  */
 int hub_lanczos_ritz(hub_t h, const double *x0_dev, int maxit, double target, double *psi_dev, double *ritz_host,
                      void *stream);

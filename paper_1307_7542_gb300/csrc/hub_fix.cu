@@ -1906,8 +1906,8 @@ int fix_lanczos(hub_ctx *h, const double *x0, int maxit, double tol, double *E0,
       f->v_cap = k;
     }
     HUB_CUDA(cudaMemcpyAsync(f->v, vv.data(), sizeof(double) * k, cudaMemcpyHostToDevice, s));
+    if ((rc = start())) return rc;        // reads x0, which psi may lie over
     HUB_CUDA(cudaMemsetAsync(psi_out, 0, sizeof(double) * D, s));
-    if ((rc = start())) return rc;
     for (int j = 0; j + 1 < k; ++j)
       if ((rc = step(f->vec[j & 1], f->vec[1 - (j & 1)], psi_out, s))) return rc;
     count_launch(h);
