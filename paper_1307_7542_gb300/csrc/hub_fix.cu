@@ -1193,7 +1193,8 @@ __global__ void __launch_bounds__(kTileThreads, kUpdateBlocks) k_fix_out(i64 n_r
     for (int j = 0; j < 2; ++j) {
       v[j] = fix_to_f64(s0[j] + s1[j], e);
       if (tabs != 1.0) v[j] *= tabs;
-      if ((j == 0 || second) && llabs(s0[j]) + llabs(s1[j]) < thr) {
+      // beyond cap only what was under way is still counted, so that the count stays far below 2^31
+      if ((j == 0 || second) && llabs(s0[j]) + llabs(s1[j]) < thr && *(volatile int *)(ctl + kCtlCount) <= cap) {
         const int at_list = atomicAdd(ctl + kCtlCount, 1);
         if (at_list < cap) list[at_list] = n + j;
       }

@@ -1,0 +1,49 @@
+"""Edges of the fixed-point path (csrc/hub_fix.cu): more entries to recompute than its list holds."""
+import numpy as np
+import pytest
+
+from oracle import hub_oracle as O
+from paper_1307_7542_gb300 import workloads as W
+
+from helpers import abs_bound, assert_entrywise
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def hub(cuda_ok):
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1307_7542_gb300 import hub as H
+    return H
+
+
+def _dense(csr, n):
+    rp, cols, vals = csr
+    A = np.zeros((n, n))
+    A[np.repeat(np.arange(n), np.diff(rp)), cols] = vals
+    return A
+
+
+def test_more_small_sums_than_the_list_holds(hub):
+    """U = 0 and a vector in the null spaces of both spins' hopping matrices: entries of ordinary
+    size, yet both hopping sums of every entry vanish, so that all of them ask to be computed
+    again, far more than the list holds (1 in 64)."""
+    M, nu, nd, b = 14, 4, 6, W.ring_bonds(14)
+    m = hub.Hubbard(M, nu, nd, b, 1.0, 0.0)
+    null = []
+    for spin, n in ((0, m.count_up), (1, m.count_dn)):
+        ev, v = np.linalg.eigh(_dense(m.csr(spin), n))
+        null.append(v[:, np.abs(ev) < 1e-9])
+    g = W.normal(21, null[0].shape[1] * null[1].shape[1]).reshape(null[1].shape[1], null[0].shape[1])
+    x = (null[1] @ g @ null[0].T).ravel()
+    x /= np.abs(x).max()
+    y = m.apply(torch.from_numpy(x).cuda()).cpu().numpy()
+    m.close()
+    om, B = O.Model(M, b, 1.0, 0.0), O.basis(M, nu, nd)
+    bound = abs_bound(om, B, x)
+    ref = O.apply(om, B, x)
+    assert (np.abs(ref) < 1e-10 * bound).mean() > 0.5 and (np.abs(x) > 2.0 ** -8).mean() > 0.9
+    assert_entrywise(y, ref, bound)
