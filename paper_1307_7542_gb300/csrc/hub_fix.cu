@@ -22,8 +22,9 @@
 // Lanczos vectors.  The vectors are kept unnormalised and monic, s_{j+1} = H s_j - alpha_j s_j -
 // beta_j^2 s_{j-1} (q_j = s_j / |s_j|, beta_{j+1} = |s_{j+1}| / |s_j|), each on its own grid, so
 // only shifts and two multiplications by a 55-bit coefficient are needed per entry, and the
-// dot products <s_j, H s_j>, <s_j, s_{j-1}> and |s_{j+1}|^2 are integer sums: no result depends on
-// the order in which blocks finish.  A start vector of random numbers keeps max |s_j| / rms(s_j)
+// dot products <s_j, H s_j>, <s_j, s_{j-1}> and |s_{j+1}|^2 are integer sums (H s_j rounded to 7 bits
+// fewer, the product of the lowest limbs to their high part, and left out of <s_j, s_{j-1}>): no
+// result depends on the order in which blocks finish.  A start vector of random numbers keeps max |s_j| / rms(s_j)
 // below 2^6.5, so an entry carries 49 bits and more below the rms, against 48 significant bits of
 // double-float arithmetic.  Against long double (12-site ring, 12 steps) alpha and beta are off by
 // 1.4e-14 and 1.8e-15 at U = 7.25, by 9.9e-10 and 4.2e-10 at U = 4000 (double-float 5.7e-14, 1.8e-15,
@@ -373,15 +374,19 @@ __device__ __forceinline__ i64 diag_term(const FixPass &P, const i64 *__restrict
 }
 
 // An entry of a pass: hopping sum s, own entry X.  Returns the output; kLz: adds to the dot
-// product <X, output 2^-7> and the maximum.
+// product <X, output 2^-7> and the maximum.  The output enters the dot product rounded to a multiple of
+// 128, not cut off: 64 units too little in every entry add up where the entries of X have one sign
+// (alpha of an all-positive vector off by 2e-15 of the operator's scale and more, now 2e-17; the
+// bound on the sums leaves room for the 64).
 template <bool kLz>
 __device__ __forceinline__ i64 pass_entry(const FixPass &P, const i64 *__restrict__ tab, i64 s, int xh, int xl,
                                           uint32_t Ir, uint32_t Ip, Dot &dot, unsigned &vmax) {
   if (P.g) s = (s + (1ll << (P.g - 1))) >> P.g;
   if (P.diag.kind) s += diag_term(P, tab, Ir, Ip, xh, xl);
   if (kLz) {
-    const int yh = (int)((u64)s >> 32);
-    dot.add(xh, xl, yh >> 3, (int)((unsigned)(s >> 7) & 0x0fffffffu));
+    const i64 r = s + 64;
+    const int yh = (int)((u64)r >> 32);
+    dot.add(xh, xl, yh >> 3, (int)((unsigned)(r >> 7) & 0x0fffffffu));
     vmax = max(vmax, (unsigned)abs(yh));
   }
   return s;

@@ -1,4 +1,5 @@
-"""Edges of the fixed-point path (csrc/hub_fix.cu): more entries to recompute than its list holds."""
+"""Edges of the fixed-point path (csrc/hub_fix.cu): more entries to recompute than its list holds; start
+vectors of one sign."""
 import numpy as np
 import pytest
 
@@ -47,3 +48,26 @@ def test_more_small_sums_than_the_list_holds(hub):
     ref = O.apply(om, B, x)
     assert (np.abs(ref) < 1e-10 * bound).mean() > 0.5 and (np.abs(x) > 2.0 ** -8).mean() > 0.9
     assert_entrywise(y, ref, bound)
+
+
+@pytest.mark.parametrize("M,nu,nd", [(13, 5, 8), (14, 9, 5), (14, 7, 7)])
+@pytest.mark.parametrize("top", [1.0001, 1.9999])
+def test_first_coefficient_of_a_positive_vector(hub, M, nu, nd, top):
+    """alpha_1 = <x, H x> / <x, x> where every entry is positive, so that errors of one sign in H x
+    add up: within 5e-16 of the operator's scale of the sum in long double.  top: the largest
+    entry's place between two powers of two, sixteen times the rms (a few roundings of FP64 numbers
+    of at most half the scale: 3 * 1.1e-16)."""
+    m = hub.Hubbard(M, nu, nd, W.ring_bonds(M), 1.0, 4.0)
+    x = np.abs(W.normal(7, m.D))
+    x *= 1.0 / np.sqrt((x * x).mean())
+    x[m.D // 3] = 16.0
+    x *= top / 16.0
+    xd = torch.from_numpy(x).cuda()
+    m.ground(xd, maxit=1, tol=0.0)
+    alpha = hub.hub_lanczos_coeffs(m.h)[0][0]
+    hub.hub_set_mode(m.h, hub.HUB_MODE_FP64)
+    y = m.apply(xd).cpu().numpy()
+    rows = sum(hub.hub_csr_info(m.h, s)[1] for s in (0, 1))
+    m.close()
+    ref = np.sum(x * y, dtype=np.longdouble) / np.sum(x * x, dtype=np.longdouble)
+    assert abs(float(alpha - ref)) <= 5e-16 * (rows + 4.0 * min(nu, nd))
