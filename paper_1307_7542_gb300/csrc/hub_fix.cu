@@ -1807,9 +1807,9 @@ int fix_lanczos(hub_ctx *h, const double *x0, int maxit, double tol, double *E0,
   HUB_CUDA(cudaMemcpyAsync(ctl, f->ctl, sizeof(ctl), cudaMemcpyDeviceToHost, s));
   HUB_CUDA(cudaMemcpyAsync(f->h_scal, f->scal, sizeof(FixScal), cudaMemcpyDeviceToHost, s));
   HUB_CUDA(cudaStreamSynchronize(s));
+  h->start_norm = std::ldexp(std::sqrt(f->h_scal->N), ctl[kCtlShift] - (p.B - 2));   // 0: hub_green_coeffs looks
   if (ctl[kCtlShift] == 2047 - 1023 || !(f->h_scal->N > 0.0))
     return fail(HUB_ERR_ARG, "hub_lanczos_ground: start vector is zero or not finite");
-  h->start_norm = std::ldexp(std::sqrt(f->h_scal->N), ctl[kCtlShift] - (p.B - 2));
 
   // graphs of one step, kept while their operands stay the same
   bool graphs = !h->prof && !f->graph_failed;

@@ -1,5 +1,5 @@
 """Edges of the fixed-point path (csrc/hub_fix.cu): more entries to recompute than its list holds; start
-vectors of one sign."""
+vectors of one sign, and of zeros."""
 import numpy as np
 import pytest
 
@@ -71,3 +71,26 @@ def test_first_coefficient_of_a_positive_vector(hub, M, nu, nd, top):
     m.close()
     ref = np.sum(x * y, dtype=np.longdouble) / np.sum(x * x, dtype=np.longdouble)
     assert abs(float(alpha - ref)) <= 5e-16 * (rows + 4.0 * min(nu, nd))
+
+
+@pytest.mark.parametrize("driver", ["fixed", "fp64", "small"])
+def test_zero_and_infinite_start_vectors(hub, driver):
+    """hub_green_coeffs of c psi0 = 0 is the empty continued fraction; a ground state from zeros,
+    and either from infinities, is refused."""
+    m = hub.Hubbard(9, 4, 3, W.ring_bonds(9), 1.0, 4.0)
+    if driver != "small":
+        hub.hub_set_small_dim(m.h, 0)
+    if driver == "fp64":
+        hub.hub_set_mode(m.h, hub.HUB_MODE_FP64)
+    x = torch.zeros(m.D, dtype=torch.float64, device="cuda")
+    a, b, n2 = hub.hub_green_coeffs(m.h, x, 5)
+    assert len(a) == 0 and len(b) == 0 and n2 == 0.0
+    with pytest.raises(hub.HubError) as e:
+        hub.hub_lanczos_ground(m.h, x, 5, 0.0)
+    assert e.value.code == hub.HUB_ERR_ARG
+    x[3] = float("inf")
+    for call in (lambda: hub.hub_green_coeffs(m.h, x, 5), lambda: hub.hub_lanczos_ground(m.h, x, 5, 0.0)):
+        with pytest.raises(hub.HubError) as e:
+            call()
+        assert e.value.code == hub.HUB_ERR_ARG
+    m.close()
