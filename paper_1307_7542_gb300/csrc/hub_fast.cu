@@ -1132,6 +1132,7 @@ static int transpose(int64_t n_r, int64_t n_c, int64_t ld_s, int64_t ld_d, const
 }
 
 static int ensure_vec(float **p, int64_t n, const char *what);
+static int64_t scratch_floats(const hub_ctx *h, const FastState *f);
 
 // z <- pass 1 (x planar double-float); with staged rows, only the row pairs p0 .. p1 - 1
 // (p1 < 0: all pairs).
@@ -1157,7 +1158,7 @@ static int run_up(hub_ctx *h, FastState *f, const float *x, float *z, cudaStream
 #undef HUB_UP
     HUB_LAUNCH_CHECK();
   } else {
-    const int64_t Dt = h->count[0] * 2 * f->ld_t;
+    const int64_t Dt = scratch_floats(h, f);   // also fast_scratch's, which takes them as they are
     if ((rc = ensure_vec(&f->xt, Dt, "transposed x")) || (rc = ensure_vec(&f->zt, Dt, "transposed z"))) return rc;
     count_launch(h, 3);
     if ((rc = transpose(h->count[1], h->count[0], f->ld, f->ld_t, x, f->xt, gate, s))) return rc;

@@ -1,12 +1,12 @@
 """Edges of the fixed-point path (csrc/hub_fix.cu): more entries to recompute than its list holds; start
-vectors of one sign, and of zeros."""
+vectors of one sign, and of zeros; scratch vectors that another path allocated."""
 import numpy as np
 import pytest
 
 from oracle import hub_oracle as O
 from paper_1307_7542_gb300 import workloads as W
 
-from helpers import abs_bound, assert_entrywise
+from helpers import abs_bound, assert_entrywise, device_bound
 
 pytestmark = pytest.mark.gpu
 
@@ -94,3 +94,20 @@ def test_zero_and_infinite_start_vectors(hub, driver):
             call()
         assert e.value.code == hub.HUB_ERR_ARG
     m.close()
+
+
+def test_scratch_vectors_of_the_double_float_path(hub):
+    """17 sites (8, 7), 24310 x 19448: both spins too long to stage.  A product at strong coupling
+    allocates the transposed scratch vectors for the double-float kernels; the fixed-point product
+    after it takes them for vectors in the other order, whose padded rows need 311,168 bytes more."""
+    m = hub.Hubbard(17, 8, 7, W.ring_bonds(17), 1.0, 4000.0)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    x = torch.randn(m.D, dtype=torch.float64, device="cuda", generator=g)
+    y = m.apply(x)
+    hub.hub_set_U(m.h, [4.0])
+    m.apply(x, y)
+    hub.hub_set_mode(m.h, hub.HUB_MODE_FP64)
+    y -= m.apply(x)
+    bound = device_bound(m, x, 4.0)
+    m.close()
+    assert bool((y.abs() <= 1.1e-13 * bound).all())       # a tenth for the FP64 product's own rounding
