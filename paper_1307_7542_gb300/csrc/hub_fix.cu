@@ -24,11 +24,15 @@
 // only shifts and two multiplications by a 55-bit coefficient are needed per entry, and the
 // dot products <s_j, H s_j>, <s_j, s_{j-1}> and |s_{j+1}|^2 are integer sums (H s_j rounded to 7 bits
 // fewer, the product of the lowest limbs to their high part, and left out of <s_j, s_{j-1}>): no
-// result depends on the order in which blocks finish.  A start vector of random numbers keeps max |s_j| / rms(s_j)
-// below 2^6.5, so an entry carries 49 bits and more below the rms, against 48 significant bits of
-// double-float arithmetic.  Against long double (12-site ring, 12 steps) alpha and beta are off by
-// 1.4e-14 and 1.8e-15 at U = 7.25, by 9.9e-10 and 4.2e-10 at U = 4000 (double-float 5.7e-14, 1.8e-15,
-// 1.1e-9 and 6.7e-10).
+// result depends on the order in which blocks finish.  A run whose vectors' rms falls below 2^48 grid
+// units (start vectors with a largest entry above some 100 times the rms: a ground state with an
+// electron added, a single configuration) is left to the FP64 driver: double-float vectors kept 48
+// bits of every entry, and below that line the grid would keep fewer.  Random start vectors have a
+// largest entry of 6 rms, their Lanczos vectors of up to 90.  Against long double (12-site ring, 24 steps,
+// largest error of alpha; in brackets with double-float vectors): random start 3.6e-15 (3.9e-14) at U = 4,
+// 7.8e-15 (9.0e-14) at U = 7.25, all entries positive 2.5e-15 (4.3e-14), one entry of 64 rms 7.7e-15 (5.0e-14),
+// a ground state of largest entry 128 rms 3.9e-13 (2.2e-12); an electron added to it, 169 rms, 3.1e-13 (1.0e-13)
+// on the grid and now 1.0e-14.
 //
 // Products for a caller (hub_apply) must keep every entry within 1e-13 (|H||x|)_n, which a grid
 // fixed by the largest entry does not give where (|H||x|)_n is small.  k_fix_out sees the entry's
@@ -1810,6 +1814,8 @@ int fix_lanczos(hub_ctx *h, const double *x0, int maxit, double tol, double *E0,
   h->start_norm = std::ldexp(std::sqrt(f->h_scal->N), ctl[kCtlShift] - (p.B - 2));   // 0: hub_green_coeffs looks
   if (ctl[kCtlShift] == 2047 - 1023 || !(f->h_scal->N > 0.0))
     return fail(HUB_ERR_ARG, "hub_lanczos_ground: start vector is zero or not finite");
+  const auto too_wide = [&](double N) { return N < 0x1p96 * (double)D; };      // rms below 2^48 (see the top)
+  if (too_wide(f->h_scal->N)) return kFixWide;
 
   // graphs of one step, kept while their operands stay the same
   bool graphs = !h->prof && !f->graph_failed;
@@ -1877,6 +1883,7 @@ int fix_lanczos(hub_ctx *h, const double *x0, int maxit, double tol, double *E0,
         if ((rc = fast_check_error(h))) return rc;
         return fail(HUB_ERR_CUDA, "hub_lanczos_ground: non-finite alpha/beta");
       }
+      if (too_wide(f->h_scal->hist[3 * b + 2])) return kFixWide;
       h->alpha.push_back(a);
       h->beta.push_back(be);
       if (tol > 0) E = lowest.next(h->alpha.data(), h->beta.data(), (int)h->alpha.size());   // else at the end

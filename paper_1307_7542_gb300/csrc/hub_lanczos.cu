@@ -380,9 +380,11 @@ extern "C" int hub_lanczos_ground(hub_t h, const double *x0_dev, int maxit, doub
       x0 = h->work[2];
     }
     rc = fix_lanczos(h, x0, maxit, tol, E0, psi_dev, iters, (cudaStream_t)stream);
-    if (rc != HUB_ERR_OOM) return rc;
-    fix_release(h);                   // its vectors do not fit: three FP64 ones may
-    h->fix_off = true;
+    if (rc != HUB_ERR_OOM && rc != kFixWide) return rc;
+    if (rc == HUB_ERR_OOM) {
+      fix_release(h);                 // its vectors do not fit: three FP64 ones may
+      h->fix_off = true;
+    }
     set_error("");
   }
   rc = ensure_workspace(h, D);
