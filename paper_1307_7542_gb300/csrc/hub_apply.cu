@@ -166,8 +166,9 @@ static int apply_kernels(hub_ctx *h, const double *x, double *y, cudaStream_t s)
   if (fix_apply_eligible(h)) {
     const int rc = fix_apply(h, x, y, s);
     if (rc != HUB_ERR_OOM) return rc;
-    h->fix_off = true;                // its vectors do not fit: the paths that need fewer
+    fast_release_scratch(h);          // its vectors do not fit (nor the double-float path's, the same ones)
     set_error("");
+    return f64_apply(h, x, y, nullptr, s);
   }
   if (use_fast(h)) return fast_apply_f64(h, x, y, s);
   return f64_apply(h, x, y, nullptr, s);

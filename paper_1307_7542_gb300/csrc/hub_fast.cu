@@ -1223,6 +1223,14 @@ int fast_exp_range(hub_ctx *h, const double *x, int64_t D, int **part, int *nblk
   return HUB_OK;
 }
 
+void fast_release_scratch(hub_ctx *h) {
+  FastState *f = fast_of(h);
+  for (float **v : {&f->xdf, &f->zdf, &f->xt, &f->zt}) {
+    dev_free(*v);
+    *v = nullptr;
+  }
+}
+
 int *fast_err(const hub_ctx *h) { return fast_of(h)->d_err; }
 
 // Conversion, both passes and the un-permutation of a product whose scale is known.

@@ -1342,7 +1342,7 @@ struct FixPlan {
 
 static FixPlan fix_plan(const hub_ctx *h) {
   FixPlan p;
-  if (h->mode != HUB_MODE_AUTO || h->fix_off || h->k0 || !h->have_hop || !h->have_U || !h->fast) return p;
+  if (h->mode != HUB_MODE_AUTO || h->k0 || !h->have_hop || !h->have_U || !h->fast) return p;
   if (h->count[0] <= 0 || h->count[1] <= 0) return p;
   // t uniform, U uniform, no site energies (the other models keep the 53-bit entries of the FP64
   // kernels, which the grid does not quite reach)

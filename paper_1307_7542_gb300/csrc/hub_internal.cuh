@@ -210,7 +210,6 @@ struct hub_ctx {
 
   // fixed-point product and Lanczos (hub_fix.cu): tables, flags and vectors
   hub::FixState *fix = nullptr;
-  bool fix_off = false;                // its vectors did not fit: the other paths until hub_hopping
 
   hub::Ham view() const;
 };
@@ -259,6 +258,7 @@ int fast_apply_host_many(hub_ctx *h, int64_t n_vec, const double *x_host, double
 int fast_apply_gated(hub_ctx *h, const double *x, double *y, const int *scale, const int *gate, cudaStream_t s);
 // The first n <= 4 scratch vectors of the handle, each large enough for a vector in either order.
 int fast_scratch(hub_ctx *h, int n, float **v);
+void fast_release_scratch(hub_ctx *h);
 // Largest and smallest biased exponents of x per block: part[0 .. nblk) and part[nblk .. 2 nblk).
 int fast_exp_range(hub_ctx *h, const double *x, int64_t D, int **part, int *nblk, cudaStream_t s);
 // The handle's device error flag.

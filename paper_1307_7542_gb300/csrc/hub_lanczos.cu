@@ -381,13 +381,21 @@ extern "C" int hub_lanczos_ground(hub_t h, const double *x0_dev, int maxit, doub
     }
     rc = fix_lanczos(h, x0, maxit, tol, E0, psi_dev, iters, (cudaStream_t)stream);
     if (rc != HUB_ERR_OOM && rc != kFixWide) return rc;
-    if (rc == HUB_ERR_OOM) {
-      fix_release(h);                 // its vectors do not fit: three FP64 ones may
-      h->fix_off = true;
-    }
     set_error("");
   }
-  rc = ensure_workspace(h, D);
+  // Where memory is short (for the fixed-point vectors, or for these beside them) the other paths' vectors
+  // go, and the FP64 kernel, which needs none, runs this call's products.
+  bool fp64 = rc == HUB_ERR_OOM;
+  if (!fp64) {
+    rc = ensure_workspace(h, D);
+    fp64 = rc == HUB_ERR_OOM && !h->k0 && h->fast;
+  }
+  if (fp64) {
+    fix_release(h);
+    if (h->fast) fast_release_scratch(h);
+    set_error("");
+    rc = ensure_workspace(h, D);
+  }
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   const int G = vec_grid(), T = kVecThreads;
@@ -424,7 +432,7 @@ extern "C" int hub_lanczos_ground(hub_t h, const double *x0_dev, int maxit, doub
   int status = HUB_ERR_NOCONV;
   // Step j, its coefficients on the way to the host.  The product carries the step's first half where it
   // runs in the FP64 kernel.
-  const bool fused = f64_product(h);
+  const bool fused = fp64 || f64_product(h);
   StepEvents ev;
   if ((rc = ev.create())) return rc;
   auto step = [&](int j) -> int {

@@ -446,7 +446,6 @@ extern "C" int hub_hopping(hub_t h, int n_bonds, const int32_t *bonds_host, cons
   }
   k0_leave(h);
   fix_release(h);
-  h->fix_off = false;
   h->have_hop = false;
   h->n_bonds = n_bonds;
   h->bonds.assign(bonds_host, bonds_host + 2 * n_bonds);

@@ -156,3 +156,43 @@ def test_vector_that_becomes_uneven(hub):
         scale = max(np.abs(a1).max(), b1.max())
         assert np.abs(a0 - a1).max() <= 1e-12 * scale and np.abs(b0 - b1).max() <= 1e-12 * scale
         assert float((p0 - p1).norm()) <= 1e-11
+
+
+def test_short_of_memory(hub):
+    """Room for three and a half more vectors: the product falls back on the FP64 kernel (room for
+    one), the Lanczos run, whose fixed-point form takes four, on the FP64 driver; both come back to the
+    fixed-point path once there is room."""
+    m = hub.Hubbard(14, 7, 7, W.ring_bonds(14), 1.0, 4.0)
+    size = 8 * m.D                                # 94 MB
+    x = torch.from_numpy(W.normal(6, m.D)).cuda()
+    y, psi = torch.empty_like(x), torch.empty_like(x)
+    hub.hub_set_mode(m.h, hub.HUB_MODE_FP64)
+    y64 = m.apply(x)
+    m.close()
+    m = hub.Hubbard(14, 7, 7, W.ring_bonds(14), 1.0, 4.0)
+    torch.cuda.empty_cache()
+
+    def fill(vectors):                            # leaves room for so many vectors
+        room = int(vectors * size)
+        return torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda")
+
+    hog = fill(1.5)
+    m.apply(x, y)
+    assert torch.equal(y, y64)
+    del hog
+    torch.cuda.empty_cache()
+    m.apply(x, y)
+    assert not torch.equal(y, y64)                # within the bound (other tests), but not the same bits
+    hub.hub_set_mode(m.h, hub.HUB_MODE_FP64)
+    E64 = hub.hub_lanczos_ground(m.h, x, 6, 0.0, psi)[0]
+    m.close()
+    m = hub.Hubbard(14, 7, 7, W.ring_bonds(14), 1.0, 4.0)
+    torch.cuda.empty_cache()
+    hog = fill(3.5)
+    E = hub.hub_lanczos_ground(m.h, x, 6, 0.0, y)[0]
+    assert E == E64 and torch.equal(y, psi)
+    del hog
+    torch.cuda.empty_cache()
+    E = hub.hub_lanczos_ground(m.h, x, 6, 0.0, y)[0]
+    assert abs(E - E64) <= 1e-11 and not torch.equal(y, psi)
+    m.close()
