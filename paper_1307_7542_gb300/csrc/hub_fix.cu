@@ -72,7 +72,9 @@ constexpr int kFixHist = 8;         // Lanczos steps recorded between two host r
 constexpr int kFixFrac = 4;         // fraction bits of the update's sums
 
 // ctl words of a product (device): see k_fix_plan
-enum { kCtlShift = 0, kCtlSkip = 1, kCtlCount = 2, kCtlDf = 3, kCtlF64 = 4, kCtlDfScale = 6, kCtlWords = 8 };
+enum { kCtlShift = 0, kCtlSkip = 1, kCtlDf = 2, kCtlF64 = 3, kCtlDfScale = 4, kCtlCount = 6, kCtlWords = 8 };
+// Entries to recompute: a 64-bit count over two words, since any number of a vector's entries may ask for it.
+__device__ __forceinline__ u64 *count_of(int *ctl) { return reinterpret_cast<u64 *>(ctl + kCtlCount); }
 
 // One spin's hopping matrix as row combinations: a row's entries are ordered adding pairs,
 // subtracting pairs, then the last adding and the last subtracting one where their numbers are odd.
@@ -288,7 +290,7 @@ __global__ void k_fix_plan(const int *__restrict__ partials, int nblk, i64 D, co
     ctl[kCtlShift] = ctl[kCtlDfScale] = emax == 0 ? 0 : emax - 1023;
     ctl[kCtlDfScale + 1] = 0;
     ctl[kCtlSkip] = out || wide ? 1 : 0;
-    ctl[kCtlCount] = 0;
+    *count_of(ctl) = 0;
     ctl[kCtlDf] = !out && wide && df_ok ? 1 : 0;
     ctl[kCtlF64] = out || (wide && !df_ok) ? 1 : 0;
   }
@@ -1202,10 +1204,9 @@ __global__ void __launch_bounds__(kTileThreads, kUpdateBlocks) k_fix_out(i64 n_r
     for (int j = 0; j < 2; ++j) {
       v[j] = fix_to_f64(s0[j] + s1[j], e);
       if (tabs != 1.0) v[j] *= tabs;
-      // beyond cap only what was under way is still counted, so that the count stays far below 2^31
-      if ((j == 0 || second) && llabs(s0[j]) + llabs(s1[j]) < thr && *(volatile int *)(ctl + kCtlCount) <= cap) {
-        const int at_list = atomicAdd(ctl + kCtlCount, 1);
-        if (at_list < cap) list[at_list] = n + j;
+      if ((j == 0 || second) && llabs(s0[j]) + llabs(s1[j]) < thr) {
+        const u64 at_list = atomicAdd(count_of(ctl), 1ull);
+        if (at_list < (u64)cap) list[at_list] = n + j;
       }
     }
     if (vec) {
@@ -1237,8 +1238,9 @@ __global__ void __launch_bounds__(256) k_fix_entries(const Ham H, const double *
                                                      int *__restrict__ ctl, const i64 *__restrict__ list, int cap,
                                                      int df_ok) {
   if (ctl[kCtlSkip]) return;
-  const int n = ctl[kCtlCount];
-  if (n > cap) {
+  const u64 all = *count_of(ctl);
+  const int n = (int)min(all, (u64)cap);
+  if (all > (u64)cap) {
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl[df_ok ? kCtlDf : kCtlF64] = 1;
     return;
   }
