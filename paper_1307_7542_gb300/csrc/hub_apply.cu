@@ -8,26 +8,29 @@
 // The diagonal (Sec. III.B) is sum_i U_i bit_i(I_up & I_dn) + eps(I_up) + eps(I_dn),
 // computed on the fly from popcount instead of Algorithm II's index_U tables.
 //
-// Kernel shape (FP64 path): a CTA takes two rows d of X and a chunk of columns u.  It stages both
-// rows in shared memory when they fit; each thread owns columns u and sums the H_up row of u
-// (gathers from shared memory; an entry is loaded once for both rows) and the H_dn rows of both d
-// (coalesced loads of the neighbour rows X[d'][u], served from L2).  The FP64 unit bounds it: one
-// multiply-add per term, at about 1/70 of the integer rate (disordered 3x4 lattice, 853,776 states,
-// 26 hops each: 56 us, with the Lanczos step around it 74 us; 47 us of FP64 issue).  Columns are cut
-// at multiples of a warp, since a partial warp costs the unit a whole one.
+// Kernel shape (FP64 path): a CTA takes two rows d of X and a chunk of columns u; each thread owns
+// columns u and sums the H_up row of u (gathers from the two rows through L1; an entry's column and
+// value are loaded once for both) and the H_dn rows of both d (coalesced loads of the neighbour rows
+// X[d'][u], served from L2).  The FP64 unit bounds it: one multiply-add per term, at about 1/70 of the
+// integer rate (12-site ring, every t and U its own, 853,776 states, 1.2e7 hops: 45 us, about 26 us of FP64
+// issue).  Staging the two rows in shared memory gained nothing at any row length (1716 entries: 0.114 ms
+// either way) and left an SM one CTA of 256 threads for rows of 6,000 to 12,800 entries: 4x4 (6,3), 8008
+// entries, 0.46 ms staged, 0.29 ms not; 3x6 (5,4) 3.67 and 1.6 ms.
+// Columns are cut at multiples of a warp, since a partial warp costs the unit a whole one.
 #include "hub_internal.cuh"
 
 namespace hub {
 
-// The diagonal with the sums over doubly occupied sites from a table: one lookup per four sites
-// instead of one divergent read of the parameters per set bit.
-__device__ __forceinline__ double f64_diag(const Ham &H, const double (*s_U)[16], uint32_t both, int64_t u, int64_t d) {
+// The diagonal with the sums over doubly occupied sites from a table: one lookup per eight sites
+// instead of one divergent read of the parameters per set bit.  (One per four sites costs up to seven
+// FP64 additions a state: 13-site ring (6,6) 146 us against 135 us.)
+__device__ __forceinline__ double f64_diag(const Ham &H, const double *s_U, uint32_t both, int64_t u, int64_t d) {
   double v;
   if (H.uniform_U) {
     v = H.U0 * (double)__popc(both);
   } else {
-    v = s_U[0][both & 15];
-    for (int k = 1; 4 * k < H.M; ++k) v += s_U[k][(both >> 4 * k) & 15];
+    v = s_U[both & 255];
+    for (int k = 1; 8 * k < H.M; ++k) v += s_U[256 * k + ((both >> 8 * k) & 255)];
   }
   if (H.has_eps) v += H.eps_up[u] + H.eps_dn[d];
   return v;
@@ -37,20 +40,24 @@ __device__ __forceinline__ double f64_diag(const Ham &H, const double (*s_U)[16]
 // kMode 2: psi += v x, y = (H x - a x - c prev) inv (second pass, known coefficients).
 // gate: null, or a device flag; the kernel does nothing while gate[0] is 0 (the other paths
 // pass their out-of-window flag, so that this kernel multiplies exactly the vectors they cannot).
-template <bool kStage, int kMode, int kF64Rows>
+template <int kMode, int kF64Rows>
 __global__ void __launch_bounds__(256, 6) k_apply_f64(const Ham H, const double *__restrict__ x, double *y,
                                                    const int *__restrict__ gate, int chunks, const F64Step L) {
   if (gate && gate[0] == 0) return;
-  extern __shared__ double xs[];
-  __shared__ double s_U[8][16];                  // sums of U_i over the set bits of each four sites
+  // Sums of U_i over the set bits of each eight sites, from those of each four; only where U varies, since
+  // the L1 that serves the gathers shrinks by it (uniform U, 17-site ring (7,2): 0.105 ms, with 9 KB 0.117).
+  extern __shared__ double s_tab[];
+  const double *s_U = s_tab + 128;
   if (!H.uniform_U) {
-    if (threadIdx.x < 128 || blockDim.x < 128)
-      for (int k = threadIdx.x; k < 128; k += min(blockDim.x, 128)) {
-        double v = 0.0;
-        for (int i = 0; i < 4; ++i)
-          if (((k >> i) & 1) && (k >> 4) * 4 + i < H.M) v += H.U[(k >> 4) * 4 + i];
-        s_U[k >> 4][k & 15] = v;
-      }
+    for (int k = threadIdx.x; k < 128; k += blockDim.x) {
+      double v = 0.0;
+      for (int i = 0; i < 4; ++i)
+        if (((k >> i) & 1) && (k >> 4) * 4 + i < H.M) v += H.U[(k >> 4) * 4 + i];
+      s_tab[k] = v;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < (H.M + 7) / 8 * 256; k += blockDim.x)
+      s_tab[128 + k] = s_tab[(k >> 8) * 32 + (k & 15)] + s_tab[(k >> 8) * 32 + 16 + ((k >> 4) & 15)];
     __syncthreads();
   }
   const int64_t nu = H.n_up, nd = H.n_dn;
@@ -63,14 +70,7 @@ __global__ void __launch_bounds__(256, 6) k_apply_f64(const Ham H, const double 
   for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
     const int64_t d = item / chunks * kF64Rows, u0 = item % chunks * width, u1 = min(nu, u0 + width);
     const int rows = kF64Rows == 1 ? 1 : (int)min((int64_t)kF64Rows, nd - d);
-    const double *__restrict__ xrow = x + d * nu;
-    if (kStage) {
-      if (item != blockIdx.x) __syncthreads();
-#pragma unroll 4
-      for (int64_t u = threadIdx.x; u < rows * nu; u += blockDim.x) xs[u] = xrow[u];
-      __syncthreads();
-    }
-    const double *r0 = kStage ? xs : xrow, *r1 = rows > 1 ? r0 + nu : r0;
+    const double *__restrict__ r0 = x + d * nu, *__restrict__ r1 = rows > 1 ? r0 + nu : r0;
     const uint32_t Id0 = H.basis_dn[d], Id1 = rows > 1 ? H.basis_dn[d + 1] : 0u;
     const int32_t k0 = H.rp_dn[d], k1 = H.rp_dn[d + 1], k2 = rows > 1 ? H.rp_dn[d + 2] : k1;
     for (int64_t u = u0 + threadIdx.x; u < u1; u += blockDim.x) {
@@ -109,11 +109,6 @@ __global__ void __launch_bounds__(256, 6) k_apply_f64(const Ham H, const double 
   }
   if (kMode == 1) f64_step_alpha(L, dot);
 }
-
-// Rows of a CTA: two; one where rows are so narrow that a CTA has few threads at work (12 columns x 924
-// rows: 8.1 us, 10.7 with two).
-static int f64_rows(const Ham &H) { return H.n_up > 128 ? 2 : 1; }
-static size_t stage_bytes(const Ham &H) { return sizeof(double) * (size_t)H.n_up * f64_rows(H); }
 
 static int apply_kernels(hub_ctx *h, const double *x, double *y, cudaStream_t s);
 
@@ -175,8 +170,14 @@ static int apply_kernels(hub_ctx *h, const double *x, double *y, cudaStream_t s)
 }
 
 // Columns of a CTA: chunks of 256 and less where the row is short, so that a small matrix still makes
-// several CTAs per SM; a quarter of a longer row, which is staged once per chunk.
+// several CTAs per SM; a quarter of a longer row.
 static int f64_chunks(const Ham &H) { return (int)std::min<int64_t>(4, (H.n_up + 255) / 256); }
+// Rows of a CTA: two, or one where rows are so narrow that a CTA has few threads at work (12 columns x 924
+// rows: 8.1 us, 10.7 with two) or the matrix is so small that two would leave SMs idle (252 x 252: 7.6 us,
+// 10.3 with two).
+static int f64_rows(const Ham &H) {
+  return H.n_up > 128 && (H.n_dn + 1) / 2 * f64_chunks(H) >= 2 * num_sms() ? 2 : 1;
+}
 int64_t f64_grid(const Ham &H) {
   const int rows = f64_rows(H);
   return std::min<int64_t>((H.n_dn + rows - 1) / rows * f64_chunks(H), (int64_t)num_sms() * 16);
@@ -188,19 +189,12 @@ template <int kMode>
 static int f64_launch(hub_ctx *h, const double *x, double *y, const int *gate, const F64Step &L, cudaStream_t s) {
   const Ham H = h->view();
   count_launch(h);
-  const size_t smem = stage_bytes(H);
   const int chunks = f64_chunks(H);
   const int64_t width = (H.n_up + chunks - 1) / chunks;
   const int threads = width > 128 ? 256 : (width > 64 ? 128 : 64);
   const int grid = (int)f64_grid(H);
-  if (smem > 200 * 1024) {
-    k_apply_f64<false, kMode, 2><<<grid, threads, 0, s>>>(H, x, y, gate, chunks, L);
-  } else if (f64_rows(H) == 1) {
-    k_apply_f64<true, kMode, 1><<<grid, threads, smem, s>>>(H, x, y, gate, chunks, L);
-  } else {
-    HUB_CUDA(cudaFuncSetAttribute(k_apply_f64<true, kMode, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    k_apply_f64<true, kMode, 2><<<grid, threads, smem, s>>>(H, x, y, gate, chunks, L);
-  }
+  const size_t tab = H.uniform_U ? 0 : sizeof(double) * (128 + (size_t)(H.M + 7) / 8 * 256);
+  (f64_rows(H) == 1 ? k_apply_f64<kMode, 1> : k_apply_f64<kMode, 2>)<<<grid, threads, tab, s>>>(H, x, y, gate, chunks, L);
   HUB_LAUNCH_CHECK();
   return HUB_OK;
 }
