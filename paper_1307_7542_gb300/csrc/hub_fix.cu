@@ -594,42 +594,198 @@ __global__ void __launch_bounds__(1024, 1) k_fix_gather(const FixPass P, const G
   if (kLz) pass_end(P, dots, vmax);
 }
 
+// Schedules, built on the device by the five kernels below (blockIdx.y: the spin), without a copy to
+// the host, beside the allocation of the scratch vectors: a handle's first product waits for them.  The
+// first product of the 13-site ring (6,6) takes 0.28 ms (0.29 without a schedule, in double-float; 0.51
+// with the groups made on the host), of 4x4 (2,8) 0.42 ms (0.30; 1.4).
+//
+// Groups of 16 positions: four quads of consecutive positions each (the outputs of a quad are one 32-byte
+// sector), chosen greedily among the next 32 quads, longest rows first, so that the group's
+// busiest bank stays low; or the quads in their own order where that needs no more steps.  At 4x4 1.17
+// steps per entry of a row against 1.26.
+constexpr int kSchedRow = 64;         // longest hopping row of the gather form
+constexpr int kSchedMax = 2 * kSchedRow;
+// Quads that a warp groups: more of them make better groups (4x4, 12,870 positions: 1.197 steps per entry with
+// 64, 1.186 with 128, 1.171 with all), but take a quarter of a microsecond each.
+constexpr int kSegFew = 64, kSegMany = 256, kSegManyFrom = 4096;
+struct SchedSpin {
+  int n, groups, idle, cap, seg;      // positions, groups (even), the position of a zero, most steps, kSeg*
+  const int32_t *rp;
+  const uint32_t *scol;
+  uint32_t *load;                     // [4 groups][8] entries of a quad by bank, two counts a word
+  uint32_t *len;                      // [4 groups] bytes: longest row of a quad
+  uint16_t *sorted, *greedy;          // [4 groups] quads by length; grouped
+  uint8_t *steps;                     // [2][groups] steps of the groups in natural order, and grouped
+  uint32_t *total;                    // [2] their sums
+  uint16_t *quad;                     // [4 groups] the groups' quads, longest groups first ...
+  uint8_t *deg;                       // [groups] ... and their steps
+  uint16_t *word;                     // the schedule (GatherLists)
+  uint32_t *meta;
+};
+struct SchedArgs {
+  SchedSpin spin[2];
+};
+
+__global__ void __launch_bounds__(256) k_fix_quads(const SchedArgs A) {
+  const SchedSpin &S = A.spin[blockIdx.y];
+  __shared__ uint32_t count[16][16];
+  const int half = threadIdx.x >> 4, lane = threadIdx.x & 15, q = blockIdx.x * 16 + half;
+  if (blockIdx.x == 0 && threadIdx.x < 2) S.total[threadIdx.x] = 0;
+  count[half][lane] = 0;
+  __syncthreads();
+  const int r0 = min(4 * q, S.n), r1 = min(4 * q + 4, S.n);
+  for (int32_t k = S.rp[r0] + lane; k < S.rp[r1]; k += 16) atomicAdd(&count[half][S.scol[k] & 15], 1u);
+  __syncthreads();
+  if (q >= 4 * S.groups) return;
+  if (lane < 8) S.load[8 * q + lane] = count[half][2 * lane] | (count[half][2 * lane + 1] << 16);
+  if (lane == 8) {
+    int m = 0;
+    for (int r = r0; r < r1; ++r) m = max(m, S.rp[r + 1] - S.rp[r]);
+    reinterpret_cast<uint8_t *>(S.len)[q] = (uint8_t)m;
+  }
+}
+
+// Place of byte i among the bytes of w, largest first and equal ones in their order.
+__device__ __forceinline__ int place_desc(const uint32_t *w, int words, int i) {
+  const uint32_t own = w[i >> 2], v = (own >> (8 * (i & 3))) & 255u, v4 = v * 0x01010101u;
+  int above = 0;
+  for (int k = 0; k < (i >> 2); ++k) above += __popc(__vcmpgeu4(w[k], v4));
+  for (int k = (i >> 2) + 1; k < words; ++k) above += __popc(__vcmpgtu4(w[k], v4));
+  above >>= 3;
+  for (int j = 0; j < 4; ++j) {
+    const uint32_t b = (own >> (8 * j)) & 255u;
+    above += b > v || (b == v && j < (i & 3)) ? 1 : 0;
+  }
+  return above;
+}
+
+constexpr int kSchedQuads = (kStageMax + 31) / 32 * 8;       // most quads of a spin
+__global__ void __launch_bounds__(256) k_fix_sort(const SchedArgs A) {
+  const SchedSpin &S = A.spin[blockIdx.y];
+  __shared__ uint32_t len[kSchedQuads / 4];
+  for (int k = threadIdx.x; k < S.groups; k += 256) len[k] = S.len[k];
+  __syncthreads();
+  const int q = blockIdx.x * 256 + threadIdx.x;
+  if (q < 4 * S.groups) S.sorted[place_desc(len, S.groups, q)] = (uint16_t)q;
+}
+
+__global__ void __launch_bounds__(32) k_fix_group(const SchedArgs A) {
+  const SchedSpin &S = A.spin[blockIdx.y];
+  __shared__ uint32_t load[kSegMany][9];
+  __shared__ uint16_t id[kSegMany], left[kSegMany];
+  __shared__ uint8_t len[kSegMany];
+  const int lane = threadIdx.x, base = blockIdx.x * S.seg, n = min(S.seg, 4 * S.groups - base);
+  if (n <= 0) return;
+  const uint8_t *lens = reinterpret_cast<const uint8_t *>(S.len);
+  for (int i = lane; i < n; i += 32) {
+    const int q = S.sorted[base + i];
+    id[i] = (uint16_t)q;
+    len[i] = lens[q];
+    left[i] = (uint16_t)i;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) load[i][w] = S.load[8 * q + w];
+  }
+  __syncwarp();
+  uint32_t natural = 0, greedy = 0;
+  for (int g = 0, head = 0; 4 * g < n; ++g) {
+    uint32_t sum[8];                             // two banks a word, at most 16 rows of kSchedRow entries: 2^10
+#pragma unroll
+    for (int w = 0; w < 8; ++w) sum[w] = 0;
+    uint32_t most = 0;
+    for (int k = 0; k < 4; ++k, ++head) {
+      const int window = k ? min(32, n - head) : 1;
+      const int own = lane < window ? left[head + lane] : 0;
+      uint32_t m2[2] = {0, 0}, sq[4] = {0, 0, 0, 0};         // sq <= 2^20 in all: the group's entries squared
+#pragma unroll
+      for (int w = 0; w < 8; ++w) {
+        const uint32_t t = sum[w] + load[own][w];
+        m2[w & 1] = __vmaxu2(m2[w & 1], t);
+        sq[w & 1] += (t & 0xffffu) * (t & 0xffffu);
+        sq[2 + (w & 1)] += (t >> 16) * (t >> 16);
+      }
+      const uint32_t mm = __vmaxu2(m2[0], m2[1]), m = max(mm & 0xffffu, mm >> 16);
+      const uint32_t key = lane < window ? (m << 21) | (sq[0] + sq[1] + sq[2] + sq[3]) : ~0u;
+      const int at = __ffs(__ballot_sync(0xffffffffu, key == __reduce_min_sync(0xffffffffu, key))) - 1;
+      const int pick = __shfl_sync(0xffffffffu, own, at);
+      __syncwarp();
+      if (lane < at) left[head + lane + 1] = (uint16_t)own;
+      if (lane == 0) {
+        left[head] = (uint16_t)pick;
+        S.greedy[base + 4 * g + k] = id[pick];
+      }
+      __syncwarp();
+#pragma unroll
+      for (int w = 0; w < 8; ++w) sum[w] += load[pick][w];
+      most = max(most, (uint32_t)len[pick]);
+    }
+#pragma unroll
+    for (int w = 0; w < 8; ++w) most = max(most, max(sum[w] & 0xffffu, sum[w] >> 16));
+    most = min(most, (uint32_t)S.cap);
+    // the same of the group in natural order
+    const int ng = base / 4 + g;
+    uint32_t v = 0;
+    if (lane < 16)
+      for (int k = 0; k < 4; ++k) v += (S.load[8 * (4 * ng + k) + (lane >> 1)] >> (16 * (lane & 1))) & 0xffffu;
+    else if (lane < 20)
+      v = lens[4 * ng + lane - 16];
+    v = min(__reduce_max_sync(0xffffffffu, v), (uint32_t)S.cap);
+    if (lane == 0) {
+      S.steps[ng] = (uint8_t)v;
+      S.steps[S.groups + ng] = (uint8_t)most;
+    }
+    natural += v;
+    greedy += most;
+  }
+  if (lane == 0) {
+    atomicAdd(S.total, natural);
+    atomicAdd(S.total + 1, greedy);
+  }
+}
+
+// The groups by length, so that the two of a slice need nearly the same number of steps.
+__global__ void __launch_bounds__(1024) k_fix_order(const SchedArgs A) {
+  const SchedSpin &S = A.spin[blockIdx.y];
+  __shared__ uint32_t deg[(kSchedQuads / 4 + 3) / 4];
+  const bool greedy = S.total[1] < S.total[0];
+  const int words = (S.groups + 3) / 4;
+  for (int k = threadIdx.x; k < words; k += 1024) {
+    uint32_t w = 0;
+    for (int j = 0; j < 4 && 4 * k + j < S.groups; ++j)
+      w |= (uint32_t)S.steps[(greedy ? S.groups : 0) + 4 * k + j] << (8 * j);
+    deg[k] = w;
+  }
+  __syncthreads();
+  for (int g = threadIdx.x; g < S.groups; g += 1024) {
+    const int at = place_desc(deg, words, g);
+    S.deg[at] = (uint8_t)(deg[g >> 2] >> (8 * (g & 3)));
+    for (int k = 0; k < 4; ++k) S.quad[4 * at + k] = greedy ? S.greedy[4 * g + k] : (uint16_t)(4 * g + k);
+  }
+}
+
 // Schedule of a group of 16 positions, the lanes of a half-warp: a colouring of the bipartite graph
 // lanes x banks (position mod 16) whose edges are the group's entries -- no two edges of a lane or
 // of a bank share a step.  By Koenig's theorem as many steps suffice as the largest degree has
 // edges; they are found edge by edge, exchanging two colours along an alternating path where the
-// lane and the bank have no free step in common.  A bank with more entries than cap_steps takes
+// lane and the bank have no free step in common.  A bank with more entries than cap steps takes
 // the rest in steps of its lanes alone (conflicts, but the schedule stays bounded).  A warp per
-// group (quads 4 g .. 4 g + 3 of quad), one lane of which colours, with the free steps of lanes and
-// banks as bit masks: 93 us at 4x4 (a thread per group and linear searches: 0.8 ms).  deg[g] = its steps.
-constexpr int kSchedRow = 64;         // longest hopping row of the gather form
-constexpr int kSchedMax = 2 * kSchedRow;
+// group, one lane of which colours, with the free steps of lanes and banks as bit masks: 93 us at 4x4
+// (a thread per group and linear searches: 0.8 ms).
 constexpr uint16_t kNoEntry = 0xffff;
-__global__ void __launch_bounds__(32) k_fix_schedule(int n, int groups, int idle, int cap_steps,
-                                                     const int32_t *__restrict__ quad,
-                                                     const int32_t *__restrict__ rp,
-                                                     const uint32_t *__restrict__ scol, uint16_t *__restrict__ word,
-                                                     uint16_t *__restrict__ deg) {
-  const int g = blockIdx.x, lane = threadIdx.x;
-  if (g >= groups) return;
+__global__ void __launch_bounds__(32) k_fix_schedule(const SchedArgs A) {
+  const SchedSpin &S = A.spin[blockIdx.y];
+  const int g = blockIdx.x, lane = threadIdx.x, n = S.n;
+  if (g >= S.groups) return;
+  const uint16_t *__restrict__ quad = S.quad;
+  const int32_t *__restrict__ rp = S.rp;
+  const uint32_t *__restrict__ scol = S.scol;
   __shared__ uint16_t at[16][kSchedMax];         // entry of a lane at a step
   __shared__ int8_t who[16][kSchedMax];          // lane that reads a bank at a step
   __shared__ u64 free_l[16][2], free_b[16][2];   // free steps
-  __shared__ int load[16];
-  if (lane < 16) load[lane] = 0;
   for (int k = lane; k < 16 * kSchedMax; k += 32) {
     at[k / kSchedMax][k % kSchedMax] = kNoEntry;
     who[k / kSchedMax][k % kSchedMax] = -1;
   }
-  __syncwarp();
-  const int own = quad[4 * g + ((lane & 15) >> 2)] * 4 + (lane & 3);
-  int steps = 0;
-  if (lane < 16 && own < n) {
-    steps = rp[own + 1] - rp[own];
-    for (int32_t k = rp[own]; k < rp[own + 1]; ++k) atomicAdd(&load[scol[k] & 15], 1);
-  }
-  __syncwarp();
-  steps = min(__reduce_max_sync(0xffffffffu, max(steps, load[lane & 15])), cap_steps);
+  const int steps = S.deg[g];
   if (lane < 16)
     for (int h = 0; h < 2; ++h) {
       const int m = min(max(steps - 64 * h, 0), 64);
@@ -694,23 +850,16 @@ __global__ void __launch_bounds__(32) k_fix_schedule(int n, int groups, int idle
     }
   }
   __syncwarp();
-  // idle lanes read the zero of a bank the step leaves free
-  uint16_t *out = word + (size_t)g * cap_steps * 16;
-  for (int j = lane; j < cap_steps; j += 32) {
+  // into the slice's layout; idle lanes read the zero of a bank the step leaves free
+  const int all = (S.deg[g & ~1] + 1) & ~1, half = g & 1;          // words hold two steps
+  for (int j = lane; j < max(8, (all + 7) & ~7); j += 32) {
     int fb = 0;
     while (fb < 15 && who[fb][j] >= 0) ++fb;
-    const uint16_t z = (uint16_t)((idle + ((fb - idle) & 15)) | 0x4000);
-    for (int l = 0; l < 16; ++l) out[j * 16 + l] = at[l][j] == kNoEntry ? z : at[l][j];
+    const uint16_t z = (uint16_t)((S.idle + ((fb - S.idle) & 15)) | 0x4000);
+    uint16_t *out = S.word + ((((size_t)(g >> 1) * (S.cap / 8) + (j >> 3)) * 32 + 16 * half) * 8 + (j & 7));
+    for (int l = 0; l < 16; ++l) out[8 * l] = at[l][j] == kNoEntry ? z : at[l][j];
   }
-  if (lane == 0) deg[g] = (uint16_t)steps;
-}
-// The groups' schedules side by side in the slices' layout.
-__global__ void k_fix_pack(const int32_t *__restrict__ group, int cap_steps, const uint16_t *__restrict__ in,
-                           uint16_t *__restrict__ word) {
-  const int sl = blockIdx.x, lane = threadIdx.x, g = group[2 * sl + (lane >> 4)];
-  for (int j = 0; j < cap_steps; ++j)
-    word[(((size_t)sl * (cap_steps / 8) + (j >> 3)) * 32 + lane) * 8 + (j & 7)] =
-        in[((size_t)g * cap_steps + j) * 16 + (lane & 15)];
+  if (lane < 16) S.meta[16 * g + lane] = (uint32_t)(quad[4 * g + (lane >> 2)] * 4 + (lane & 3)) | ((uint32_t)all << 16);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1385,131 +1534,71 @@ static FixState *fix_state(hub_ctx *h) {
 static i64 fix_ld(i64 n) { return (n + 3) & ~(i64)3; }
 static int grid_of(i64 n) { return (int)std::max<i64>(1, std::min<i64>((n + 255) / 256, (i64)num_sms() * 16)); }
 
-// Groups of 16 positions for a gather schedule: four quads of consecutive positions each (the
-// outputs of a quad are one 32-byte sector), chosen greedily among the next 32 quads, longest rows
-// first, so that the group's busiest bank stays low; or the quads in their own order where that
-// needs no more steps.  At 4x4 1.17 steps per entry of a row against 1.26.
-static std::vector<int32_t> gather_groups(int n, const SpinCSR &c, int *rc) {
-  const int groups = (n + 31) / 32 * 2, quads = 4 * groups;
-  std::vector<int32_t> rp(n + 1), natural(quads), best(quads);
-  std::vector<uint32_t> sc(std::max<i64>(c.nnz, 1));
-  cudaError_t e = cudaMemcpy(rp.data(), c.rowptr, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess && c.nnz) e = cudaMemcpy(sc.data(), c.scol, sizeof(uint32_t) * c.nnz, cudaMemcpyDeviceToHost);
-  *rc = e == cudaSuccess ? HUB_OK : cuda_fail(e, "gather groups", __FILE__, __LINE__);
-  if (*rc) return natural;
-  std::vector<int32_t> load(16 * (size_t)quads, 0), len(quads, 0);
-  for (int r = 0; r < n; ++r) {
-    len[r / 4] = std::max(len[r / 4], rp[r + 1] - rp[r]);
-    for (int32_t k = rp[r]; k < rp[r + 1]; ++k) ++load[16 * (size_t)(r / 4) + (sc[k] & 15)];
-  }
-  for (int q = 0; q < quads; ++q) natural[q] = q;
-  auto steps = [&](const std::vector<int32_t> &order) {
-    i64 total = 0;
-    for (int g = 0; g < groups; ++g) {
-      int m = 0;
-      for (int b = 0; b < 16; ++b) {
-        int s = 0;
-        for (int k = 0; k < 4; ++k) s += load[16 * (size_t)order[4 * g + k] + b];
-        m = std::max(m, s);
-      }
-      for (int k = 0; k < 4; ++k) m = std::max(m, len[order[4 * g + k]]);
-      total += m;
-    }
-    return total;
-  };
-  std::vector<int32_t> left = natural;
-  std::stable_sort(left.begin(), left.end(), [&](int a, int b) { return len[a] > len[b]; });
-  size_t head = 0;
-  for (int g = 0; g < groups; ++g) {
-    int32_t sum[16] = {0};               // at most 4 quads of 4 rows of kSchedRow entries: 2^10
-    for (int k = 0; k < 4; ++k) {
-      size_t pick = head;
-      int64_t score = INT64_MAX;
-      for (size_t i = head; i < std::min(left.size(), head + (k ? 32 : 1)); ++i) {
-        const int32_t *l = &load[16 * (size_t)left[i]];
-        int32_t m = 0, sq = 0;
-        for (int b = 0; b < 16; ++b) {
-          const int32_t v = sum[b] + l[b];
-          m = std::max(m, v);
-          sq += v * v;
-        }
-        const int64_t sc2 = ((int64_t)m << 32) + sq;
-        if (sc2 < score) {
-          score = sc2;
-          pick = i;
-        }
-      }
-      best[4 * g + k] = left[pick];
-      for (int b = 0; b < 16; ++b) sum[b] += load[16 * (size_t)left[pick] + b];
-      for (size_t i = pick; i > head; --i) left[i] = left[i - 1];
-      ++head;
-    }
-  }
-  return steps(best) < steps(natural) ? best : natural;
-}
-
-// Gather schedule of a spin: the groups coloured on the device, then paired by length into slices.
-// One allocation for the schedule and what it is made from (a first product pays for each).
-static int gather_tables(FixState *f, int s, int n, const SpinCSR &c) {
+// Arrays of a spin's gather schedule and of what it is made from, in one allocation (a first product
+// pays for each).
+static int gather_arrays(FixState *f, int s, int n, const SpinCSR &c, SchedSpin *S) {
   const int slices = (n + 31) / 32, groups = 2 * slices;
   const int cap = std::min(kSchedMax, (2 * std::max(c.max_row, 1) + 7) / 8 * 8);
-  std::vector<uint16_t> d(groups);
-  std::vector<int32_t> order(groups);
-  int rc = HUB_OK;
-  const std::vector<int32_t> q = gather_groups(n, c, &rc);
-  if (rc) return rc;
-  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
-  const size_t words = up(sizeof(uint16_t) * 32 * (size_t)slices * cap), lanes = 32 * (size_t)slices;
-  const size_t o_meta = 2 * words, o_quad = o_meta + up(sizeof(uint32_t) * (lanes + groups));
-  const size_t o_deg = o_quad + up(sizeof(int32_t) * q.size()), bytes = o_deg + up(sizeof(uint16_t) * groups);
-  if (!f->sched[s] && !dev_alloc((void **)&f->sched[s], bytes, "gather schedule")) return HUB_ERR_OOM;
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    const size_t o = at;
+    at += (bytes + 255) / 256 * 256;
+    return o;
+  };
+  const size_t o_word = take(sizeof(uint16_t) * 32 * (size_t)slices * cap);
+  const size_t o_meta = take(sizeof(uint32_t) * 32 * (size_t)slices);
+  const size_t o_load = take(sizeof(uint32_t) * 8 * 4 * groups), o_len = take(4 * (size_t)groups);
+  const size_t o_sorted = take(sizeof(uint16_t) * 4 * groups), o_greedy = take(sizeof(uint16_t) * 4 * groups);
+  const size_t o_quad = take(sizeof(uint16_t) * 4 * groups), o_steps = take(2 * (size_t)groups);
+  const size_t o_deg = take((size_t)groups), o_total = take(2 * sizeof(uint32_t));
+  if (!f->sched[s] && !dev_alloc((void **)&f->sched[s], at, "gather schedule")) return HUB_ERR_OOM;
   char *base = (char *)f->sched[s];
   f->meta[s] = (uint32_t *)(base + o_meta);
   f->cap_steps[s] = cap;
   f->slices[s] = slices;
-  uint16_t *tmp = (uint16_t *)(base + words), *deg = (uint16_t *)(base + o_deg);
-  int32_t *quad = (int32_t *)(base + o_quad), *grp = (int32_t *)(f->meta[s] + lanes);
-  HUB_CUDA(cudaMemcpy(quad, q.data(), sizeof(int32_t) * q.size(), cudaMemcpyHostToDevice));
-  k_fix_schedule<<<groups, 32>>>(n, groups, (int)fix_ld(n), cap, quad, c.rowptr, c.scol, tmp, deg);
-  HUB_LAUNCH_CHECK();
-  HUB_CUDA(cudaMemcpy(d.data(), deg, sizeof(uint16_t) * groups, cudaMemcpyDeviceToHost));
-  for (int g = 0; g < groups; ++g) order[g] = g;
-  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return d[a] > d[b]; });
-  std::vector<uint32_t> meta(lanes + groups);
-  for (int k = 0; k < slices; ++k)
-    for (int l = 0; l < 32; ++l) {          // words hold two steps
-      const uint32_t steps = (d[order[2 * k]] + 1u) & ~1u;
-      const uint32_t at = (uint32_t)q[4 * order[2 * k + (l >> 4)] + ((l >> 2) & 3)] * 4 + (l & 3);
-      meta[32 * (size_t)k + l] = at | (steps << 16);
-    }
-  for (int g = 0; g < groups; ++g) meta[lanes + g] = (uint32_t)order[g];
-  HUB_CUDA(cudaMemcpy(f->meta[s], meta.data(), sizeof(uint32_t) * meta.size(), cudaMemcpyHostToDevice));
-  k_fix_pack<<<slices, 32>>>(grp, cap, tmp, f->sched[s]);
-  HUB_LAUNCH_CHECK();
+  *S = SchedSpin{n, groups, (int)fix_ld(n), cap, n < kSegManyFrom ? kSegFew : kSegMany, c.rowptr, c.scol, (uint32_t *)(base + o_load),
+                 (uint32_t *)(base + o_len), (uint16_t *)(base + o_sorted), (uint16_t *)(base + o_greedy),
+                 (uint8_t *)(base + o_steps), (uint32_t *)(base + o_total), (uint16_t *)(base + o_quad),
+                 (uint8_t *)(base + o_deg), f->sched[s], f->meta[s]};
   return HUB_OK;
 }
 
-// Tables of the plan: entry lists, coefficients and diagonal.
+// Tables of the plan, entry lists of the spins: enqueued on the legacy stream, to be waited for
+// (fix_tables_wait) before the first launch that reads them.
 static int fix_tables(hub_ctx *h, FixState *f, const FixPlan &p) {
-  if (!f->lists_ready) {
-    for (int s = 0; s < (h->shared ? 1 : 2); ++s) {
-      const SpinCSR &c = h->csr[s];
-      const i64 nnz = c.nnz, n = h->count[s];
-      if (p.gather[s]) {
-        const int rc = gather_tables(f, s, (int)n, c);
-        if (rc) return rc;
-        continue;
-      }
-      if ((!f->cnt[s] && !dev_alloc((void **)&f->cnt[s], sizeof(uint32_t) * n, "hopping entry counts")) ||
-          (!f->word[s] && !dev_alloc((void **)&f->word[s], sizeof(uint32_t) * (nnz + 32), "hopping entries")))
-        return HUB_ERR_OOM;
-      HUB_CUDA(cudaMemset(f->word[s], 0, sizeof(uint32_t) * (nnz + 32)));
-      k_fix_lists<<<grid_of(n), 256>>>(n, c.rowptr, c.scol, f->cnt[s], f->word[s]);
-      HUB_LAUNCH_CHECK();
+  if (f->lists_ready) return HUB_OK;
+  SchedArgs A{};
+  int gathers = 0, groups = 0, segs = 0;
+  for (int s = 0; s < (h->shared ? 1 : 2); ++s) {
+    const SpinCSR &c = h->csr[s];
+    const i64 nnz = c.nnz, n = h->count[s];
+    if (p.gather[s]) {
+      const int rc = gather_arrays(f, s, (int)n, c, &A.spin[gathers]);
+      if (rc) return rc;
+      const SchedSpin &S = A.spin[gathers++];
+      groups = std::max(groups, S.groups);
+      segs = std::max(segs, (4 * S.groups + S.seg - 1) / S.seg);
+      continue;
     }
-    HUB_CUDA(cudaDeviceSynchronize());
-    f->lists_ready = true;
+    if ((!f->cnt[s] && !dev_alloc((void **)&f->cnt[s], sizeof(uint32_t) * n, "hopping entry counts")) ||
+        (!f->word[s] && !dev_alloc((void **)&f->word[s], sizeof(uint32_t) * (nnz + 32), "hopping entries")))
+      return HUB_ERR_OOM;
+    HUB_CUDA(cudaMemsetAsync(f->word[s], 0, sizeof(uint32_t) * (nnz + 32), nullptr));
+    k_fix_lists<<<grid_of(n), 256>>>(n, c.rowptr, c.scol, f->cnt[s], f->word[s]);
+    HUB_LAUNCH_CHECK();
   }
+  if (!gathers) return HUB_OK;
+  k_fix_quads<<<dim3((4 * groups + 15) / 16, gathers), 256>>>(A);
+  k_fix_sort<<<dim3((4 * groups + 255) / 256, gathers), 256>>>(A);
+  k_fix_group<<<dim3(segs, gathers), 32>>>(A);
+  k_fix_order<<<dim3(1, gathers), 1024>>>(A);
+  k_fix_schedule<<<dim3(groups, gathers), 32>>>(A);
+  HUB_LAUNCH_CHECK();
+  return HUB_OK;
+}
+static int fix_tables_wait(FixState *f) {
+  if (!f->lists_ready) HUB_CUDA(cudaStreamSynchronize(nullptr));
+  f->lists_ready = true;
   return HUB_OK;
 }
 
@@ -1687,6 +1776,7 @@ int fix_apply(hub_ctx *h, const double *x, double *y, cudaStream_t s) {
     f->cap = (int)std::min<i64>(std::max<i64>(D / 64, 1024), (i64)1 << 24);
     if (!dev_alloc((void **)&f->list, sizeof(i64) * f->cap, "entries to recompute")) return HUB_ERR_OOM;
   }
+  if ((rc = fix_tables_wait(f))) return rc;
   const int df_ok = use_fast(h) ? 1 : 0;
   if ((rc = plan_vector(h, f, x, D, df_ok, s))) return rc;
   // X: rows spin down (the caller's order); XT: rows spin up
@@ -1755,6 +1845,7 @@ int fix_lanczos(hub_ctx *h, const double *x0, int maxit, double tol, double *E0,
       (!f->ctl && !dev_alloc((void **)&f->ctl, sizeof(int) * kCtlWords, "product flags")))
     return HUB_ERR_OOM;
   if (!f->h_scal) HUB_CUDA(cudaMallocHost((void **)&f->h_scal, sizeof(FixScal)));
+  if ((rc = fix_tables_wait(f))) return rc;
   const int tb = (int)tile_blocks(h), ub = std::min(tb, kUpdateBlocks * num_sms());
   const int swap = F.a == 0;
   const bool st32 = small_tiles(h);

@@ -196,3 +196,26 @@ def test_short_of_memory(hub):
     E = hub.hub_lanczos_ground(m.h, x, 6, 0.0, y)[0]
     assert abs(E - E64) <= 1e-11 and not torch.equal(y, psi)
     m.close()
+
+
+@pytest.mark.parametrize("M,nu,nd", [(4, 4, 2), (6, 2, 3), (9, 4, 3), (11, 5, 2), (12, 6, 1), (16, 5, 1), (16, 8, 1),
+                                     (16, 1, 8)])
+@pytest.mark.parametrize("lattice", ["ring", "square"])
+def test_schedules_of_all_lengths(hub, M, nu, nd, lattice):
+    """Gather schedules from one position to 12,870: counts that are no multiple of a group, of a
+    slice or of a warp's share of the grouping, few and many quads, a long spin beside a short one."""
+    b = W.ring_bonds(M)
+    if lattice == "square":                      # longer rows, uneven ones
+        b = W.square_bonds(4, 4, True) if M == 16 else [(i, j) for i in range(M) for j in range(i + 1, M) if (i * j) % 3 != 1]
+    m = hub.Hubbard(M, nu, nd, b, 1.0, 4.0)
+    hub.hub_set_small_dim(m.h, 0)
+    x = torch.from_numpy(W.normal(9, m.D)).cuda()
+    steps = min(5, m.D)
+    a0, b0, p0 = _run(hub, m, x, steps)
+    hub.hub_set_mode(m.h, hub.HUB_MODE_FP64)
+    a1, b1, p1 = _run(hub, m, x, steps)
+    m.close()
+    k = min(len(a0), len(a1))
+    scale = max(np.abs(a1).max(), b1.max(), 1.0)
+    assert np.abs(a0[:k] - a1[:k]).max() <= 1e-12 * scale and np.abs(b0[:k] - b1[:k]).max() <= 1e-12 * scale
+    assert float((p0 - p1).norm()) <= 1e-10
