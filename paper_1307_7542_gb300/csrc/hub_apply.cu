@@ -43,7 +43,8 @@ __device__ __forceinline__ double f64_diag(const Ham &H, const double *s_U, uint
 template <int kMode, int kF64Rows>
 __global__ void __launch_bounds__(256, 6) k_apply_f64(const Ham H, const double *__restrict__ x, double *y,
                                                    const int *__restrict__ gate, int chunks, const F64Step L) {
-  if (gate && gate[0] == 0) return;
+  after_previous();
+  if (gate && flag_of(gate) == 0) return;
   // Sums of U_i over the set bits of each eight sites, from those of each four; only where U varies, since
   // the L1 that serves the gathers shrinks by it (uniform U, 17-site ring (7,2): 0.105 ms, with 9 KB 0.117).
   extern __shared__ double s_tab[];
@@ -192,10 +193,11 @@ static int f64_launch(hub_ctx *h, const double *x, double *y, const int *gate, c
   const int chunks = f64_chunks(H);
   const int64_t width = (H.n_up + chunks - 1) / chunks;
   const int threads = width > 128 ? 256 : (width > 64 ? 128 : 64);
-  const int grid = (int)f64_grid(H);
+  // behind the other paths' kernels (gate) it has nothing to do as a rule: no more CTAs than are resident
+  const int grid = (int)(gate ? std::min<int64_t>(f64_grid(H), (int64_t)num_sms() * 6) : f64_grid(H));
   const size_t tab = H.uniform_U ? 0 : sizeof(double) * (128 + (size_t)(H.M + 7) / 8 * 256);
-  (f64_rows(H) == 1 ? k_apply_f64<kMode, 1> : k_apply_f64<kMode, 2>)<<<grid, threads, tab, s>>>(H, x, y, gate, chunks, L);
-  HUB_LAUNCH_CHECK();
+  HUB_CUDA(launch_kernel(gate && !h->prof, f64_rows(H) == 1 ? k_apply_f64<kMode, 1> : k_apply_f64<kMode, 2>, grid,
+                         threads, tab, s, H, x, y, gate, chunks, L));
   return HUB_OK;
 }
 int f64_apply(hub_ctx *h, const double *x, double *y, const int *gate, cudaStream_t s) {

@@ -264,7 +264,8 @@ __global__ void k_scale_all(const int *__restrict__ partials, int nblk, int n_se
 __global__ void k_f64_to_df(int64_t r0, int64_t r1, int64_t n_up, int64_t ld, const double *__restrict__ x,
                             const int *__restrict__ scale, const int32_t *__restrict__ slot_row,
                             float *__restrict__ out, const int *__restrict__ gate) {
-  if (gate && gate[0] == 0) return;
+  after_previous();
+  if (gate && flag_of(gate) == 0) return;
   const int shift = scale ? scale[0] : 0;
   for (int64_t d = r0 + blockIdx.x; d < r1; d += gridDim.x) {
     float *__restrict__ row = out + d * 2 * ld;
@@ -284,7 +285,8 @@ __global__ void k_f64_to_df(int64_t r0, int64_t r1, int64_t n_up, int64_t ld, co
 __global__ void k_unpermute(int64_t r0, int64_t r1, int64_t n_up, int64_t ld, const float *__restrict__ v,
                             const int32_t *__restrict__ slot_of, const int *__restrict__ scale, double tabs,
                             double *__restrict__ y, const int *__restrict__ gate) {
-  if (scale[1] || (gate && gate[0] == 0)) return;
+  after_previous();
+  if (flag_of(scale + 1) || (gate && flag_of(gate) == 0)) return;
   const int shift = scale[0];
   for (int64_t d = r0 + blockIdx.x; d < r1; d += gridDim.x) {
     const float *__restrict__ row = v + d * 2 * ld;
@@ -324,7 +326,8 @@ static_assert(kUpThreads % 32 == 0 && kUpThreads >= 512 && kUpThreads <= 1024, "
 template <typename Col>
 __global__ void __launch_bounds__(kUpThreads, 1) k_up(const FastView F, const float *__restrict__ x,
                                                       float *__restrict__ z, int64_t p_begin, int64_t p_end) {
-  if (F.gate && F.gate[0] == 0) return;
+  after_previous();
+  if (F.gate && flag_of(F.gate) == 0) return;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float *xs = reinterpret_cast<float *>(smem_raw);
   __shared__ __align__(8) uint64_t bar;
@@ -511,7 +514,8 @@ constexpr int kTile = 32;
 __global__ void __launch_bounds__(256) k_transpose(int64_t n_r, int64_t n_c, int64_t ld_s, int64_t ld_d,
                                                    const float *__restrict__ src, float *__restrict__ dst,
                                                    const int *__restrict__ gate) {
-  if (gate && gate[0] == 0) return;
+  after_previous();
+  if (gate && flag_of(gate) == 0) return;
   __shared__ float th[kTile][kTile + 1], tl[kTile][kTile + 1];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int64_t c0 = (int64_t)blockIdx.x * kTile, r0 = (int64_t)blockIdx.y * kTile;
@@ -660,7 +664,8 @@ __device__ __forceinline__ void dn_group(DfSumP (&acc)[kLane], const Side &S, co
 template <typename Col, int kMode>
 __global__ void __launch_bounds__(kDnThreads, HUB_DN_MINB) k_dn(const FastView F, const Side S, const float *__restrict__ x,
                                                   const float *z, float *w) {
-  if (F.gate && F.gate[0] == 0) return;
+  after_previous();
+  if (F.gate && flag_of(F.gate) == 0) return;
   constexpr int kLane = kDnLaneCols / 2;               // packed pairs per lane
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t ld = S.ld;
@@ -1107,27 +1112,27 @@ static dim3 dn_grid(const Side &S) {
 }
 
 template <typename Col, int kMode>
-static int launch_dn_t(const FastView &v, const Side &S, const float *x, const float *z, float *w, cudaStream_t s) {
+static int launch_dn_t(const FastView &v, const Side &S, const float *x, const float *z, float *w, bool chained,
+                       cudaStream_t s) {
   const dim3 g = dn_grid(S);
   if (g.y > 65535) return fail(HUB_ERR_ARG, "fast apply: too many column strips");
-  k_dn<Col, kMode><<<g, kDnThreads, 0, s>>>(v, S, x, z, w);
-  HUB_LAUNCH_CHECK();
+  HUB_CUDA(launch_kernel(chained, k_dn<Col, kMode>, g, kDnThreads, 0, s, v, S, x, z, w));
   return HUB_OK;
 }
 
 template <int kMode>
 static int launch_dn(const FastState *f, const FastView &v, const Side &S, const float *x, const float *z, float *w,
-                     cudaStream_t s) {
-  return f->col16 ? launch_dn_t<uint16_t, kMode>(v, S, x, z, w, s) : launch_dn_t<uint32_t, kMode>(v, S, x, z, w, s);
+                     bool chained, cudaStream_t s) {
+  return f->col16 ? launch_dn_t<uint16_t, kMode>(v, S, x, z, w, chained, s)
+                  : launch_dn_t<uint32_t, kMode>(v, S, x, z, w, chained, s);
 }
 
 // dst = src^T for planar matrices (see k_transpose)
 static int transpose(int64_t n_r, int64_t n_c, int64_t ld_s, int64_t ld_d, const float *src, float *dst,
-                     const int *gate, cudaStream_t s) {
+                     const int *gate, bool chained, cudaStream_t s) {
   const dim3 g((unsigned)((n_c + kTile - 1) / kTile), (unsigned)((ld_d + kTile - 1) / kTile));
   if (g.y > 65535) return fail(HUB_ERR_ARG, "fast apply: matrix too large to transpose");
-  k_transpose<<<g, dim3(kTile, 8), 0, s>>>(n_r, n_c, ld_s, ld_d, src, dst, gate);
-  HUB_LAUNCH_CHECK();
+  HUB_CUDA(launch_kernel(chained, k_transpose, g, dim3(kTile, 8), 0, s, n_r, n_c, ld_s, ld_d, src, dst, gate));
   return HUB_OK;
 }
 
@@ -1139,6 +1144,7 @@ static int64_t scratch_floats(const hub_ctx *h, const FastState *f);
 static int run_up(hub_ctx *h, FastState *f, const float *x, float *z, cudaStream_t s, int64_t p0 = 0, int64_t p1 = -1,
                   const int *gate = nullptr) {
   const FastView v = fast_view(h, f, gate);
+  const bool chained = gate && !h->prof;
   if (p1 < 0) p1 = (v.n_dn + 1) / 2;
   if (!f->staged && (p0 != 0 || p1 != (v.n_dn + 1) / 2)) return fail(HUB_ERR_STATE, "pass 1: partial range");
   if (p1 <= p0) return HUB_OK;
@@ -1152,18 +1158,17 @@ static int run_up(hub_ctx *h, FastState *f, const float *x, float *z, cudaStream
 #define HUB_UP(C)                                                                                          \
   do {                                                                                                     \
     HUB_CUDA(cudaFuncSetAttribute(k_up<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxStage));  \
-    k_up<C><<<grid, threads, smem, s>>>(v, x, z, p0, p1);                                                  \
+    HUB_CUDA(launch_kernel(chained, k_up<C>, grid, threads, smem, s, v, x, z, p0, p1));                     \
   } while (0)
     if (f->col16) HUB_UP(uint16_t); else HUB_UP(uint32_t);
 #undef HUB_UP
-    HUB_LAUNCH_CHECK();
   } else {
     const int64_t Dt = scratch_floats(h, f);   // also fast_scratch's, which takes them as they are
     if ((rc = ensure_vec(&f->xt, Dt, "transposed x")) || (rc = ensure_vec(&f->zt, Dt, "transposed z"))) return rc;
     count_launch(h, 3);
-    if ((rc = transpose(h->count[1], h->count[0], f->ld, f->ld_t, x, f->xt, gate, s))) return rc;
-    if ((rc = launch_dn<2>(f, v, side_up(h, f), f->xt, nullptr, f->zt, s))) return rc;
-    if ((rc = transpose(h->count[0], h->count[1], f->ld_t, f->ld, f->zt, z, gate, s))) return rc;
+    if ((rc = transpose(h->count[1], h->count[0], f->ld, f->ld_t, x, f->xt, gate, chained, s))) return rc;
+    if ((rc = launch_dn<2>(f, v, side_up(h, f), f->xt, nullptr, f->zt, chained, s))) return rc;
+    if ((rc = transpose(h->count[0], h->count[1], f->ld_t, f->ld, f->zt, z, gate, chained, s))) return rc;
   }
   return prof_mark(h, HUB_PROF_UP, false, s);
 }
@@ -1179,7 +1184,7 @@ static int run_dn(hub_ctx *h, FastState *f, const float *x, const float *z, floa
   S.r_begin = r0;
   if (r1 >= 0) S.n_rows = r1;
   if (S.n_rows <= S.r_begin) return prof_mark(h, HUB_PROF_DN, false, s);
-  if ((rc = launch_dn<0>(f, v, S, x, z, w, s))) return rc;
+  if ((rc = launch_dn<0>(f, v, S, x, z, w, gate && !h->prof, s))) return rc;
   return prof_mark(h, HUB_PROF_DN, false, s);
 }
 
@@ -1213,7 +1218,7 @@ int fast_scratch(hub_ctx *h, int n, float **v) {
   return HUB_OK;
 }
 
-int fast_exp_range(hub_ctx *h, const double *x, int64_t D, int **part, int *nblk, cudaStream_t s) {
+static int fast_exp_range(hub_ctx *h, const double *x, int64_t D, int **part, int *nblk, cudaStream_t s) {
   FastState *f = fast_of(h);
   *nblk = grid_vec();
   if (!(*part = range_buf(f))) return HUB_ERR_OOM;
@@ -1238,14 +1243,14 @@ static int df_apply(hub_ctx *h, FastState *f, const double *x, double *y, const 
                     cudaStream_t s) {
   int rc;
   count_launch(h);
-  k_f64_to_df<<<row_grid(h), 256, 0, s>>>(0, h->count[1], h->count[0], f->ld, x, scale, f->slot_row, f->xdf, gate);
-  HUB_LAUNCH_CHECK();
+  const bool chained = gate && !h->prof;
+  HUB_CUDA(launch_kernel(chained, k_f64_to_df, row_grid(h), 256, 0, s, 0, h->count[1], h->count[0], f->ld, x, scale,
+                         f->slot_row, f->xdf, gate));
   if ((rc = run_up(h, f, f->xdf, f->zdf, s, 0, -1, gate))) return rc;
   if ((rc = run_dn(h, f, f->xdf, f->zdf, f->zdf, s, 0, -1, gate))) return rc;
   count_launch(h);
-  k_unpermute<<<row_grid(h), 512, 0, s>>>(0, h->count[1], h->count[0], f->ld, f->zdf, f->slot_of, scale,
-                                          std::fabs(h->t[0]), y, gate);
-  HUB_LAUNCH_CHECK();
+  HUB_CUDA(launch_kernel(chained, k_unpermute, row_grid(h), 512, 0, s, 0, h->count[1], h->count[0], f->ld, f->zdf,
+                         f->slot_of, scale, std::fabs(h->t[0]), y, gate));
   return HUB_OK;
 }
 

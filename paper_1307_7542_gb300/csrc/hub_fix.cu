@@ -114,6 +114,7 @@ struct FixPass {
   int t_neg;                          // uniform t < 0: the sums change sign
   int *err;                           // device error flag
   int fail_waits;                     // test hook
+  int chained;                        // launch_kernel's
   const int *skip;                    // apply: device flag, nothing to do
   u64 *acc;                           // Lanczos: dot product and maximum into these slots
   struct FixScal *scal;               // Lanczos, second pass of a step: its last block ends the step
@@ -245,55 +246,91 @@ __device__ __forceinline__ double fix_to_f64(i64 v, int e) {
   return __longlong_as_double((i64)(sign | (((u64)(unsigned)(E - 1) << 52) + r)));
 }
 
+// True in exactly one block, the last to arrive; all slots are then complete.  Leaves the
+// ticket at zero.
+__device__ __forceinline__ bool last_block(unsigned *ticket) {
+  __shared__ bool last;
+  if (threadIdx.x < 32) __threadfence();     // the adding threads
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (last && threadIdx.x == 0) *ticket = 0;
+  return last;
+}
+
 // ---------------------------------------------------------------------------------------
-// Scale and route of a caller's vector.  partials: k_exp_range's, nblk maxima then nblk minima
-// of the biased exponents.  ctl[kCtlShift]: exponent of max |x|; [kCtlSkip]: not for this path;
-// [kCtlF64] / [kCtlDf]: the FP64 / double-float kernels multiply it instead.  A vector outside
-// the double-float window (kExp*) goes to FP64 as before.  `wide` vectors -- more than one in
-// eight of 4096 sampled entries below 2^-8 of the largest -- would fill the list of entries to
-// recompute; random numbers have 2 % there (max 6 sigma), a ground state of the 12-site ring
-// 40 % and more.  Only time depends on the sample: the list catches what it misses.
+// Scale and route of a caller's vector, from the range of its exponents.  ctl[kCtlShift]: exponent of
+// max |x|; [kCtlSkip]: not for this path; [kCtlF64] / [kCtlDf]: the FP64 / double-float kernels
+// multiply it instead.  A vector outside the double-float window (kExp*) goes to FP64 as before.
+// `wide` vectors -- more than one in eight of 4096 sampled entries below 2^-8 of the largest -- would
+// fill the list of entries to recompute; random numbers have 2 % there (max 6 sigma), a ground
+// state of the 12-site ring 40 % and more.  Only time depends on the sample: the list catches what
+// it misses.  The last block to finish decides; it leaves the ticket at zero.
 // ---------------------------------------------------------------------------------------
 constexpr int kPlanThreads = 256, kPlanSamples = 4096;
-__global__ void k_fix_plan(const int *__restrict__ partials, int nblk, i64 D, const double *__restrict__ x, int df_ok,
-                           int *__restrict__ ctl) {
-  __shared__ int smax, smin, small;
-  if (threadIdx.x == 0) {
-    smax = 0;
-    smin = 2048;
-    small = 0;
-  }
-  __syncthreads();
+struct FixRange {                     // what the blocks hand to the last one
+  unsigned ticket;
+  uint16_t sample[kPlanSamples];      // exponents of every D / kPlanSamples-th entry (0: none)
+  int part[1];                        // largest exponent, then smallest one, of each block
+};
+__global__ void __launch_bounds__(kPlanThreads) k_fix_plan(i64 D, const double *__restrict__ x, int df_ok,
+                                                           FixRange *__restrict__ R, int *__restrict__ ctl) {
+  __shared__ int wmax[kPlanThreads / 32], wmin[kPlanThreads / 32], sum;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nblk = gridDim.x;
+  const i64 first = blockIdx.x * (i64)kPlanThreads + tid, step = D > kPlanSamples ? D / kPlanSamples : 1;
+  if (first < kPlanSamples)
+    R->sample[first] = first * step < D ? (uint16_t)(((u64)__double_as_longlong(x[first * step]) >> 52) & 0x7ff) : 0;
   int a = 0, c = 2048;
-  for (int k = threadIdx.x; k < nblk; k += blockDim.x) {
-    a = max(a, partials[k]);
-    c = min(c, partials[nblk + k]);
-  }
-  atomicMax(&smax, a);
-  atomicMin(&smin, c);
-  __syncthreads();
-  const int emax = smax, emin = smin;
-  int n = 0;
-  {
-    const i64 step = D > kPlanSamples ? D / kPlanSamples : 1;
-    for (int k = threadIdx.x; k < kPlanSamples; k += blockDim.x) {
-      const i64 at = k * step;
-      if (at < D) n += (int)(((u64)__double_as_longlong(x[at]) >> 52) & 0x7ff) < emax - 8 ? 1 : 0;
+  auto across = [&]() {               // the block's range, in every thread
+    a = __reduce_max_sync(0xffffffffu, a);
+    c = __reduce_min_sync(0xffffffffu, c);
+    if (lane == 0) {
+      wmax[warp] = a;
+      wmin[warp] = c;
     }
-    atomicAdd(&small, n);
+    __syncthreads();
+    for (int k = 0; k < kPlanThreads / 32; ++k) {
+      a = max(a, wmax[k]);
+      c = min(c, wmin[k]);
+    }
+  };
+  for (i64 k = first; k < D; k += (i64)nblk * kPlanThreads) {
+    const u64 b = (u64)__double_as_longlong(x[k]);
+    const int e = (int)((b >> 52) & 0x7ff);
+    a = max(a, e);
+    if (b << 1) c = min(c, e);
+  }
+  across();
+  if (tid == 0) {
+    R->part[blockIdx.x] = a;
+    R->part[nblk + blockIdx.x] = c;
+    sum = 0;
+  }
+  __threadfence();                    // the samples are every thread's
+  if (!last_block(&R->ticket)) return;
+  __threadfence();
+  a = 0;
+  c = 2048;
+  for (int k = tid; k < nblk; k += kPlanThreads) {
+    a = max(a, __ldcg(R->part + k));
+    c = min(c, __ldcg(R->part + nblk + k));
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const bool out = emax != 0 && (emax < kExpLo || emax > kExpHi || emin < emax - kExpSpan);
-    const i64 samples = D < kPlanSamples ? D : kPlanSamples;
-    const bool wide = emax == 0 || 8 * (i64)small > samples;
-    ctl[kCtlShift] = ctl[kCtlDfScale] = emax == 0 ? 0 : emax - 1023;
-    ctl[kCtlDfScale + 1] = 0;
-    ctl[kCtlSkip] = out || wide ? 1 : 0;
-    *count_of(ctl) = 0;
-    ctl[kCtlDf] = !out && wide && df_ok ? 1 : 0;
-    ctl[kCtlF64] = out || (wide && !df_ok) ? 1 : 0;
-  }
+  across();
+  int n = 0;
+  const int samples = (int)min(D, (i64)kPlanSamples);
+  for (int k = tid; k < samples; k += kPlanThreads) n += __ldcg(R->sample + k) < a - 8 ? 1 : 0;
+  atomicAdd(&sum, n);
+  __syncthreads();
+  if (tid != 0) return;
+  const bool out = a != 0 && (a < kExpLo || a > kExpHi || c < a - kExpSpan);
+  const bool wide = a == 0 || 8 * sum > samples;
+  ctl[kCtlShift] = ctl[kCtlDfScale] = a == 0 ? 0 : a - 1023;
+  ctl[kCtlDfScale + 1] = 0;
+  ctl[kCtlSkip] = out || wide ? 1 : 0;
+  *count_of(ctl) = 0;
+  ctl[kCtlDf] = !out && wide && df_ok ? 1 : 0;
+  ctl[kCtlF64] = out || (wide && !df_ok) ? 1 : 0;
 }
 
 // A thread's sums (N = 4: one dot product, 8: two) into the block's slot; vmax (top word of the
@@ -318,18 +355,6 @@ __device__ __forceinline__ void block_sums(i64 (&v)[N], unsigned vmax, int which
     vmax = __reduce_max_sync(0xffffffffu, lane < nw ? sm[lane] : 0u);
     if (lane == 0) atomicMax(slot + 4 + which, (u64)vmax);
   }
-}
-
-// True in exactly one block, the last to arrive; all slots are then complete.  Leaves the
-// ticket at zero.
-__device__ __forceinline__ bool last_block(unsigned *ticket) {
-  __shared__ bool last;
-  if (threadIdx.x < 32) __threadfence();     // the adding threads
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (last && threadIdx.x == 0) *ticket = 0;
-  return last;
 }
 
 // hh 2^56 + mid 2^28 of summed halves as a double, exact to 2^-53 of the total
@@ -464,7 +489,8 @@ __global__ void __launch_bounds__(1024, 1) k_fix_gather(const FixPass P, const G
   int2 *const x0 = reinterpret_cast<int2 *>(smem), *const x1 = x0 + kPlane;   // entries ld .. ld + 15 are zero
   __shared__ __align__(8) uint64_t bar;
   __shared__ i64 utab[32];
-  if (P.skip && __ldg(P.skip)) return;
+  after_previous();
+  if (P.skip && flag_of(P.skip)) return;
   const int tid = threadIdx.x, lane = tid & 31;
   if (tid < 32) {
     utab[tid] = P.diag.tab[tid];
@@ -939,7 +965,8 @@ template <bool kLz>
 __global__ void __launch_bounds__(kCombThreads, 2) k_fix_comb(const FixPass P, const CombLists S) {
   constexpr int kWarps = kCombThreads / 32;
   __shared__ i64 utab[32];
-  if (P.skip && __ldg(P.skip)) return;
+  after_previous();
+  if (P.skip && flag_of(P.skip)) return;
   if (P.fail_waits) {                       // test hook: report as a given-up wait would
     if (threadIdx.x == 0) atomicExch(P.err, 1);
     return;
@@ -1073,6 +1100,10 @@ __device__ __forceinline__ void tile_at(uint32_t tile, i64 n_c, i64 *r0, i64 *c0
   *c0 = (i64)(tile - by * tx) * T;
   *r0 = (i64)by * T;
 }
+template <int T>
+__device__ __forceinline__ uint32_t tiles_of(i64 n_r, i64 n_c) {      // below 2^31 (fix_fits)
+  return (uint32_t)(((n_c + T - 1) / T) * ((n_r + T - 1) / T));
+}
 __device__ __forceinline__ double2 ld_two(const double *p, bool vec, bool second) {
   if (vec) return *reinterpret_cast<const double2 *>(p);
   return make_double2(p[0], second ? p[1] : 0.0);
@@ -1086,48 +1117,51 @@ __global__ void __launch_bounds__(kTileThreads) k_fix_in(i64 n_r, i64 n_c, i64 l
                                                          int use_skip, int B, i64 *__restrict__ X,
                                                          i64 *__restrict__ XT, u64 *__restrict__ acc) {
   __shared__ TileBuf<T> t;
-  if (use_skip && __ldg(ctl + kCtlSkip)) return;
+  after_previous();
+  if (use_skip && flag_of(ctl + kCtlSkip)) return;
   const int e = ctl[kCtlShift] - (B - 2);
-  i64 r0, c0;
-  tile_at<T>(blockIdx.x, n_c, &r0, &c0);
   const TileAt<T> at;
-  const i64 u = c0 + at.c;
-  const bool in = u < n_c, second = u + 1 < n_c;
   const bool vec = (n_c & 1) == 0 && ((uintptr_t)x & 15) == 0;
   constexpr int kN = T / TileAt<T>::kStep;
-  double2 xv[kN];
+  DotLong dots{{0, 0, 0, 0}};
+  const uint32_t tiles = tiles_of<T>(n_r, n_c);
+  for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    i64 r0, c0;
+    tile_at<T>(tile, n_c, &r0, &c0);
+    const i64 u = c0 + at.c;
+    const bool in = u < n_c, second = u + 1 < n_c;
+    double2 xv[kN];
 #pragma unroll
-  for (int i = 0; i < kN; ++i) {
-    const i64 d = r0 + at.k0 + i * TileAt<T>::kStep;
-    xv[i] = make_double2(0.0, 0.0);
-    if (d < n_r && in) xv[i] = ld_two(x + d * n_c + u, vec, second);
-  }
-  Dot dot{0, 0};
-#pragma unroll
-  for (int i = 0; i < kN; ++i) {
-    const int k = at.k0 + i * TileAt<T>::kStep;
-    i64 v[2] = {f64_to_fix(xv[i].x, e), f64_to_fix(xv[i].y, e)};
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      if (acc) {
-        int h, l;
-        limbs28(v[j], h, l);
-        dot.square(h, l);
-      }
-      v[j] = fix_store<kLimb>(v[j]);
-      t.v[k][at.c + j] = v[j];
+    for (int i = 0; i < kN; ++i) {
+      const i64 d = r0 + at.k0 + i * TileAt<T>::kStep;
+      xv[i] = make_double2(0.0, 0.0);
+      if (d < n_r && in) xv[i] = ld_two(x + d * n_c + u, vec, second);
     }
-    if (X && r0 + k < n_r && in) *reinterpret_cast<longlong2 *>(X + (r0 + k) * ld + u) = make_longlong2(v[0], v[1]);
-  }
-  if (XT) {
-    __syncthreads();
-    tile_out_t<T>(t, XT, ldt, r0, c0, n_r, n_c);
-  }
-  if (acc) {
-    DotLong dots{{0, 0, 0, 0}};
+    if (XT && tile != blockIdx.x) __syncthreads();        // the tile before has been written out
+    Dot dot{0, 0};
+#pragma unroll
+    for (int i = 0; i < kN; ++i) {
+      const int k = at.k0 + i * TileAt<T>::kStep;
+      i64 v[2] = {f64_to_fix(xv[i].x, e), f64_to_fix(xv[i].y, e)};
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        if (acc) {
+          int h, l;
+          limbs28(v[j], h, l);
+          dot.square(h, l);
+        }
+        v[j] = fix_store<kLimb>(v[j]);
+        t.v[k][at.c + j] = v[j];
+      }
+      if (X && r0 + k < n_r && in) *reinterpret_cast<longlong2 *>(X + (r0 + k) * ld + u) = make_longlong2(v[0], v[1]);
+    }
+    if (XT) {
+      __syncthreads();
+      tile_out_t<T>(t, XT, ldt, r0, c0, n_r, n_c);
+    }
     dots.take(dot);
-    block_sums<4>(dots.v, 0u, 0, acc);
   }
+  if (acc) block_sums<4>(dots.v, 0u, 0, acc);
 }
 
 // Scalars of a Lanczos start: |S_1|^2 from k_fix_in's slots.
@@ -1175,7 +1209,7 @@ __global__ void __launch_bounds__(kTileThreads, kUpdateBlocks) k_fix_update(i64 
   unsigned vmax = 0;
   const TileAt<T> at;
   const int c = at.c;
-  const uint32_t tiles = (uint32_t)(((n_c + T - 1) / T) * ((n_r + T - 1) / T));   // below 2^31 (fix_fits)
+  const uint32_t tiles = tiles_of<T>(n_r, n_c);
   for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     i64 r0, c0;
     tile_at<T>(tile, n_c, &r0, &c0);
@@ -1321,48 +1355,53 @@ __global__ void __launch_bounds__(kTileThreads, kUpdateBlocks) k_fix_out(i64 n_r
   static_assert(T == 32 || !(kAt && kBt), "two tiles in 48 KB");
   __shared__ TileBuf<T> t;
   __shared__ TileBuf<kAt && kBt ? T : 2> t2;
-  if (ctl[kCtlSkip]) return;
+  after_previous();
+  if (flag_of(ctl + kCtlSkip)) return;
   const int e = ctl[kCtlShift] + eg;
-  i64 r0, c0;
-  tile_at<T>(blockIdx.x, n_c, &r0, &c0);
   const TileAt<T> at;
-  const i64 u = c0 + at.c;
-  const bool second = u + 1 < n_c;
   const bool vec = (n_c & 1) == 0 && ((uintptr_t)y & 15) == 0;
-  if (kBt) tile_in_t<T>(t, b, ldt, r0, c0, n_r, n_c);
-  if constexpr (kAt && kBt)
-    tile_in_t<T>(t2, a, ldt, r0, c0, n_r, n_c);
-  else if (kAt)
-    tile_in_t<T>(t, a, ldt, r0, c0, n_r, n_c);
-  if (kAt || kBt) __syncthreads();
-#pragma unroll 1
-  for (int k = at.k0; k < T; k += TileAt<T>::kStep) {
-    const i64 d = r0 + k;
-    if (d >= n_r || u >= n_c) continue;
-    longlong2 va;
+  const uint32_t tiles = tiles_of<T>(n_r, n_c);
+  for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    i64 r0, c0;
+    tile_at<T>(tile, n_c, &r0, &c0);
+    const i64 u = c0 + at.c;
+    const bool second = u + 1 < n_c;
+    if ((kAt || kBt) && tile != blockIdx.x) __syncthreads();          // the tile before has been read
+    if (kBt) tile_in_t<T>(t, b, ldt, r0, c0, n_r, n_c);
     if constexpr (kAt && kBt)
-      va = make_longlong2(t2.v[k][at.c], t2.v[k][at.c + 1]);
-    else
-      va = kAt ? make_longlong2(t.v[k][at.c], t.v[k][at.c + 1]) : *reinterpret_cast<const longlong2 *>(a + d * ld + u);
-    const longlong2 vb = kBt ? make_longlong2(t.v[k][at.c], t.v[k][at.c + 1])
-                             : *reinterpret_cast<const longlong2 *>(b + d * ld + u);
-    const i64 n = d * n_c + u;
-    const i64 s0[2] = {va.x, va.y}, s1[2] = {vb.x, vb.y};
-    double v[2];
+      tile_in_t<T>(t2, a, ldt, r0, c0, n_r, n_c);
+    else if (kAt)
+      tile_in_t<T>(t, a, ldt, r0, c0, n_r, n_c);
+    if (kAt || kBt) __syncthreads();
+#pragma unroll 1
+    for (int k = at.k0; k < T; k += TileAt<T>::kStep) {
+      const i64 d = r0 + k;
+      if (d >= n_r || u >= n_c) continue;
+      longlong2 va;
+      if constexpr (kAt && kBt)
+        va = make_longlong2(t2.v[k][at.c], t2.v[k][at.c + 1]);
+      else
+        va = kAt ? make_longlong2(t.v[k][at.c], t.v[k][at.c + 1]) : *reinterpret_cast<const longlong2 *>(a + d * ld + u);
+      const longlong2 vb = kBt ? make_longlong2(t.v[k][at.c], t.v[k][at.c + 1])
+                               : *reinterpret_cast<const longlong2 *>(b + d * ld + u);
+      const i64 n = d * n_c + u;
+      const i64 s0[2] = {va.x, va.y}, s1[2] = {vb.x, vb.y};
+      double v[2];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      v[j] = fix_to_f64(s0[j] + s1[j], e);
-      if (tabs != 1.0) v[j] *= tabs;
-      if ((j == 0 || second) && llabs(s0[j]) + llabs(s1[j]) < thr) {
-        const u64 at_list = atomicAdd(count_of(ctl), 1ull);
-        if (at_list < (u64)cap) list[at_list] = n + j;
+      for (int j = 0; j < 2; ++j) {
+        v[j] = fix_to_f64(s0[j] + s1[j], e);
+        if (tabs != 1.0) v[j] *= tabs;
+        if ((j == 0 || second) && llabs(s0[j]) + llabs(s1[j]) < thr) {
+          const u64 at_list = atomicAdd(count_of(ctl), 1ull);
+          if (at_list < (u64)cap) list[at_list] = n + j;
+        }
       }
-    }
-    if (vec) {
-      *reinterpret_cast<double2 *>(y + n) = make_double2(v[0], v[1]);
-    } else {
-      y[n] = v[0];
-      if (second) y[n + 1] = v[1];
+      if (vec) {
+        *reinterpret_cast<double2 *>(y + n) = make_double2(v[0], v[1]);
+      } else {
+        y[n] = v[0];
+        if (second) y[n + 1] = v[1];
+      }
     }
   }
 }
@@ -1386,7 +1425,8 @@ __global__ void k_fix_axpy(i64 n_r, i64 n_c, i64 ld, const i64 *__restrict__ cur
 __global__ void __launch_bounds__(256) k_fix_entries(const Ham H, const double *__restrict__ x, double *__restrict__ y,
                                                      int *__restrict__ ctl, const i64 *__restrict__ list, int cap,
                                                      int df_ok) {
-  if (ctl[kCtlSkip]) return;
+  after_previous();
+  if (flag_of(ctl + kCtlSkip)) return;
   const u64 all = *count_of(ctl);
   const int n = (int)min(all, (u64)cap);
   if (all > (u64)cap) {
@@ -1441,6 +1481,7 @@ struct FixState {
   uint32_t *meta[2] = {nullptr, nullptr};
   int cap_steps[2] = {0, 0}, slices[2] = {0, 0};
   int *ctl = nullptr;
+  FixRange *range = nullptr;          // in ctl's allocation
   i64 *list = nullptr;
   int cap = 0;
   u64 *acc = nullptr;
@@ -1647,6 +1688,14 @@ static i64 tile_blocks(const hub_ctx *h, i64 T) {
   return ((h->count[0] + T - 1) / T) * ((h->count[1] + T - 1) / T);
 }
 static i64 tile_blocks(const hub_ctx *h) { return tile_blocks(h, small_tiles(h) ? 32 : 64); }
+// CTAs of the kernels that take tiles in turn: as many as are resident.  (One per tile cost 8 us where the
+// kernel finds nothing to do, 2916 CTAs, and 17 us with 7600.)
+static int in_blocks(const hub_ctx *h) {
+  return (int)std::min<i64>(tile_blocks(h), (i64)(small_tiles(h) ? 8 : 3) * num_sms());
+}
+static int out_blocks(const hub_ctx *h, i64 T) {
+  return (int)std::min<i64>(tile_blocks(h, T), (i64)kUpdateBlocks * num_sms());
+}
 // grids are one-dimensional, row strides in bytes 32-bit
 static bool fix_fits(const hub_ctx *h) {
   const i64 lim = ((i64)1 << 31) - 1;
@@ -1660,8 +1709,7 @@ static int launch_comb(const hub_ctx *h, const FixState *f, const FixPass &P, in
   const int t = h->shared ? 0 : a;
   CombLists L{tile_rows(P.n_rows, P.n_pos), h->csr[t].rowptr, f->cnt[t], f->word[t]};
   const int g = (int)comb_blocks(P.n_rows, P.n_pos);
-  (P.acc ? k_fix_comb<true> : k_fix_comb<false>)<<<g, kCombThreads, 0, s>>>(P, L);
-  HUB_LAUNCH_CHECK();
+  HUB_CUDA(launch_kernel(P.chained, P.acc ? k_fix_comb<true> : k_fix_comb<false>, g, kCombThreads, 0, s, P, L));
   return HUB_OK;
 }
 template <int kPlane, bool kLimb>
@@ -1673,8 +1721,7 @@ static int launch_gather_t(const FixPass &P, const GatherLists &L, cudaStream_t 
   const int grid = (int)std::min<i64>((P.n_rows + 1) / 2, per_sm * num_sms());
   const auto k = P.acc ? k_fix_gather<kPlane, true, kLimb> : k_fix_gather<kPlane, false, kLimb>;
   HUB_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k<<<grid, threads, smem, s>>>(P, L);
-  HUB_LAUNCH_CHECK();
+  HUB_CUDA(launch_kernel(P.chained, k, grid, threads, smem, s, P, L));
   return HUB_OK;
 }
 template <int kPlane>
@@ -1718,6 +1765,7 @@ static int fix_product(hub_ctx *h, FixState *f, const FixPlan &p, const FixShape
   P1.x = F.both ? ST : S;
   P1.out = out1;
   P0.skip = P1.skip = skip;
+  P0.chained = P1.chained = skip && !h->prof ? 1 : 0;
   if (lz) {
     P0.acc = P1.acc = f->acc;
     P0.scal = P1.scal = f->scal;
@@ -1739,13 +1787,17 @@ static int fix_product(hub_ctx *h, FixState *f, const FixPlan &p, const FixShape
   return HUB_OK;
 }
 
-// Scale and route words of x (k_exp_range's partials live with the double-float path)
+// Scale and route words of x
 static int plan_vector(hub_ctx *h, FixState *f, const double *x, i64 D, int df_ok, cudaStream_t s) {
-  int *part = nullptr, nblk = 0;
-  const int rc = fast_exp_range(h, x, D, &part, &nblk, s);
-  if (rc) return rc;
+  const int nblk = 4 * num_sms();
+  if (!f->ctl) {
+    const size_t words = 256;           // bytes, for the words and the padding behind them
+    if (!dev_alloc((void **)&f->ctl, words + sizeof(FixRange) + 2 * sizeof(int) * nblk, "product flags")) return HUB_ERR_OOM;
+    f->range = (FixRange *)((char *)f->ctl + words);
+    HUB_CUDA(cudaMemsetAsync(f->range, 0, sizeof(unsigned), s));
+  }
   count_launch(h);
-  k_fix_plan<<<1, kPlanThreads, 0, s>>>(part, nblk, D, x, df_ok, f->ctl);
+  k_fix_plan<<<nblk, kPlanThreads, 0, s>>>(D, x, df_ok, f->range, f->ctl);
   HUB_LAUNCH_CHECK();
   return HUB_OK;
 }
@@ -1771,7 +1823,6 @@ int fix_apply(hub_ctx *h, const double *x, double *y, cudaStream_t s) {
   const i64 n_up = h->count[0], n_dn = h->count[1], D = n_up * n_dn;
   float *buf[4] = {nullptr, nullptr, nullptr, nullptr};
   if ((rc = fast_scratch(h, scratch_vectors(p, F), buf))) return rc;
-  if (!f->ctl && !dev_alloc((void **)&f->ctl, sizeof(int) * kCtlWords, "product flags")) return HUB_ERR_OOM;
   if (!f->list) {
     f->cap = (int)std::min<i64>(std::max<i64>(D / 64, 1024), (i64)1 << 24);
     if (!dev_alloc((void **)&f->list, sizeof(i64) * f->cap, "entries to recompute")) return HUB_ERR_OOM;
@@ -1783,13 +1834,15 @@ int fix_apply(hub_ctx *h, const double *x, double *y, cudaStream_t s) {
   const bool cx = F.both || F.a == 1, ct = F.both || F.a == 0;
   i64 *X = (i64 *)buf[0], *XT = (i64 *)buf[1];
   const i64 ld = fix_ld(n_up), ldt = fix_ld(n_dn);
-  const int tb = (int)tile_blocks(h), *skip = f->ctl + kCtlSkip;
+  const int *skip = f->ctl + kCtlSkip;
   count_launch(h, 3);
   const bool st = small_tiles(h);
-  (p.limbs() ? (st ? k_fix_in<32, true> : k_fix_in<64, true>)
-             : (st ? k_fix_in<32, false> : k_fix_in<64, false>))<<<tb, kTileThreads, 0, s>>>(
-      n_dn, n_up, ld, ldt, x, f->ctl, 1, p.B, cx ? X : nullptr, ct ? XT : nullptr, nullptr);
-  HUB_LAUNCH_CHECK();
+  const bool chained = !h->prof;
+  HUB_CUDA(launch_kernel(chained,
+                         p.limbs() ? (st ? k_fix_in<32, true> : k_fix_in<64, true>)
+                                   : (st ? k_fix_in<32, false> : k_fix_in<64, false>),
+                         in_blocks(h), kTileThreads, 0, s, n_dn, n_up, ld, ldt, x, f->ctl, 1, p.B, cx ? X : nullptr,
+                         ct ? XT : nullptr, nullptr));
   i64 *in0 = F.a == 1 ? X : XT, *in1 = F.a == 1 ? XT : X, *out0 = in0, *out1 = in1;   // gathers: in place
   if (F.both && !p.gather[0]) {
     out0 = (i64 *)buf[2];
@@ -1798,9 +1851,9 @@ int fix_apply(hub_ctx *h, const double *x, double *y, cudaStream_t s) {
   if ((rc = fix_product(h, f, p, F, in0, in1, out0, out1, skip, false, s))) return rc;
   const i64 thr = ((i64)std::ceil(p.units * 1.25e13) >> p.g) + 1;   // |error| <= units 2^e <= 0.8e-13 thr 2^(e + g)
   const int eg = p.g - (p.B - 2);
-#define FIX_OUT(T, AT, BT)                                                                                      \
-  k_fix_out<T, AT, BT><<<(int)tile_blocks(h, T), kTileThreads, 0, s>>>(n_dn, n_up, ld, ldt, out0, out1, eg, thr, \
-                                                                       p.tau, f->ctl, f->list, f->cap, y)
+#define FIX_OUT(T, AT, BT)                                                                                   \
+  HUB_CUDA(launch_kernel(chained, k_fix_out<T, AT, BT>, out_blocks(h, T), kTileThreads, 0, s, n_dn, n_up, ld, \
+                         ldt, out0, out1, eg, thr, p.tau, f->ctl, f->list, f->cap, y))
   if (F.both && st)
     FIX_OUT(32, false, true);
   else if (F.both)
@@ -1810,9 +1863,8 @@ int fix_apply(hub_ctx *h, const double *x, double *y, cudaStream_t s) {
   else
     FIX_OUT(32, true, true);
 #undef FIX_OUT
-  HUB_LAUNCH_CHECK();
-  k_fix_entries<<<num_sms() * 4, 256, 0, s>>>(h->view(), x, y, f->ctl, f->list, f->cap, df_ok);
-  HUB_LAUNCH_CHECK();
+  HUB_CUDA(launch_kernel(chained, k_fix_entries, num_sms() * 4, 256, 0, s, h->view(), x, y, f->ctl, f->list, f->cap,
+                         df_ok));
   if (df_ok && (rc = fast_apply_gated(h, x, y, f->ctl + kCtlDfScale, f->ctl + kCtlDf, s))) return rc;
   return f64_apply(h, x, y, f->ctl + kCtlF64, s);
 }
@@ -1841,12 +1893,11 @@ int fix_lanczos(hub_ctx *h, const double *x0, int maxit, double tol, double *E0,
   for (int k = 0; k < 2; ++k)
     if (!f->vec[k] && !dev_alloc((void **)&f->vec[k], sizeof(i64) * n_r * ld, "Lanczos vector")) return HUB_ERR_OOM;
   if ((!f->acc && !dev_alloc((void **)&f->acc, sizeof(u64) * kFixSlots * kAcc, "Lanczos sums")) ||
-      (!f->scal && !dev_alloc((void **)&f->scal, sizeof(FixScal), "Lanczos scalars")) ||
-      (!f->ctl && !dev_alloc((void **)&f->ctl, sizeof(int) * kCtlWords, "product flags")))
+      (!f->scal && !dev_alloc((void **)&f->scal, sizeof(FixScal), "Lanczos scalars")))
     return HUB_ERR_OOM;
   if (!f->h_scal) HUB_CUDA(cudaMallocHost((void **)&f->h_scal, sizeof(FixScal)));
   if ((rc = fix_tables_wait(f))) return rc;
-  const int tb = (int)tile_blocks(h), ub = std::min(tb, kUpdateBlocks * num_sms());
+  const int ub = (int)std::min<i64>(tile_blocks(h), (i64)kUpdateBlocks * num_sms());
   const int swap = F.a == 0;
   const bool st32 = small_tiles(h);
 
@@ -1858,7 +1909,7 @@ int fix_lanczos(hub_ctx *h, const double *x0, int maxit, double tol, double *E0,
     HUB_CUDA(cudaMemsetAsync(f->acc, 0, sizeof(u64) * kFixSlots * kAcc, s));
     HUB_CUDA(cudaMemsetAsync(f->vec[1], 0, sizeof(i64) * n_r * ld, s));
     (p.limbs() ? (st32 ? k_fix_in<32, true> : k_fix_in<64, true>)
-               : (st32 ? k_fix_in<32, false> : k_fix_in<64, false>))<<<tb, kTileThreads, 0, s>>>(
+               : (st32 ? k_fix_in<32, false> : k_fix_in<64, false>))<<<in_blocks(h), kTileThreads, 0, s>>>(
         n_dn, n_up, fix_ld(n_up), fix_ld(n_dn), x0, f->ctl, 0, p.B, swap ? nullptr : f->vec[0],
         swap ? f->vec[0] : (F.both ? ST : nullptr), f->acc);
     HUB_LAUNCH_CHECK();

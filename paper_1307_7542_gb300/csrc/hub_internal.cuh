@@ -66,6 +66,35 @@ struct Ham {
   int has_eps;
 };
 
+// chained: a launch that need not wait for the kernel before it on the stream to drain; its blocks are
+// placed while that one ends, and wait (after_previous, the first thing such a kernel does) for its
+// results.  For rows of kernels of which most find on a device flag that there is nothing to do: a vector of
+// the 13-site ring (6,6) that goes to the double-float kernels takes 146 us with plain launches, 142 chained,
+// 115 chained with no more CTAs than are resident and with flags through L1 (120 in double-float alone).
+template <typename... P, typename... A>
+inline cudaError_t launch_kernel(bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                 cudaStream_t s, A... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &attr;
+  c.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A flag written by a kernel before this one, read after after_previous(): an ordinary load that the compiler
+// can neither move nor make a read-only one.  (A volatile one goes past L1: 5 us in a kernel of 20 us.)
+__device__ __forceinline__ int flag_of(const int *p) {
+  int v;
+  asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
 // Lane l of the warp: the warp's total of v[l % N].  Each of the first log2(N) exchanges sends one of
 // a pair and keeps the other, so that N totals take N + 4 - log2(N) shuffles instead of 5 N.
 template <int N, typename T>
@@ -259,8 +288,6 @@ int fast_apply_gated(hub_ctx *h, const double *x, double *y, const int *scale, c
 // The first n <= 4 scratch vectors of the handle, each large enough for a vector in either order.
 int fast_scratch(hub_ctx *h, int n, float **v);
 void fast_release_scratch(hub_ctx *h);
-// Largest and smallest biased exponents of x per block: part[0 .. nblk) and part[nblk .. 2 nblk).
-int fast_exp_range(hub_ctx *h, const double *x, int64_t D, int **part, int *nblk, cudaStream_t s);
 // The handle's device error flag.
 int *fast_err(const hub_ctx *h);
 int fast_check_error(hub_ctx *h);
