@@ -24,15 +24,16 @@
 // only shifts and two multiplications by a 55-bit coefficient are needed per entry, and the
 // dot products <s_j, H s_j>, <s_j, s_{j-1}> and |s_{j+1}|^2 are integer sums (H s_j rounded to 7 bits
 // fewer, the product of the lowest limbs to their high part, and left out of <s_j, s_{j-1}>): no
-// result depends on the order in which blocks finish.  A run whose vectors' rms falls below 2^48 grid
-// units (start vectors with a largest entry above some 100 times the rms: a ground state with an
-// electron added, a single configuration) is left to the FP64 driver: double-float vectors kept 48
-// bits of every entry, and below that line the grid would keep fewer.  Random start vectors have a
-// largest entry of 6 rms, their Lanczos vectors of up to 90.  Against long double (12-site ring, 24 steps,
-// largest error of alpha; in brackets with double-float vectors): random start 3.6e-15 (3.9e-14) at U = 4,
-// 7.8e-15 (9.0e-14) at U = 7.25, all entries positive 2.5e-15 (4.3e-14), one entry of 64 rms 7.7e-15 (5.0e-14),
-// a ground state of largest entry 128 rms 3.9e-13 (2.2e-12); an electron added to it, 169 rms, 3.1e-13 (1.0e-13)
-// on the grid and now 1.0e-14.
+// result depends on the order in which blocks finish.  A rounding is 2^-57 of a vector's largest entry,
+// so that an entry of rms size keeps 53 bits of a random start vector, 46 after sixty steps at 4x4 half
+// filling, 45 to 41 of a 4x4 ground state with an electron added.  Its start vector uses the whole grid
+// (k_fix_plan).  Largest error of alpha over the first steps against long double (12-site ring, 24 steps;
+// in brackets with double-float vectors, which kept 48 bits of every entry): random start 3.7e-15
+// (3.9e-14) at U = 4, 5.4e-15 (9.0e-14) at U = 7.25, all entries positive 4.3e-15 (4.3e-14), one entry of
+// 400 rms 1.6e-14 (4.8e-14), one configuration 4.1e-15 (5.8e-14), a ground state 1.2e-13 (2.2e-12), an
+// electron added to it 8.2e-14 (1.0e-13), at U = 12 8.7e-14 (1.7e-13).  Against FP64 vectors, whose own
+// errors are of that size: 4x4 half filling, 60 steps, 1e-14 (9e-14) at U = 4, 4e-14 (3e-13) at U = 8;
+// an electron added, 20 steps, 4e-14 (7e-14).
 //
 // Products for a caller (hub_apply) must keep every entry within 1e-13 (|H||x|)_n, which a grid
 // fixed by the largest entry does not give where (|H||x|)_n is small.  k_fix_out sees the entry's
@@ -72,7 +73,7 @@ constexpr int kFixHist = 8;         // Lanczos steps recorded between two host r
 constexpr int kFixFrac = 4;         // fraction bits of the update's sums
 
 // ctl words of a product (device): see k_fix_plan
-enum { kCtlShift = 0, kCtlSkip = 1, kCtlDf = 2, kCtlF64 = 3, kCtlDfScale = 4, kCtlCount = 6, kCtlWords = 8 };
+enum { kCtlShift = 0, kCtlSkip = 1, kCtlDf = 2, kCtlF64 = 3, kCtlDfScale = 4, kCtlCount = 6, kCtlScale = 8, kCtlWords = 10 };
 // Entries to recompute: a 64-bit count over two words, since any number of a vector's entries may ask for it.
 __device__ __forceinline__ u64 *count_of(int *ctl) { return reinterpret_cast<u64 *>(ctl + kCtlCount); }
 
@@ -232,6 +233,18 @@ __device__ __forceinline__ i64 f64_to_fix(double x, int e) {
   return (b >> 63) ? -(i64)v : (i64)v;
 }
 
+// x c 2^-31 = X 2^e rounded to the nearest integer X, |X| < 2^57 (Lanczos start vectors: see k_fix_plan)
+__device__ __forceinline__ i64 f64_to_fix_scaled(double x, unsigned c, int e) {
+  const u64 b = (u64)__double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  if (ex == 0) return 0;
+  const u64 m = ((b & 0x000fffffffffffffull) | 0x0010000000000000ull) << 11;
+  const u64 p = __umul64hi(m, (u64)c << 32);             // x c 2^-31 = p 2^(ex - 1085)
+  const int r = e + 1085 - ex;                           // 7 and more
+  const u64 v = r > 64 ? 0ull : ((p >> (r - 1)) + 1) >> 1;
+  return (b >> 63) ? -(i64)v : (i64)v;
+}
+
 // v 2^e rounded to FP64 (results in the normal range)
 __device__ __forceinline__ double fix_to_f64(i64 v, int e) {
   if (v == 0) return 0.0;
@@ -265,13 +278,15 @@ __device__ __forceinline__ bool last_block(unsigned *ticket) {
 // `wide` vectors -- more than one in eight of 4096 sampled entries below 2^-8 of the largest -- would
 // fill the list of entries to recompute; random numbers have 2 % there (max 6 sigma), a ground
 // state of the 12-site ring 40 % and more.  Only time depends on the sample: the list catches what
-// it misses.  The last block to finish decides; it leaves the ticket at zero.
+// it misses.  [kCtlScale]: 2^31 times a factor, from just below 1 to 2, that takes max |x| to just below
+// the next power of two but one: a Lanczos run is free to scale its start vector, so that it uses the whole
+// grid.  The last block to finish decides; it leaves the ticket at zero.
 // ---------------------------------------------------------------------------------------
 constexpr int kPlanThreads = 256, kPlanSamples = 4096;
 struct FixRange {                     // what the blocks hand to the last one
   unsigned ticket;
   uint16_t sample[kPlanSamples];      // exponents of every D / kPlanSamples-th entry (0: none)
-  int part[1];                        // largest exponent, then smallest one, of each block
+  int part[1];                        // top word of the largest magnitude, then smallest exponent, of each block
 };
 __global__ void __launch_bounds__(kPlanThreads) k_fix_plan(i64 D, const double *__restrict__ x, int df_ok,
                                                            FixRange *__restrict__ R, int *__restrict__ ctl) {
@@ -296,9 +311,9 @@ __global__ void __launch_bounds__(kPlanThreads) k_fix_plan(i64 D, const double *
   };
   for (i64 k = first; k < D; k += (i64)nblk * kPlanThreads) {
     const u64 b = (u64)__double_as_longlong(x[k]);
-    const int e = (int)((b >> 52) & 0x7ff);
-    a = max(a, e);
-    if (b << 1) c = min(c, e);
+    const int top = (int)(b >> 32) & 0x7fffffff;
+    a = max(a, top);
+    if (b << 1) c = min(c, top >> 20);
   }
   across();
   if (tid == 0) {
@@ -317,6 +332,8 @@ __global__ void __launch_bounds__(kPlanThreads) k_fix_plan(i64 D, const double *
   }
   __syncthreads();
   across();
+  const unsigned mant = ((unsigned)a & 0xfffffu) + 0x100001u;       // max |x| is below mant 2^-20 of its power of two
+  a >>= 20;
   int n = 0;
   const int samples = (int)min(D, (i64)kPlanSamples);
   for (int k = tid; k < samples; k += kPlanThreads) n += __ldcg(R->sample + k) < a - 8 ? 1 : 0;
@@ -327,6 +344,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_fix_plan(i64 D, const double *
   const bool wide = a == 0 || 8 * sum > samples;
   ctl[kCtlShift] = ctl[kCtlDfScale] = a == 0 ? 0 : a - 1023;
   ctl[kCtlDfScale + 1] = 0;
+  ctl[kCtlScale] = (int)(unsigned)(((1ull << 52) - (1ull << 38)) / mant);
   ctl[kCtlSkip] = out || wide ? 1 : 0;
   *count_of(ctl) = 0;
   ctl[kCtlDf] = !out && wide && df_ok ? 1 : 0;
@@ -1110,7 +1128,7 @@ __device__ __forceinline__ double2 ld_two(const double *p, bool vec, bool second
 }
 
 // X (stride ld) and XT (transposed, stride ldt), either may be null, from FP64 x (n_r x n_c) on the
-// grid of ctl[kCtlShift].  acc != null: also |X|^2 into the slots.
+// grid of ctl[kCtlShift].  acc != null: a Lanczos run's, scaled by ctl[kCtlScale]; also |X|^2 into the slots.
 template <int T, bool kLimb>
 __global__ void __launch_bounds__(kTileThreads) k_fix_in(i64 n_r, i64 n_c, i64 ld, i64 ldt,
                                                          const double *__restrict__ x, const int *__restrict__ ctl,
@@ -1119,7 +1137,8 @@ __global__ void __launch_bounds__(kTileThreads) k_fix_in(i64 n_r, i64 n_c, i64 l
   __shared__ TileBuf<T> t;
   after_previous();
   if (use_skip && flag_of(ctl + kCtlSkip)) return;
-  const int e = ctl[kCtlShift] - (B - 2);
+  const int e = ctl[kCtlShift] - (acc ? B - 1 : B - 2);
+  const unsigned c = (unsigned)ctl[kCtlScale];
   const TileAt<T> at;
   const bool vec = (n_c & 1) == 0 && ((uintptr_t)x & 15) == 0;
   constexpr int kN = T / TileAt<T>::kStep;
@@ -1142,7 +1161,14 @@ __global__ void __launch_bounds__(kTileThreads) k_fix_in(i64 n_r, i64 n_c, i64 l
 #pragma unroll
     for (int i = 0; i < kN; ++i) {
       const int k = at.k0 + i * TileAt<T>::kStep;
-      i64 v[2] = {f64_to_fix(xv[i].x, e), f64_to_fix(xv[i].y, e)};
+      i64 v[2];
+      if (acc) {
+        v[0] = f64_to_fix_scaled(xv[i].x, c, e);
+        v[1] = f64_to_fix_scaled(xv[i].y, c, e);
+      } else {
+        v[0] = f64_to_fix(xv[i].x, e);
+        v[1] = f64_to_fix(xv[i].y, e);
+      }
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         if (acc) {
@@ -1172,7 +1198,7 @@ __global__ void k_fix_start(u64 *acc, int B, FixScal *q) {
     q->overlap = 0.0;
     q->N_prev = 1.0;
     q->alpha = q->beta2 = 0.0;
-    q->max_cur = ldexp(1.0, B - 1);
+    q->max_cur = ldexp(1.0, B);
     q->rescale = 0;
     q->max_prev = 0.0;
     q->ratio = 0.5;
@@ -1955,11 +1981,9 @@ int fix_lanczos(hub_ctx *h, const double *x0, int maxit, double tol, double *E0,
   HUB_CUDA(cudaMemcpyAsync(ctl, f->ctl, sizeof(ctl), cudaMemcpyDeviceToHost, s));
   HUB_CUDA(cudaMemcpyAsync(f->h_scal, f->scal, sizeof(FixScal), cudaMemcpyDeviceToHost, s));
   HUB_CUDA(cudaStreamSynchronize(s));
-  h->start_norm = std::ldexp(std::sqrt(f->h_scal->N), ctl[kCtlShift] - (p.B - 2));   // 0: hub_green_coeffs looks
-  if (ctl[kCtlShift] == 2047 - 1023 || !(f->h_scal->N > 0.0))
+  h->start_norm = std::ldexp(std::sqrt(f->h_scal->N) / (unsigned)ctl[kCtlScale], 31 + ctl[kCtlShift] - (p.B - 1));
+  if (ctl[kCtlShift] == 2047 - 1023 || !(f->h_scal->N > 0.0))          // N = 0: hub_green_coeffs looks at the norm
     return fail(HUB_ERR_ARG, "hub_lanczos_ground: start vector is zero or not finite");
-  const auto too_wide = [&](double N) { return N < 0x1p96 * (double)D; };      // rms below 2^48 (see the top)
-  if (too_wide(f->h_scal->N)) return kFixWide;
 
   // graphs of one step, kept while their operands stay the same
   bool graphs = !h->prof && !f->graph_failed;
@@ -2027,7 +2051,6 @@ int fix_lanczos(hub_ctx *h, const double *x0, int maxit, double tol, double *E0,
         if ((rc = fast_check_error(h))) return rc;
         return fail(HUB_ERR_CUDA, "hub_lanczos_ground: non-finite alpha/beta");
       }
-      if (too_wide(f->h_scal->hist[3 * b + 2])) return kFixWide;
       h->alpha.push_back(a);
       h->beta.push_back(be);
       if (tol > 0) E = lowest.next(h->alpha.data(), h->beta.data(), (int)h->alpha.size());   // else at the end

@@ -318,8 +318,6 @@ constexpr int kExpSpan = 80, kExpLo = 200, kExpHi = 1900;
 bool fix_apply_eligible(const hub_ctx *h);
 int fix_apply(hub_ctx *h, const double *x, double *y, cudaStream_t s);
 bool fix_lanczos_eligible(const hub_ctx *h);
-// kFixWide: a vector of the run is too uneven for the grid; nothing has been written.
-constexpr int kFixWide = 1000;
 int fix_lanczos(hub_ctx *h, const double *x0, int maxit, double tol, double *E0, double *psi_out, int *iters,
                 cudaStream_t s);
 void fix_release(hub_ctx *h);

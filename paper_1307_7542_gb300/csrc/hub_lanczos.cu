@@ -370,6 +370,7 @@ extern "C" int hub_lanczos_ground(hub_t h, const double *x0_dev, int maxit, doub
   const int64_t D = vec_len(h);
   if (D == 0) return fail(HUB_ERR_ARG, "hub_lanczos_ground: empty sector");
   if (small_eligible(h)) return small_lanczos(h, x0_dev, maxit, tol, E0, psi_dev, iters, (cudaStream_t)stream);
+  bool fp64 = false;
   if (fix_lanczos_eligible(h)) {
     const double *x0 = x0_dev;
     if (!x0) {
@@ -380,22 +381,15 @@ extern "C" int hub_lanczos_ground(hub_t h, const double *x0_dev, int maxit, doub
       x0 = h->work[2];
     }
     rc = fix_lanczos(h, x0, maxit, tol, E0, psi_dev, iters, (cudaStream_t)stream);
-    if (rc != HUB_ERR_OOM && rc != kFixWide) return rc;
-    set_error("");
-  }
-  // Where memory is short (for the fixed-point vectors, or for these beside them) the other paths' vectors
-  // go, and the FP64 kernel, which needs none, runs this call's products.
-  bool fp64 = rc == HUB_ERR_OOM;
-  if (!fp64) {
-    rc = ensure_workspace(h, D);
-    fp64 = rc == HUB_ERR_OOM && !h->k0 && h->fast;
-  }
-  if (fp64) {
+    if (rc != HUB_ERR_OOM) return rc;
+    // its vectors do not fit: three FP64 ones may, without the other paths' beside them; the FP64 kernel,
+    // which needs none, runs this call's products
     fix_release(h);
-    if (h->fast) fast_release_scratch(h);
+    fast_release_scratch(h);
+    fp64 = true;
     set_error("");
-    rc = ensure_workspace(h, D);
   }
+  rc = ensure_workspace(h, D);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   const int G = vec_grid(), T = kVecThreads;
