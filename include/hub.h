@@ -58,6 +58,12 @@ extern "C" {
                              integer-pipe sums when t is uniform                         */
 #define HUB_MODE_FP64 1   /* always the native FP64 kernels                              */
 
+#define HUB_ROUTE_NONE 0  /* no product yet                                         */
+#define HUB_ROUTE_FP64 1  /* the native FP64 kernel                                 */
+#define HUB_ROUTE_FIX 2   /* 64-bit fixed point                                     */
+#define HUB_ROUTE_DF 3    /* double-float                                           */
+#define HUB_ROUTE_SYM 4   /* a momentum sector's kernel                             */
+
 #define HUB_SYM_NONE 0    /* the full sector (N_up, N_dn)                              */
 #define HUB_SYM_K0 1      /* its k = 0 subspace under the translation i -> i-1 mod M   */
 #define HUB_SYM_KPI 2     /* its k = pi subspace (T eigenvalue -1; M even)             */
@@ -436,6 +442,14 @@ int hub_set_small_dim(hub_t h, int64_t max_dim);
  * HUB_ERR_CUDA on a CUDA error, else HUB_OK.  hub_lanczos_ground checks this itself.
  */
 int hub_check(hub_t h);
+
+/*
+ * Which kernels wrote the result of the handle's last product (HUB_ROUTE_*; of the last vector
+ * of hub_apply_host_many).  The choice between them is made on the device (see hub_apply), so
+ * this waits for the queued work; for tests and diagnosis.  Products inside the Lanczos drivers
+ * of hub_fix.cu and hub_small.cu do not count.  HUB_ERR_ARG for NULL arguments.
+ */
+int hub_last_route(hub_t h, int *route);
 
 /*
  * Test hook (no counterpart in the paper; off by default).  While enabled, every CTA of the

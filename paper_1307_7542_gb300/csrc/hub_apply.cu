@@ -157,6 +157,7 @@ static bool f64_is_faster(const hub_ctx *h) {
 static int apply_kernels(hub_ctx *h, const double *x, double *y, cudaStream_t s) {
   const Ham H = h->view();
   if (H.n_up == 0 || H.n_dn == 0) return HUB_OK;
+  set_route(h, h->k0 ? HUB_ROUTE_SYM : HUB_ROUTE_FP64);
   if (h->k0) return k0_apply(h, x, y, s);
   if (f64_is_faster(h)) return f64_apply(h, x, y, nullptr, s);
   if (fix_apply_eligible(h)) {
@@ -164,10 +165,17 @@ static int apply_kernels(hub_ctx *h, const double *x, double *y, cudaStream_t s)
     if (rc != HUB_ERR_OOM) return rc;
     fast_release_scratch(h);          // its vectors do not fit (nor the double-float path's, the same ones)
     set_error("");
+    set_route(h, HUB_ROUTE_FP64);
     return f64_apply(h, x, y, nullptr, s);
   }
   if (use_fast(h)) return fast_apply_f64(h, x, y, s);
   return f64_apply(h, x, y, nullptr, s);
+}
+
+void set_route(hub_ctx *h, int route, const int *f64_flag, const int *df_flag) {
+  h->route = route;
+  h->route_flag[0] = f64_flag;
+  h->route_flag[1] = df_flag;
 }
 
 // Columns of a CTA: chunks of 256 and less where the row is short, so that a small matrix still makes
@@ -241,6 +249,22 @@ static int host_apply_buffers(hub_ctx *h, double **x, double **y) {
     dev_free(*x);
     *x = nullptr;
     return HUB_ERR_OOM;
+  }
+  return HUB_OK;
+}
+
+extern "C" int hub_last_route(hub_t h, int *route) {
+  if (!h || !route) return fail(HUB_ERR_ARG, "hub_last_route: NULL argument");
+  const int to[2] = {HUB_ROUTE_FP64, HUB_ROUTE_DF};
+  *route = h->route;
+  HUB_CUDA(cudaDeviceSynchronize());
+  for (int k = 0; k < 2; ++k) {
+    int flag = 0;
+    if (h->route_flag[k]) HUB_CUDA(cudaMemcpy(&flag, h->route_flag[k], sizeof(int), cudaMemcpyDeviceToHost));
+    if (flag) {
+      *route = to[k];
+      break;
+    }
   }
   return HUB_OK;
 }

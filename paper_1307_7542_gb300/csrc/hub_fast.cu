@@ -785,6 +785,7 @@ void fast_release(hub_ctx *h) {
   dev_free(f->zdf);
   dev_free(f->xt);
   dev_free(f->zt);
+  if (h->route == HUB_ROUTE_DF) set_route(h, HUB_ROUTE_NONE);     // its flag goes
   dev_free(f->d_range);
   dev_free(f->d_err);
   dev_free(f->d_range_chunks);
@@ -1275,6 +1276,7 @@ int fast_apply_f64(hub_ctx *h, const double *x, double *y, cudaStream_t s) {
   count_launch(h);
   k_scale<<<1, 256, 0, s>>>(part, G, scale);
   HUB_LAUNCH_CHECK();
+  set_route(h, HUB_ROUTE_DF, scale + 1);
   if ((rc = df_apply(h, f, x, y, scale, nullptr, s))) return rc;
   return f64_apply(h, x, y, scale + 1, s);
 }
@@ -1432,6 +1434,7 @@ static int pipeline_host(hub_ctx *h, FastState *f, const double *x_host, double 
   }
   if ((rc = host_pass1(h, f, xd, C.bi, C.nci, C.per, ev_in, s))) return rc;
   HUB_CUDA(cudaStreamSynchronize(s));
+  set_route(h, *f->h_flag == 2 ? HUB_ROUTE_FP64 : HUB_ROUTE_DF);
   if (*f->h_flag == 2) {   // outside the double-float window: the FP64 kernel, one copy back
     if ((rc = f64_apply(h, xd, yd, nullptr, s))) return rc;
     HUB_CUDA(cudaMemcpyAsync(y_host, yd, sizeof(double) * n_dn * n_up, cudaMemcpyDeviceToHost, s));
@@ -1523,6 +1526,7 @@ int fast_apply_host_many(hub_ctx *h, int64_t n_vec, const double *x_host, double
       if (v + 1 < n_vec && (rc = copy_in(v + 1))) return rc;
       HUB_CUDA(cudaStreamSynchronize(s));
       const int route = *f->h_flag;
+      set_route(h, route == 2 ? HUB_ROUTE_FP64 : HUB_ROUTE_DF);
       if (route == 1 && (rc = host_redo(h, f, xd[p], s))) return rc;
       if (v >= 2) HUB_CUDA(cudaStreamWaitEvent(s, y_free[p], 0));
       if (route == 2) {   // outside the double-float window: the FP64 kernel, one copy back

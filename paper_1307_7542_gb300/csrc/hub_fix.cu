@@ -1531,6 +1531,7 @@ void fix_release(hub_ctx *h) {
     dev_free(f->vec[s]);
     if (f->graph[s]) cudaGraphExecDestroy(f->graph[s]);
   }
+  if (h->route == HUB_ROUTE_FIX) set_route(h, HUB_ROUTE_NONE);    // its flags go
   dev_free(f->ctl);
   dev_free(f->list);
   dev_free(f->acc);
@@ -1856,6 +1857,7 @@ int fix_apply(hub_ctx *h, const double *x, double *y, cudaStream_t s) {
   if ((rc = fix_tables_wait(f))) return rc;
   const int df_ok = use_fast(h) ? 1 : 0;
   if ((rc = plan_vector(h, f, x, D, df_ok, s))) return rc;
+  set_route(h, HUB_ROUTE_FIX, f->ctl + kCtlF64, f->ctl + kCtlDf);
   // X: rows spin down (the caller's order); XT: rows spin up
   const bool cx = F.both || F.a == 1, ct = F.both || F.a == 0;
   i64 *X = (i64 *)buf[0], *XT = (i64 *)buf[1];

@@ -240,6 +240,11 @@ struct hub_ctx {
   // fixed-point product and Lanczos (hub_fix.cu): tables, flags and vectors
   hub::FixState *fix = nullptr;
 
+  // the last product's kernels (hub_last_route): HUB_ROUTE_*, or the one that the words of a path's own
+  // flags decide
+  int route = 0;
+  const int *route_flag[2] = {nullptr, nullptr};   // device: nonzero for FP64, for double-float
+
   hub::Ham view() const;
 };
 
@@ -262,6 +267,7 @@ int reduce_partials_2stage(const double *partials, int n, double *tmp, int ntmp,
 
 // Apply entry used by Lanczos and the VJP (no argument checks).
 int apply_launch(hub_ctx *h, const double *x, double *y, cudaStream_t s);
+void set_route(hub_ctx *h, int route, const int *f64_flag = nullptr, const int *df_flag = nullptr);
 // The FP64 product kernel of the full sector; with a gate it does nothing unless gate[0] != 0
 // when it runs (a device flag written earlier on the stream).
 int f64_apply(hub_ctx *h, const double *x, double *y, const int *gate, cudaStream_t s);

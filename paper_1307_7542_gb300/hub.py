@@ -26,6 +26,7 @@ HUB_ERR_CUDA = -3
 HUB_ERR_NOCONV = -4
 HUB_ERR_STATE = -5
 HUB_ERR_TIMEOUT = -6
+HUB_ROUTE_NONE, HUB_ROUTE_FP64, HUB_ROUTE_FIX, HUB_ROUTE_DF, HUB_ROUTE_SYM = 0, 1, 2, 3, 4
 HUB_SYM_NONE = 0
 HUB_SYM_K0 = 1
 HUB_SYM_KPI = 2
@@ -66,6 +67,7 @@ SIGNATURES = {
     "hub_k_project": (_i, [_p, _p, _p, _p]),
     "hub_set_mode": (_i, [_p, _i]),
     "hub_check": (_i, [_p]),
+    "hub_last_route": (_i, [_p, ctypes.POINTER(_i)]),
     "hub_test_fail_waits": (_i, [_p, _i]),
     "hub_profile": (_i, [_p, _i]),
     "hub_profile_read": (_i, [_p, _i, ctypes.POINTER(_d), ctypes.POINTER(_i64), ctypes.POINTER(_i64)]),
@@ -345,6 +347,13 @@ def hub_set_mode(h, mode):
 
 def hub_check(h):
     _check(lib().hub_check(h))
+
+
+def hub_last_route(h):
+    """HUB_ROUTE_* of the handle's last product."""
+    r = _i()
+    _check(lib().hub_last_route(h, ctypes.byref(r)))
+    return r.value
 
 
 def hub_set_small_dim(h, max_dim):
