@@ -43,8 +43,10 @@ __device__ __forceinline__ double f64_diag(const Ham &H, const double *s_U, uint
 template <int kMode, int kF64Rows>
 __global__ void __launch_bounds__(256, 6) k_apply_f64(const Ham H, const double *__restrict__ x, double *y,
                                                    const int *__restrict__ gate, int chunks, const F64Step L) {
-  after_previous();
-  if (gate && flag_of(gate) == 0) return;
+  if (gate) {
+    after_previous();
+    if (flag_of(gate) == 0) return;
+  }
   // Sums of U_i over the set bits of each eight sites, from those of each four; only where U varies, since
   // the L1 that serves the gathers shrinks by it (uniform U, 17-site ring (7,2): 0.105 ms, with 9 KB 0.117).
   extern __shared__ double s_tab[];

@@ -264,8 +264,10 @@ __global__ void k_scale_all(const int *__restrict__ partials, int nblk, int n_se
 __global__ void k_f64_to_df(int64_t r0, int64_t r1, int64_t n_up, int64_t ld, const double *__restrict__ x,
                             const int *__restrict__ scale, const int32_t *__restrict__ slot_row,
                             float *__restrict__ out, const int *__restrict__ gate) {
-  after_previous();
-  if (gate && flag_of(gate) == 0) return;
+  if (gate) {
+    after_previous();
+    if (flag_of(gate) == 0) return;
+  }
   const int shift = scale ? scale[0] : 0;
   for (int64_t d = r0 + blockIdx.x; d < r1; d += gridDim.x) {
     float *__restrict__ row = out + d * 2 * ld;
@@ -285,7 +287,7 @@ __global__ void k_f64_to_df(int64_t r0, int64_t r1, int64_t n_up, int64_t ld, co
 __global__ void k_unpermute(int64_t r0, int64_t r1, int64_t n_up, int64_t ld, const float *__restrict__ v,
                             const int32_t *__restrict__ slot_of, const int *__restrict__ scale, double tabs,
                             double *__restrict__ y, const int *__restrict__ gate) {
-  after_previous();
+  if (gate) after_previous();
   if (flag_of(scale + 1) || (gate && flag_of(gate) == 0)) return;
   const int shift = scale[0];
   for (int64_t d = r0 + blockIdx.x; d < r1; d += gridDim.x) {
@@ -326,8 +328,10 @@ static_assert(kUpThreads % 32 == 0 && kUpThreads >= 512 && kUpThreads <= 1024, "
 template <typename Col>
 __global__ void __launch_bounds__(kUpThreads, 1) k_up(const FastView F, const float *__restrict__ x,
                                                       float *__restrict__ z, int64_t p_begin, int64_t p_end) {
-  after_previous();
-  if (F.gate && flag_of(F.gate) == 0) return;
+  if (F.gate) {
+    after_previous();
+    if (flag_of(F.gate) == 0) return;
+  }
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float *xs = reinterpret_cast<float *>(smem_raw);
   __shared__ __align__(8) uint64_t bar;
@@ -514,8 +518,10 @@ constexpr int kTile = 32;
 __global__ void __launch_bounds__(256) k_transpose(int64_t n_r, int64_t n_c, int64_t ld_s, int64_t ld_d,
                                                    const float *__restrict__ src, float *__restrict__ dst,
                                                    const int *__restrict__ gate) {
-  after_previous();
-  if (gate && flag_of(gate) == 0) return;
+  if (gate) {
+    after_previous();
+    if (flag_of(gate) == 0) return;
+  }
   __shared__ float th[kTile][kTile + 1], tl[kTile][kTile + 1];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int64_t c0 = (int64_t)blockIdx.x * kTile, r0 = (int64_t)blockIdx.y * kTile;
@@ -664,8 +670,10 @@ __device__ __forceinline__ void dn_group(DfSumP (&acc)[kLane], const Side &S, co
 template <typename Col, int kMode>
 __global__ void __launch_bounds__(kDnThreads, HUB_DN_MINB) k_dn(const FastView F, const Side S, const float *__restrict__ x,
                                                   const float *z, float *w) {
-  after_previous();
-  if (F.gate && flag_of(F.gate) == 0) return;
+  if (F.gate) {
+    after_previous();
+    if (flag_of(F.gate) == 0) return;
+  }
   constexpr int kLane = kDnLaneCols / 2;               // packed pairs per lane
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t ld = S.ld;
@@ -1454,7 +1462,8 @@ static int pipeline_host(hub_ctx *h, FastState *f, const double *x_host, double 
 // pass 2 the output goes back in row chunks while later chunks are un-permuted.  The
 // power-of-two scale of the conversion is taken from the first chunk's largest exponent; if
 // the whole vector's largest exponent is larger, conversion and pass 1 are redone with it, so
-// the result is bit for bit that of hub_apply.  xd, yd: the handle's FP64 device buffers.
+// the result is that of these kernels on the whole vector (hub_apply itself runs sectors of this
+// size in fixed point).  xd, yd: the handle's FP64 device buffers.
 int fast_apply_host(hub_ctx *h, const double *x_host, double *y_host, double *xd, double *yd, cudaStream_t s) {
   FastState *f = fast_of(h);
   if (!f || !f->built) return fail(HUB_ERR_STATE, "fast apply: not built");

@@ -116,7 +116,7 @@ struct FixPass {
   int *err;                           // device error flag
   int fail_waits;                     // test hook
   int chained;                        // launch_kernel's
-  const int *skip;                    // apply: device flag, nothing to do
+  const int *skip;                    // products: device flag, nothing to do
   u64 *acc;                           // Lanczos: dot product and maximum into these slots
   struct FixScal *scal;               // Lanczos, second pass of a step: its last block ends the step
   int second;
@@ -124,7 +124,7 @@ struct FixPass {
 
 // Lanczos scalars on the device.
 struct FixScal {
-  double N, N_prev;                   // |S_j|^2 and |S_{j-1}|^2 (integers on their grids)
+  double N;                           // |S_j|^2 (an integer on its grid)
   double alpha, beta2;                // of step j
   double overlap;                     // <S_j, S_{j-1}>
   double max_cur, max_prev;           // bounds on |S_j|, |S_{j-1}|
@@ -507,8 +507,10 @@ __global__ void __launch_bounds__(1024, 1) k_fix_gather(const FixPass P, const G
   int2 *const x0 = reinterpret_cast<int2 *>(smem), *const x1 = x0 + kPlane;   // entries ld .. ld + 15 are zero
   __shared__ __align__(8) uint64_t bar;
   __shared__ i64 utab[32];
-  after_previous();
-  if (P.skip && flag_of(P.skip)) return;
+  if (!kLz) {
+    after_previous();
+    if (flag_of(P.skip)) return;
+  }
   const int tid = threadIdx.x, lane = tid & 31;
   if (tid < 32) {
     utab[tid] = P.diag.tab[tid];
@@ -650,10 +652,11 @@ __global__ void __launch_bounds__(1024, 1) k_fix_gather(const FixPass P, const G
 constexpr int kSchedRow = 64;         // longest hopping row of the gather form
 constexpr int kSchedMax = 2 * kSchedRow;
 // Quads that a warp groups: more of them make better groups (4x4, 12,870 positions: 1.197 steps per entry with
-// 64, 1.186 with 128, 1.171 with all), but take a quarter of a microsecond each.
-constexpr int kSegFew = 64, kSegMany = 256, kSegManyFrom = 4096;
+// 64, 1.186 with 128, 1.171 with all), but take a quarter of a microsecond each, before the first product.
+constexpr int kSegMax = 1024;
+static int seg_quads(double D) { return D < 0x1p22 ? 64 : (D < 0x1p25 ? 256 : kSegMax); }
 struct SchedSpin {
-  int n, groups, idle, cap, seg;      // positions, groups (even), the position of a zero, most steps, kSeg*
+  int n, groups, idle, cap, seg;      // positions, groups (even), the position of a zero, most steps, seg_quads
   const int32_t *rp;
   const uint32_t *scol;
   uint32_t *load;                     // [4 groups][8] entries of a quad by bank, two counts a word
@@ -715,9 +718,9 @@ __global__ void __launch_bounds__(256) k_fix_sort(const SchedArgs A) {
 
 __global__ void __launch_bounds__(32) k_fix_group(const SchedArgs A) {
   const SchedSpin &S = A.spin[blockIdx.y];
-  __shared__ uint32_t load[kSegMany][9];
-  __shared__ uint16_t id[kSegMany], left[kSegMany];
-  __shared__ uint8_t len[kSegMany];
+  __shared__ uint32_t load[kSegMax][9];
+  __shared__ uint16_t id[kSegMax], left[kSegMax];
+  __shared__ uint8_t len[kSegMax];
   const int lane = threadIdx.x, base = blockIdx.x * S.seg, n = min(S.seg, 4 * S.groups - base);
   if (n <= 0) return;
   const uint8_t *lens = reinterpret_cast<const uint8_t *>(S.len);
@@ -983,7 +986,7 @@ template <bool kLz>
 __global__ void __launch_bounds__(kCombThreads, 2) k_fix_comb(const FixPass P, const CombLists S) {
   constexpr int kWarps = kCombThreads / 32;
   __shared__ i64 utab[32];
-  after_previous();
+  if (P.chained) after_previous();          // tested at run time: the Lanczos form without a test ran 10 % slower
   if (P.skip && flag_of(P.skip)) return;
   if (P.fail_waits) {                       // test hook: report as a given-up wait would
     if (threadIdx.x == 0) atomicExch(P.err, 1);
@@ -1129,22 +1132,25 @@ __device__ __forceinline__ double2 ld_two(const double *p, bool vec, bool second
 
 // X (stride ld) and XT (transposed, stride ldt), either may be null, from FP64 x (n_r x n_c) on the
 // grid of ctl[kCtlShift].  acc != null: a Lanczos run's, scaled by ctl[kCtlScale]; also |X|^2 into the slots.
-template <int T, bool kLimb>
+template <int T, bool kLimb, bool kTurns>
 __global__ void __launch_bounds__(kTileThreads) k_fix_in(i64 n_r, i64 n_c, i64 ld, i64 ldt,
                                                          const double *__restrict__ x, const int *__restrict__ ctl,
                                                          int use_skip, int B, i64 *__restrict__ X,
                                                          i64 *__restrict__ XT, u64 *__restrict__ acc) {
   __shared__ TileBuf<T> t;
-  after_previous();
-  if (use_skip && flag_of(ctl + kCtlSkip)) return;
+  if (use_skip) {
+    after_previous();
+    if (flag_of(ctl + kCtlSkip)) return;
+  }
   const int e = ctl[kCtlShift] - (acc ? B - 1 : B - 2);
   const unsigned c = (unsigned)ctl[kCtlScale];
   const TileAt<T> at;
   const bool vec = (n_c & 1) == 0 && ((uintptr_t)x & 15) == 0;
   constexpr int kN = T / TileAt<T>::kStep;
   DotLong dots{{0, 0, 0, 0}};
-  const uint32_t tiles = tiles_of<T>(n_r, n_c);
-  for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+  const uint32_t tiles = kTurns ? tiles_of<T>(n_r, n_c) : 0;
+  uint32_t tile = blockIdx.x;
+  do {
     i64 r0, c0;
     tile_at<T>(tile, n_c, &r0, &c0);
     const i64 u = c0 + at.c;
@@ -1156,7 +1162,7 @@ __global__ void __launch_bounds__(kTileThreads) k_fix_in(i64 n_r, i64 n_c, i64 l
       xv[i] = make_double2(0.0, 0.0);
       if (d < n_r && in) xv[i] = ld_two(x + d * n_c + u, vec, second);
     }
-    if (XT && tile != blockIdx.x) __syncthreads();        // the tile before has been written out
+    if (kTurns && XT && tile != blockIdx.x) __syncthreads();          // the tile before has been written out
     Dot dot{0, 0};
 #pragma unroll
     for (int i = 0; i < kN; ++i) {
@@ -1186,7 +1192,8 @@ __global__ void __launch_bounds__(kTileThreads) k_fix_in(i64 n_r, i64 n_c, i64 l
       tile_out_t<T>(t, XT, ldt, r0, c0, n_r, n_c);
     }
     dots.take(dot);
-  }
+    tile += gridDim.x;
+  } while (kTurns && tile < tiles);
   if (acc) block_sums<4>(dots.v, 0u, 0, acc);
 }
 
@@ -1196,7 +1203,6 @@ __global__ void k_fix_start(u64 *acc, int B, FixScal *q) {
   if (threadIdx.x == 0) {
     q->N = N;
     q->overlap = 0.0;
-    q->N_prev = 1.0;
     q->alpha = q->beta2 = 0.0;
     q->max_cur = ldexp(1.0, B);
     q->rescale = 0;
@@ -1341,7 +1347,6 @@ __global__ void __launch_bounds__(kTileThreads, kUpdateBlocks) k_fix_update(i64 
     }
     q->hist_n = i + 1;
     q->step += 1;
-    q->N_prev = q->N;
     q->N = N;
     q->beta2 = b2;
     q->rel = -(q->sh + r);
@@ -1373,7 +1378,7 @@ __global__ void __launch_bounds__(256) k_fix_rescale(const FixScal *__restrict__
 // not reach thr is recorded in list (see k_fix_entries).  Memory bounds it (24 bytes per entry, 0.59 ms
 // at 4x4): 0.69 ms with four CTAs per SM and loads as they are needed, 0.85 ms with a tile's loads in
 // registers first (116 of them, two CTAs); unrolled by 2 or 4, or five CTAs, 0 to 0.09 ms slower.
-template <int T, bool kAt, bool kBt>
+template <int T, bool kAt, bool kBt, bool kTurns>
 __global__ void __launch_bounds__(kTileThreads, kUpdateBlocks) k_fix_out(i64 n_r, i64 n_c, i64 ld, i64 ldt,
                                                                          const i64 *__restrict__ a, const i64 *__restrict__ b, int eg, i64 thr, double tabs,
                                                           int *__restrict__ ctl, i64 *__restrict__ list, int cap,
@@ -1386,13 +1391,14 @@ __global__ void __launch_bounds__(kTileThreads, kUpdateBlocks) k_fix_out(i64 n_r
   const int e = ctl[kCtlShift] + eg;
   const TileAt<T> at;
   const bool vec = (n_c & 1) == 0 && ((uintptr_t)y & 15) == 0;
-  const uint32_t tiles = tiles_of<T>(n_r, n_c);
-  for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+  const uint32_t tiles = kTurns ? tiles_of<T>(n_r, n_c) : 0;
+  uint32_t tile = blockIdx.x;
+  do {
     i64 r0, c0;
     tile_at<T>(tile, n_c, &r0, &c0);
     const i64 u = c0 + at.c;
     const bool second = u + 1 < n_c;
-    if ((kAt || kBt) && tile != blockIdx.x) __syncthreads();          // the tile before has been read
+    if (kTurns && (kAt || kBt) && tile != blockIdx.x) __syncthreads();          // the tile before has been read
     if (kBt) tile_in_t<T>(t, b, ldt, r0, c0, n_r, n_c);
     if constexpr (kAt && kBt)
       tile_in_t<T>(t2, a, ldt, r0, c0, n_r, n_c);
@@ -1429,7 +1435,8 @@ __global__ void __launch_bounds__(kTileThreads, kUpdateBlocks) k_fix_out(i64 n_r
         if (second) y[n + 1] = v[1];
       }
     }
-  }
+    tile += gridDim.x;
+  } while (kTurns && tile < tiles);
 }
 
 // psi += v_j q_j alone (the last vector)
@@ -1604,7 +1611,7 @@ static int grid_of(i64 n) { return (int)std::max<i64>(1, std::min<i64>((n + 255)
 
 // Arrays of a spin's gather schedule and of what it is made from, in one allocation (a first product
 // pays for each).
-static int gather_arrays(FixState *f, int s, int n, const SpinCSR &c, SchedSpin *S) {
+static int gather_arrays(FixState *f, int s, int n, int seg, const SpinCSR &c, SchedSpin *S) {
   const int slices = (n + 31) / 32, groups = 2 * slices;
   const int cap = std::min(kSchedMax, (2 * std::max(c.max_row, 1) + 7) / 8 * 8);
   size_t at = 0;
@@ -1624,7 +1631,7 @@ static int gather_arrays(FixState *f, int s, int n, const SpinCSR &c, SchedSpin 
   f->meta[s] = (uint32_t *)(base + o_meta);
   f->cap_steps[s] = cap;
   f->slices[s] = slices;
-  *S = SchedSpin{n, groups, (int)fix_ld(n), cap, n < kSegManyFrom ? kSegFew : kSegMany, c.rowptr, c.scol, (uint32_t *)(base + o_load),
+  *S = SchedSpin{n, groups, (int)fix_ld(n), cap, seg, c.rowptr, c.scol, (uint32_t *)(base + o_load),
                  (uint32_t *)(base + o_len), (uint16_t *)(base + o_sorted), (uint16_t *)(base + o_greedy),
                  (uint8_t *)(base + o_steps), (uint32_t *)(base + o_total), (uint16_t *)(base + o_quad),
                  (uint8_t *)(base + o_deg), f->sched[s], f->meta[s]};
@@ -1641,7 +1648,7 @@ static int fix_tables(hub_ctx *h, FixState *f, const FixPlan &p) {
     const SpinCSR &c = h->csr[s];
     const i64 nnz = c.nnz, n = h->count[s];
     if (p.gather[s]) {
-      const int rc = gather_arrays(f, s, (int)n, c, &A.spin[gathers]);
+      const int rc = gather_arrays(f, s, (int)n, seg_quads((double)h->count[0] * (double)h->count[1]), c, &A.spin[gathers]);
       if (rc) return rc;
       const SchedSpin &S = A.spin[gathers++];
       groups = std::max(groups, S.groups);
@@ -1715,14 +1722,23 @@ static i64 tile_blocks(const hub_ctx *h, i64 T) {
   return ((h->count[0] + T - 1) / T) * ((h->count[1] + T - 1) / T);
 }
 static i64 tile_blocks(const hub_ctx *h) { return tile_blocks(h, small_tiles(h) ? 32 : 64); }
-// CTAs of the kernels that take tiles in turn: as many as are resident.  (One per tile cost 8 us where the
-// kernel finds nothing to do, 2916 CTAs, and 17 us with 7600.)
+// k_fix_in and k_fix_out: a CTA per tile, or (kTurns) as many as are resident, which take tiles in turn.  The
+// first costs 8 us where the kernel finds nothing to do (2916 tiles) and 17 us with 7600; the second is
+// slower where there is (4x4 half filling: 0.67 and 0.77 ms against 0.60 and 0.69; k_fix_out at 2916 tiles of
+// 64 x 64 60 us against 54, k_fix_in 46 either way).
+constexpr i64 kTurnTiles = 8192;
+static bool in_turns(const hub_ctx *h) { return tile_blocks(h) <= kTurnTiles; }
 static int in_blocks(const hub_ctx *h) {
-  return (int)std::min<i64>(tile_blocks(h), (i64)(small_tiles(h) ? 8 : 3) * num_sms());
+  const i64 tiles = tile_blocks(h);
+  return (int)(in_turns(h) ? std::min<i64>(tiles, (i64)(small_tiles(h) ? 8 : 3) * num_sms()) : tiles);
 }
-static int out_blocks(const hub_ctx *h, i64 T) {
-  return (int)std::min<i64>(tile_blocks(h, T), (i64)kUpdateBlocks * num_sms());
+template <bool kTurns>
+static auto in_kernel(const hub_ctx *h, bool limbs) {
+  return limbs ? (small_tiles(h) ? k_fix_in<32, true, kTurns> : k_fix_in<64, true, kTurns>)
+               : (small_tiles(h) ? k_fix_in<32, false, kTurns> : k_fix_in<64, false, kTurns>);
 }
+static auto in_kernel(const hub_ctx *h, bool limbs) { return in_turns(h) ? in_kernel<true>(h, limbs) : in_kernel<false>(h, limbs); }
+
 // grids are one-dimensional, row strides in bytes 32-bit
 static bool fix_fits(const hub_ctx *h) {
   const i64 lim = ((i64)1 << 31) - 1;
@@ -1866,11 +1882,8 @@ int fix_apply(hub_ctx *h, const double *x, double *y, cudaStream_t s) {
   count_launch(h, 3);
   const bool st = small_tiles(h);
   const bool chained = !h->prof;
-  HUB_CUDA(launch_kernel(chained,
-                         p.limbs() ? (st ? k_fix_in<32, true> : k_fix_in<64, true>)
-                                   : (st ? k_fix_in<32, false> : k_fix_in<64, false>),
-                         in_blocks(h), kTileThreads, 0, s, n_dn, n_up, ld, ldt, x, f->ctl, 1, p.B, cx ? X : nullptr,
-                         ct ? XT : nullptr, nullptr));
+  HUB_CUDA(launch_kernel(chained, in_kernel(h, p.limbs()), in_blocks(h), kTileThreads, 0, s, n_dn, n_up, ld, ldt, x,
+                         f->ctl, 1, p.B, cx ? X : nullptr, ct ? XT : nullptr, nullptr));
   i64 *in0 = F.a == 1 ? X : XT, *in1 = F.a == 1 ? XT : X, *out0 = in0, *out1 = in1;   // gathers: in place
   if (F.both && !p.gather[0]) {
     out0 = (i64 *)buf[2];
@@ -1879,17 +1892,23 @@ int fix_apply(hub_ctx *h, const double *x, double *y, cudaStream_t s) {
   if ((rc = fix_product(h, f, p, F, in0, in1, out0, out1, skip, false, s))) return rc;
   const i64 thr = ((i64)std::ceil(p.units * 1.25e13) >> p.g) + 1;   // |error| <= units 2^e <= 0.8e-13 thr 2^(e + g)
   const int eg = p.g - (p.B - 2);
-#define FIX_OUT(T, AT, BT)                                                                                   \
-  HUB_CUDA(launch_kernel(chained, k_fix_out<T, AT, BT>, out_blocks(h, T), kTileThreads, 0, s, n_dn, n_up, ld, \
-                         ldt, out0, out1, eg, thr, p.tau, f->ctl, f->list, f->cap, y))
-  if (F.both && st)
-    FIX_OUT(32, false, true);
+#define FIX_OUT(T, AT, BT, TURNS)                                                                                \
+  HUB_CUDA(launch_kernel(chained, k_fix_out<T, AT, BT, TURNS>,                                                  \
+                         (int)(TURNS ? std::min<i64>(tile_blocks(h, T), (i64)kUpdateBlocks * num_sms()) : tile_blocks(h, T)), \
+                         kTileThreads, 0, s, n_dn, n_up, ld, ldt, out0, out1, eg, thr, p.tau, f->ctl, f->list, f->cap, y))
+  const bool turns = tile_blocks(h, 32) <= kTurnTiles;
+  if (F.both && st && turns)
+    FIX_OUT(32, false, true, true);
+  else if (F.both && st)
+    FIX_OUT(32, false, true, false);
   else if (F.both)
-    FIX_OUT(64, false, true);
+    FIX_OUT(64, false, true, false);
   else if (F.a == 1)
-    FIX_OUT(64, false, false);
+    FIX_OUT(64, false, false, false);
+  else if (turns)
+    FIX_OUT(32, true, true, true);
   else
-    FIX_OUT(32, true, true);
+    FIX_OUT(32, true, true, false);
 #undef FIX_OUT
   HUB_CUDA(launch_kernel(chained, k_fix_entries, num_sms() * 4, 256, 0, s, h->view(), x, y, f->ctl, f->list, f->cap,
                          df_ok));
@@ -1936,8 +1955,7 @@ int fix_lanczos(hub_ctx *h, const double *x0, int maxit, double tol, double *E0,
     count_launch(h, 2);
     HUB_CUDA(cudaMemsetAsync(f->acc, 0, sizeof(u64) * kFixSlots * kAcc, s));
     HUB_CUDA(cudaMemsetAsync(f->vec[1], 0, sizeof(i64) * n_r * ld, s));
-    (p.limbs() ? (st32 ? k_fix_in<32, true> : k_fix_in<64, true>)
-               : (st32 ? k_fix_in<32, false> : k_fix_in<64, false>))<<<in_blocks(h), kTileThreads, 0, s>>>(
+    in_kernel(h, p.limbs())<<<in_blocks(h), kTileThreads, 0, s>>>(
         n_dn, n_up, fix_ld(n_up), fix_ld(n_dn), x0, f->ctl, 0, p.B, swap ? nullptr : f->vec[0],
         swap ? f->vec[0] : (F.both ? ST : nullptr), f->acc);
     HUB_LAUNCH_CHECK();
