@@ -53,9 +53,9 @@ extern "C" {
 #define HUB_SPIN_UP 0
 #define HUB_SPIN_DN 1
 
-#define HUB_MODE_AUTO 0   /* fixed-point or double-float path when t and U are uniform (window
-                             and bound: see hub_apply), else FP64; in a momentum sector:
-                             integer-pipe sums when t is uniform                         */
+#define HUB_MODE_AUTO 0   /* fixed-point or double-float path when t and U are uniform and there
+                             are no site energies (window and bound: see hub_apply), else
+                             FP64; in a momentum sector: integer-pipe sums when t is uniform */
 #define HUB_MODE_FP64 1   /* always the native FP64 kernels                              */
 
 #define HUB_ROUTE_NONE 0  /* no product yet                                         */
@@ -69,9 +69,9 @@ extern "C" {
 #define HUB_SYM_KPI 2     /* its k = pi subspace (T eigenvalue -1; M even)             */
 
 #define HUB_PROF_APPLY 0  /* a whole product H x (both passes on the fast path)       */
-#define HUB_PROF_UP 1     /* fast path pass 1: spin-up hops + diagonal                 */
-#define HUB_PROF_DN 2     /* fast path pass 2: spin-down hops + epilogue               */
-#define HUB_PROF_UPDATE 3 /* fast Lanczos: the update r_j = w - c r_{j-1} (its own pass) */
+#define HUB_PROF_UP 1     /* fixed-point or double-float pass 1                        */
+#define HUB_PROF_DN 2     /* fixed-point or double-float pass 2                        */
+#define HUB_PROF_UPDATE 3 /* fixed-point Lanczos: the update that forms the next vector */
 
 typedef struct hub_ctx *hub_t;
 
@@ -122,19 +122,25 @@ int hub_get_csr(hub_t h, int spin, int32_t *rowptr_host, int32_t *cols_host, dou
  * Accuracy: every entry satisfies |y_n - (Hx)_n| <= 1e-13 (|H||x|)_n, |H| the entrywise
  * absolute matrix.  The native FP64 kernel (HUB_MODE_FP64; non-uniform t or U) does
  * this with FP64 multiply-adds, also for products of few terms (one launch).  In
- * HUB_MODE_AUTO with uniform t and U larger products run in 64-bit fixed point: the entries on
- * one power-of-two grid, 2^-(B+1) of the largest |x_n| (B = 56 or 62 minus the bits of the
- * number of hopping terms), sums exact; an entry whose two sums are too small for the grid to
- * meet the bound is computed again in FP64, and a vector with many such entries is multiplied in
+ * HUB_MODE_AUTO with uniform t and U and no site energies, larger products (more than 2.2e7
+ * terms) run in 64-bit fixed point: the entries on one power-of-two grid, rounded to 2^-(B-1) of
+ * the power of two below the largest |x_n| at worst (B = 56 or 62 minus the bits of the number of
+ * hopping terms), sums exact; an entry whose two sums are too small for the grid to meet the
+ * bound is computed again in FP64, and a vector with many such entries is multiplied in
  * double-float arithmetic (pairs of FP32 numbers, 48 significant bits; compensated
  * sums) with a derived worst-case error of max(N + 10.1, 16) * 2^-48 (|H||x|)_n, N <= 15 the
  * most terms one low-part accumulator takes (N = 9 on the 4x4 lattice: 6.8e-14 (|H||x|)_n).
- * These need a window, checked on the device for every call: the largest |x_n| in
+ * Both need a window, checked on the device for every call: the largest |x_n| in
  * [2^-823, 2^877], every nonzero |x_n| at least 2^-80 times the largest (no FP64
- * subnormals, infinities or NaN); and a model with uniform t != 0 and U, no site energies,
- * |t| and U/|t| either 0 or in [2^-16, 2^16].  A vector or model outside it is multiplied by the FP64 kernel
- * instead, on the same stream and with no host synchronisation, so every call meets the
- * bound.
+ * subnormals, infinities or NaN).  Of the models with uniform t != 0 and U and no site energies
+ * the fixed point takes those with |t| in [2^-500, 2^500] and hopping terms per entry plus
+ * min(N_up, N_dn) |U/t| up to about 190 (4x4 half filling: U/|t| up to 19), the double-float
+ * kernels those with |t| and U/|t| either 0 or in [2^-16, 2^16]: stronger coupling runs in
+ * double-float, as fast as it did before there was a fixed point.  A vector or model outside is
+ * multiplied by the FP64 kernel instead, on the same stream and with no host synchronisation, so
+ * every call meets the bound.  Device memory: two vectors, four where neither spin's rows can be
+ * staged (more than 14384 states each); where they do not fit the FP64 kernel, which needs none, runs the call.
+ * hub_last_route tells which kernels ran.
  */
 int hub_apply(hub_t h, const double *x_dev, double *y_dev, void *stream);
 
@@ -172,12 +178,13 @@ int hub_apply_host_many(hub_t h, int64_t n_vec, const double *x_host, double *y_
  * (beta_j <= 1e-14 |alpha_j|, returns HUB_CONVERGED_BREAKDOWN) or at maxit (returns
  * HUB_ERR_NOCONV, *E0 still set).  If psi_dev != NULL the recurrence is run a second
  * time to form the normalised ground-state vector, which may lie over x0.  Blocks until done;
- * *E0 and *iters are host pointers (iters may be NULL).  Workspace: three device vectors.
- * In HUB_MODE_AUTO with uniform t and U and no site energies (and t, U in hub_apply's parameter
- * range) the Lanczos vectors are held in 64-bit fixed point, each on a grid of its own
- * 2^-56 of about its largest entry, and the dot products are integer sums.  This does not change
- * E0 at the 1e-10
- * level; HUB_MODE_FP64 keeps every vector in FP64.  Sectors of at most hub_set_small_dim's
+ * *E0 and *iters are host pointers (iters may be NULL).  Workspace: three device vectors and what hub_apply needs.
+ * In HUB_MODE_AUTO with uniform t and U and no site energies (|t| in [2^-500, 2^500], min(N_up,
+ * N_dn) |U/t| up to 2^24) the Lanczos vectors are held in 64-bit fixed point, each on a grid of its
+ * own 2^-56 of about its largest entry, and the dot products are integer sums (workspace: four
+ * device vectors, five where neither spin's rows can be staged; where they do not fit the run
+ * takes FP64 vectors and products).  alpha_j and beta_j are closer to those of exact arithmetic
+ * than with vectors of 48 significant bits; HUB_MODE_FP64 keeps every vector in FP64.  Sectors of at most hub_set_small_dim's
  * bound (default 262144 states; not in a momentum sector) run instead in one cooperative
  * kernel per batch of iterations, FP64 throughout, in either mode: the same recurrence and
  * stopping rule, alpha_j and beta_j equal to the other drivers' up to rounding.
@@ -414,12 +421,11 @@ int hub_k_columns(hub_t h, uint32_t *dn_host, int32_t *sign_host);
 int hub_k_project(hub_t h, const double *x_dev, double *y_dev, void *stream);
 
 /*
- * Arithmetic path (no counterpart in the paper).  HUB_MODE_AUTO (default) runs products
- * with uniform t and U on the fast path: vectors held as pairs of FP32 numbers (about 48
- * significant bits), sums by error-free transformations on the FP32 pipe, because the
- * FP64 unit of this GPU issues about 1/70 of the FP32 rate.  Its per-entry error is at
- * most 6.8e-14 (|H||x|)_n at 4x4 inside the window stated at hub_apply, and inputs outside
- * the window go to the FP64 kernel, so both modes meet 1e-13 (|H||x|)_n.  Inputs and
+ * Arithmetic path (no counterpart in the paper).  HUB_MODE_AUTO (default) runs products and
+ * Lanczos steps with uniform t and U in 64-bit fixed point on the integer pipe, or in pairs of
+ * FP32 numbers (about 48 significant bits) with sums by error-free transformations, because the
+ * FP64 unit of this GPU issues about 1/70 of the integer and FP32 rates.  Which one is chosen,
+ * and the bound that all of them meet, stand at hub_apply and hub_lanczos_ground.  Inputs and
  * outputs of every entry point stay FP64.  HUB_MODE_FP64 forces the native FP64 kernels.
  */
 int hub_set_mode(hub_t h, int mode);
@@ -455,8 +461,8 @@ int hub_last_route(hub_t h, int *route);
  * Test hook (no counterpart in the paper; off by default).  While enabled, every CTA of the
  * fast path's first pass, once the bulk copies of its first row pair have landed, and every
  * CTA of the small-sector Lanczos, before its first grid barrier, takes the exit a given-up
- * bounded wait takes: it sets the handle's device error flag and returns without computing.  No wait runs out and no copy is left in flight; the hook exists so
- * that the error path (hub_check and hub_lanczos_ground returning HUB_ERR_TIMEOUT) can be
+ * bounded wait takes: it sets the handle's device error flag and returns without computing.  No wait runs out
+ * and no copy is left in flight; the hook exists so that the error path (hub_check and hub_lanczos_ground returning HUB_ERR_TIMEOUT) can be
  * exercised.  Results computed while it is enabled are meaningless.
  */
 int hub_test_fail_waits(hub_t h, int enable);
