@@ -16,16 +16,16 @@
 // contribution each, the second with the diagonal; k_fix_out or k_fix_update adds them.
 //
 // Grid.  |X_m| <= 2^B, B = min(56, 62 - hh), 2^hh >= the largest number of hopping terms of an
-// entry, so that no sum overflows.  A rounded entry is off by at most 1/2 of 2^e, 2^-(B+1) of
-// the vector's largest entry.  Y is kept on the grid 2^(e + g), g >= 0 chosen for the diagonal.
+// entry, so that no sum overflows.  A rounded entry is off by at most 1/2 of 2^e: of the
+// vector's largest entry 2^-B in a Lanczos run, 2^-(B-1) in a product.  Y is kept on the grid 2^(e + g), g >= 0 chosen for the diagonal.
 //
 // Lanczos vectors.  The vectors are kept unnormalised and monic, s_{j+1} = H s_j - alpha_j s_j -
 // beta_j^2 s_{j-1} (q_j = s_j / |s_j|, beta_{j+1} = |s_{j+1}| / |s_j|), each on its own grid, so
 // only shifts and two multiplications by a 55-bit coefficient are needed per entry, and the
 // dot products <s_j, H s_j>, <s_j, s_{j-1}> and |s_{j+1}|^2 are integer sums (H s_j rounded to 7 bits
 // fewer, the product of the lowest limbs to their high part, and left out of <s_j, s_{j-1}>): no
-// result depends on the order in which blocks finish.  A rounding is 2^-57 of a vector's largest entry,
-// so that an entry of rms size keeps 53 bits of a random start vector, 46 after sixty steps at 4x4 half
+// result depends on the order in which blocks finish.  A rounding is 2^-56 of a vector's largest entry
+// at most, so that an entry of rms size keeps 53 bits of a random start vector, 46 after sixty steps at 4x4 half
 // filling, 45 to 41 of a 4x4 ground state with an electron added.  Its start vector uses the whole grid
 // (k_fix_plan).  Largest error of alpha over the first steps against long double (12-site ring, 24 steps;
 // in brackets with double-float vectors, which kept 48 bits of every entry): random start 3.7e-15
